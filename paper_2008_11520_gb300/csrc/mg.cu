@@ -72,35 +72,6 @@ template <typename T> __device__ __forceinline__ int patch_mask(const MgLev<T> &
            (fluid(L, 2 * m, 2 * n + 1) ? 4 : 0) | (fluid(L, 2 * m + 1, 2 * n + 1) ? 8 : 0);
 }
 
-// Values and derivatives of (u, v) at the 4 Gauss points of cell (ci, cj).
-template <typename T>
-struct GaussVel {
-    T U[4], V[4], Ux[4], Uy[4], Vx[4], Vy[4];
-    __device__ __forceinline__ void eval(const MgLev<T> &L, const T *u, const T *v, int ci, int cj) {
-        const int nxn = L.nx + 1;
-        T ub[4], vb[4];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int n = (cj + (b >> 1)) * nxn + ci + (b & 1);
-            ub[b] = u[n];
-            vb[b] = v[n];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            U[q] = V[q] = Ux[q] = Uy[q] = Vx[q] = Vy[q] = T(0);
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                U[q] += L.fc.qphi[q][b] * ub[b];
-                V[q] += L.fc.qphi[q][b] * vb[b];
-                Ux[q] += L.fc.qdx[q][b] * ub[b];
-                Uy[q] += L.fc.qdy[q][b] * ub[b];
-                Vx[q] += L.fc.qdx[q][b] * vb[b];
-                Vy[q] += L.fc.qdy[q][b] * vb[b];
-            }
-        }
-    }
-};
-
 template <typename T> __device__ __forceinline__ T inflow(const MgLev<T> &L, int J, double up) {
     const double y = J * L.hy;
     return (T)(up * 4.0 * y * (L.ly - y) / (L.ly * L.ly));
@@ -157,103 +128,142 @@ template <typename T> __device__ __forceinline__ T lps_row(const MgLev<T> &L, co
     return acc;
 }
 
+// Values of (u, v) at the 2 x 2 Gauss points (i along x, j along y) of a cell
+// and their derivatives, in tensor form: a bilinear field's x-derivative
+// depends on j only, its y-derivative on i only.
+template <typename T>
+struct CellVel {
+    T U[2][2], V[2][2], Ux[2], Uy[2], Vx[2], Vy[2];   // [j][i], [j], [i]
+    static __device__ __forceinline__ void field(const FemCoef<T> &fc, const T (&w)[4], T (&W)[2][2], T (&Wx)[2],
+                                                 T (&Wy)[2]) {
+        const T db = w[1] - w[0], dt = w[3] - w[2], dd = dt - db;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const T g = i ? fc.cg1 : fc.cg0;
+            const T b = w[0] + g * db, t = w[2] + g * dt, e = t - b;
+            W[0][i] = b + fc.cg0 * e;
+            W[1][i] = b + fc.cg1 * e;
+            Wy[i] = e * fc.inv_hy;
+            Wx[i] = (db + g * dd) * fc.inv_hx;
+        }
+    }
+    __device__ __forceinline__ void eval(const FemCoef<T> &fc, const T *u, const T *v, int n0, int nxn) {
+        const T ub[4] = {u[n0], u[n0 + 1], u[n0 + nxn], u[n0 + nxn + 1]};
+        const T vb[4] = {v[n0], v[n0 + 1], v[n0 + nxn], v[n0 + nxn + 1]};
+        field(fc, ub, U, Ux, Uy);
+        field(fc, vb, V, Vx, Vy);
+    }
+};
+
 // mode 0: F = A(x) - b on free rows, x - g(t) on fixed rows (the Newton defect).
-// mode 1: b = Rhs(x) (velocity rows; Dirichlet rows and pressure rows 0).
+// mode 1: F = Rhs(x) (velocity rows; Dirichlet rows and pressure rows 0).
+// mode 2: F = J(x) dx, J the Newton matrix of the defect at x (fixed rows: identity).
+//
+// A CTA owns 32 x 4 nodes.  The convection of every cell around them is
+// formed once, in the tensor form of the Gauss rule, and its four corners'
+// sums go through shared memory; each node then adds its four cells' corners
+// to the linear terms.  One thread a node, evaluating its four cells by
+// itself, did every cell four times over (FP64 runs at two FMA a clock and
+// SM): J(x) dx on 256 x 64 cells in FP64 86 -> 23 us, on
+// 1024 x 256 in FP32 20.5 -> 13.9 us (ncu, cold caches).
+constexpr int MR_X = 32, MR_Y = 4, MR_CX = MR_X + 1, MR_CELLS = MR_CX * (MR_Y + 1), MR_THREADS = MR_X * MR_Y;
+
 template <typename T, int MODE>
-__global__ void __launch_bounds__(MG_THREADS) k_mg_defect(MgLev<T> L, const T *__restrict__ x,
-                                                          const T *__restrict__ b, double up, T *__restrict__ F) {
-    const int node = blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= L.N) return;
-    const int nxn = L.nx + 1, I = node % nxn, J = node / nxn;
-    const T *u = x, *v = x + L.N, *p = x + 2 * L.N;
+__global__ void __launch_bounds__(MR_THREADS) k_mg_rows(const __grid_constant__ MgLev<T> L, const T *__restrict__ x,
+                                                        const T *__restrict__ dx, const T *__restrict__ b, double up,
+                                                        T *__restrict__ F) {
+    __shared__ T cc[8][MR_CELLS];   // corner sums of 1/2 convection: u rows of SW, SE, NW, NE, then v rows
+    __shared__ unsigned char cf[MR_CELLS];
+    const FemCoef<T> &fc = L.fc;
+    const int nxn = L.nx + 1, N = L.N;
+    const int nbx = (L.nx + MR_X) / MR_X;
+    const int I0 = (blockIdx.x % nbx) * MR_X, J0 = (blockIdx.x / nbx) * MR_Y;
+    const T g0 = fc.cg0, g1 = fc.cg1, hq = T(0.5) * fc.qw;
+    for (int e = threadIdx.x; e < MR_CELLS; e += MR_THREADS) {
+        const int ey = e / MR_CX, ex = e - ey * MR_CX, ci = I0 - 1 + ex, cj = J0 - 1 + ey;
+        const bool f = fluid(L, ci, cj);
+        cf[e] = f;
+        if (!f) continue;
+        const int n0 = cj * nxn + ci;
+        CellVel<T> g, h;
+        g.eval(fc, x, x + N, n0, nxn);
+        if constexpr (MODE == 2) h.eval(fc, dx, dx + N, n0, nxn);
+        T tu[2][2], tv[2][2];   // [j][corner along x]
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            T cu[2], cv[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                if constexpr (MODE == 2) {
+                    cu[i] = g.U[j][i] * h.Ux[j] + g.V[j][i] * h.Uy[i] + h.U[j][i] * g.Ux[j] + h.V[j][i] * g.Uy[i];
+                    cv[i] = g.U[j][i] * h.Vx[j] + g.V[j][i] * h.Vy[i] + h.U[j][i] * g.Vx[j] + h.V[j][i] * g.Vy[i];
+                } else {
+                    cu[i] = g.U[j][i] * g.Ux[j] + g.V[j][i] * g.Uy[i];
+                    cv[i] = g.U[j][i] * g.Vx[j] + g.V[j][i] * g.Vy[i];
+                }
+            }
+            tu[j][0] = g1 * cu[0] + g0 * cu[1];
+            tu[j][1] = g0 * cu[0] + g1 * cu[1];
+            tv[j][0] = g1 * cv[0] + g0 * cv[1];
+            tv[j][1] = g0 * cv[0] + g1 * cv[1];
+        }
+#pragma unroll
+        for (int ax = 0; ax < 2; ++ax) {
+            cc[ax][e] = hq * (g1 * tu[0][ax] + g0 * tu[1][ax]);
+            cc[2 + ax][e] = hq * (g0 * tu[0][ax] + g1 * tu[1][ax]);
+            cc[4 + ax][e] = hq * (g1 * tv[0][ax] + g0 * tv[1][ax]);
+            cc[6 + ax][e] = hq * (g0 * tv[0][ax] + g1 * tv[1][ax]);
+        }
+    }
+    __syncthreads();
+    const int tx = threadIdx.x % MR_X, ty = threadIdx.x / MR_X, I = I0 + tx, J = J0 + ty;
+    if (I > L.nx || J > L.ny) return;
+    const int node = J * nxn + I;
+    const T *d = MODE == 2 ? dx : x;   // the field of the linear terms
+    const T *u = d, *v = d + N, *p = d + 2 * (size_t)N;
     const uint8_t fl = L.flags[node];
     T Au = T(0), Av = T(0), Ap = T(0);
 #pragma unroll
     for (int cy = 0; cy < 2; ++cy)
 #pragma unroll
         for (int cx = 0; cx < 2; ++cx) {
-            const int ci = I - 1 + cx, cj = J - 1 + cy;
-            if (!fluid(L, ci, cj)) continue;
+            const int e = (ty + cy) * MR_CX + tx + cx;
+            if (!cf[e]) continue;
             const int a = (1 - cx) + 2 * (1 - cy);       // the node's corner in this cell
-            linear_rows(L, u, v, p, ci, cj, a, MODE == 1, Au, Av, Ap);
-            GaussVel<T> gv;
-            gv.eval(L, u, v, ci, cj);
-            T cu = T(0), cv = T(0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const T w = L.fc.qw * L.fc.qphi[q][a];
-                cu += w * (gv.U[q] * gv.Ux[q] + gv.V[q] * gv.Uy[q]);
-                cv += w * (gv.U[q] * gv.Vx[q] + gv.V[q] * gv.Vy[q]);
-            }
-            const T s = MODE == 1 ? T(-0.5) : T(0.5);
-            Au += s * cu;
-            Av += s * cv;
+            linear_rows(L, u, v, p, I - 1 + cx, J - 1 + cy, a, MODE == 1, Au, Av, Ap);
+            Au += MODE == 1 ? -cc[a][e] : cc[a][e];
+            Av += MODE == 1 ? -cc[4 + a][e] : cc[4 + a][e];
         }
     if (MODE == 1) {
         const bool fixed = fl & 1;
         F[node] = fixed ? T(0) : Au;
-        F[L.N + node] = fixed ? T(0) : Av;
-        F[2 * L.N + node] = T(0);
+        F[N + node] = fixed ? T(0) : Av;
+        F[2 * (size_t)N + node] = T(0);
         return;
     }
     Ap += lps_row(L, p, I, J);
+    if (MODE == 2) {
+        F[node] = (fl & 1) ? u[node] : Au;
+        F[N + node] = (fl & 1) ? v[node] : Av;
+        F[2 * (size_t)N + node] = (fl & 4) ? Ap : p[node];
+        return;
+    }
     if (fl & 1) {
         F[node] = u[node] - ((fl & 2) ? inflow(L, J, up) : T(0));
-        F[L.N + node] = v[node];
+        F[N + node] = v[node];
     } else {
         F[node] = Au - b[node];
-        F[L.N + node] = Av - b[L.N + node];
+        F[N + node] = Av - b[N + node];
     }
-    F[2 * L.N + node] = (fl & 4) ? Ap - b[2 * L.N + node] : p[node];
+    F[2 * (size_t)N + node] = (fl & 4) ? Ap - b[2 * (size_t)N + node] : p[node];
 }
 
-// Row (I, J) of J(x) dx, J the Newton matrix of the defect at x (fixed rows: identity).
-template <typename T>
-__device__ __forceinline__ void jvp_rows(const MgLev<T> &L, const T *x, const T *dx, int I, int J, T (&y)[3]) {
-    const int nxn = L.nx + 1, node = J * nxn + I;
-    const T *du = dx, *dv = dx + L.N, *dp = dx + 2 * L.N;
-    const uint8_t fl = L.flags[node];
-    T Au = T(0), Av = T(0), Ap = T(0);
-#pragma unroll
-    for (int cy = 0; cy < 2; ++cy)
-#pragma unroll
-        for (int cx = 0; cx < 2; ++cx) {
-            const int ci = I - 1 + cx, cj = J - 1 + cy;
-            if (!fluid(L, ci, cj)) continue;
-            const int a = (1 - cx) + 2 * (1 - cy);
-            linear_rows(L, du, dv, dp, ci, cj, a, false, Au, Av, Ap);
-            GaussVel<T> g0, g1;   // at x and of the increment
-            g0.eval(L, x, x + L.N, ci, cj);
-            g1.eval(L, du, dv, ci, cj);
-            T cu = T(0), cv = T(0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const T w = L.fc.qw * L.fc.qphi[q][a];
-                cu += w * (g0.U[q] * g1.Ux[q] + g0.V[q] * g1.Uy[q] + g1.U[q] * g0.Ux[q] + g1.V[q] * g0.Uy[q]);
-                cv += w * (g0.U[q] * g1.Vx[q] + g0.V[q] * g1.Vy[q] + g1.U[q] * g0.Vx[q] + g1.V[q] * g0.Vy[q]);
-            }
-            Au += T(0.5) * cu;
-            Av += T(0.5) * cv;
-        }
-    Ap += lps_row(L, dp, I, J);
-    y[0] = (fl & 1) ? du[node] : Au;
-    y[1] = (fl & 1) ? dv[node] : Av;
-    y[2] = (fl & 4) ? Ap : dp[node];
-}
-
-// y = J(x) dx on every node.
-template <typename T>
-__global__ void __launch_bounds__(MG_THREADS) k_mg_jvp(MgLev<T> L, const T *__restrict__ x, const T *__restrict__ dx,
-                                                       T *__restrict__ y) {
-    const int node = blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= L.N) return;
-    const int nxn = L.nx + 1, I = node % nxn, J = node / nxn;
-    T r[3];
-    jvp_rows(L, x, dx, I, J, r);
-    y[node] = r[0];
-    y[L.N + node] = r[1];
-    y[2 * L.N + node] = r[2];
-}
+// Programmatic dependent launch: the colour passes of a sweep are launched
+// so that a pass may start while the one before it drains; what depends on
+// that one comes after the wait (which ends when the pass before has
+// completed and its writes are visible).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // One colour pass of the Vanka smoother for J(x) d = rhs: every fluid cell
 // (ci, cj) with ci = cx (mod 4), cj = cy (mod 4) solves the 12 x 12 block of
@@ -262,152 +272,430 @@ __global__ void __launch_bounds__(MG_THREADS) k_mg_jvp(MgLev<T> L, const T *__re
 // omega times the solution to d.  Cells of one colour
 // are four cells apart: none reads a node another one writes, so the pass is
 // a block Gauss-Seidel step in any order.
+//
+// A pass has few cells (1/16 of the level) and much serial work in each, so a
+// cell is spread over 4 lanes (8 cells a warp): the lanes evaluate the Gauss
+// data of the nine cells around it into shared memory, then lane a holds the
+// three rows of node a in registers, and the lanes eliminate together
+// (Gauss-Jordan; the pivot row comes by shuffle).  One thread a cell, with its
+// 12 x 12 block in local memory, left the chip idle: one sweep of 1024 x 256
+// cells in FP32 took 0.80 ms (now 0.21), of 256 x 64 in FP64 5.7 ms (now
+// 0.245).  16 lanes a cell, one row each, measured 0.65 and 0.6 ms: pivot
+// search and role divergence cost more instructions than the lanes save.
+// What bounds it now: instruction issue on full levels (0.42 of the slots),
+// on small ones the chain of 16 dependent passes (about 5 us each in FP32).
+//
+// Everything is indexed relative to the row's node a: (ex, ey) says whether a
+// cell around the node is in the own cell's column / row (0) or the
+// neighbour's (1); b = (bx, by) is the other node of a pair inside that cell,
+// 0 = the node itself along that direction.  Node a ^ b of the own cell is in
+// cell (ex, ey) iff (bx & ex) == (by & ey) == 0.  Gauss points count from the
+// node (0 near, 1 far).
+constexpr int VK_LANES = 4, VK_THREADS = 32, VK_CELLS = VK_THREADS / VK_LANES;
+constexpr int VK_ROWS = 36 + 7 * 4;
+// AHEAD: the block does not depend on d, so it is assembled and eliminated
+// before the wait for the colour before (the next colours' CTAs do that while
+// this one runs), the multipliers staying in registers and the rows that the
+// defect needs in shared memory; after the wait only the defect and its
+// elimination remain.  It shortens the chain of 16 colours (one sweep,
+// FP64 256 x 64 cells: 535 -> 245 us, 1024 x 256: 2620 -> 2120; FP32
+// 256 x 64: 145 -> 88) but takes 164 registers instead of 109 in FP32, so
+// there colours that fill the chip go without: 768 x 192 cells (9216 a
+// colour) 163 against 179 us, 1024 x 256 (16384) 281 against 212.
+constexpr long long VK_AHEAD_CELLS = 10000;
+constexpr int VK_G = 17;   // shared values per neighbour cell: U 4, V 4, Ux 2, Vx 2, Uy 2, Vy 2 (odd pitch)
+
+// Magnitudes compared as integers: for values without their sign bit the bit
+// patterns order like the values (a NaN above all), and the comparison stays
+// off the FP64 pipe.
+__device__ __forceinline__ int mag_key(float v) { return __float_as_int(v) & 0x7fffffff; }
+__device__ __forceinline__ long long mag_key(double v) { return __double_as_longlong(v) & 0x7fffffffffffffffll; }
+__device__ __forceinline__ float key_mag(int k) { return __int_as_float(k); }
+__device__ __forceinline__ double key_mag(long long k) { return __longlong_as_double(k); }
+
+// The element operator of one cell around a node, row by row: products of
+// 1D factors of the Gauss rule (2 x 2 points, weights folded into hq).
 template <typename T>
-__global__ void __launch_bounds__(128) k_mg_vanka(MgLev<T> L, const T *__restrict__ x, const T *__restrict__ rhs,
-                                                  T *__restrict__ dx, T omega, int cx, int cy) {
+struct RowCell {
+    T X[2], Y[2];            // (v.grad phi_b, phi_a) / 2, the x and y parts, by (by, bx)
+    T jx[2], jv[2];          // (d_x u phi_b, phi_a), (d_x v ...) / 2: factor along y, by by
+    T iy[2], iv[2];          // (d_y u phi_b, phi_a), (d_y v ...) / 2: factor along x, by bx
+    T sx, sy;                // side of the node in the cell: +1 at its right / upper edge
+    __device__ __forceinline__ void set(const FemCoef<T> &fc, const T *q, int cax, int cay) {
+        const T g0 = fc.cg0, g1 = fc.cg1, hq = T(0.5) * fc.qw;
+        const T w11 = g1 * g1, w00 = g0 * g0, w01 = g0 * g1;
+        side(cax, cay);
+        T PU[2], PV[2];
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const int jn = n ^ cay, in = n ^ cax;
+            PU[n] = g1 * q[2 * jn + cax] + g0 * q[2 * jn + 1 - cax];
+            PV[n] = g1 * q[4 + 2 * cay + in] + g0 * q[4 + 2 * (1 - cay) + in];
+        }
+        const T cxh = sx * (hq * fc.inv_hx), cyh = sy * (hq * fc.inv_hy);
+        X[0] = cxh * (w11 * PU[0] + w00 * PU[1]);
+        X[1] = cxh * (w01 * (PU[0] + PU[1]));
+        Y[0] = cyh * (w11 * PV[0] + w00 * PV[1]);
+        Y[1] = cyh * (w01 * (PV[0] + PV[1]));
+        auto pair = [&](const T *d, int near, T (&o)[2]) {
+            const T n = hq * d[near], f = hq * d[1 - near];
+            o[0] = w11 * n + w00 * f;
+            o[1] = w01 * (n + f);
+        };
+        pair(q + 8, cay, jx);
+        pair(q + 10, cay, jv);
+        pair(q + 12, cax, iy);
+        pair(q + 14, cax, iv);
+    }
+    __device__ __forceinline__ void side(int cax, int cay) {
+        sx = cax ? T(1) : T(-1);
+        sy = cay ? T(1) : T(-1);
+    }
+    // entries of rows (u, v, p) of node a against (u, v, p) of node b: the
+    // velocity block, and those that do not depend on x
+    __device__ __forceinline__ void velocity(const FemCoef<T> &fc, int bx, int by, T &uu, T &uv, T &vu, T &vv) const {
+        const T g0 = fc.cg0, g1 = fc.cg1, m0 = g1 * g1 + g0 * g0, m1 = T(2) * (g0 * g1);
+        const T mx = bx ? m1 : m0, my = by ? m1 : m0;
+        const T nl = (bx ? -X[by] : X[by]) + (by ? -Y[bx] : Y[bx]) + fc.Av[0][bx + 2 * by];
+        uu = nl + mx * jx[by];
+        uv = my * iy[bx];
+        vu = mx * jv[by];
+        vv = nl + my * iv[bx];
+    }
+    __device__ __forceinline__ void constants(const FemCoef<T> &fc, int bx, int by, T &up, T &vp, T &pu, T &pv) const {
+        const T gx = sx * fc.Gx[1][1 + 2 * by], gy = sy * fc.Gy[2][2 + bx];
+        up = -gx;
+        vp = -gy;
+        pu = bx ? -gx : gx;
+        pv = by ? -gy : gy;
+    }
+};
+
+template <typename T, bool AHEAD>
+__global__ void __launch_bounds__(VK_THREADS) k_mg_vanka(const __grid_constant__ MgLev<T> L, const T *__restrict__ x,
+                                                         const T *__restrict__ rhs, T *dx, T omega, int cx, int cy) {
+    __shared__ T sm[VK_CELLS][9 * VK_G];
+    // AHEAD: this lane's rows of J, the own cell's columns, then the others
+    __shared__ T rows[AHEAD ? VK_ROWS : 1][VK_THREADS];
+    constexpr unsigned FULL = 0xffffffffu;
+    if constexpr (AHEAD) pdl_trigger();   // the next colour may start on what does not depend on d
+    const FemCoef<T> &fc = L.fc;
     const int nx4 = (L.nx - cx + 3) / 4, ny4 = (L.ny - cy + 3) / 4;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nx4 * ny4) return;
-    const int cj = cy + 4 * (k / nx4), ci = cx + 4 * (k % nx4);
-    const int cell = cj * L.nx + ci;
-    if (L.solid[cell]) return;
-    const int nxn = L.nx + 1;
-    T A[12][12];
+    const int lane = threadIdx.x, a = lane & 3, slot = lane / VK_LANES;
+    const int id = blockIdx.x * VK_CELLS + slot;
+    bool live = id < nx4 * ny4;
+    const int cj = live ? cy + 4 * (id / nx4) : cy, ci = live ? cx + 4 * (id % nx4) : cx;
+    live = live && !L.solid[(size_t)cj * L.nx + ci];
+    const int nxn = L.nx + 1, N = L.N;
+    T *gs = sm[slot];
+    // ---- Gauss data of the nine cells at x, cell 3 (dj + 1) + di + 1 by lane (that mod 4)
+    unsigned fmask = 0;
 #pragma unroll
-    for (int i = 0; i < 12; ++i)
+    for (int r = 0; r < 3; ++r) {
+        const int c9 = 4 * r + a, di = c9 % 3 - 1, dj = c9 / 3 - 1;
+        const bool f = live && c9 < 9 && fluid(L, ci + di, cj + dj);
+        if (f) {
+            CellVel<T> g;
+            g.eval(fc, x, x + N, (cj + dj) * nxn + ci + di, nxn);
+            T *o = gs + c9 * VK_G;
 #pragma unroll
-        for (int j = 0; j < 12; ++j) A[i][j] = T(0);
-    // element contributions of the cells that share a node with this one
-    for (int dj = -1; dj <= 1; ++dj)
-        for (int di = -1; di <= 1; ++di) {
-            const int ck = ci + di, cl = cj + dj;
-            if (!fluid(L, ck, cl)) continue;
-            GaussVel<T> g;
-            g.eval(L, x, x + L.N, ck, cl);
-            for (int a = 0; a < 4; ++a) {
-                const int la = di + (a & 1), lb_a = dj + (a >> 1);   // offset of test node a from (ci, cj)
-                if (la < 0 || la > 1 || lb_a < 0 || lb_a > 1) continue;
-                const int ra = 3 * (la + 2 * lb_a);
-                for (int b = 0; b < 4; ++b) {
-                    const int ka = di + (b & 1), kb = dj + (b >> 1);
-                    if (ka < 0 || ka > 1 || kb < 0 || kb > 1) continue;
-                    const int cb = 3 * (ka + 2 * kb);
-                    T nl = T(0), ruu = T(0), ruv = T(0), rvu = T(0), rvv = T(0);
+            for (int j = 0; j < 2; ++j) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const T w = L.fc.qw * L.fc.qphi[q][a];
-                        nl += w * (g.U[q] * L.fc.qdx[q][b] + g.V[q] * L.fc.qdy[q][b]);
-                        const T wb = w * L.fc.qphi[q][b];
-                        ruu += wb * g.Ux[q];
-                        ruv += wb * g.Uy[q];
-                        rvu += wb * g.Vx[q];
-                        rvv += wb * g.Vy[q];
+                for (int i = 0; i < 2; ++i) {
+                    o[2 * j + i] = g.U[j][i];
+                    o[4 + 2 * j + i] = g.V[j][i];
+                }
+                o[8 + j] = g.Ux[j];
+                o[10 + j] = g.Vx[j];
+                o[12 + j] = g.Uy[j];
+                o[14 + j] = g.Vy[j];
+            }
+        }
+        fmask |= ((__ballot_sync(FULL, f) >> (lane & 28)) & 15u) << (4 * r);
+    }
+    __syncwarp();
+    // ---- rows of node a: columns 3 b + component, b relative to the node
+    const int ax = a & 1, ay = a >> 1;
+    const int I = ci + ax, J = cj + ay, node = J * nxn + I;
+    const int dcx = ax ? -1 : 1, dcy = ay ? -1 : 1;   // towards the own cell's other node
+    const uint8_t fl = live ? L.flags[node] : 1;      // (a dead slot solves the identity)
+    T R[3][12];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int i = 0; i < 12; ++i) R[c][i] = T(0);
+    bool has[4];   // cell (ex, ey) is fluid
+    {
+        int o = 36;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int ex = e & 1, ey = e >> 1;
+            const int c9 = 3 * ((ey ? -dcy : 0) + 1) + (ex ? -dcx : 0) + 1;
+            has[e] = (fmask >> c9) & 1;
+            RowCell<T> rc;
+            if (has[e]) rc.set(fc, gs + c9 * VK_G, ex ? 1 - ax : ax, ey ? 1 - ay : ay);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int bx = b & 1, by = b >> 1;
+                const bool outer = (bx & ex) || (by & ey);
+                if (has[e]) {
+                    T uu, uv, up, vu, vv, vp, pu, pv;
+                    rc.velocity(fc, bx, by, uu, uv, vu, vv);
+                    rc.constants(fc, bx, by, up, vp, pu, pv);
+                    if (outer && AHEAD) {
+                        // kept for the defect (the constant entries are formed again there)
+                        rows[o][lane] = uu;
+                        rows[o + 1][lane] = uv;
+                        rows[o + 2][lane] = vu;
+                        rows[o + 3][lane] = vv;
+                    } else if (!outer) {
+                        R[0][3 * b] += uu;
+                        R[0][3 * b + 1] += uv;
+                        R[0][3 * b + 2] += up;
+                        R[1][3 * b] += vu;
+                        R[1][3 * b + 1] += vv;
+                        R[1][3 * b + 2] += vp;
+                        R[2][3 * b] += pu;
+                        R[2][3 * b + 1] += pv;
                     }
-                    A[ra][cb] += L.fc.Av[a][b] + T(0.5) * (nl + ruu);
-                    A[ra][cb + 1] += T(0.5) * ruv;
-                    A[ra + 1][cb] += T(0.5) * rvu;
-                    A[ra + 1][cb + 1] += L.fc.Av[a][b] + T(0.5) * (nl + rvv);
-                    A[ra][cb + 2] -= L.fc.Gx[a][b];
-                    A[ra + 1][cb + 2] -= L.fc.Gy[a][b];
-                    A[ra + 2][cb] += L.fc.Dx[a][b];
-                    A[ra + 2][cb + 1] += L.fc.Dy[a][b];
                 }
-            }
-        }
-    // projection term: patches that hold both nodes of a pair
-    int gI[4], gJ[4], gn[4];
-    for (int a = 0; a < 4; ++a) {
-        gI[a] = ci + (a & 1);
-        gJ[a] = cj + (a >> 1);
-        gn[a] = gJ[a] * nxn + gI[a];
-    }
-    for (int m = (ci - 1) >> 1; m <= (ci + 1) >> 1; ++m)
-        for (int n = (cj - 1) >> 1; n <= (cj + 1) >> 1; ++n) {
-            const int pm_ = patch_mask(L, m, n);
-            if (!pm_) continue;
-            const T *S = L.lps + pm_ * 81;
-            for (int a = 0; a < 4; ++a) {
-                const int ia = gI[a] - 2 * m, ja = gJ[a] - 2 * n;
-                if (ia < 0 || ia > 2 || ja < 0 || ja > 2) continue;
-                for (int b = 0; b < 4; ++b) {
-                    const int ib = gI[b] - 2 * m, jb = gJ[b] - 2 * n;
-                    if (ib < 0 || ib > 2 || jb < 0 || jb > 2) continue;
-                    A[3 * a + 2][3 * b + 2] += S[(3 * ja + ia) * 9 + 3 * jb + ib];
-                }
-            }
-        }
-    // right-hand side: the defect rhs - J(x) d on the cell's unknowns.  Rows of
-    // fixed unknowns are identity rows of J, so their correction is exactly
-    // their defect (the first cell that holds one sets it, later ones add 0).
-    T z[12];
-    for (int a = 0; a < 4; ++a) {
-        const uint8_t fl = L.flags[gn[a]];
-        T jd[3];
-        jvp_rows(L, x, dx, gI[a], gJ[a], jd);
-        for (int c = 0; c < 3; ++c) {
-            const int i = 3 * a + c;
-            const bool fixed = c < 2 ? (fl & 1) : !(fl & 4);
-            z[i] = rhs[c * L.N + gn[a]] - jd[c];
-            if (fixed) {
-                for (int j = 0; j < 12; ++j) A[i][j] = T(0);
-                A[i][i] = T(1);
+                if (outer && AHEAD) o += 4;
             }
         }
     }
-    // Gaussian elimination with partial pivoting.  A block can be singular: a
-    // cell whose 4 nodes all hold Dirichlet velocities couples its pressures
-    // only through the projection term, which vanishes on linear functions.
-    // A pivot below a relative threshold leaves that unknown's correction 0.
-    T scale = T(0);
-    for (int i = 0; i < 12; ++i)
-        for (int j = 0; j < 12; ++j) scale = fmax(scale, fabs(A[i][j]));
-    const T tiny = scale * (sizeof(T) == 8 ? T(1e-12) : T(1e-6));
+    if constexpr (AHEAD) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int i = 0; i < 12; ++i) rows[12 * c + i][lane] = R[c][i];
+    }
+    // projection term of the node's pressure row: its entries in the own cell
+    // (lp), and where its (up to four) patches' rows are
+    T lp[4] = {T(0), T(0), T(0), T(0)};
+    const T *Sp[4];
+    int pbase[4];   // first node of the patch, -1: no such patch
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int qx = q & 1, qy = q >> 1;
+        const int m = (I - qx) >> 1, n = (J - qy) >> 1;   // 2m <= I <= 2m + 2, 2n <= J <= 2n + 2
+        int mask = 0;
+        if (live && !(qx && (I & 1)) && !(qy && (J & 1))) mask = patch_mask(L, m, n);
+        const int il = I - 2 * m, jl = J - 2 * n;
+        pbase[q] = mask ? 2 * n * nxn + 2 * m : -1;
+        Sp[q] = L.lps + (mask ? (mask * 9 + 3 * jl + il) * 9 : 0);
+        if (mask) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int ib = il + ((b & 1) ? dcx : 0), jb = jl + ((b >> 1) ? dcy : 0);
+                if (ib >= 0 && ib <= 2 && jb >= 0 && jb <= 2) lp[b] += Sp[q][3 * jb + ib];
+            }
+        }
+    }
+    // ---- the defect rhs - J(x) d on the node's unknowns (everything that
+    // depends on d, which the pass before wrote)
+    T z[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) z[c] = live ? rhs[(size_t)c * N + node] : T(0);
+    auto defect = [&]() {
+        if constexpr (!AHEAD) pdl_trigger();
+        pdl_wait();
+        if (!live) return;
+        const T *du = dx, *dv = dx + N, *dp = dx + 2 * (size_t)N;
+        const T own[3] = {du[node], dv[node], dp[node]};
+        T jd[3] = {T(0), T(0), T(0)};
+        // the own cell's nodes
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int n = node + ((b & 1) ? dcx : 0) + ((b >> 1) ? dcy * nxn : 0);
+            const T d0 = du[n], d1 = dv[n], d2 = dp[n];
+            auto at = [&](int c, int i) { return AHEAD ? rows[AHEAD ? 12 * c + i : 0][lane] : R[c][i]; };
+#pragma unroll
+            for (int c = 0; c < 3; ++c) jd[c] += at(c, 3 * b) * d0 + at(c, 3 * b + 1) * d1 + at(c, 3 * b + 2) * d2;
+        }
+        // the other nodes of the cells around the node
+        int o = 36;
+#pragma unroll
+        for (int e = 1; e < 4; ++e) {
+            const int ex = e & 1, ey = e >> 1;
+            if (!has[e]) {
+                o += ex && ey ? 12 : 8;
+                continue;
+            }
+            RowCell<T> rc;
+            if constexpr (AHEAD) rc.side(ex ? 1 - ax : ax, ey ? 1 - ay : ay);
+            else rc.set(fc, gs + (3 * ((ey ? -dcy : 0) + 1) + (ex ? -dcx : 0) + 1) * VK_G, ex ? 1 - ax : ax, ey ? 1 - ay : ay);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int bx = b & 1, by = b >> 1;
+                if (!((bx & ex) || (by & ey))) continue;
+                const int n = node + (bx ? (ex ? -dcx : dcx) : 0) + (by ? (ey ? -dcy : dcy) * nxn : 0);
+                const T d0 = du[n], d1 = dv[n], d2 = dp[n];
+                T uu, uv, up, vu, vv, vp, pu, pv;
+                rc.constants(fc, bx, by, up, vp, pu, pv);
+                if constexpr (AHEAD) {
+                    uu = rows[o][lane];
+                    uv = rows[o + 1][lane];
+                    vu = rows[o + 2][lane];
+                    vv = rows[o + 3][lane];
+                    o += 4;
+                } else {
+                    rc.velocity(fc, bx, by, uu, uv, vu, vv);
+                }
+                jd[0] += uu * d0 + uv * d1 + up * d2;
+                jd[1] += vu * d0 + vv * d1 + vp * d2;
+                jd[2] += pu * d0 + pv * d1;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (pbase[q] < 0) continue;
+            const T *pp = dp + pbase[q];
+#pragma unroll
+            for (int kb = 0; kb < 3; ++kb)
+#pragma unroll
+                for (int ka = 0; ka < 3; ++ka) jd[2] += Sp[q][3 * kb + ka] * pp[kb * nxn + ka];
+        }
+        z[0] -= (fl & 1) ? own[0] : jd[0];
+        z[1] -= (fl & 1) ? own[1] : jd[1];
+        z[2] -= (fl & 4) ? jd[2] : own[2];
+    };
+    if constexpr (!AHEAD) defect();
+#pragma unroll
+    for (int b = 0; b < 4; ++b) R[2][3 * b + 2] += lp[b];
+    // rows of fixed unknowns: identity; columns by absolute node, b ^ a
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const bool fixed = c < 2 ? (fl & 1) : !(fl & 4);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) R[c][i] = fixed ? (i == c ? T(1) : T(0)) : R[c][i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            if (ax) {
+                const T t0 = R[c][i], t1 = R[c][6 + i];
+                R[c][i] = R[c][3 + i];
+                R[c][3 + i] = t0;
+                R[c][6 + i] = R[c][9 + i];
+                R[c][9 + i] = t1;
+            }
+            if (ay) {
+                const T t0 = R[c][i], t1 = R[c][3 + i];
+                R[c][i] = R[c][6 + i];
+                R[c][6 + i] = t0;
+                R[c][3 + i] = R[c][9 + i];
+                R[c][9 + i] = t1;
+            }
+        }
+    }
+    // ---- Gauss-Jordan elimination with partial pivoting over the 12 rows; the
+    // multipliers stay in the eliminated columns.  A
+    // block can be singular: a cell whose 4 nodes all hold Dirichlet velocities
+    // couples its pressures only through the projection term, which vanishes
+    // on linear functions.  A pivot below a relative threshold leaves that
+    // unknown's correction 0 and drops its row.  pos is a row's place under
+    // the exchanges (ties go to the first row); unk the unknown it became.
+    using Key = decltype(mag_key(T(0)));
+    Key scale = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int i = 0; i < 12; ++i) scale = max(scale, mag_key(R[c][i]));
+    scale = max(scale, __shfl_xor_sync(FULL, scale, 1));
+    scale = max(scale, __shfl_xor_sync(FULL, scale, 2));
+    const T tiny = key_mag(scale) * (sizeof(T) == 8 ? T(1e-12) : T(1e-6));
+    int pos[3] = {3 * a, 3 * a + 1, 3 * a + 2}, unk[3] = {-1, -1, -1};
+    T dinv[3] = {T(0), T(0), T(0)};
+    unsigned long long prows = 0;   // pivot row of each column, 4 bits
+    unsigned deads = 0;
+#pragma unroll
     for (int k = 0; k < 12; ++k) {
-        int piv = k;
-        T best = fabs(A[k][k]);
-        for (int i = k + 1; i < 12; ++i)
-            if (fabs(A[i][k]) > best) {
-                best = fabs(A[i][k]);
-                piv = i;
+        // the largest |entry| of column k among the rows not used yet, as (value, place, row);
+        // a NaN is the largest key, so every lane agrees on it and it spreads to the whole block
+        Key best = -1;
+        int idx = 0xffff;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const Key v = unk[c] >= 0 ? Key(-1) : mag_key(R[c][k]);
+            const int iv = (pos[c] << 4) | (3 * a + c);
+            if (v > best || (v == best && iv < idx)) {
+                best = v;
+                idx = iv;
             }
-        if (piv != k) {
-            for (int j = 0; j < 12; ++j) {
-                const T tmp = A[k][j];
-                A[k][j] = A[piv][j];
-                A[piv][j] = tmp;
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            const Key ov = __shfl_xor_sync(FULL, best, o);
+            const int oi = __shfl_xor_sync(FULL, idx, o);
+            if (ov > best || (ov == best && oi < idx)) {
+                best = ov;
+                idx = oi;
             }
-            const T tz = z[k];
-            z[k] = z[piv];
-            z[piv] = tz;
         }
-        if (best <= tiny) {
-            A[k][k] = T(1);
-            for (int j = k + 1; j < 12; ++j) A[k][j] = T(0);
-            z[k] = T(0);
-            continue;
+        const int prow = idx & 15, ppos = idx >> 4, pl = prow / 3, pc = prow - 3 * pl;
+        const bool dead = key_mag(best) <= tiny;
+        prows |= (unsigned long long)prow << (4 * k);
+        deads |= (dead ? 1u : 0u) << k;
+        // the pivot row, from lane pl of the cell
+        T pv[12];
+#pragma unroll
+        for (int j = k; j < 12; ++j) {
+            const T v = pc == 0 ? R[0][j] : (pc == 1 ? R[1][j] : R[2][j]);
+            pv[j] = __shfl_sync(FULL, v, pl, 4);
         }
-        const T inv = T(1) / A[k][k];
-        for (int i = k + 1; i < 12; ++i) {
-            const T f = A[i][k] * inv;
-            if (f == T(0)) continue;
-            for (int j = k; j < 12; ++j) A[i][j] -= f * A[k][j];
-            z[i] -= f * z[k];
+        T pz = T(0);
+        if constexpr (!AHEAD) pz = __shfl_sync(FULL, pc == 0 ? z[0] : (pc == 1 ? z[1] : z[2]), pl, 4);
+        const T inv = dead ? T(0) : T(1) / pv[k];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const bool piv = prow == 3 * a + c;
+            const T f = piv ? T(0) : R[c][k] * inv;
+            R[c][k] = f;
+#pragma unroll
+            for (int j = k + 1; j < 12; ++j) R[c][j] -= f * pv[j];
+            if constexpr (!AHEAD) z[c] -= f * pz;
+            if (pos[c] == k) pos[c] = ppos;
+            if (piv) {
+                pos[c] = k;
+                unk[c] = k;
+                dinv[c] = inv;
+                if (dead) {
+                    if constexpr (!AHEAD) z[c] = T(0);
+#pragma unroll
+                    for (int j = k + 1; j < 12; ++j) R[c][j] = T(0);
+                }
+            }
         }
     }
-    for (int k = 11; k >= 0; --k) {
-        T s = z[k];
-        for (int j = k + 1; j < 12; ++j) s -= A[k][j] * z[j];
-        z[k] = s / A[k][k];
+    if constexpr (AHEAD) {
+        // the elimination of the right-hand side
+        defect();
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const int prow = (int)(prows >> (4 * k)) & 15, pl = prow / 3, pc = prow - 3 * pl;
+            const T pz = __shfl_sync(FULL, pc == 0 ? z[0] : (pc == 1 ? z[1] : z[2]), pl, 4);
+            const bool dead = (deads >> k) & 1;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                z[c] -= R[c][k] * pz;
+                if (dead && prow == 3 * a + c) z[c] = T(0);
+            }
+        }
     }
-    for (int a = 0; a < 4; ++a)
-        for (int c = 0; c < 3; ++c) dx[c * L.N + gn[a]] += omega * z[3 * a + c];
+    if (live) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (unk[c] < 0) continue;
+            const int ua = unk[c] / 3, uc = unk[c] - 3 * ua;
+            dx[(size_t)uc * N + (cj + (ua >> 1)) * nxn + ci + (ua & 1)] += omega * (z[c] * dinv[c]);
+        }
+    }
 }
 
 // End of a Vanka sweep: every fixed unknown (an identity row of J) takes its
 // exact correction, its defect: d = rhs there.  This also reaches the nodes
 // that no fluid cell holds (inside an obstacle), which no cell block visits.
 template <typename T>
-__global__ void __launch_bounds__(MG_THREADS) k_mg_fixed(MgLev<T> L, const T *__restrict__ rhs, T *__restrict__ dx) {
+__global__ void __launch_bounds__(MG_THREADS) k_mg_fixed(MgLev<T> L, const T *__restrict__ rhs, T *dx) {
+    pdl_wait();   // the last colour pass of the sweep
     const int node = blockIdx.x * blockDim.x + threadIdx.x;
     if (node >= L.N) return;
     const uint8_t fl = L.flags[node];
@@ -578,6 +866,9 @@ int check_level(const dnnmg_mg_s *m, int level, int need_coarser = 0) {
 }
 
 unsigned blocks(long long n, int th) { return (unsigned)((n + th - 1) / th); }
+unsigned rows_grid(const dnnmg_mg_s *m, int l) {
+    return blocks(m->levels[l].nx + 1, MR_X) * blocks(m->levels[l].ny + 1, MR_Y);
+}
 
 // Projection patch matrices by the patch's fluid cells: for each subset (bit
 // 2 cb + ca), the sum over its cells T of alpha (grad(p - pi p), grad(q - pi q))_T
@@ -624,6 +915,36 @@ void lps_tables(const FemCoef<double> &f, double hx, double hy, double alpha0, d
         for (int c = 0; c < 4; ++c)
             if (mask & (1 << c))
                 for (int i = 0; i < 81; ++i) (*out)[mask * 81 + i] += (&Lc[c][0][0])[i];
+}
+
+// One sweep: the 16 colour passes and the fixed unknowns.  Each pass may start
+// while the one before it drains (programmatic launch), except the first,
+// whose inputs the work before the sweep may still be writing.
+template <typename T>
+cudaError_t vanka_sweep(const dnnmg_mg_s &m, int level, const T *x, const T *r, T *dx, T omega, cudaStream_t st) {
+    const MgLev<T> L = dev_level<T>(m, level);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cudaError_t e;
+    for (int c = 0; c < 16; ++c) {
+        const int cx = c & 3, cy = c >> 2;
+        const long long nc = (long long)((L.nx - cx + 3) / 4) * ((L.ny - cy + 3) / 4);
+        if (nc <= 0) continue;
+        cfg.gridDim = dim3(blocks(nc, VK_CELLS));
+        cfg.blockDim = dim3(VK_THREADS);
+        auto k = k_mg_vanka<T, true>;
+        if constexpr (sizeof(T) == 4)
+            if (nc > VK_AHEAD_CELLS) k = k_mg_vanka<T, false>;
+        if ((e = cudaLaunchKernelEx(&cfg, k, L, x, r, dx, omega, cx, cy)) != cudaSuccess) return e;
+        cfg.numAttrs = 1;
+    }
+    cfg.gridDim = dim3(blocks(L.N, MG_THREADS));
+    cfg.blockDim = dim3(MG_THREADS);
+    return cudaLaunchKernelEx(&cfg, k_mg_fixed<T>, L, r, dx);
 }
 
 }  // namespace
@@ -747,12 +1068,11 @@ int dnnmg_mg_defect(dnnmg_mg_t m, int level, const void *x, const void *b, doubl
     clear_error();
     if (int e = check_level(m, level)) return e;
     if (!x || !b || !F) return fail(DNNMG_EINVAL, "NULL array");
-    const int N = m->levels[level].N;
     const double up = inflow_peak_mg(m->desc, t);
-    MG_DISPATCH((k_mg_defect<double, 0><<<blocks(N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<double>(*m, level), (const double *)x, (const double *)b, up, (double *)F)),
-                (k_mg_defect<float, 0><<<blocks(N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<float>(*m, level), (const float *)x, (const float *)b, up, (float *)F)));
+    MG_DISPATCH((k_mg_rows<double, 0><<<rows_grid(m, level), MR_THREADS, 0, s>>>(
+                    dev_level<double>(*m, level), (const double *)x, nullptr, (const double *)b, up, (double *)F)),
+                (k_mg_rows<float, 0><<<rows_grid(m, level), MR_THREADS, 0, s>>>(
+                    dev_level<float>(*m, level), (const float *)x, nullptr, (const float *)b, up, (float *)F)));
     return DNNMG_OK;
 }
 
@@ -761,11 +1081,10 @@ int dnnmg_mg_rhs(dnnmg_mg_t m, int level, const void *x, void *b, cudaStream_t s
     if (int e = check_level(m, level)) return e;
     if (!x || !b) return fail(DNNMG_EINVAL, "NULL array");
     if (x == b) return fail(DNNMG_EINVAL, "x and b must not alias");
-    const int N = m->levels[level].N;
-    MG_DISPATCH((k_mg_defect<double, 1><<<blocks(N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<double>(*m, level), (const double *)x, nullptr, 0.0, (double *)b)),
-                (k_mg_defect<float, 1><<<blocks(N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<float>(*m, level), (const float *)x, nullptr, 0.0, (float *)b)));
+    MG_DISPATCH((k_mg_rows<double, 1><<<rows_grid(m, level), MR_THREADS, 0, s>>>(
+                    dev_level<double>(*m, level), (const double *)x, nullptr, nullptr, 0.0, (double *)b)),
+                (k_mg_rows<float, 1><<<rows_grid(m, level), MR_THREADS, 0, s>>>(
+                    dev_level<float>(*m, level), (const float *)x, nullptr, nullptr, 0.0, (float *)b)));
     return DNNMG_OK;
 }
 
@@ -774,11 +1093,10 @@ int dnnmg_mg_jvp(dnnmg_mg_t m, int level, const void *x, const void *dx, void *y
     if (int e = check_level(m, level)) return e;
     if (!x || !dx || !y) return fail(DNNMG_EINVAL, "NULL array");
     if (y == dx || y == x) return fail(DNNMG_EINVAL, "y must not alias x or dx");
-    const int N = m->levels[level].N;
-    MG_DISPATCH((k_mg_jvp<double><<<blocks(N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<double>(*m, level), (const double *)x, (const double *)dx, (double *)y)),
-                (k_mg_jvp<float><<<blocks(N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<float>(*m, level), (const float *)x, (const float *)dx, (float *)y)));
+    MG_DISPATCH((k_mg_rows<double, 2><<<rows_grid(m, level), MR_THREADS, 0, s>>>(
+                    dev_level<double>(*m, level), (const double *)x, (const double *)dx, nullptr, 0.0, (double *)y)),
+                (k_mg_rows<float, 2><<<rows_grid(m, level), MR_THREADS, 0, s>>>(
+                    dev_level<float>(*m, level), (const float *)x, (const float *)dx, nullptr, 0.0, (float *)y)));
     return DNNMG_OK;
 }
 
@@ -787,19 +1105,9 @@ int dnnmg_mg_vanka(dnnmg_mg_t m, int level, const void *x, const void *r, void *
     if (int e = check_level(m, level)) return e;
     if (!x || !r || !dx) return fail(DNNMG_EINVAL, "NULL array");
     if (dx == r || dx == x) return fail(DNNMG_EINVAL, "dx must not alias x or r");
-    const MgLevelHost &h = m->levels[level];
-    const long long nc = (long long)((h.nx + 3) / 4) * ((h.ny + 3) / 4);
-    for (int cy = 0; cy < 4; ++cy)
-        for (int cx = 0; cx < 4; ++cx)
-            MG_DISPATCH((k_mg_vanka<double><<<blocks(nc, 128), 128, 0, s>>>(
-                            dev_level<double>(*m, level), (const double *)x, (const double *)r, (double *)dx, omega, cx, cy)),
-                        (k_mg_vanka<float><<<blocks(nc, 128), 128, 0, s>>>(
-                            dev_level<float>(*m, level), (const float *)x, (const float *)r, (float *)dx, (float)omega,
-                            cx, cy)));
-    MG_DISPATCH((k_mg_fixed<double><<<blocks(h.N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<double>(*m, level), (const double *)r, (double *)dx)),
-                (k_mg_fixed<float><<<blocks(h.N, MG_THREADS), MG_THREADS, 0, s>>>(
-                    dev_level<float>(*m, level), (const float *)r, (float *)dx)));
+    DNNMG_CUDA_TRY(m->desc.precision == DNNMG_F64
+                       ? vanka_sweep(*m, level, (const double *)x, (const double *)r, (double *)dx, omega, s)
+                       : vanka_sweep(*m, level, (const float *)x, (const float *)r, (float *)dx, (float)omega, s));
     return DNNMG_OK;
 }
 
