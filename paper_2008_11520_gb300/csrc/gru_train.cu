@@ -18,6 +18,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "gru_win.cuh"
 
 namespace dnnmg {
 namespace {
@@ -345,6 +346,8 @@ struct dnnmg_trainer_s {
     // BF16 products (dnnmg_trainer_set_precision)
     int bf16;
     int *d_status;
+    float *wpart;   // the fused window's partial weight gradients; null: one kernel per product
+    int tiled;      // the saved activations are in the fused window's layout (h_0 .. h_{T-1} in rh)
     // BF16 copies, each tensor rounded once (offsets into arena, in elements;
     // row strides kx = kpad(n_in), kh = kpad(H), k2 = kpad(2H), ko = kpad(n_out),
     // kt = kpad(T P), ks = kpad((T+1) P))
@@ -490,6 +493,64 @@ cudaError_t seq_backward_bf16(dnnmg_trainer_s *t, const float *dD, const float *
     return cudaSuccess;
 }
 
+// [T][P][H] rows to the fused window's tiles (rows past P zero) or back.
+__global__ void k_relayout(int T, int P, int ntiles, int H, const float *__restrict__ src, float *__restrict__ dst,
+                           int to_tiles) {
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // element of the tiled array
+    const long long n = (long long)T * ntiles * 128 * H;
+    if (e >= n) return;
+    const int blk = 128 * H;
+    const long long st = e / blk;
+    const int in = (int)(e - st * blk), s = (int)(st / ntiles), tile = (int)(st - (long long)s * ntiles);
+    const int row = (in / 4) % 128, c = in / 512 * 4 + in % 4, p = tile * 128 + row;
+    const long long r = ((long long)s * P + p) * H + c;
+    if (to_tiles) dst[e] = p < P ? src[r] : 0.0f;
+    else if (p < P) dst[r] = src[e];
+}
+__global__ void k_mul(long long n, const float *__restrict__ a, const float *__restrict__ b, float *__restrict__ c) {
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) c[e] = a[e] * b[e];
+}
+
+// The saved activations in the layout the backward about to run reads: only
+// where the precision was changed between a window's forward and backward
+// does that differ from the one its forward wrote.
+cudaError_t want_layout(dnnmg_trainer_s *t, int tiled, cudaStream_t st) {
+    if (t->tiled == tiled) return cudaSuccess;
+    const int nt = win_tiles(t->P), H = t->H;
+    const long long nb = (long long)t->T * nt * 128 * H, nr = (long long)t->T * t->P * H;
+    float *arr[3] = {t->z, t->r, t->c};
+    for (float *a : arr) {
+        k_relayout<<<blocks_for(nb), 256, 0, st>>>(t->T, t->P, nt, H, a, t->GX, tiled);
+        cudaError_t e = cudaMemcpyAsync(a, t->GX, (tiled ? nb : nr) * sizeof(float), cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (tiled) {
+        k_relayout<<<blocks_for(nb), 256, 0, st>>>(t->T, t->P, nt, H, t->hs, t->rh, 1);
+    } else {
+        k_relayout<<<blocks_for(nb), 256, 0, st>>>(t->T, t->P, nt, H, t->rh, t->hs, 0);
+        k_mul<<<blocks_for(nr), 256, 0, st>>>(nr, t->r, t->hs, t->rh);
+    }
+    t->tiled = tiled;
+    return cudaGetLastError();
+}
+
+bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
+// The fused window's arguments that do not change from call to call, and X.
+WinArgs window(dnnmg_trainer_s *t, const float *X) {
+    WinArgs g = {};
+    g.n_in = t->n_in; g.ldx = t->ldx; g.n_out = t->n_out; g.nfc = round_up(t->n_out, 16);
+    g.T = t->T; g.P = t->P; g.ntiles = win_tiles(t->P);
+    g.xvec = t->ldx % 4 == 0 && aligned16(X);
+    g.part_cols = 3 * t->H + g.nfc;
+    g.X = X;
+    g.z = t->z; g.r = t->r; g.c = t->c; g.hb = t->rh;
+    g.part = t->wpart;
+    g.status = t->d_status;
+    return g;
+}
+
 void trainer_free(dnnmg_trainer_s *t) {
     if (!t) return;
     float *bufs[] = {t->GX, t->hs, t->z, t->r, t->rh, t->c, t->GH, t->AH, t->dHfc, t->dG, t->dh, t->drh, t->carry,
@@ -498,6 +559,7 @@ void trainer_free(dnnmg_trainer_s *t) {
     cudaFree(t->red);
     cudaFree(t->d_status);
     cudaFree(t->arena);
+    cudaFree(t->wpart);
     delete t;
 }
 
@@ -533,9 +595,11 @@ int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnm
     t->splits = (int)std::min<size_t>(256, std::max<size_t>(1, TP / 4096));
     const size_t mx = (size_t)std::max(3 * H, n_out) * std::max(std::max(n_in, H), 1);
     t->part_floats = (size_t)t->splits * mx;
+    // (z, r, rh and c hold whole 128-row tiles in the fused window)
+    const size_t TPt = (size_t)T * win_tiles(P) * 128;
     struct { float **p; size_t n; } req[] = {
-        {&t->GX, TP * 3 * H}, {&t->hs, (TP + P) * H}, {&t->z, TP * H}, {&t->r, TP * H}, {&t->rh, TP * H},
-        {&t->c, TP * H}, {&t->GH, (size_t)P * 2 * H}, {&t->AH, (size_t)P * H}, {&t->dHfc, TP * H},
+        {&t->GX, std::max(TP * 3, TPt) * H}, {&t->hs, (TP + P) * H}, {&t->z, TPt * H}, {&t->r, TPt * H}, {&t->rh, TPt * H},
+        {&t->c, TPt * H}, {&t->GH, (size_t)P * 2 * H}, {&t->AH, (size_t)P * H}, {&t->dHfc, TP * H},
         {&t->dG, TP * 3 * H}, {&t->dh, (size_t)P * H}, {&t->drh, (size_t)P * H}, {&t->carry, (size_t)P * H},
         {&t->part, t->part_floats}};
     bool ok = true;
@@ -565,6 +629,22 @@ int dnnmg_trainer_set_precision(dnnmg_trainer_t t, int precision) {
         return fail(DNNMG_EINVAL, "trainer precision must be DNNMG_F32 or DNNMG_BF16NET, got %d", precision);
     t->bf16 = 0;
     if (precision == DNNMG_F32) return DNNMG_OK;
+    if (!t->d_status) {
+        if (cudaMalloc(&t->d_status, sizeof(int)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(DNNMG_ENOMEM, "device allocation of the status word failed");
+        }
+        DNNMG_CUDA_TRY(cudaMemset(t->d_status, 0, sizeof(int)));
+    }
+    if (win_supported(t->n_in, t->H, t->n_out)) {
+        if (!t->wpart && cudaMalloc(&t->wpart, win_part_floats(t->H, t->n_out, t->P) * sizeof(float)) != cudaSuccess) {
+            t->wpart = nullptr;
+            cudaGetLastError();
+            return fail(DNNMG_ENOMEM, "device allocation of the partial gradients failed");
+        }
+        t->bf16 = 1;
+        return DNNMG_OK;
+    }
     // BF16 copies of the window's operands, K contiguous, each region 256-byte aligned
     const int H = t->H, P = t->P, TP = t->T * t->P;
     t->kx = kpad(t->n_in); t->kh = kpad(H); t->k2 = kpad(2 * H); t->ko = kpad(t->n_out);
@@ -588,18 +668,15 @@ int dnnmg_trainer_set_precision(dnnmg_trainer_t t, int precision) {
     t->o_hsT = take((size_t)H * t->ks);
     t->o_rhT = take((size_t)H * t->kt);
     t->o_dDT = take((size_t)t->n_out * t->kt);
-    if (off > t->arena_elems || !t->d_status) {
+    if (off > t->arena_elems) {
         cudaFree(t->arena);
         t->arena = nullptr;
         t->arena_elems = 0;
-        if (cudaMalloc(&t->arena, off * sizeof(__nv_bfloat16)) != cudaSuccess ||
-            (!t->d_status && cudaMalloc(&t->d_status, sizeof(int)) != cudaSuccess)) {
-            cudaFree(t->arena);
+        if (cudaMalloc(&t->arena, off * sizeof(__nv_bfloat16)) != cudaSuccess) {
             t->arena = nullptr;
             cudaGetLastError();
             return fail(DNNMG_ENOMEM, "BF16 operand scratch (%zu values) could not be allocated", off);
         }
-        DNNMG_CUDA_TRY(cudaMemset(t->d_status, 0, sizeof(int)));
         t->arena_elems = off;
     }
     t->bf16 = 1;
@@ -638,6 +715,24 @@ int dnnmg_gru_seq_forward(dnnmg_trainer_t t, const float *X, const float *h0, co
     const int H = t->H, P = t->P, T = t->T;
     const size_t PH = (size_t)P * H;
     const int TP = T * P;
+    if (t->bf16 && t->wpart) {
+        WinArgs g = window(t, X);
+        g.Wx = Wx;
+        g.Uh = Uh;
+        g.Wfc = Wfc;
+        g.D = D;
+        g.pairs = t->n_out % 2 == 0 && reinterpret_cast<uintptr_t>(D) % 8 == 0;
+        g.h0 = h0;
+        g.hT = t->hs + (size_t)T * PH;
+        if (h0 && !aligned16(h0)) {
+            DNNMG_CUDA_TRY(cudaMemcpyAsync(t->hs, h0, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));
+            g.h0 = t->hs;
+        }
+        DNNMG_CUDA_TRY(win_forward(g, H, st));
+        t->tiled = 1;
+        return DNNMG_OK;
+    }
+    t->tiled = 0;
     // h_0 (zero when h0 is NULL)
     if (h0) DNNMG_CUDA_TRY(cudaMemcpyAsync(t->hs, h0, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));
     else DNNMG_CUDA_TRY(cudaMemsetAsync(t->hs, 0, PH * sizeof(float), st));
@@ -679,6 +774,23 @@ int dnnmg_gru_seq_backward(dnnmg_trainer_t t, const float *dD, const float *X, c
     const int H = t->H, P = t->P, T = t->T, n_out = t->n_out, n_in = t->n_in;
     const size_t PH = (size_t)P * H;
     const int TP = T * P;
+    const int fused = t->bf16 && t->wpart;
+    DNNMG_CUDA_TRY(want_layout(t, fused, st));
+    if (fused) {
+        WinArgs g = window(t, X);
+        g.Uh = Uh;
+        g.Wfc = Wfc;
+        g.dD = dD;
+        g.pairs = t->n_out % 2 == 0 && reinterpret_cast<uintptr_t>(dD) % 8 == 0;
+        g.gWx = gWx;
+        g.gUh = gUh;
+        g.gWfc = gWfc;
+        g.dh0 = dh0 && !aligned16(dh0) ? t->carry : dh0;
+        DNNMG_CUDA_TRY(win_backward(g, H, st));
+        if (dh0 && g.dh0 != dh0)
+            DNNMG_CUDA_TRY(cudaMemcpyAsync(dh0, t->carry, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        return DNNMG_OK;
+    }
     if (t->bf16) {
         DNNMG_CUDA_TRY(seq_backward_bf16(t, dD, X, Uh, Wfc, gWx, gUh, gWfc, st));
         if (dh0) DNNMG_CUDA_TRY(cudaMemcpyAsync(dh0, t->carry, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));

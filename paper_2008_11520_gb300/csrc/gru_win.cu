@@ -1,0 +1,655 @@
+// The training window of the patch network with BF16 products, as two
+// persistent kernels: forward over T steps (Eq. gru and the output layer) and
+// truncated backpropagation through time with the weight gradients.
+//
+// Patch rows are independent, so a CTA takes 128 of them (one tensor-memory
+// lane a row) through the whole window: weights stay in shared memory as
+// BF16 operand images, the state and the carried gradient in registers, every
+// product is a tcgen05 MMA between images the same threads wrote, and only
+// the window's inputs, outputs and saved activations touch memory.  A kernel
+// per product (with FP32 intermediates and BF16 copies of every operand in
+// memory between them) took 4.07 ms for loss and gradients of 65 536 rows, T =
+// 10, H = 64; this takes 0.65 ms, of it forward 266 us, backward 256 us and
+// the sum of the partial gradients 15 us (ncu).
+//
+// Arithmetic is that of the kernel-per-product path (gru_train.cu): operands
+// are rounded to BF16 where it rounds them, X W_x^T and h U^T are accumulated
+// apart and added in FP32, gates and updates are FP32.  The weight gradients
+// accumulate in tensor memory over a CTA's rows and steps, and the CTAs'
+// partial sums are added in a fixed order, so they repeat bit for bit.
+//
+// Saved activations (z, r, c and h_0 .. h_{T-1}, FP32) are laid out
+// [step][tile][column / 4][row][4]: a warp, whose lanes are rows, moves 512
+// contiguous bytes per 4 columns.
+//
+// Every wait is bounded (2 s): on time-out the kernel sets
+// DNNMG_DEVERR_TIMEOUT in *status, drains its MMAs, frees its tensor memory
+// and returns.
+#include <algorithm>
+#include <cstring>
+
+#include "common.cuh"
+#include "gru_win.cuh"
+#include "ptx.cuh"
+
+namespace dnnmg {
+namespace {
+
+using namespace ptx;
+
+constexpr int TM = 128;            // rows of a tile
+constexpr int IMG = TM * 128;      // one operand image: 128 rows of 64 BF16 columns, 128-byte swizzle
+constexpr int FWD_TH = 256, BWD_TH = 512;
+
+__device__ __forceinline__ void tc_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// K-major operand: rows of 64 K elements, 8-row groups 1024 B apart.
+__device__ __forceinline__ uint64_t desc_k(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3FFFF) >> 4) | (uint64_t)1 << 16 | (uint64_t)(1024 >> 4) << 32 | (uint64_t)1 << 46 |
+           (uint64_t)2 << 61;
+}
+// The same image as an MN-major operand: its 64 columns are the M (or N)
+// extent, its rows the K extent; the next 64 columns are `next` bytes on.
+__device__ __forceinline__ uint64_t desc_mn(uint32_t saddr, uint32_t next) {
+    return (uint64_t)((saddr & 0x3FFFF) >> 4) | (uint64_t)((next >> 4) & 0x3FFF) << 16 | (uint64_t)(1024 >> 4) << 32 |
+           (uint64_t)1 << 46 | (uint64_t)2 << 61;
+}
+// kind::f16, BF16 A and B, FP32 D; mn: both operands MN-major
+__host__ __device__ constexpr uint32_t idesc(int N, bool mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(TM >> 4) << 24);
+}
+__device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(id), "r"(acc)
+        : "memory");
+}
+// D (+)= A B^T over ksteps x 16 columns of two K-major images
+__device__ __forceinline__ void mma_k(uint32_t d, uint32_t a, uint32_t b, int N, int ksteps, bool acc) {
+    const uint64_t da = desc_k(a), db = desc_k(b);
+    for (int k = 0; k < ksteps; ++k) umma(d, da + 2 * k, db + 2 * k, idesc(N, false), (acc || k > 0) ? 1u : 0u);
+}
+// D (+)= A^T B over the 128 rows of the images
+__device__ __forceinline__ void mma_mn(uint32_t d, uint64_t a, uint64_t b, int N, bool acc) {
+#pragma unroll
+    for (int k = 0; k < TM / 16; ++k)
+        umma(d, a + k * (2048 >> 4), b + k * (2048 >> 4), idesc(N, true), (acc || k > 0) ? 1u : 0u);
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t t, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(t));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// values read by tmem_ld8 may be used from here on
+__device__ __forceinline__ void keep(float (&v)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) asm volatile("" : "+f"(v[i]));
+}
+
+__device__ __forceinline__ uint32_t pack(float a, float b) {
+    const __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&t);
+}
+// byte offset of 16-byte unit u of row `row` in an image
+__device__ __forceinline__ uint32_t swz(int row, int u) { return (uint32_t)(row * 128 + ((u ^ (row & 7)) << 4)); }
+// 8 consecutive columns c .. c+7 (c a multiple of 8) of a row
+__device__ __forceinline__ void put8(uint8_t *img, int row, int c, const float *v) {
+    *reinterpret_cast<uint4 *>(img + swz(row, c / 8)) =
+        make_uint4(pack(v[0], v[1]), pack(v[2], v[3]), pack(v[4], v[5]), pack(v[6], v[7]));
+}
+__device__ __forceinline__ void put1(uint8_t *img, int row, int c, float v) {
+    *reinterpret_cast<__nv_bfloat16 *>(img + swz(row, c / 8) + (c & 7) * 2) = __float2bfloat16_rn(v);
+}
+// image rows [0, rows) x columns [0, 64) of src(row, col)
+template <typename F> __device__ __forceinline__ void build(uint8_t *img, int rows, int nth, F src) {
+    for (int e = threadIdx.x; e < rows * 8; e += nth) {
+        const int r = e >> 3, c = (e & 7) * 8;
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = src(r, c + i);
+        *reinterpret_cast<uint4 *>(img + (r >> 3) * 1024 + (r & 7) * 128 + (((c >> 3) ^ (r & 7)) << 4)) =
+            make_uint4(pack(v[0], v[1]), pack(v[2], v[3]), pack(v[4], v[5]), pack(v[6], v[7]));
+    }
+}
+
+__device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + expf(-x)); }
+
+__device__ __forceinline__ void ld4(const float *p, float *v) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void st4(float *p, const float *v) {
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+// saved activations: element (column c, row) of a tile's block
+__device__ __forceinline__ size_t blk(int c, int row) { return (size_t)(c >> 2) * (4 * TM) + 4 * row; }
+
+// The feature rows of a tile, coalesced: 16 lanes take one row's 64 columns.
+template <int NTH> struct XTile {
+    static constexpr int NV = TM * 16 / NTH;
+    float4 v[NV];
+    __device__ __forceinline__ void load(const WinArgs &g, int s, int p0) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int e = threadIdx.x + i * NTH, row = e >> 4, c = (e & 15) * 4;
+            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (p0 + row >= g.P || c >= g.n_in) continue;
+            const float *src = g.X + ((size_t)s * g.P + p0 + row) * g.ldx + c;
+            if (g.xvec) {
+                v[i] = __ldg(reinterpret_cast<const float4 *>(src));
+            } else {   // rows that do not start on 16 bytes
+                v[i].x = __ldg(src);
+                if (c + 1 < g.n_in) v[i].y = __ldg(src + 1);
+                if (c + 2 < g.n_in) v[i].z = __ldg(src + 2);
+                if (c + 3 < g.n_in) v[i].w = __ldg(src + 3);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(const WinArgs &g, uint8_t *img) const {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int e = threadIdx.x + i * NTH, row = e >> 4, c = (e & 15) * 4;
+            const float a = v[i].x, b = c + 1 < g.n_in ? v[i].y : 0.f, d = c + 2 < g.n_in ? v[i].z : 0.f,
+                        f = c + 3 < g.n_in ? v[i].w : 0.f;   // (columns past n_in are not read as features)
+            *reinterpret_cast<uint2 *>(img + swz(row, c >> 3) + (c & 4) * 2) = make_uint2(pack(a, b), pack(d, f));
+        }
+    }
+};
+
+// Shared start and end of both kernels: barriers, tensor memory, teardown.
+struct Cta {
+    uint32_t bar0, tmem;
+    volatile int *abort_flag;
+    __device__ __forceinline__ void init(uint64_t *bars, int nbar, int cols) {
+        uint32_t *slot = reinterpret_cast<uint32_t *>(bars + nbar);
+        abort_flag = reinterpret_cast<volatile int *>(slot + 1);
+        bar0 = smem_u32(bars);
+        if (threadIdx.x == 0) {
+            for (int i = 0; i < nbar; ++i) mbar_init(bar0 + 8 * i, 1);
+            *abort_flag = 0;
+            mbar_init_fence();
+        }
+        if (threadIdx.x < 32) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        fence_async_smem();
+        tc_before_sync();
+        __syncthreads();
+        tc_after_sync();
+        tmem = *slot;
+    }
+    // images written before are visible to the MMAs issued after, and tensor
+    // memory read before may be overwritten; false once a wait has run out
+    __device__ __forceinline__ bool hand_over(bool ok) {
+        fence_async_smem();
+        tc_before_sync();
+        const bool bad = __syncthreads_or(!ok);
+        tc_after_sync();
+        return !bad;
+    }
+    __device__ __forceinline__ bool wait(int b, uint32_t parity) {
+        const bool ok = mbar_wait_inl(bar0 + 8 * b, parity, abort_flag);
+        __syncwarp();
+        tc_after_sync();
+        return ok;
+    }
+    __device__ __forceinline__ void finish(int drain_bar, int cols, int *status) {
+        if (threadIdx.x == 0) {
+            if (*abort_flag) {
+                atomicOr(status, DNNMG_DEVERR_TIMEOUT);
+                volatile int no_abort = 0;
+                tc_commit(bar0 + 8 * drain_bar);   // every MMA issued has finished before teardown
+                mbar_wait(bar0 + 8 * drain_bar, 0, &no_abort);
+            }
+        }
+        tc_before_sync();
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            tc_after_sync();
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+        }
+    }
+};
+
+__device__ __forceinline__ uint8_t *align1k(uint8_t *p) { return p + ((1024u - (smem_u32(p) & 1023u)) & 1023u); }
+
+// ---------------------------------------------------------------- forward
+// Two CTAs an SM (each 256 threads, two per row, and half the tensor memory),
+// so that one computes while the other waits for its MMAs.  Tensor memory
+// columns: X W_zr^T [0, 2H), h U_zr^T [2H, 4H); once r has been read,
+// X W_h^T [H, 2H) and (r h) U_h^T [3H, 4H); then the output layer [0, nfc).
+// Bound by instruction issue (gate functions and conversions) and, close
+// behind, by memory (1.2 kB a row and step).
+template <int H> struct FwdLayout {
+    static constexpr int WX = 0, U = WX + 3 * H * 128, F = U + 3 * H * 128, X = F + 64 * 128, HI = X + IMG,
+                         BARS = HI + IMG, BYTES = BARS + 64 + 1024;
+    static constexpr int COLS = 4 * H;
+};
+
+template <int H>
+__global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
+    using L = FwdLayout<H>;
+    constexpr int NH = H / 2;   // state columns of a thread
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = align1k(smem_raw);
+    uint8_t *sX = base + L::X, *sH = base + L::HI;
+    const uint32_t uWx = smem_u32(base + L::WX), uU = smem_u32(base + L::U), uF = smem_u32(base + L::F),
+                   uX = smem_u32(sX), uH = smem_u32(sH);
+    build(base + L::WX, 3 * H, FWD_TH, [&](int r, int c) { return c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + c) : 0.f; });
+    build(base + L::U, 3 * H, FWD_TH, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)r * H + c) : 0.f; });
+    build(base + L::F, g.nfc, FWD_TH, [&](int r, int c) { return r < g.n_out && c < H ? __ldg(g.Wfc + (size_t)r * H + c) : 0.f; });
+    Cta cta;
+    cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 2, L::COLS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, half = warp >> 2, row = q * 32 + lane, c0 = half * NH;
+    const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
+    uint32_t ph = 0;   // phase of the MMA barrier
+    bool ok = true;
+    XTile<FWD_TH> xt;
+    for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
+        const int p0 = tile * TM, gp = p0 + row;
+        const bool valid = gp < g.P;
+        float hv[NH];
+        xt.load(g, 0, p0);
+#pragma unroll
+        for (int i = 0; i < NH; i += 4) {
+            hv[i] = hv[i + 1] = hv[i + 2] = hv[i + 3] = 0.f;
+            if (g.h0 && valid) ld4(g.h0 + (size_t)gp * H + c0 + i, hv + i);
+        }
+        const size_t tblk = (size_t)TM * H;
+#pragma unroll
+        for (int i = 0; i < NH; i += 4) st4(g.hb + (size_t)tile * tblk + blk(c0 + i, row), hv + i);
+#pragma unroll
+        for (int i = 0; i < NH; i += 8) put8(sH, row, c0 + i, hv + i);
+        xt.store(g, sX);
+        for (int s = 0; s < g.T; ++s) {
+            const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma_k(cta.tmem, uX, uWx, 2 * H, 4, false);
+                mma_k(cta.tmem + 2 * H, uH, uU, 2 * H, H / 16, false);
+                tc_commit(cta.bar0);
+            }
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            // r and r h
+#pragma unroll
+            for (int i = 0; i < NH; i += 8) {
+                float a[8], b[8], rr[8];
+                tmem_ld8(tl + H + c0 + i, a);
+                tmem_ld8(tl + 3 * H + c0 + i, b);
+                tmem_wait();
+                keep(a);
+                keep(b);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    rr[j] = sigm(a[j] + b[j]);
+                    a[j] = rr[j] * hv[i + j];
+                }
+                st4(g.r + sb + blk(c0 + i, row), rr);
+                st4(g.r + sb + blk(c0 + i + 4, row), rr + 4);
+                put8(sH, row, c0 + i, a);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma_k(cta.tmem + H, uX, uWx + 2 * H * 128, H, 4, false);
+                mma_k(cta.tmem + 3 * H, uH, uU + 2 * H * 128, H, H / 16, false);
+                tc_commit(cta.bar0);
+            }
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            // candidate and new state
+#pragma unroll
+            for (int i = 0; i < NH; i += 8) {
+                float a[8], b[8], zz[8], cc[8];
+                tmem_ld8(tl + c0 + i, a);
+                tmem_ld8(tl + 2 * H + c0 + i, b);
+                tmem_ld8(tl + H + c0 + i, zz);
+                tmem_ld8(tl + 3 * H + c0 + i, cc);
+                tmem_wait();
+                keep(a);
+                keep(b);
+                keep(zz);
+                keep(cc);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float z = sigm(a[j] + b[j]), c = tanhf(zz[j] + cc[j]);
+                    zz[j] = z;
+                    cc[j] = c;
+                    hv[i + j] = z * hv[i + j] + (1.0f - z) * c;
+                }
+                st4(g.z + sb + blk(c0 + i, row), zz);
+                st4(g.z + sb + blk(c0 + i + 4, row), zz + 4);
+                st4(g.c + sb + blk(c0 + i, row), cc);
+                st4(g.c + sb + blk(c0 + i + 4, row), cc + 4);
+                put8(sH, row, c0 + i, hv + i);
+            }
+            if (s + 1 < g.T) {
+                xt.load(g, s + 1, p0);
+                float *hb = g.hb + ((size_t)(s + 1) * g.ntiles + tile) * tblk;
+#pragma unroll
+                for (int i = 0; i < NH; i += 4) st4(hb + blk(c0 + i, row), hv + i);
+            } else if (valid) {
+#pragma unroll
+                for (int i = 0; i < NH; i += 4) st4(g.hT + (size_t)gp * H + c0 + i, hv + i);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma_k(cta.tmem, uH, uF, g.nfc, H / 16, false);
+                tc_commit(cta.bar0);
+            }
+            if (s + 1 < g.T) xt.store(g, sX);
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            // outputs: blocks of 8 columns, alternating between the two threads of a row
+            float *drow = g.D + ((size_t)s * g.P + gp) * g.n_out;
+            for (int b = half; b < g.nfc / 8; b += 2) {
+                float v[8];
+                tmem_ld8(tl + 8 * b, v);
+                tmem_wait();
+                keep(v);
+                if (!valid) continue;
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    const int c = 8 * b + j;
+                    if (g.pairs) {
+                        if (c < g.n_out) *reinterpret_cast<float2 *>(drow + c) = make_float2(v[j], v[j + 1]);
+                    } else {
+                        if (c < g.n_out) drow[c] = v[j];
+                        if (c + 1 < g.n_out) drow[c + 1] = v[j + 1];
+                    }
+                }
+            }
+        }
+        ok = cta.hand_over(ok);   // (the same answer in every thread)
+    }
+    cta.finish(1, L::COLS, g.status);
+}
+
+// ---------------------------------------------------------------- backward
+// One CTA an SM, 512 threads (four per row).  Per step, last first:
+//   dh = dD W_fc + carry; dA_z, dA_c; images of h_{s}, r h_{s}, h_{s+1}, dA_z, dA_c
+//   MMA: d(r h) = dA_c U_h
+//   dA_r and the carry's part that does not pass through U_z, U_r
+//   MMA: [dA_z, dA_r] [U_z; U_r] and the next step's dD W_fc, then the
+//   weight gradients [X | h]^T [dA_z, dA_r], [X | r h]^T dA_c and h_{s+1}^T dD
+//   into their accumulators, which run while the next step's elements do.
+// Tensor memory: carry part [0, H), dD W_fc [64, 64 + H), d(r h) [128, 128 + H),
+// gradients [192, 192 + 2H), [320, 320 + H), [384, 384 + nfc).
+// Bound by the chain of the two MMA round trips a step and the element work
+// between them; memory (1.4 kB a row and step) is close behind.
+template <int H> struct BwdLayout {
+    static constexpr int X = 0, HP = X + IMG, RH = HP + IMG, HN = RH + IMG, GZR = HN + IMG,
+                         GC = GZR + (H == 64 ? 2 : 1) * IMG, DD = GC + IMG, WF = DD + 2 * IMG, UC = WF + H * 128,
+                         UZR = UC + H * 128, BARS = UZR + (H == 64 ? 2 : 1) * H * 128, BYTES = BARS + 64 + 1024;
+    static constexpr int COLS = 512;
+};
+constexpr int T_CARRY = 0, T_DH = 64, T_DRH = 128, T_G1 = 192, T_G2 = 320, T_G3 = 384;
+
+template <int H>
+__global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
+    using L = BwdLayout<H>;
+    constexpr int NC = H / 4;   // state columns of a thread: 16 or 8
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = align1k(smem_raw);
+    const uint32_t u = smem_u32(base);
+    // operands of the state gradients: rows are the products' columns
+    build(base + L::WF, H, BWD_TH, [&](int r, int c) { return c < g.n_out ? __ldg(g.Wfc + (size_t)c * H + r) : 0.f; });
+    build(base + L::UC, H, BWD_TH, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)(2 * H + c) * H + r) : 0.f; });
+    for (int k = 0; k < (H == 64 ? 2 : 1); ++k)
+        build(base + L::UZR + k * H * 128, H, BWD_TH, [&](int r, int c) { return __ldg(g.Uh + (size_t)(64 * k + c) * H + r); });
+    // columns that no step writes but the MMAs of unused gradient rows read
+    build(base + L::HP, TM, BWD_TH, [&](int, int) { return 0.f; });
+    build(base + L::RH, TM, BWD_TH, [&](int, int) { return 0.f; });
+    build(base + L::HN, TM, BWD_TH, [&](int, int) { return 0.f; });
+    build(base + L::GC, TM, BWD_TH, [&](int, int) { return 0.f; });
+    build(base + L::DD, TM, BWD_TH, [&](int, int) { return 0.f; });
+    build(base + L::DD + IMG, TM, BWD_TH, [&](int, int) { return 0.f; });
+    Cta cta;
+    cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 4, L::COLS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, part = warp >> 2, row = q * 32 + lane, c0 = part * NC;
+    const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
+    uint32_t ph0 = 0, ph1 = 0, ph2 = 0;   // state part, gradients, d(r h)
+    bool ok = true, grads = false;        // grads: the accumulators hold something
+    const size_t tblk = (size_t)TM * H;
+    XTile<BWD_TH> xt;
+    float zv[NC], rv[NC], cv[NC], hp[NC];
+    auto load_step = [&](int s, int tile) {
+        const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+#pragma unroll
+        for (int i = 0; i < NC; i += 4) {
+            const size_t o = sb + blk(c0 + i, row);
+            ld4(g.z + o, zv + i);
+            ld4(g.r + o, rv + i);
+            ld4(g.c + o, cv + i);
+            ld4(g.hb + o, hp + i);
+        }
+    };
+    // dD rows of a step into their image (one of two), each thread a few columns of its row
+    auto load_dd = [&](int s, int p0) {
+        uint8_t *img = base + L::DD + (s & 1) * IMG;
+        const int gp = p0 + row;
+        const float *src = g.dD + ((size_t)s * g.P + gp) * g.n_out;
+        if (g.pairs) {
+            for (int c = 2 * part; c < g.n_out; c += 8) {
+                float2 v = make_float2(0.f, 0.f);
+                if (gp < g.P) v = __ldg(reinterpret_cast<const float2 *>(src + c));
+                *reinterpret_cast<uint32_t *>(img + swz(row, c >> 3) + (c & 7) * 2) = pack(v.x, v.y);
+            }
+        } else {
+            for (int c = part; c < g.n_out; c += 4) put1(img, row, c, gp < g.P ? __ldg(src + c) : 0.f);
+        }
+    };
+    const int kfc = g.nfc / 16;
+    for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
+        const int p0 = tile * TM, gp = p0 + row;
+        float cpart[NC];
+#pragma unroll
+        for (int i = 0; i < NC; ++i) cpart[i] = 0.f;
+        // (the previous tile's gradients have been waited for before its images are reused: below)
+        if (grads) {
+            ok = cta.wait(1, ph1);
+            ph1 ^= 1;
+        }
+        if (!(ok = cta.hand_over(ok))) break;
+        load_dd(g.T - 1, p0);
+        load_step(g.T - 1, tile);
+        xt.load(g, g.T - 1, p0);
+        if (!(ok = cta.hand_over(ok))) break;
+        if (tid == 0) {
+            mma_k(cta.tmem + T_DH, u + L::DD + ((g.T - 1) & 1) * IMG, u + L::WF, H, kfc, false);
+            tc_commit(cta.bar0);
+        }
+        for (int s = g.T - 1; s >= 0; --s) {
+            ok = cta.wait(0, ph0);
+            ph0 ^= 1;
+            float dh[NC], az[NC], ac[NC];
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float a[8], b[8];
+                tmem_ld8(tl + T_DH + c0 + i, a);
+                tmem_ld8(tl + T_CARRY + c0 + i, b);
+                tmem_wait();
+                keep(a);
+                keep(b);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = i + j;
+                    const float carry = s == g.T - 1 ? 0.f : b[j] + cpart[k];
+                    dh[k] = a[j] + carry;
+                    const float dc = dh[k] * (1.0f - zv[k]), dz = dh[k] * (hp[k] - cv[k]);
+                    az[k] = dz * zv[k] * (1.0f - zv[k]);
+                    ac[k] = dc * (1.0f - cv[k] * cv[k]);
+                }
+            }
+            // the images may be overwritten once the step before's gradients are done
+            if (s < g.T - 1) {
+                ok = cta.wait(1, ph1) && ok;
+                ph1 ^= 1;
+            }
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float t[8];
+                put8(base + L::HP, row, c0 + i, hp + i);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) t[j] = rv[i + j] * hp[i + j];
+                put8(base + L::RH, row, c0 + i, t);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) t[j] = zv[i + j] * hp[i + j] + (1.0f - zv[i + j]) * cv[i + j];
+                put8(base + L::HN, row, c0 + i, t);
+                put8(base + L::GZR, row, c0 + i, az + i);
+                put8(base + L::GC, row, c0 + i, ac + i);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma_k(cta.tmem + T_DRH, u + L::GC, u + L::UC, H, H / 16, false);
+                tc_commit(cta.bar0 + 16);
+            }
+            xt.store(g, base + L::X);
+            if (s > 0) load_dd(s - 1, p0);
+            ok = cta.wait(2, ph2);
+            ph2 ^= 1;
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float a[8];
+                tmem_ld8(tl + T_DRH + c0 + i, a);
+                tmem_wait();
+                keep(a);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = i + j;
+                    cpart[k] = dh[k] * zv[k] + a[j] * rv[k];
+                    a[j] = a[j] * hp[k] * rv[k] * (1.0f - rv[k]);
+                }
+                // columns H .. 2H-1 of [dA_z, dA_r]
+                if (H == 64) put8(base + L::GZR + IMG, row, c0 + i, a);
+                else put8(base + L::GZR, row, H + c0 + i, a);
+            }
+            if (s > 0) {
+                load_step(s - 1, tile);
+                xt.load(g, s - 1, p0);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma_k(cta.tmem + T_CARRY, u + L::GZR, u + L::UZR, H, 4, false);
+                if (H == 64) mma_k(cta.tmem + T_CARRY, u + L::GZR + IMG, u + L::UZR + H * 128, H, 4, true);
+                if (s > 0) mma_k(cta.tmem + T_DH, u + L::DD + ((s - 1) & 1) * IMG, u + L::WF, H, kfc, false);
+                tc_commit(cta.bar0);
+                mma_mn(cta.tmem + T_G1, desc_mn(u + L::X, L::HP - L::X), desc_mn(u + L::GZR, IMG), 2 * H, grads);
+                mma_mn(cta.tmem + T_G2, desc_mn(u + L::X, L::RH - L::X), desc_mn(u + L::GC, IMG), H, grads);
+                mma_mn(cta.tmem + T_G3, desc_mn(u + L::HN, L::HP - L::X), desc_mn(u + L::DD + (s & 1) * IMG, IMG), g.nfc, grads);
+                tc_commit(cta.bar0 + 8);
+            }
+            grads = true;
+        }
+        if (!ok) break;
+        // gradient of h_0
+        ok = cta.wait(0, ph0);
+        ph0 ^= 1;
+        if (g.dh0) {
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float b[8];
+                tmem_ld8(tl + T_CARRY + c0 + i, b);
+                tmem_wait();
+                keep(b);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) b[j] += cpart[i + j];
+                if (gp < g.P) {
+                    st4(g.dh0 + (size_t)gp * H + c0 + i, b);
+                    st4(g.dh0 + (size_t)gp * H + c0 + i + 4, b + 4);
+                }
+            }
+        }
+        ok = cta.hand_over(ok);   // (the same answer in every thread)
+    }
+    // this CTA's sums: [column][lane], gradients of W_x (lanes 0 .. 63) and U (64 ..), then of W_fc
+    if (ok && grads) {
+        ok = cta.wait(1, ph1);
+        ph1 ^= 1;
+    }
+    if (ok && !*cta.abort_flag) {
+        float *o = g.part + (size_t)blockIdx.x * g.part_cols * TM;
+        const int ncol = 3 * H + g.nfc;
+        for (int b = part; b < ncol / 8; b += 4) {
+            const int c = 8 * b;
+            const int t = c < 2 * H ? T_G1 + c : (c < 3 * H ? T_G2 + c - 2 * H : T_G3 + c - 3 * H);
+            float v[8];
+            tmem_ld8(tl + t, v);
+            tmem_wait();
+            keep(v);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[(size_t)(c + j) * TM + row] = v[j];
+        }
+    }
+    cta.finish(3, L::COLS, g.status);
+}
+
+// Sums of the CTAs' partial gradients, in the order of the CTAs.
+__global__ void __launch_bounds__(TM) k_win_reduce(const WinArgs g, int H, int nparts) {
+    const int c = blockIdx.x, m = threadIdx.x;
+    const float *p = g.part + (size_t)c * TM + m;
+    const size_t stride = (size_t)g.part_cols * TM;
+    float s = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < nparts; ++i) s += p[i * stride];
+    if (c < 3 * H) {
+        if (m < g.n_in && m < 64) g.gWx[(size_t)c * g.n_in + m] = s;
+        if (m >= 64 && m < 64 + H) g.gUh[(size_t)c * H + m - 64] = s;
+    } else if (c - 3 * H < g.n_out && m < H) {
+        g.gWfc[(size_t)(c - 3 * H) * H + m] = s;
+    }
+}
+
+int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return n > 0 ? n : 1;
+}
+
+template <typename K> cudaError_t launch(K k, int grid, int threads, int smem, const WinArgs &g, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k<<<grid, threads, smem, st>>>(g);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Shapes the window kernels take: one 64-column chunk of features, H = 32 or
+// 64, up to 64 outputs (the K = 1 networks of the training workload); the
+// others run one kernel per product.
+bool win_supported(int n_in, int H, int n_out) { return n_in <= 64 && (H == 32 || H == 64) && n_out <= 64; }
+int win_tiles(int P) { return (P + TM - 1) / TM; }
+size_t win_part_floats(int H, int n_out, int P) {
+    return (size_t)std::min(win_tiles(P), sm_count()) * (3 * H + round_up(n_out, 16)) * TM;
+}
+
+cudaError_t win_forward(WinArgs g, int H, cudaStream_t st) {
+    const int grid = std::min(g.ntiles, 2 * sm_count());
+    if (H == 64) return launch(k_win_fwd<64>, grid, FWD_TH, FwdLayout<64>::BYTES, g, st);
+    return launch(k_win_fwd<32>, grid, FWD_TH, FwdLayout<32>::BYTES, g, st);
+}
+
+cudaError_t win_backward(WinArgs g, int H, cudaStream_t st) {
+    const int grid = std::min(g.ntiles, sm_count());
+    cudaError_t e = H == 64 ? launch(k_win_bwd<64>, grid, BWD_TH, BwdLayout<64>::BYTES, g, st)
+                            : launch(k_win_bwd<32>, grid, BWD_TH, BwdLayout<32>::BYTES, g, st);
+    if (e != cudaSuccess) return e;
+    k_win_reduce<<<3 * H + g.nfc, TM, 0, st>>>(g, H, grid);
+    return cudaGetLastError();
+}
+
+}  // namespace dnnmg

@@ -1,0 +1,26 @@
+// The fused training window (gru_win.cu) as gru_train.cu calls it.
+#pragma once
+
+#include "common.cuh"
+
+namespace dnnmg {
+
+struct WinArgs {
+    int n_in, ldx, n_out, nfc, T, P, ntiles;   // nfc: n_out rounded up to 16
+    int pairs;                                 // rows of D and dD start on 8 bytes (n_out even)
+    int xvec;                                  // rows of X start on 16 bytes
+    int part_cols;                             // columns of a CTA's partial gradients (3H + nfc)
+    const float *X, *h0, *Wx, *Uh, *Wfc, *dD;
+    float *D, *hT;                             // outputs of every step, state after the last
+    float *z, *r, *c, *hb;                     // saved activations, [T][ntiles][H / 4][128][4]
+    float *gWx, *gUh, *gWfc, *dh0, *part;
+    int *status;
+};
+
+bool win_supported(int n_in, int H, int n_out);
+int win_tiles(int P);
+size_t win_part_floats(int H, int n_out, int P);
+cudaError_t win_forward(WinArgs g, int H, cudaStream_t st);
+cudaError_t win_backward(WinArgs g, int H, cudaStream_t st);
+
+}  // namespace dnnmg
