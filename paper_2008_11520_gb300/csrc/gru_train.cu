@@ -347,7 +347,6 @@ struct dnnmg_trainer_s {
     int bf16;
     int *d_status;
     float *wpart;   // the fused window's partial weight gradients; null: one kernel per product
-    int tiled;      // the saved activations are in the fused window's layout (h_0 .. h_{T-1} in rh)
     // BF16 copies, each tensor rounded once (offsets into arena, in elements;
     // row strides kx = kpad(n_in), kh = kpad(H), k2 = kpad(2H), ko = kpad(n_out),
     // kt = kpad(T P), ks = kpad((T+1) P))
@@ -493,48 +492,6 @@ cudaError_t seq_backward_bf16(dnnmg_trainer_s *t, const float *dD, const float *
     return cudaSuccess;
 }
 
-// [T][P][H] rows to the fused window's tiles (rows past P zero) or back.
-__global__ void k_relayout(int T, int P, int ntiles, int H, const float *__restrict__ src, float *__restrict__ dst,
-                           int to_tiles) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // element of the tiled array
-    const long long n = (long long)T * ntiles * 128 * H;
-    if (e >= n) return;
-    const int blk = 128 * H;
-    const long long st = e / blk;
-    const int in = (int)(e - st * blk), s = (int)(st / ntiles), tile = (int)(st - (long long)s * ntiles);
-    const int row = (in / 4) % 128, c = in / 512 * 4 + in % 4, p = tile * 128 + row;
-    const long long r = ((long long)s * P + p) * H + c;
-    if (to_tiles) dst[e] = p < P ? src[r] : 0.0f;
-    else if (p < P) dst[r] = src[e];
-}
-__global__ void k_mul(long long n, const float *__restrict__ a, const float *__restrict__ b, float *__restrict__ c) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) c[e] = a[e] * b[e];
-}
-
-// The saved activations in the layout the backward about to run reads: only
-// where the precision was changed between a window's forward and backward
-// does that differ from the one its forward wrote.
-cudaError_t want_layout(dnnmg_trainer_s *t, int tiled, cudaStream_t st) {
-    if (t->tiled == tiled) return cudaSuccess;
-    const int nt = win_tiles(t->P), H = t->H;
-    const long long nb = (long long)t->T * nt * 128 * H, nr = (long long)t->T * t->P * H;
-    float *arr[3] = {t->z, t->r, t->c};
-    for (float *a : arr) {
-        k_relayout<<<blocks_for(nb), 256, 0, st>>>(t->T, t->P, nt, H, a, t->GX, tiled);
-        cudaError_t e = cudaMemcpyAsync(a, t->GX, (tiled ? nb : nr) * sizeof(float), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-    }
-    if (tiled) {
-        k_relayout<<<blocks_for(nb), 256, 0, st>>>(t->T, t->P, nt, H, t->hs, t->rh, 1);
-    } else {
-        k_relayout<<<blocks_for(nb), 256, 0, st>>>(t->T, t->P, nt, H, t->rh, t->hs, 0);
-        k_mul<<<blocks_for(nr), 256, 0, st>>>(nr, t->r, t->hs, t->rh);
-    }
-    t->tiled = tiled;
-    return cudaGetLastError();
-}
-
 bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
 // The fused window's arguments that do not change from call to call, and X.
@@ -547,6 +504,8 @@ WinArgs window(dnnmg_trainer_s *t, const float *X) {
     g.X = X;
     g.z = t->z; g.r = t->r; g.c = t->c; g.hb = t->rh;
     g.part = t->wpart;
+    g.dG = t->dG;
+    g.hT = t->hs + (size_t)t->T * t->P * t->H;
     g.status = t->d_status;
     return g;
 }
@@ -598,13 +557,16 @@ int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnm
     // (z, r, rh and c hold whole 128-row tiles in the fused window)
     const size_t TPt = (size_t)T * win_tiles(P) * 128;
     struct { float **p; size_t n; } req[] = {
-        {&t->GX, std::max(TP * 3, TPt) * H}, {&t->hs, (TP + P) * H}, {&t->z, TPt * H}, {&t->r, TPt * H}, {&t->rh, TPt * H},
+        {&t->GX, TP * 3 * H}, {&t->hs, (TP + P) * H}, {&t->z, TPt * H}, {&t->r, TPt * H}, {&t->rh, TPt * H},
         {&t->c, TPt * H}, {&t->GH, (size_t)P * 2 * H}, {&t->AH, (size_t)P * H}, {&t->dHfc, TP * H},
-        {&t->dG, TP * 3 * H}, {&t->dh, (size_t)P * H}, {&t->drh, (size_t)P * H}, {&t->carry, (size_t)P * H},
+        {&t->dG, TPt * 3 * H}, {&t->dh, (size_t)P * H}, {&t->drh, (size_t)P * H}, {&t->carry, (size_t)P * H},
         {&t->part, t->part_floats}};
     bool ok = true;
     for (auto &q : req) ok = ok && cudaMalloc(q.p, q.n * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&t->red, kRedBlocks * sizeof(double)) == cudaSuccess;
+    ok = ok && cudaMalloc(&t->d_status, sizeof(int)) == cudaSuccess && cudaMemset(t->d_status, 0, sizeof(int)) == cudaSuccess;
+    if (win_supported(n_in, H, n_out))
+        ok = ok && cudaMalloc(&t->wpart, win_part_floats(H, n_out, T, P) * sizeof(float)) == cudaSuccess;
     if (!ok) {
         trainer_free(t);
         cudaGetLastError();
@@ -629,19 +591,7 @@ int dnnmg_trainer_set_precision(dnnmg_trainer_t t, int precision) {
         return fail(DNNMG_EINVAL, "trainer precision must be DNNMG_F32 or DNNMG_BF16NET, got %d", precision);
     t->bf16 = 0;
     if (precision == DNNMG_F32) return DNNMG_OK;
-    if (!t->d_status) {
-        if (cudaMalloc(&t->d_status, sizeof(int)) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(DNNMG_ENOMEM, "device allocation of the status word failed");
-        }
-        DNNMG_CUDA_TRY(cudaMemset(t->d_status, 0, sizeof(int)));
-    }
-    if (win_supported(t->n_in, t->H, t->n_out)) {
-        if (!t->wpart && cudaMalloc(&t->wpart, win_part_floats(t->H, t->n_out, t->P) * sizeof(float)) != cudaSuccess) {
-            t->wpart = nullptr;
-            cudaGetLastError();
-            return fail(DNNMG_ENOMEM, "device allocation of the partial gradients failed");
-        }
+    if (t->wpart) {   // the fused window: no operand copies
         t->bf16 = 1;
         return DNNMG_OK;
     }
@@ -688,7 +638,6 @@ int dnnmg_trainer_status(dnnmg_trainer_t t, int *status, int reset) {
     if (int e = check_trainer(t)) return e;
     if (!status) return fail(DNNMG_EINVAL, "status is NULL");
     *status = 0;
-    if (!t->d_status) return DNNMG_OK;
     DNNMG_CUDA_TRY(cudaMemcpy(status, t->d_status, sizeof(int), cudaMemcpyDeviceToHost));
     if (reset) DNNMG_CUDA_TRY(cudaMemset(t->d_status, 0, sizeof(int)));
     return DNNMG_OK;
@@ -715,7 +664,7 @@ int dnnmg_gru_seq_forward(dnnmg_trainer_t t, const float *X, const float *h0, co
     const int H = t->H, P = t->P, T = t->T;
     const size_t PH = (size_t)P * H;
     const int TP = T * P;
-    if (t->bf16 && t->wpart) {
+    if (t->wpart) {
         WinArgs g = window(t, X);
         g.Wx = Wx;
         g.Uh = Uh;
@@ -723,16 +672,13 @@ int dnnmg_gru_seq_forward(dnnmg_trainer_t t, const float *X, const float *h0, co
         g.D = D;
         g.pairs = t->n_out % 2 == 0 && reinterpret_cast<uintptr_t>(D) % 8 == 0;
         g.h0 = h0;
-        g.hT = t->hs + (size_t)T * PH;
         if (h0 && !aligned16(h0)) {
             DNNMG_CUDA_TRY(cudaMemcpyAsync(t->hs, h0, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));
             g.h0 = t->hs;
         }
-        DNNMG_CUDA_TRY(win_forward(g, H, st));
-        t->tiled = 1;
+        DNNMG_CUDA_TRY(t->bf16 ? win_forward(g, H, st) : win32_forward(g, H, st));
         return DNNMG_OK;
     }
-    t->tiled = 0;
     // h_0 (zero when h0 is NULL)
     if (h0) DNNMG_CUDA_TRY(cudaMemcpyAsync(t->hs, h0, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));
     else DNNMG_CUDA_TRY(cudaMemsetAsync(t->hs, 0, PH * sizeof(float), st));
@@ -774,9 +720,7 @@ int dnnmg_gru_seq_backward(dnnmg_trainer_t t, const float *dD, const float *X, c
     const int H = t->H, P = t->P, T = t->T, n_out = t->n_out, n_in = t->n_in;
     const size_t PH = (size_t)P * H;
     const int TP = T * P;
-    const int fused = t->bf16 && t->wpart;
-    DNNMG_CUDA_TRY(want_layout(t, fused, st));
-    if (fused) {
+    if (t->wpart) {
         WinArgs g = window(t, X);
         g.Uh = Uh;
         g.Wfc = Wfc;
@@ -786,7 +730,7 @@ int dnnmg_gru_seq_backward(dnnmg_trainer_t t, const float *dD, const float *X, c
         g.gUh = gUh;
         g.gWfc = gWfc;
         g.dh0 = dh0 && !aligned16(dh0) ? t->carry : dh0;
-        DNNMG_CUDA_TRY(win_backward(g, H, st));
+        DNNMG_CUDA_TRY(t->bf16 ? win_backward(g, H, st) : win32_backward(g, H, st));
         if (dh0 && g.dh0 != dh0)
             DNNMG_CUDA_TRY(cudaMemcpyAsync(dh0, t->carry, PH * sizeof(float), cudaMemcpyDeviceToDevice, st));
         return DNNMG_OK;

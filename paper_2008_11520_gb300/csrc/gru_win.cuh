@@ -1,4 +1,4 @@
-// The fused training window (gru_win.cu) as gru_train.cu calls it.
+// The fused training window (gru_win.cu, gru_win32.cu) as gru_train.cu calls it.
 #pragma once
 
 #include "common.cuh"
@@ -14,13 +14,18 @@ struct WinArgs {
     float *D, *hT;                             // outputs of every step, state after the last
     float *z, *r, *c, *hb;                     // saved activations, [T][ntiles][H / 4][128][4]
     float *gWx, *gUh, *gWfc, *dh0, *part;
+    float *dG;                                 // FP32: gate gradients, [T][ntiles][3][H / 4][128][4]
     int *status;
 };
 
 bool win_supported(int n_in, int H, int n_out);
 int win_tiles(int P);
-size_t win_part_floats(int H, int n_out, int P);
-cudaError_t win_forward(WinArgs g, int H, cudaStream_t st);
-cudaError_t win_backward(WinArgs g, int H, cudaStream_t st);
+size_t win_part_floats(int H, int n_out, int T, int P);
+cudaError_t win_forward(const WinArgs &g, int H, cudaStream_t st);        // BF16 products (gru_win.cu)
+cudaError_t win_backward(const WinArgs &g, int H, cudaStream_t st);
+cudaError_t win32_forward(const WinArgs &g, int H, cudaStream_t st);      // FP32 products (gru_win32.cu)
+cudaError_t win32_backward(const WinArgs &g, int H, cudaStream_t st);
+int win32_parts(int T, int P);
+cudaError_t win_reduce(const WinArgs &g, int H, int nparts, cudaStream_t st);
 
 }  // namespace dnnmg

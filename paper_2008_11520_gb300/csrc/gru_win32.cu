@@ -1,0 +1,654 @@
+// The training window of the patch network with FP32 products, on the tensor
+// cores: forward over T steps, backpropagation of the state gradients, and
+// the weight gradients, as three persistent kernels.
+//
+// An FP32 operand is the sum of three BF16 values (8 significant bits each,
+// so all 24), and a product of two is the sum of six BF16 products (the three
+// left out are below 2^-24 of it).  Accumulation in tensor memory truncates,
+// so the order matters: the small products are accumulated first and the
+// leading one last, over at most 128 terms, and longer sums are added in FP32
+// registers.  Measured against 64 bits on N(0, 1) operands: 0.8e-7 for K = 64
+// and 1.3e-7 for K = 128, against 1.5e-7 and 2.1e-7 for FP32 FMA in sequence
+// (the leading product first: 7e-7 and 1.4e-6); sums of 4096 terms drained
+// every 128: 1.6e-7 against 1.1e-6.
+//
+// Six tcgen05 products of BF16 are 316 TFLOP/s of FP32 at the measured BF16
+// rate; the CUDA cores' FMAs give 74.  With the fused window (see gru_win.cu,
+// whose layouts these kernels share) loss and gradients of 65 536 rows, T =
+// 10, H = 64 take 1.27 ms instead of 5.5 ms with one FP32 kernel per
+// product, and of 762 rows, H = 32, 0.46 ms instead of 2.7 ms.
+//
+// Values beyond the largest BF16 number are clamped to it (an infinite
+// feature saturates the gates as it does in FP32); a NaN stays one.
+#include <algorithm>
+#include <cstring>
+
+#include "common.cuh"
+#include "gru_win.cuh"
+#include "gru_win_dev.cuh"
+
+namespace dnnmg {
+namespace {
+
+constexpr int W32_TH = 512;   // four threads a row
+
+// the products of the three-part operands, small ones first
+__device__ constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
+
+// D = A B^T of two K-major operands whose parts are astep / bstep bytes apart;
+// with a second pair of operands (a2, b2), whose K follows the first one's
+__device__ __forceinline__ void mma3_k(uint32_t d, uint32_t a, uint32_t astep, uint32_t b, uint32_t bstep, int N, int ksteps) {
+    uint32_t acc = 0;
+    for (int p = 0; p < 6; ++p) {
+        const uint64_t da = desc_k(a + PA[p] * astep), db = desc_k(b + PB[p] * bstep);
+        for (int k = 0; k < ksteps; ++k) {
+            umma(d, da + 2 * k, db + 2 * k, idesc(N, false), acc);
+            acc = 1;
+        }
+    }
+}
+// D = A^T B over `rows` rows of MN-major operands; anext / bnext: the next 64 columns
+__device__ __forceinline__ void mma3_mn(uint32_t d, uint32_t a, uint32_t astep, uint32_t anext, uint32_t b, uint32_t bstep,
+                                        uint32_t bnext, int N, int rows) {
+    uint32_t acc = 0;
+    for (int p = 0; p < 6; ++p) {
+        const uint64_t da = desc_mn(a + PA[p] * astep, anext), db = desc_mn(b + PB[p] * bstep, bnext);
+        for (int k = 0; k < rows / 16; ++k) {
+            umma(d, da + k * (2048 >> 4), db + k * (2048 >> 4), idesc(N, true), acc);
+            acc = 1;
+        }
+    }
+}
+
+// Each accumulation at a product's full magnitude (one per 16 terms of its
+// leading part) drops on average 2.1e-8 of the sum (measured: 0.85e-7 for K =
+// 64, 1.7e-7 for K = 128, all of one sign).  That much is put back, so that
+// long sums of products do not keep the bias.
+__device__ __forceinline__ float whole(float v, int ksteps) { return fmaf(v, 2.1e-8f * (float)ksteps, v); }
+
+__device__ __forceinline__ float clamp_bf16(float x) {
+    float y;
+    asm("{\n.reg .f32 t;\nmin.NaN.f32 t, %1, 0f7F7F0000;\nmax.NaN.f32 %0, t, 0fFF7F0000;\n}\n" : "=f"(y) : "f"(x));
+    return y;
+}
+// the three parts of two values, each pair packed
+__device__ __forceinline__ void split2(float x, float y, uint32_t (&o)[3]) {
+    x = clamp_bf16(x);
+    y = clamp_bf16(y);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const __nv_bfloat162 t = __floats2bfloat162_rn(x, y);
+        o[p] = *reinterpret_cast<const uint32_t *>(&t);
+        x -= __low2float(t);
+        y -= __high2float(t);
+    }
+}
+// 8 consecutive columns of a row into the three images, `step` bytes apart
+__device__ __forceinline__ void put8_3(uint8_t *img, int step, int row, int c, const float *v) {
+    uint32_t o[4][3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) split2(v[2 * i], v[2 * i + 1], o[i]);
+    const uint32_t at = swz(row, c >> 3);
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+        *reinterpret_cast<uint4 *>(img + p * step + at) = make_uint4(o[0][p], o[1][p], o[2][p], o[3][p]);
+}
+// 4 consecutive columns (c a multiple of 4)
+__device__ __forceinline__ void put4_3(uint8_t *img, int step, int row, int c, const float *v) {
+    uint32_t a[3], b[3];
+    split2(v[0], v[1], a);
+    split2(v[2], v[3], b);
+    const uint32_t at = swz(row, c >> 3) + (c & 4) * 2;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2 *>(img + p * step + at) = make_uint2(a[p], b[p]);
+}
+template <typename F> __device__ __forceinline__ void build3(uint8_t *img, int step, int rows, F src) {
+    for (int e = threadIdx.x; e < rows * 8; e += W32_TH) {
+        const int r = e >> 3, c = (e & 7) * 8;
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = src(r, c + i);
+        put8_3(img, step, r, c, v);   // (8-row groups are 1024 bytes apart: row * 128 throughout)
+    }
+}
+__device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &x, uint8_t *img) {
+#pragma unroll
+    for (int i = 0; i < XTile<W32_TH>::NV; ++i) {
+        const int e = threadIdx.x + i * W32_TH, row = e >> 4, c = (e & 15) * 4;
+        const float v[4] = {x.v[i].x, c + 1 < g.n_in ? x.v[i].y : 0.f, c + 2 < g.n_in ? x.v[i].z : 0.f,
+                            c + 3 < g.n_in ? x.v[i].w : 0.f};
+        put4_3(img, IMG, row, c, v);
+    }
+}
+
+// ---------------------------------------------------------------- forward
+// One CTA an SM: the weights' three parts take 172 KB (H = 64), so the three
+// images of one operand share the rest and h, X and r h pass through them in
+// turn: the previous state for h U_zr^T and the previous step's outputs, X
+// for X W_x^T, r h for the candidate.  Tensor memory: X W_x^T [0, 3H),
+// h U_zr^T [3H, 5H), (r h) U_h^T [5H, 6H), outputs [6H, 6H + nfc).
+// Bound by the chain of three MMA round trips a step with the splits and gate
+// functions between them.
+template <int H> struct Fwd32Layout {
+    static constexpr int WS = 3 * H * 128, FS = 64 * 128;   // bytes of one part
+    static constexpr int WX = 0, U = WX + 3 * WS, F = U + 3 * WS, A = F + 3 * FS, BARS = A + 3 * IMG, BYTES = BARS + 64 + 1024;
+    static constexpr int COLS = H == 64 ? 512 : 256;
+};
+
+template <int H>
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
+    using L = Fwd32Layout<H>;
+    constexpr int NC = H / 4;   // state columns of a thread
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = align1k(smem_raw), *sA = base + L::A;
+    const uint32_t u = smem_u32(base), uA = u + L::A;
+    build3(base + L::WX, L::WS, 3 * H, [&](int r, int c) { return c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + c) : 0.f; });
+    build3(base + L::U, L::WS, 3 * H, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)r * H + c) : 0.f; });
+    build3(base + L::F, L::FS, g.nfc, [&](int r, int c) { return r < g.n_out && c < H ? __ldg(g.Wfc + (size_t)r * H + c) : 0.f; });
+    Cta cta;
+    cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 2, L::COLS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, part = warp >> 2, row = q * 32 + lane, c0 = part * NC;
+    const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
+    const size_t tblk = (size_t)TM * H;
+    uint32_t ph = 0;
+    bool ok = true;
+    XTile<W32_TH> xt;
+    for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
+        const int p0 = tile * TM, gp = p0 + row;
+        const bool valid = gp < g.P;
+        float hv[NC];
+#pragma unroll
+        for (int i = 0; i < NC; i += 4) {
+            hv[i] = hv[i + 1] = hv[i + 2] = hv[i + 3] = 0.f;
+            if (g.h0 && valid) ld4(g.h0 + (size_t)gp * H + c0 + i, hv + i);
+            st4(g.hb + (size_t)tile * tblk + blk(c0 + i, row), hv + i);
+        }
+        xt.load(g, 0, p0);
+#pragma unroll
+        for (int i = 0; i < NC; i += 8) put8_3(sA, IMG, row, c0 + i, hv + i);
+        if (!(ok = cta.hand_over(ok))) break;
+        if (tid == 0) {
+            mma3_k(cta.tmem + 3 * H, uA, IMG, u + L::U, L::WS, 2 * H, H / 16);
+            tc_commit(cta.bar0);
+        }
+        auto outputs = [&](int s) {   // of step s, from tensor memory
+            float *drow = g.D + ((size_t)s * g.P + gp) * g.n_out;
+            for (int b = part; b < g.nfc / 8; b += 4) {
+                float v[8];
+                tmem_ld8(tl + 6 * H + 8 * b, v);
+                tmem_wait();
+                keep(v);
+                if (!valid) continue;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = whole(v[j], H / 16);
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    const int c = 8 * b + j;
+                    if (g.pairs) {
+                        if (c < g.n_out) *reinterpret_cast<float2 *>(drow + c) = make_float2(v[j], v[j + 1]);
+                    } else {
+                        if (c < g.n_out) drow[c] = v[j];
+                        if (c + 1 < g.n_out) drow[c + 1] = v[j + 1];
+                    }
+                }
+            }
+        };
+        for (int s = 0; s < g.T; ++s) {
+            const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            store_x3(g, xt, sA);
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma3_k(cta.tmem, uA, IMG, u + L::WX, L::WS, 3 * H, 4);
+                tc_commit(cta.bar0);
+            }
+            if (s > 0) outputs(s - 1);
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float a[8], b[8], rr[8];
+                tmem_ld8(tl + H + c0 + i, a);
+                tmem_ld8(tl + 4 * H + c0 + i, b);
+                tmem_wait();
+                keep(a);
+                keep(b);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    rr[j] = sigm(whole(a[j], 4) + whole(b[j], H / 16));
+                    a[j] = rr[j] * hv[i + j];
+                }
+                st4(g.r + sb + blk(c0 + i, row), rr);
+                st4(g.r + sb + blk(c0 + i + 4, row), rr + 4);
+                put8_3(sA, IMG, row, c0 + i, a);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma3_k(cta.tmem + 5 * H, uA, IMG, u + L::U + 2 * H * 128, L::WS, H, H / 16);
+                tc_commit(cta.bar0);
+            }
+            if (s + 1 < g.T) xt.load(g, s + 1, p0);
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float a[8], b[8], zz[8], cc[8];
+                tmem_ld8(tl + c0 + i, a);
+                tmem_ld8(tl + 3 * H + c0 + i, b);
+                tmem_ld8(tl + 2 * H + c0 + i, zz);
+                tmem_ld8(tl + 5 * H + c0 + i, cc);
+                tmem_wait();
+                keep(a);
+                keep(b);
+                keep(zz);
+                keep(cc);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float z = sigm(whole(a[j], 4) + whole(b[j], H / 16)),
+                                c = tanhf(whole(zz[j], 4) + whole(cc[j], H / 16));
+                    zz[j] = z;
+                    cc[j] = c;
+                    hv[i + j] = z * hv[i + j] + (1.0f - z) * c;
+                }
+                st4(g.z + sb + blk(c0 + i, row), zz);
+                st4(g.z + sb + blk(c0 + i + 4, row), zz + 4);
+                st4(g.c + sb + blk(c0 + i, row), cc);
+                st4(g.c + sb + blk(c0 + i + 4, row), cc + 4);
+                put8_3(sA, IMG, row, c0 + i, hv + i);
+            }
+            if (s + 1 < g.T) {
+                float *hb = g.hb + ((size_t)(s + 1) * g.ntiles + tile) * tblk;
+#pragma unroll
+                for (int i = 0; i < NC; i += 4) st4(hb + blk(c0 + i, row), hv + i);
+            } else if (valid) {
+#pragma unroll
+                for (int i = 0; i < NC; i += 4) st4(g.hT + (size_t)gp * H + c0 + i, hv + i);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma3_k(cta.tmem + 6 * H, uA, IMG, u + L::F, L::FS, g.nfc, H / 16);
+                if (s + 1 < g.T) mma3_k(cta.tmem + 3 * H, uA, IMG, u + L::U, L::WS, 2 * H, H / 16);
+                tc_commit(cta.bar0);
+            }
+        }
+        if (ok) {
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            if (ok) outputs(g.T - 1);
+        }
+        ok = cta.hand_over(ok);   // (the same answer in every thread)
+    }
+    cta.finish(1, L::COLS, g.status);
+}
+
+// ---------------------------------------------------------------- backward
+// The state gradients, last step first (as k_win_bwd), with dA written to
+// memory for the weight gradients: the images of three-part operands leave no
+// room for them here.  Two operands' images (B0, B1): dA_z and dA_c, then
+// dD of the next step and dA_r.  Tensor memory: dD W_fc [0, H), d(r h)
+// [64, 64 + H), dA_z U_z [128, ..), dA_r U_r [192, ..).
+template <int H> struct Bwd32Layout {
+    static constexpr int WS = H * 128;
+    static constexpr int WF = 0, UC = WF + 3 * WS, UZ = UC + 3 * WS, UR = UZ + 3 * WS, B0 = UR + 3 * WS, B1 = B0 + 3 * IMG,
+                         BARS = B1 + 3 * IMG, BYTES = BARS + 64 + 1024;
+    static constexpr int COLS = 256;
+};
+
+template <int H>
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
+    using L = Bwd32Layout<H>;
+    constexpr int NC = H / 4;
+    constexpr int T_DH = 0, T_DRH = 64, T_CZ = 128, T_CR = 192;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = align1k(smem_raw), *B0 = base + L::B0, *B1 = base + L::B1;
+    const uint32_t u = smem_u32(base);
+    build3(base + L::WF, L::WS, H, [&](int r, int c) { return c < g.n_out ? __ldg(g.Wfc + (size_t)c * H + r) : 0.f; });
+    build3(base + L::UC, L::WS, H, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)(2 * H + c) * H + r) : 0.f; });
+    build3(base + L::UZ, L::WS, H, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)c * H + r) : 0.f; });
+    build3(base + L::UR, L::WS, H, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)(H + c) * H + r) : 0.f; });
+    Cta cta;
+    cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 2, L::COLS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, part = warp >> 2, row = q * 32 + lane, c0 = part * NC;
+    const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
+    const size_t tblk = (size_t)TM * H;
+    const int kfc = g.nfc / 16;
+    uint32_t ph = 0;
+    bool ok = true;
+    // dD of a step: each thread up to 16 columns of its row (blocks of 4 dealt to the row's threads)
+    constexpr int DDN = 4;
+    float dd[DDN][4];
+    auto load_dd = [&](int s, int gp) {
+#pragma unroll
+        for (int i = 0; i < DDN; ++i) {
+            const int c = 4 * (part + 4 * i);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                dd[i][j] = gp < g.P && c + j < g.n_out ? __ldg(g.dD + ((size_t)s * g.P + gp) * g.n_out + c + j) : 0.f;
+        }
+    };
+    auto put_dd = [&](uint8_t *img) {
+#pragma unroll
+        for (int i = 0; i < DDN; ++i) {
+            const int c = 4 * (part + 4 * i);
+            if (c < g.nfc) put4_3(img, IMG, row, c, dd[i]);
+        }
+    };
+    for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
+        const int p0 = tile * TM, gp = p0 + row;
+        float zv[NC], rv[NC], cv[NC], hp[NC], cpart[NC];
+        auto load_step = [&](int s) {
+            const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+#pragma unroll
+            for (int i = 0; i < NC; i += 4) {
+                const size_t o = sb + blk(c0 + i, row);
+                ld4(g.z + o, zv + i);
+                ld4(g.r + o, rv + i);
+                ld4(g.c + o, cv + i);
+                ld4(g.hb + o, hp + i);
+            }
+        };
+        load_dd(g.T - 1, gp);
+        load_step(g.T - 1);
+        put_dd(B0);
+        if (!(ok = cta.hand_over(ok))) break;
+        if (tid == 0) {
+            mma3_k(cta.tmem + T_DH, u + L::B0, IMG, u + L::WF, L::WS, H, kfc);
+            tc_commit(cta.bar0);
+        }
+        for (int s = g.T - 1; s >= 0; --s) {
+            const size_t gb = ((size_t)s * g.ntiles + tile) * 3 * tblk;   // dA: gates z, r, c one after the other
+            if (s > 0) load_dd(s - 1, gp);
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            float dh[NC];
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float a[8], b[8], c[8], az[8], ac[8];
+                tmem_ld8(tl + T_DH + c0 + i, a);
+                tmem_ld8(tl + T_CZ + c0 + i, b);
+                tmem_ld8(tl + T_CR + c0 + i, c);
+                tmem_wait();
+                keep(a);
+                keep(b);
+                keep(c);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = i + j;
+                    const float carry = s == g.T - 1 ? 0.f : whole(b[j] + c[j], H / 16) + cpart[k];
+                    dh[k] = whole(a[j], kfc) + carry;
+                    const float dc = dh[k] * (1.0f - zv[k]), dz = dh[k] * (hp[k] - cv[k]);
+                    az[j] = dz * zv[k] * (1.0f - zv[k]);
+                    ac[j] = dc * (1.0f - cv[k] * cv[k]);
+                }
+                put8_3(B0, IMG, row, c0 + i, az);
+                put8_3(B1, IMG, row, c0 + i, ac);
+#pragma unroll
+                for (int j = 0; j < 8; j += 4) {
+                    st4(g.dG + gb + blk(c0 + i + j, row), az + j);
+                    st4(g.dG + gb + 2 * tblk + blk(c0 + i + j, row), ac + j);
+                }
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma3_k(cta.tmem + T_DRH, u + L::B1, IMG, u + L::UC, L::WS, H, H / 16);
+                mma3_k(cta.tmem + T_CZ, u + L::B0, IMG, u + L::UZ, L::WS, H, H / 16);
+                tc_commit(cta.bar0);
+            }
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+#pragma unroll
+            for (int i = 0; i < NC; i += 8) {
+                float a[8];
+                tmem_ld8(tl + T_DRH + c0 + i, a);
+                tmem_wait();
+                keep(a);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = i + j;
+                    a[j] = whole(a[j], H / 16);
+                    cpart[k] = dh[k] * zv[k] + a[j] * rv[k];
+                    a[j] = a[j] * hp[k] * rv[k] * (1.0f - rv[k]);
+                }
+                put8_3(B1, IMG, row, c0 + i, a);
+#pragma unroll
+                for (int j = 0; j < 8; j += 4) st4(g.dG + gb + tblk + blk(c0 + i + j, row), a + j);
+            }
+            if (s > 0) {
+                put_dd(B0);
+                load_step(s - 1);
+            }
+            if (!(ok = cta.hand_over(ok))) break;
+            if (tid == 0) {
+                mma3_k(cta.tmem + T_CR, u + L::B1, IMG, u + L::UR, L::WS, H, H / 16);
+                if (s > 0) mma3_k(cta.tmem + T_DH, u + L::B0, IMG, u + L::WF, L::WS, H, kfc);
+                tc_commit(cta.bar0);
+            }
+        }
+        if (ok) {
+            ok = cta.wait(0, ph);
+            ph ^= 1;
+            if (ok && g.dh0) {
+#pragma unroll
+                for (int i = 0; i < NC; i += 8) {
+                    float b[8], c[8];
+                    tmem_ld8(tl + T_CZ + c0 + i, b);
+                    tmem_ld8(tl + T_CR + c0 + i, c);
+                    tmem_wait();
+                    keep(b);
+                    keep(c);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) b[j] = whole(b[j] + c[j], H / 16) + cpart[i + j];
+                    if (gp < g.P) {
+                        st4(g.dh0 + (size_t)gp * H + c0 + i, b);
+                        st4(g.dh0 + (size_t)gp * H + c0 + i + 4, b + 4);
+                    }
+                }
+            }
+        }
+        ok = cta.hand_over(ok);   // (the same answer in every thread)
+    }
+    cta.finish(1, L::COLS, g.status);
+}
+
+// ---------------------------------------------------------------- weight gradients
+// [X | h_s]^T [dA_z, dA_r], [X | r h_s]^T dA_c and h_{s+1}^T dD over all
+// steps and rows, in blocks of 64 rows (whose operands' three parts fill the
+// shared memory): a CTA takes a contiguous range of blocks, accumulates each
+// in tensor memory, adds it to FP32 registers and these, every few blocks, to
+// a sum kept in tensor memory (a sum in one run of 67 blocks loses twice as much).
+// Bound by memory (2.6 kB a row and step at H = 64) and the splits.
+constexpr int GR = 64, GIMG = GR * 128;   // rows of a block, one image
+constexpr int G32_RUN = 8;                // blocks added up in registers before they join the sum in tensor memory
+template <int H> struct Grad32Layout {
+    // parts of one operand GIMG apart
+    static constexpr int X = 0, HP = X + 3 * GIMG, RH = HP + 3 * GIMG, HN = RH + 3 * GIMG, GZ = HN + 3 * GIMG,
+                         GRR = GZ + 3 * GIMG, GC = GRR + 3 * GIMG, DD = GC + 3 * GIMG, BARS = DD + 3 * GIMG,
+                         BYTES = BARS + 64 + 1024;
+    static constexpr int COLS = 512;        // the block's products, then sums of G32_RUN blocks from SUM on
+    static constexpr int SUM = 256;
+    static constexpr int NB = (3 * H + 64) / 8 / 4;   // blocks of 8 gradient columns a thread adds up
+};
+
+template <int H>
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
+    using L = Grad32Layout<H>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = align1k(smem_raw);
+    const uint32_t u = smem_u32(base);
+    // columns that no block writes but products of unused gradient rows read
+    for (int e = threadIdx.x; e < L::BARS / 16; e += W32_TH) reinterpret_cast<uint4 *>(base)[e] = make_uint4(0, 0, 0, 0);
+    Cta cta;
+    cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 2, L::COLS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, part = warp >> 2, row = q * 32 + lane;
+    const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
+    const int ncol = 3 * H + g.nfc;
+    const size_t tblk = (size_t)TM * H;
+    float acc[L::NB][8];
+#pragma unroll
+    for (int b = 0; b < L::NB; ++b)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[b][j] = 0.f;
+    const long long n = 2LL * g.T * g.ntiles;   // blocks: (tile, half, step), steps fastest
+    const long long i0 = n * blockIdx.x / gridDim.x, i1 = n * (blockIdx.x + 1) / gridDim.x;
+    uint32_t ph = 0;
+    bool ok = true;
+    auto drain = [&]() {   // the block's products into the registers
+        ok = cta.wait(0, ph);
+        ph ^= 1;
+#pragma unroll
+        for (int b = 0; b < L::NB; ++b) {
+            const int c = 8 * (part + 4 * b);
+            if (c < ncol) {
+                float v[8];
+                tmem_ld8(tl + c, v);
+                tmem_wait();
+                keep(v);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[b][j] += whole(v[j], GR / 16);
+            }
+        }
+    };
+    bool summed = false;
+    auto flush = [&]() {   // the registers' sums into tensor memory
+#pragma unroll
+        for (int b = 0; b < L::NB; ++b) {
+            const int c = 8 * (part + 4 * b);
+            if (c < ncol) {
+                if (summed) {
+                    float v[8];
+                    tmem_ld8(tl + L::SUM + c, v);
+                    tmem_wait();
+                    keep(v);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[b][j] += v[j];
+                }
+                tmem_st8(tl + L::SUM + c, acc[b]);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[b][j] = 0.f;
+        }
+        tmem_wait_st();
+        summed = true;
+    };
+    for (long long it = i0; it < i1; ++it) {
+        const int s = (int)(it % g.T), th = (int)(it / g.T), tile = th >> 1, r0 = (th & 1) * GR;
+        const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+        const bool last = s + 1 == g.T;
+        // the block's operands: 8 columns of a row a thread (rows fastest, so that reads are contiguous)
+        constexpr int NV = GR * (H / 8) / W32_TH > 0 ? GR * (H / 8) / W32_TH : 1;
+        const bool mine = tid < GR * (H / 8);
+        const int lr = tid & (GR - 1), lc = (tid / GR) * 8, tr = r0 + lr;   // row in the block and in the tile
+        static_assert(NV == 1, "one piece of every operand a thread");
+        float hp[8], rr[8], hn[8], az[8], ar[8], ac[8];
+        if (mine) {
+            const size_t o = sb + blk(lc, tr), o4 = sb + blk(lc + 4, tr);
+            const size_t gz = ((size_t)s * g.ntiles + tile) * 3 * tblk + blk(lc, tr), gz4 = gz + 4 * TM;
+            ld4(g.hb + o, hp); ld4(g.hb + o4, hp + 4);
+            ld4(g.r + o, rr); ld4(g.r + o4, rr + 4);
+            ld4(g.dG + gz, az); ld4(g.dG + gz4, az + 4);
+            ld4(g.dG + gz + tblk, ar); ld4(g.dG + gz4 + tblk, ar + 4);
+            ld4(g.dG + gz + 2 * tblk, ac); ld4(g.dG + gz4 + 2 * tblk, ac + 4);
+            if (!last) {
+                const size_t step = (size_t)g.ntiles * tblk;
+                ld4(g.hb + o + step, hn); ld4(g.hb + o4 + step, hn + 4);
+            } else if (tile * TM + tr < g.P) {
+                ld4(g.hT + (size_t)(tile * TM + tr) * H + lc, hn); ld4(g.hT + (size_t)(tile * TM + tr) * H + lc + 4, hn + 4);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) hn[j] = 0.f;
+            }
+        }
+        float xv[8], dv[8];   // features and dD: 8 columns of a row, 8 threads a row
+        const int xr = tid >> 3, xc = (tid & 7) * 8, gp = tile * TM + r0 + xr;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) xv[j] = dv[j] = 0.f;
+        if (gp < g.P) {
+            const float *src = g.X + ((size_t)s * g.P + gp) * g.ldx + xc;
+            if (g.xvec) {
+                if (xc < g.n_in) ld4(src, xv);
+                if (xc + 4 < g.n_in) ld4(src + 4, xv + 4);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) xv[j] = xc + j < g.n_in ? xv[j] : 0.f;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) xv[j] = xc + j < g.n_in ? __ldg(src + j) : 0.f;
+            }
+            const float *dsrc = g.dD + ((size_t)s * g.P + gp) * g.n_out + xc;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (xc + j < g.n_out) dv[j] = __ldg(dsrc + j);
+        }
+        if (it > i0) {
+            drain();   // the images are free again
+            if ((it - i0) % G32_RUN == 0) flush();
+        }
+        if (mine) {
+            put8_3(base + L::HP, GIMG, lr, lc, hp);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) rr[j] *= hp[j];
+            put8_3(base + L::RH, GIMG, lr, lc, rr);
+            put8_3(base + L::HN, GIMG, lr, lc, hn);
+            put8_3(base + L::GZ, GIMG, lr, lc, az);
+            // H = 32: dA_z and dA_r side by side in one image
+            if (H == 64) put8_3(base + L::GRR, GIMG, lr, lc, ar);
+            else put8_3(base + L::GZ, GIMG, lr, H + lc, ar);
+            put8_3(base + L::GC, GIMG, lr, lc, ac);
+        }
+        put8_3(base + L::X, GIMG, xr, xc, xv);
+        if (xc < g.nfc) put8_3(base + L::DD, GIMG, xr, xc, dv);
+        if (!(ok = cta.hand_over(ok))) break;
+        if (tid == 0) {
+            mma3_mn(cta.tmem, u + L::X, GIMG, L::HP - L::X, u + L::GZ, GIMG, L::GRR - L::GZ, 2 * H, GR);
+            mma3_mn(cta.tmem + 2 * H, u + L::X, GIMG, L::RH - L::X, u + L::GC, GIMG, GIMG, H, GR);
+            mma3_mn(cta.tmem + 3 * H, u + L::HN, GIMG, L::HP - L::X, u + L::DD, GIMG, GIMG, g.nfc, GR);
+            tc_commit(cta.bar0);
+        }
+    }
+    if (ok && i1 > i0) {
+        drain();
+        flush();
+    }
+    if (ok && summed && !*cta.abort_flag) {
+        float *o = g.part + (size_t)blockIdx.x * g.part_cols * TM;
+#pragma unroll
+        for (int b = 0; b < L::NB; ++b) {
+            const int c = 8 * (part + 4 * b);
+            if (c >= ncol) continue;
+            float v[8];
+            tmem_ld8(tl + L::SUM + c, v);
+            tmem_wait();
+            keep(v);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[(size_t)(c + j) * TM + row] = v[j];
+        }
+    }
+    cta.finish(1, L::COLS, g.status);
+}
+
+}  // namespace
+
+cudaError_t win32_forward(const WinArgs &g, int H, cudaStream_t st) {
+    const int grid = std::min(g.ntiles, sm_count());
+    if (H == 64) return launch(k_win32_fwd<64>, grid, W32_TH, Fwd32Layout<64>::BYTES, g, st);
+    return launch(k_win32_fwd<32>, grid, W32_TH, Fwd32Layout<32>::BYTES, g, st);
+}
+
+cudaError_t win32_backward(const WinArgs &g, int H, cudaStream_t st) {
+    const int sms = sm_count(), grid = std::min(g.ntiles, sms), ggrid = win32_parts(g.T, g.P);
+    cudaError_t e = H == 64 ? launch(k_win32_bwd<64>, grid, W32_TH, Bwd32Layout<64>::BYTES, g, st)
+                            : launch(k_win32_bwd<32>, grid, W32_TH, Bwd32Layout<32>::BYTES, g, st);
+    if (e != cudaSuccess) return e;
+    e = H == 64 ? launch(k_win32_grad<64>, ggrid, W32_TH, Grad32Layout<64>::BYTES, g, st)
+                : launch(k_win32_grad<32>, ggrid, W32_TH, Grad32Layout<32>::BYTES, g, st);
+    if (e != cudaSuccess) return e;
+    return win_reduce(g, H, ggrid, st);
+}
+
+// CTAs of the weight-gradient kernel, each with a partial sum of its own
+int win32_parts(int T, int P) { return (int)std::min<long long>(2LL * T * win_tiles(P), sm_count()); }
+
+}  // namespace dnnmg

@@ -1,8 +1,8 @@
-"""The fused training window (BF16 products) at the edges of its range: rows
+"""The fused training window at the edges of its range: rows
 that end inside, at and past a 128-row tile, more tiles than CTAs, the
 smallest and largest layers it takes, feature rows and arrays that do not
-start on 16 bytes, no initial state, and a precision changed between a
-window's forward and backward."""
+start on 16 bytes, no initial state, infinite features, and a precision
+changed between a window's forward and backward."""
 
 import numpy as np
 import pytest
@@ -14,7 +14,7 @@ from test_train_gpu import cu, problem
 
 pytestmark = pytest.mark.gpu
 
-TOL = 2e-2   # BF16 operands against FP64
+TOL = {"bf16": 2e-2, "f32": 1e-5}   # BF16 operands, FP32 products against FP64
 
 
 @pytest.fixture(scope="module")
@@ -37,12 +37,14 @@ def off_by_one(a):
     (3, 129, 64, 64, 64, 64, True), (2, 257, 51, 51, 64, 18, False), (1, 39000, 51, 64, 64, 18, False),
     (5, 700, 50, 52, 32, 18, True)])
 @pytest.mark.parametrize("state", [True, False])
-def test_window_matches_oracle(dn, T, P, n_in, ldx, H, n_out, shift, state):
+@pytest.mark.parametrize("prec", ["bf16", "f32"])
+def test_window_matches_oracle(dn, T, P, n_in, ldx, H, n_out, shift, state, prec):
     (X, h0, Y), W = problem(T, P, n_in, ldx, H, n_out, seed=T + P)
     h0 = h0 if state else np.zeros_like(h0)
+    tol = TOL[prec]
     wrap = off_by_one if shift else (lambda a: a)
     Xg, Wg = wrap(cu(X)), [wrap(cu(w)) for w in W]
-    tr = dn.Trainer(n_in, ldx, H, n_out, T, P, precision="bf16")
+    tr = dn.Trainer(n_in, ldx, H, n_out, T, P, precision=prec)
     D = wrap(torch.zeros(T, P, n_out, device="cuda"))
     tr.forward(Xg, wrap(cu(h0)) if state else None, *Wg, D)
     Do, cache = otrain.seq_forward(X[:, :, :n_in], h0, *W)
@@ -53,16 +55,17 @@ def test_window_matches_oracle(dn, T, P, n_in, ldx, H, n_out, shift, state):
     go = otrain.seq_backward(dD, cache, *W)
     torch.cuda.synchronize()
     assert tr.status() == 0
-    assert rel_l2(D.cpu().numpy(), Do) <= TOL
-    assert rel_l2(tr.state().cpu().numpy(), cache["hs"][-1]) <= TOL
+    assert rel_l2(D.cpu().numpy(), Do) <= tol
+    assert rel_l2(tr.state().cpu().numpy(), cache["hs"][-1]) <= tol
     for a, b, name in zip(g + [dh0], go, ("Wx", "Uh", "Wfc", "h0")):
-        assert rel_l2(a.cpu().numpy(), b) <= TOL, name
+        assert rel_l2(a.cpu().numpy(), b) <= tol, name
 
 
 @pytest.mark.parametrize("first,then", [("bf16", "f32"), ("f32", "bf16")])
 def test_precision_changed_between_forward_and_backward(dn, first, then):
     # the backward reads what the other precision's forward saved
     T, P, n_in, ldx, H, n_out = 3, 150, 51, 64, 32, 18
+    tol = TOL["bf16"]
     (X, h0, Y), W = problem(T, P, n_in, ldx, H, n_out, seed=2)
     Xg, Wg = cu(X), [cu(w) for w in W]
     tr = dn.Trainer(n_in, ldx, H, n_out, T, P)
@@ -78,4 +81,18 @@ def test_precision_changed_between_forward_and_backward(dn, first, then):
     go = otrain.seq_backward(dD, cache, *W)
     torch.cuda.synchronize()
     for a, b, name in zip(g, go, ("Wx", "Uh", "Wfc")):
-        assert rel_l2(a.cpu().numpy(), b) <= TOL, name
+        assert rel_l2(a.cpu().numpy(), b) <= tol, name
+
+
+def test_infinite_feature_saturates_the_gates(dn):
+    # FP32 operands are clamped to the largest BF16 number before they are split
+    T, P, n_in, ldx, H, n_out = 2, 5, 51, 64, 32, 18
+    (X, h0, Y), W = problem(T, P, n_in, ldx, H, n_out, seed=4)
+    X[0, 2, 7], X[1, 3, 9] = np.inf, -np.inf
+    tr = dn.Trainer(n_in, ldx, H, n_out, T, P)
+    D = torch.empty(T, P, n_out, device="cuda")
+    tr.forward(cu(X), cu(h0), *[cu(w) for w in W], D)
+    with np.errstate(over="ignore"):
+        Do, _ = otrain.seq_forward(X[:, :, :n_in], h0, *W)
+    assert np.isfinite(Do).all()
+    assert rel_l2(D.cpu().numpy(), Do) <= TOL["f32"]
