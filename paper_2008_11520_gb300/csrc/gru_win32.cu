@@ -15,7 +15,7 @@
 // Six tcgen05 products of BF16 are 316 TFLOP/s of FP32 at the measured BF16
 // rate; the CUDA cores' FMAs give 74.  With the fused window (see gru_win.cu,
 // whose layouts these kernels share) loss and gradients of 65 536 rows, T =
-// 10, H = 64 take 1.27 ms instead of 5.5 ms with one FP32 kernel per
+// 10, H = 64 take 1.23 ms instead of 5.5 ms with one FP32 kernel per
 // product, and of 762 rows, H = 32, 0.46 ms instead of 2.7 ms.
 //
 // Values beyond the largest BF16 number are clamped to it (an infinite
@@ -71,10 +71,13 @@ __device__ __forceinline__ float clamp_bf16(float x) {
     asm("{\n.reg .f32 t;\nmin.NaN.f32 t, %1, 0f7F7F0000;\nmax.NaN.f32 %0, t, 0fFF7F0000;\n}\n" : "=f"(y) : "f"(x));
     return y;
 }
-// the three parts of two values, each pair packed
-__device__ __forceinline__ void split2(float x, float y, uint32_t (&o)[3]) {
-    x = clamp_bf16(x);
-    y = clamp_bf16(y);
+// the three parts of two values, each pair packed; CL: of values that may be
+// beyond the BF16 range (the caller's arrays; states, gates and gradients are not)
+template <bool CL> __device__ __forceinline__ void split2(float x, float y, uint32_t (&o)[3]) {
+    if (CL) {
+        x = clamp_bf16(x);
+        y = clamp_bf16(y);
+    }
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const __nv_bfloat162 t = __floats2bfloat162_rn(x, y);
@@ -84,31 +87,33 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t (&o)[3]) {
     }
 }
 // 8 consecutive columns of a row into the three images, `step` bytes apart
-__device__ __forceinline__ void put8_3(uint8_t *img, int step, int row, int c, const float *v) {
+template <bool CL = false> __device__ __forceinline__ void put8_3(uint8_t *img, int step, int row, int c, const float *v) {
     uint32_t o[4][3];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) split2(v[2 * i], v[2 * i + 1], o[i]);
+    for (int i = 0; i < 4; ++i) split2<CL>(v[2 * i], v[2 * i + 1], o[i]);
     const uint32_t at = swz(row, c >> 3);
 #pragma unroll
     for (int p = 0; p < 3; ++p)
         *reinterpret_cast<uint4 *>(img + p * step + at) = make_uint4(o[0][p], o[1][p], o[2][p], o[3][p]);
 }
 // 4 consecutive columns (c a multiple of 4)
-__device__ __forceinline__ void put4_3(uint8_t *img, int step, int row, int c, const float *v) {
+template <bool CL = false> __device__ __forceinline__ void put4_3(uint8_t *img, int step, int row, int c, const float *v) {
     uint32_t a[3], b[3];
-    split2(v[0], v[1], a);
-    split2(v[2], v[3], b);
+    split2<CL>(v[0], v[1], a);
+    split2<CL>(v[2], v[3], b);
     const uint32_t at = swz(row, c >> 3) + (c & 4) * 2;
 #pragma unroll
     for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2 *>(img + p * step + at) = make_uint2(a[p], b[p]);
 }
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 template <typename F> __device__ __forceinline__ void build3(uint8_t *img, int step, int rows, F src) {
     for (int e = threadIdx.x; e < rows * 8; e += W32_TH) {
         const int r = e >> 3, c = (e & 7) * 8;
         float v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = src(r, c + i);
-        put8_3(img, step, r, c, v);   // (8-row groups are 1024 bytes apart: row * 128 throughout)
+        put8_3<true>(img, step, r, c, v);   // (8-row groups are 1024 bytes apart: row * 128 throughout)
     }
 }
 __device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &x, uint8_t *img) {
@@ -117,7 +122,7 @@ __device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &
         const int e = threadIdx.x + i * W32_TH, row = e >> 4, c = (e & 15) * 4;
         const float v[4] = {x.v[i].x, c + 1 < g.n_in ? x.v[i].y : 0.f, c + 2 < g.n_in ? x.v[i].z : 0.f,
                             c + 3 < g.n_in ? x.v[i].w : 0.f};
-        put4_3(img, IMG, row, c, v);
+        put4_3<true>(img, IMG, row, c, v);
     }
 }
 
@@ -333,7 +338,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
 #pragma unroll
         for (int i = 0; i < DDN; ++i) {
             const int c = 4 * (part + 4 * i);
-            if (c < g.nfc) put4_3(img, IMG, row, c, dd[i]);
+            if (c < g.nfc) put4_3<true>(img, IMG, row, c, dd[i]);
         }
     };
     for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
@@ -538,34 +543,33 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
         const int s = (int)(it % g.T), th = (int)(it / g.T), tile = th >> 1, r0 = (th & 1) * GR;
         const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
         const bool last = s + 1 == g.T;
-        // the block's operands: 8 columns of a row a thread (rows fastest, so that reads are contiguous)
-        constexpr int NV = GR * (H / 8) / W32_TH > 0 ? GR * (H / 8) / W32_TH : 1;
+        // the block's operands: 8 columns of a row a thread (rows fastest, so
+        // that reads are contiguous); h, r and X are read while the products
+        // of the block before run, the others brought into L2 meanwhile
         const bool mine = tid < GR * (H / 8);
         const int lr = tid & (GR - 1), lc = (tid / GR) * 8, tr = r0 + lr;   // row in the block and in the tile
-        static_assert(NV == 1, "one piece of every operand a thread");
-        float hp[8], rr[8], hn[8], az[8], ar[8], ac[8];
+        const size_t o = sb + blk(lc, tr), gz = ((size_t)s * g.ntiles + tile) * 3 * tblk + blk(lc, tr);
+        const float *hnp = last ? g.hT + (size_t)(tile * TM + tr) * H + lc : g.hb + o + (size_t)g.ntiles * tblk;
+        const int hstep = last ? 4 : 4 * TM;
+        const bool hnok = !last || tile * TM + tr < g.P;
+        const int xr = tid >> 3, xc = (tid & 7) * 8, gp = tile * TM + r0 + xr;   // X and dD: 8 threads a row
+        const float *dsrc = g.dD + ((size_t)s * g.P + gp) * g.n_out + xc;
+        float hp[8], rr[8], xv[8];
         if (mine) {
-            const size_t o = sb + blk(lc, tr), o4 = sb + blk(lc + 4, tr);
-            const size_t gz = ((size_t)s * g.ntiles + tile) * 3 * tblk + blk(lc, tr), gz4 = gz + 4 * TM;
-            ld4(g.hb + o, hp); ld4(g.hb + o4, hp + 4);
-            ld4(g.r + o, rr); ld4(g.r + o4, rr + 4);
-            ld4(g.dG + gz, az); ld4(g.dG + gz4, az + 4);
-            ld4(g.dG + gz + tblk, ar); ld4(g.dG + gz4 + tblk, ar + 4);
-            ld4(g.dG + gz + 2 * tblk, ac); ld4(g.dG + gz4 + 2 * tblk, ac + 4);
-            if (!last) {
-                const size_t step = (size_t)g.ntiles * tblk;
-                ld4(g.hb + o + step, hn); ld4(g.hb + o4 + step, hn + 4);
-            } else if (tile * TM + tr < g.P) {
-                ld4(g.hT + (size_t)(tile * TM + tr) * H + lc, hn); ld4(g.hT + (size_t)(tile * TM + tr) * H + lc + 4, hn + 4);
-            } else {
+            ld4(g.hb + o, hp); ld4(g.hb + o + 4 * TM, hp + 4);
+            ld4(g.r + o, rr); ld4(g.r + o + 4 * TM, rr + 4);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) hn[j] = 0.f;
+            for (int k = 0; k < 3; ++k) {
+                prefetch_l2(g.dG + gz + k * tblk);
+                prefetch_l2(g.dG + gz + k * tblk + 4 * TM);
+            }
+            if (hnok) {
+                prefetch_l2(hnp);
+                prefetch_l2(hnp + hstep);
             }
         }
-        float xv[8], dv[8];   // features and dD: 8 columns of a row, 8 threads a row
-        const int xr = tid >> 3, xc = (tid & 7) * 8, gp = tile * TM + r0 + xr;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) xv[j] = dv[j] = 0.f;
+        for (int j = 0; j < 8; ++j) xv[j] = 0.f;
         if (gp < g.P) {
             const float *src = g.X + ((size_t)s * g.P + gp) * g.ldx + xc;
             if (g.xvec) {
@@ -577,29 +581,44 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) xv[j] = xc + j < g.n_in ? __ldg(src + j) : 0.f;
             }
-            const float *dsrc = g.dD + ((size_t)s * g.P + gp) * g.n_out + xc;
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (xc + j < g.n_out) dv[j] = __ldg(dsrc + j);
+            if (xc < g.n_out) prefetch_l2(dsrc);
         }
         if (it > i0) {
             drain();   // the images are free again
             if ((it - i0) % G32_RUN == 0) flush();
         }
+        float az[8], ar[8];
+        if (mine) {
+            ld4(g.dG + gz, az); ld4(g.dG + gz + 4 * TM, az + 4);
+            ld4(g.dG + gz + tblk, ar); ld4(g.dG + gz + tblk + 4 * TM, ar + 4);
+        }
+        put8_3<true>(base + L::X, GIMG, xr, xc, xv);
         if (mine) {
             put8_3(base + L::HP, GIMG, lr, lc, hp);
 #pragma unroll
             for (int j = 0; j < 8; ++j) rr[j] *= hp[j];
             put8_3(base + L::RH, GIMG, lr, lc, rr);
-            put8_3(base + L::HN, GIMG, lr, lc, hn);
+            ld4(g.dG + gz + 2 * tblk, hp); ld4(g.dG + gz + 2 * tblk + 4 * TM, hp + 4);   // dA_c
+#pragma unroll
+            for (int j = 0; j < 8; ++j) rr[j] = 0.f;
+            if (hnok) {
+                ld4(hnp, rr);
+                ld4(hnp + hstep, rr + 4);
+            }
             put8_3(base + L::GZ, GIMG, lr, lc, az);
             // H = 32: dA_z and dA_r side by side in one image
             if (H == 64) put8_3(base + L::GRR, GIMG, lr, lc, ar);
             else put8_3(base + L::GZ, GIMG, lr, H + lc, ar);
-            put8_3(base + L::GC, GIMG, lr, lc, ac);
         }
-        put8_3(base + L::X, GIMG, xr, xc, xv);
-        if (xc < g.nfc) put8_3(base + L::DD, GIMG, xr, xc, dv);
+        if (xc < g.nfc) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) xv[j] = gp < g.P && xc + j < g.n_out ? __ldg(dsrc + j) : 0.f;
+            put8_3<true>(base + L::DD, GIMG, xr, xc, xv);
+        }
+        if (mine) {
+            put8_3(base + L::GC, GIMG, lr, lc, hp);
+            put8_3(base + L::HN, GIMG, lr, lc, rr);
+        }
         if (!(ok = cta.hand_over(ok))) break;
         if (tid == 0) {
             mma3_mn(cta.tmem, u + L::X, GIMG, L::HP - L::X, u + L::GZ, GIMG, L::GRR - L::GZ, 2 * H, GR);
