@@ -538,7 +538,8 @@ int dnnmg_net_create(int n_in, int hidden, int n_out, const double *Wx, const do
     n->H = hidden;
     n->n_out = n_out;
     n->precision = precision;
-    n->WxT = n->UhT = n->WfcT = n->tc_weights = nullptr;
+    n->WxT = n->UhT = n->WfcT = n->WfcTp = n->tc_weights = nullptr;
+    n->ldo = round_up(n_out, 4);
     n->tc = nullptr;
     n->d_status = nullptr;
     n->tc_bytes = 0;
@@ -576,10 +577,17 @@ int dnnmg_net_create(int n_in, int hidden, int n_out, const double *Wx, const do
     int e = upload(wx, &n->WxT);
     if (!e) e = upload(uh, &n->UhT);
     if (!e) e = upload(wfc, &n->WfcT);
+    if (!e && precision != DNNMG_BF16NET) {
+        std::vector<double> pad((size_t)hidden * n->ldo, 0.0);
+        for (int k = 0; k < hidden; ++k)
+            for (int o = 0; o < n_out; ++o) pad[(size_t)k * n->ldo + o] = wfc[(size_t)k * n_out + o];
+        e = upload(pad, &n->WfcTp);
+    }
     if (e) {
         cudaFree(n->WxT);
         cudaFree(n->UhT);
         cudaFree(n->WfcT);
+        cudaFree(n->WfcTp);
         cudaFree(n->d_status);
         delete n;
         cudaGetLastError();
@@ -601,6 +609,7 @@ int dnnmg_net_destroy(dnnmg_net_t net) {
     cudaFree(net->WxT);
     cudaFree(net->UhT);
     cudaFree(net->WfcT);
+    cudaFree(net->WfcTp);
     cudaFree(net->tc_weights);
     cudaFree(net->d_status);
     tc_release(*net);

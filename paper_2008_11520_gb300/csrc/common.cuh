@@ -116,6 +116,9 @@ struct Net {
     void *tc;                     // tensor-core schedule (gru_tc.cu), null if not used
     // transposed weights for the CUDA-core kernel: WxT [ldx][3H], UhT [H][3H], WfcT [H][n_out]
     void *WxT, *UhT, *WfcT;
+    // WfcT with rows padded by zeros to ldo = round_up(n_out, 4) (F32 and F64 nets)
+    void *WfcTp;
+    int ldo;
     // K-major bf16 operands for the tensor-core kernel (BF16NET only, may be null)
     void *tc_weights;
     size_t tc_bytes;
