@@ -11,6 +11,8 @@
 //            bfloat16), float accumulation and float gate arithmetic; the
 //            stored state h stays float.  This is the same arithmetic as the
 //            tensor-core kernel, so the two can be compared tightly.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace dnnmg {
@@ -145,7 +147,7 @@ k_gru(int n_in, int ldx, int H, int n_out, const TW *__restrict__ X, const TW *_
 // after the other from zero, as k_gru's does: the same bits.
 // FP32: 8 patches and 4 columns a thread, operations on patch pairs in packed
 // form.  16 336 patches, 99 inputs, H = 64, 50 outputs: k_gru 123 us,
-// this 64 us; bound by the weights' way from L2 (each CTA reads all of them).  FP64 runs at two FMA a clock and SM, so
+// this 58 us; bound by latency (the weights' way from L2, staging).  FP64 runs at two FMA a clock and SM, so
 // there the tile is small (2 columns of 1 patch) and few patches are spread
 // over the chip: 254 patches, 51 inputs, H = 32: k_gru 83 us (32 CTAs), this
 // 38 us (both under ncu, cold caches).
@@ -158,50 +160,68 @@ template <typename T, int JT, int PT> struct RTile {
             for (int p = 0; p < PT; ++p) a[j][p] = T(0);
     }
     // a += W[0 .. n)[j] x[0 .. n)[p], rows of W ldw apart, of x ldp apart
-    __device__ __forceinline__ void mac(const T *__restrict__ W, int ldw, const T *x, int ldp, int n);
+    template <bool SW> __device__ __forceinline__ void mac(const T *W, int ldw, const T *x, int ldp, int n);
 };
-template <> __device__ __forceinline__ void RTile<float, 4, 8>::mac(const float *__restrict__ W, int ldw, const float *x,
-                                                                   int ldp, int n) {
-    unsigned long long c[4][4];   // patch pairs
+// a weight vector from shared memory (SW) or, through the read-only path, from global
+template <bool SW, typename V, typename T> __device__ __forceinline__ V load_w(const T *p) {
+    if constexpr (SW) return *reinterpret_cast<const V *>(p);
+    else return __ldg(reinterpret_cast<const V *>(p));
+}
+// PT patches (4 or 8) of 4 columns, patch pairs packed
+template <bool SW, int PT>
+__device__ __forceinline__ void mac_f32(float (&a)[4][PT], const float *W, int ldw, const float *x, int ldp, int n) {
+    unsigned long long c[4][PT / 2];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int p = 0; p < 4; ++p) asm("mov.b64 %0, {%1, %2};" : "=l"(c[j][p]) : "f"(a[j][2 * p]), "f"(a[j][2 * p + 1]));
+        for (int p = 0; p < PT / 2; ++p) asm("mov.b64 %0, {%1, %2};" : "=l"(c[j][p]) : "f"(a[j][2 * p]), "f"(a[j][2 * p + 1]));
 #pragma unroll 4
     for (int k = 0; k < n; ++k) {
-        const float4 w = __ldg(reinterpret_cast<const float4 *>(W + (size_t)k * ldw));
-        const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(x + k * ldp);
-        const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(x + k * ldp + 4);
-        const unsigned long long xv[4] = {x0.x, x0.y, x1.x, x1.y};
+        const float4 w = load_w<SW, float4>(W + (size_t)k * ldw);
+        unsigned long long xv[PT / 2];
+#pragma unroll
+        for (int p = 0; p < PT / 2; p += 2) {
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(x + k * ldp + 2 * p);
+            xv[p] = t.x;
+            xv[p + 1] = t.y;
+        }
         const float wv[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             unsigned long long ww;
             asm("mov.b64 %0, {%1, %1};" : "=l"(ww) : "f"(wv[j]));
 #pragma unroll
-            for (int p = 0; p < 4; ++p) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[j][p]) : "l"(ww), "l"(xv[p]));
+            for (int p = 0; p < PT / 2; ++p) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[j][p]) : "l"(ww), "l"(xv[p]));
         }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int p = 0; p < 4; ++p) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[j][2 * p]), "=f"(a[j][2 * p + 1]) : "l"(c[j][p]));
+        for (int p = 0; p < PT / 2; ++p) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[j][2 * p]), "=f"(a[j][2 * p + 1]) : "l"(c[j][p]));
 }
-template <> __device__ __forceinline__ void RTile<double, 2, 1>::mac(const double *__restrict__ W, int ldw, const double *x,
-                                                                    int ldp, int n) {
+template <> template <bool SW>
+__device__ __forceinline__ void RTile<float, 4, 8>::mac(const float *W, int ldw, const float *x, int ldp, int n) {
+    mac_f32<SW, 8>(a, W, ldw, x, ldp, n);
+}
+template <> template <bool SW>
+__device__ __forceinline__ void RTile<float, 4, 4>::mac(const float *W, int ldw, const float *x, int ldp, int n) {
+    mac_f32<SW, 4>(a, W, ldw, x, ldp, n);
+}
+template <> template <bool SW>
+__device__ __forceinline__ void RTile<double, 2, 1>::mac(const double *W, int ldw, const double *x, int ldp, int n) {
 #pragma unroll 4
     for (int k = 0; k < n; ++k) {
-        const double2 w = __ldg(reinterpret_cast<const double2 *>(W + (size_t)k * ldw));
+        const double2 w = load_w<SW, double2>(W + (size_t)k * ldw);
         const double xv = x[k * ldp];
         a[0][0] = fma(w.x, xv, a[0][0]);
         a[1][0] = fma(w.y, xv, a[1][0]);
     }
 }
 
-template <typename T, int TP, int JT, int PT, int THREADS>
+template <typename T, int TP, int JT, int PT, int THREADS, bool SW>
 __global__ void __launch_bounds__(THREADS)
-k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, const T *__restrict__ WxT,
-         const T *__restrict__ UhT, const T *__restrict__ WfcT, T *__restrict__ h, T *__restrict__ d, int P) {
+k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, const T *WxT, const T *UhT, const T *WfcT, T *__restrict__ h, T *__restrict__ d, int P) {
+    static_assert(TP % PT == 0, "whole tiles");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int LP = TP + (TP > 4 ? 16 / (int)sizeof(T) : 0);   // staged row length (padded against bank conflicts)
     T *xs = reinterpret_cast<T *>(smem_raw);   // [n_in][LP] features
@@ -209,78 +229,122 @@ k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, 
     T *zs = hs + H * LP;                       // [H][LP] update gate
     T *rh = zs + H * LP;                       // [H][LP] r * h
     T *gh = rh + H * LP;                       // [H][LP] W_h x, then the new state
-    const int p0 = blockIdx.x * TP, np = min(TP, P - p0), G = 3 * H;
-    for (int i = threadIdx.x; i < TP * n_in; i += THREADS) {
-        const int p = i / n_in, k = i - p * n_in;
-        xs[k * LP + p] = p < np ? __ldg(X + (size_t)(p0 + p) * ldx + k) : T(0);
+    const int G = 3 * H;
+    if constexpr (SW) {
+        // the weights stay in shared memory for all of this CTA's patches (sizes are whole 16-byte pieces)
+        T *ws = gh + H * LP;
+        const T *src[3] = {WxT, UhT, WfcT};
+        const int cnt[3] = {n_in * G, H * G, H * ldo};
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            constexpr int EPC = 16 / sizeof(T);
+            for (int i = threadIdx.x * EPC; i < cnt[m]; i += THREADS * EPC)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(ws + i)),
+                             "l"(src[m] + i)
+                             : "memory");
+            if (m == 0) WxT = ws;
+            else if (m == 1) UhT = ws;
+            else WfcT = ws;
+            ws += cnt[m];
+        }
     }
-    for (int i = threadIdx.x; i < TP * H; i += THREADS) {
-        const int p = i / H, k = i - p * H;
-        hs[k * LP + p] = p < np ? h[(size_t)(p0 + p) * H + k] : T(0);
-    }
-    __syncthreads();
-    constexpr int PG = TP / PT;
-    RTile<T, JT, PT> t;
-    // z, r and W_h x: a tile lies in one gate (H is a multiple of JT)
-    for (int e = threadIdx.x; e < G / JT * PG; e += THREADS) {
-        const int jg = e % (G / JT), pg = e / (G / JT), j = jg * JT, p = pg * PT, gate = j / H, jj = j - gate * H;
-        t.zero();
-        t.mac(WxT + j, G, xs + p, LP, n_in);
-        if (gate < 2) t.mac(UhT + j, G, hs + p, LP, H);
-#pragma unroll
-        for (int a = 0; a < JT; ++a)
-#pragma unroll
-            for (int b = 0; b < PT; ++b) {
-                const int o = (jj + a) * LP + p + b;
-                if (gate == 0) zs[o] = sigm(t.a[a][b]);
-                else if (gate == 1) rh[o] = sigm(t.a[a][b]) * hs[o];
-                else gh[o] = t.a[a][b];
-            }
-    }
-    __syncthreads();
-    // candidate and state update
-    for (int e = threadIdx.x; e < H / JT * PG; e += THREADS) {
-        const int jg = e % (H / JT), pg = e / (H / JT), j = jg * JT, p = pg * PT;
-#pragma unroll
-        for (int a = 0; a < JT; ++a)
-#pragma unroll
-            for (int b = 0; b < PT; ++b) t.a[a][b] = gh[(j + a) * LP + p + b];
-        t.mac(UhT + 2 * H + j, G, rh + p, LP, H);
-#pragma unroll
-        for (int a = 0; a < JT; ++a)
-#pragma unroll
-            for (int b = 0; b < PT; ++b) {
-                const int o = (j + a) * LP + p + b;
-                const T z = zs[o];
-                gh[o] = z * hs[o] + (T(1) - z) * tanh_(t.a[a][b]);
-            }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < np * H; i += THREADS) {
-        const int p = i / H, k = i - p * H;
-        h[(size_t)(p0 + p) * H + k] = gh[k * LP + p];
-    }
-    // output layer d = W_fc h' (rows of WfcT ldo long, zero past n_out)
-    for (int e = threadIdx.x; e < ldo / JT * PG; e += THREADS) {
-        const int og = e % (ldo / JT), pg = e / (ldo / JT), o = og * JT, p = pg * PT;
-        t.zero();
-        t.mac(WfcT + o, ldo, gh + p, LP, H);
-#pragma unroll
-        for (int b = 0; b < PT; ++b)
+    for (long long q0 = (long long)blockIdx.x * TP; q0 < P; q0 += (long long)gridDim.x * TP) {
+        const int p0 = (int)q0, np = min(TP, P - p0);
+        for (int i = threadIdx.x; i < TP * n_in; i += THREADS) {
+            const int p = i / n_in, k = i - p * n_in;
+            xs[k * LP + p] = p < np ? __ldg(X + (size_t)(p0 + p) * ldx + k) : T(0);
+        }
+        for (int i = threadIdx.x; i < TP * H; i += THREADS) {
+            const int p = i / H, k = i - p * H;
+            hs[k * LP + p] = p < np ? h[(size_t)(p0 + p) * H + k] : T(0);
+        }
+        if constexpr (SW) asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        constexpr int PG = TP / PT;
+        RTile<T, JT, PT> t;
+        // the two short products have a third of the columns: half the patches a tile
+        constexpr int PT2 = PT > 4 ? PT / 2 : PT, PG2 = TP / PT2;
+        RTile<T, JT, PT2> t2;
+        // z, r and W_h x: a tile lies in one gate (H is a multiple of JT)
+        for (int e = threadIdx.x; e < G / JT * PG; e += THREADS) {
+            const int jg = e % (G / JT), pg = e / (G / JT), j = jg * JT, p = pg * PT, gate = j / H, jj = j - gate * H;
+            t.zero();
+            t.template mac<SW>(WxT + j, G, xs + p, LP, n_in);
+            if (gate < 2) t.template mac<SW>(UhT + j, G, hs + p, LP, H);
 #pragma unroll
             for (int a = 0; a < JT; ++a)
-                if (p + b < np && o + a < n_out) d[(size_t)(p0 + p + b) * n_out + o + a] = t.a[a][b];
+#pragma unroll
+                for (int b = 0; b < PT; ++b) {
+                    const int o = (jj + a) * LP + p + b;
+                    if (gate == 0) zs[o] = sigm(t.a[a][b]);
+                    else if (gate == 1) rh[o] = sigm(t.a[a][b]) * hs[o];
+                    else gh[o] = t.a[a][b];
+                }
+        }
+        __syncthreads();
+        // candidate and state update
+        for (int e = threadIdx.x; e < H / JT * PG2; e += THREADS) {
+            const int jg = e % (H / JT), pg = e / (H / JT), j = jg * JT, p = pg * PT2;
+#pragma unroll
+            for (int a = 0; a < JT; ++a)
+#pragma unroll
+                for (int b = 0; b < PT2; ++b) t2.a[a][b] = gh[(j + a) * LP + p + b];
+            t2.template mac<SW>(UhT + 2 * H + j, G, rh + p, LP, H);
+#pragma unroll
+            for (int a = 0; a < JT; ++a)
+#pragma unroll
+                for (int b = 0; b < PT2; ++b) {
+                    const int o = (j + a) * LP + p + b;
+                    const T z = zs[o];
+                    gh[o] = z * hs[o] + (T(1) - z) * tanh_(t2.a[a][b]);
+                }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < np * H; i += THREADS) {
+            const int p = i / H, k = i - p * H;
+            h[(size_t)(p0 + p) * H + k] = gh[k * LP + p];
+        }
+        // output layer d = W_fc h' (rows of WfcT ldo long, zero past n_out)
+        for (int e = threadIdx.x; e < ldo / JT * PG2; e += THREADS) {
+            const int og = e % (ldo / JT), pg = e / (ldo / JT), o = og * JT, p = pg * PT2;
+            t2.zero();
+            t2.template mac<SW>(WfcT + o, ldo, gh + p, LP, H);
+#pragma unroll
+            for (int b = 0; b < PT2; ++b)
+#pragma unroll
+                for (int a = 0; a < JT; ++a)
+                    if (p + b < np && o + a < n_out) d[(size_t)(p0 + p + b) * n_out + o + a] = t2.a[a][b];
+        }
+        __syncthreads();   // the staged values are free for the next patches
     }
 }
 
-template <typename T, int TP, int JT, int PT, int THREADS>
+int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return n > 0 ? n : 1;
+}
+size_t weight_count(const Net &n) { return (size_t)3 * n.H * (n.n_in + n.H) + (size_t)n.H * n.ldo; }
+// bytes of the weights and the staged values of TP patches (row length LP)
+size_t rt_bytes(const Net &n, int LP, size_t elem) {
+    return elem * ((size_t)LP * (n.n_in + 4 * n.H) + weight_count(n));
+}
+
+template <typename T, int TP, int JT, int PT, int THREADS, bool SW>
 cudaError_t run_rt(const Net &n, const void *X, void *h, void *d, int P, cudaStream_t st) {
     constexpr int LP = TP + (TP > 4 ? 16 / (int)sizeof(T) : 0);
-    const size_t sm = sizeof(T) * (size_t)LP * (n.n_in + 4 * n.H);
-    auto k = k_gru_rt<T, TP, JT, PT, THREADS>;
+    const size_t sm = sizeof(T) * ((size_t)LP * (n.n_in + 4 * n.H) + (SW ? weight_count(n) : 0));
+    auto k = k_gru_rt<T, TP, JT, PT, THREADS, SW>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<(P + TP - 1) / TP, THREADS, sm, st>>>(n.n_in, n.ldx, n.H, n.n_out, n.ldo, (const T *)X, (const T *)n.WxT,
+    int grid = (P + TP - 1) / TP;
+    if (SW) {   // persistent: as many CTAs as fit
+        int per = 1;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, THREADS, sm)) != cudaSuccess) return e;
+        grid = std::min(grid, std::max(1, per) * sm_count());
+    }
+    k<<<grid, THREADS, sm, st>>>(n.n_in, n.ldx, n.H, n.n_out, n.ldo, (const T *)X, (const T *)n.WxT,
                                               (const T *)n.UhT, (const T *)n.WfcTp, (T *)h, (T *)d, P);
     return cudaGetLastError();
 }
@@ -303,11 +367,22 @@ cudaError_t run(const Net &n, const void *X, void *h, void *d, int P, cudaStream
 cudaError_t launch_gru_cuda_core(const Net &n, const void *X, void *h, void *d, int P,
                                  cudaStream_t st) {
     if (P == 0) return cudaSuccess;
-    // the register-tiled kernel where its staged values fit a quarter of an SM's
-    // shared memory (several CTAs an SM cover the staging); else one column a thread
+    // the register-tiled kernel, its weights in shared memory where they fit; else
+    // one column a thread
     if (n.WfcTp && n.H % 4 == 0 && n.n_in + 4 * n.H <= 512) {
-        if (n.precision == DNNMG_F32) return run_rt<float, 32, 4, 8, 192>(n, X, h, d, P, st);
-        if (n.precision == DNNMG_F64) return run_rt<double, 2, 2, 1, 128>(n, X, h, d, P, st);
+        constexpr size_t lim = 225 * 1024;
+        if (n.precision == DNNMG_F32) {
+            // one tile or less an SM: weights staged once, narrow tiles on twice the warps
+            // (99 -> 64 -> 50: 4000 patches 25 against 35 us); more tiles: several CTAs an SM
+            // read them from L2 (16 336 patches 58 against 78 us)
+            if ((P + 31) / 32 <= sm_count() && rt_bytes(n, 36, 4) <= lim)
+                return run_rt<float, 32, 4, 4, 384, true>(n, X, h, d, P, st);
+            return run_rt<float, 32, 4, 8, 192, false>(n, X, h, d, P, st);
+        }
+        if (n.precision == DNNMG_F64) {
+            if (rt_bytes(n, 2, 8) <= lim) return run_rt<double, 2, 2, 1, 128, true>(n, X, h, d, P, st);
+            return run_rt<double, 2, 2, 1, 128, false>(n, X, h, d, P, st);
+        }
     }
     if (n.precision == DNNMG_F64) return run<double, double, 8>(n, X, h, d, P, st);
     if (n.precision == DNNMG_F32) return run<float, float, 16>(n, X, h, d, P, st);
