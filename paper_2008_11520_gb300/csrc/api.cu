@@ -407,8 +407,10 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
     g.solid = m->d_solid;
     g.patch_id = m->d_patch_id;
     g.patch_cell = m->d_patch_cell;
-    std::vector<int> tab((size_t)I.ldx);
-    feature_table(g, tab.data());
+    // the column tables of both tile sizes, one after the other
+    std::vector<int> tab(2 * (size_t)I.ldx);
+    feature_table(g, tab.data(), false);
+    feature_table(g, tab.data() + I.ldx, true);
     m->d_feat_tab = nullptr;
     if (cudaMalloc(&m->d_feat_tab, tab.size() * sizeof(int)) != cudaSuccess ||
         cudaMemcpy(m->d_feat_tab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -421,6 +423,7 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
         return fail(DNNMG_ENOMEM, "device allocation of the feature table failed");
     }
     g.feat_tab = m->d_feat_tab;
+    g.feat_tab_small = m->d_feat_tab + I.ldx;
     tile_counts(g, &g.ntx, &g.nty);
     std::vector<uint8_t> tflags((size_t)g.ntx * g.nty);
     tile_flags(g, solid.data(), tflags.data());
@@ -457,12 +460,17 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
     std::vector<int> slow;
     residual_cf_slow_tiles(g, tflags.data(), &slow);
     g.n_slow_tiles = (int)slow.size();
+    std::vector<int> small;
+    small_tiles_of(g, slow, &small);
+    g.n_slow_small = (int)small.size();
+    slow.insert(slow.end(), small.begin(), small.end());
     m->d_slow_tiles = nullptr;
     if (cudaMalloc(&m->d_slow_tiles, (slow.size() ? slow.size() : 1) * sizeof(int)) != cudaSuccess ||
         (slow.size() && cudaMemcpy(m->d_slow_tiles, slow.data(), slow.size() * sizeof(int),
                                    cudaMemcpyHostToDevice) != cudaSuccess))
         return undo("boundary tile list");
     g.slow_tiles = m->d_slow_tiles;
+    g.slow_small = m->d_slow_tiles + g.n_slow_tiles;
     std::vector<uint16_t> ctab((size_t)I.ldx);
     residual_cf_table(g, ctab.data());
     m->d_cf_tab = nullptr;

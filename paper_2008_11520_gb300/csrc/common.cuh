@@ -50,10 +50,13 @@ struct MeshGeom {
     const int *patch_id;          // device [npy][npx], fluid patch number or -1
     const int *patch_cell;        // device [P], pj npx + pi
     const int *feat_tab;          // device [ldx], source of each feature column (stencil.cu)
+    const int *feat_tab_small;    // the same for 8 x 8-cell tiles
     const uint8_t *tile_flags;    // device [nty][ntx], all-fluid bits of each 32 x 16-cell tile
     int ntx, nty;
     const int *slow_tiles;        // device [n_slow_tiles]: tiles without the all-fluid bit (ty ntx + tx)
     int n_slow_tiles;
+    const int *slow_small;        // the 8 x 8-cell tiles of those, in their own numbering
+    int n_slow_small;
     const uint16_t *cf_tab;       // device [ldx]: feature column sources of the closed-form tiles
     int *status;                  // device status word of the mesh (DNNMG_DEVERR_* bits)
 };
@@ -190,8 +193,9 @@ cudaError_t launch_gemm_tc(int M, int N, int K, const void *A, int lda, const vo
 int gemm_tc_splits_used(int K, int splits);
 void tc_release(Net &n);
 // Per feature column: (kind << 24) | offset into the residual / node tiles of stencil.cu.
-void feature_table(const MeshGeom &g, int *tab);
+void feature_table(const MeshGeom &g, int *tab, bool small);
 int feature_table_capacity();
+void small_tiles_of(const MeshGeom &g, const std::vector<int> &big, std::vector<int> *out);
 // Per 32 x 16-cell stencil tile (ntx x nty of them): bit 0 = every fine cell
 // within two cells of the tile exists and is fluid, bit 1 = the same within one.
 void tile_flags(const MeshGeom &g, const uint8_t *solid, uint8_t *flags);

@@ -19,12 +19,28 @@
 namespace dnnmg {
 namespace {
 
-constexpr int TXC = 32;            // fine cells per tile in x
+constexpr int TXC = 32;            // fine cells per tile in x (the tile flags' grid, and every FP32 tile)
 constexpr int TYC = 16;            // fine cells per tile in y
-constexpr int NXN = TXC + 1;       // tile nodes in x
-constexpr int NYN = TYC + 1;
 constexpr int NTHREADS = 256;
-constexpr int RES_THREADS = 256;   // residual/feature kernels (10 warps measured slower)
+// A tile of X x Y fine cells and the threads that work on it (10 warps for
+// the residual of a 32 x 16 tile measured slower).
+template <int X, int Y, int TH> struct TileDim {
+    static constexpr int TXC = X, TYC = Y, NXN = X + 1, NYN = Y + 1, THREADS = TH;
+    static constexpr int LX = X == 32 ? 5 : X == 16 ? 4 : 3;   // log2 X
+    static_assert(X == 1 << LX, "power of two");
+};
+using BigTile = TileDim<TXC, TYC, 256>;
+// Few tiles: a 32 x 16 tile is 16 us of latency in FP32 and 80 us of work in
+// FP64 (two FMA a clock and SM) on one SM while the rest of the chip idles.
+// 64 x 16 cells in FP64 (2 tiles): residual and features 80 -> 26 us,
+// right-hand side 29 -> 9 us; 256 x 64 in FP32 (32 tiles): 24.5 -> 9 and
+// 5.7 -> 4.6 us; bound by the chain of staging, cell and node passes.
+using SmallTile = TileDim<8, 8, 128>;
+// Whether a launch over n tiles of 32 x 16 cells takes 8 x 8 ones instead:
+// where the large ones would not fill the chip twice over (patches have to
+// fit a tile).  Every node's arithmetic is the same in both.
+inline bool use_small(const MeshGeom &g, long long n) { return g.S <= SmallTile::TXC && n < 304; }
+inline long long tiles_of(const MeshGeom &g) { return (long long)g.ntx * g.nty; }
 
 template <typename TX, typename T> __device__ __forceinline__ TX store_as(T v) { return (TX)v; }
 template <> __device__ __forceinline__ __nv_bfloat16 store_as<__nv_bfloat16, float>(float v) {
@@ -67,6 +83,7 @@ __device__ __forceinline__ bool tile_fluid(const MeshGeom &g, int tx, int ty, in
 __device__ __forceinline__ bool node_tile_fluid(const MeshGeom &g, int bx, int by) {
     return tile_fluid(g, 2 * bx, by, 2) && tile_fluid(g, 2 * bx + 1, by, 2);
 }
+
 
 // Asynchronous 16-byte copy global -> shared; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_bytes) {
@@ -389,11 +406,12 @@ __device__ __forceinline__ void convection(const ConvK<V> &k, const V (&u)[4], c
 }
 
 // Shared-memory layout of the residual/feature tile (element counts).  The
-// node window of x~ spans columns I0-4 .. I0+35 (16-byte aligned; node I0+ii
-// at column ii+4) and rows J0-2 .. J0+18 (node J0+jj at row jj+2).
-struct ResLayout {
-    static constexpr int HX = 40, HY = NYN + 4, XO = 4, YO = 2, HP = HX * HY;
-    static constexpr int BX = 36;                              // b_f window: columns I0 .. I0+35
+// node window of x~ spans columns I0-4 .. I0+TXC+3 (16-byte aligned; node I0+ii
+// at column ii+4) and rows J0-2 .. J0+TYC+2 (node J0+jj at row jj+2).
+template <typename D> struct ResLayout {
+    static constexpr int TXC = D::TXC, TYC = D::TYC, NXN = D::NXN, NYN = D::NYN;
+    static constexpr int HX = TXC + 8, HY = NYN + 4, XO = 4, YO = 2, HP = HX * HY;
+    static constexpr int BX = TXC + 4;                         // b_f window: columns I0 .. I0+TXC+3
     static constexpr int CX = TXC + 2, CY = TYC + 2;           // cells -1 .. 32 x -1 .. 16
     static constexpr int NCELL = CX * CY;
     // cell contributions: one array per (component, corner), pitch NCP; the
@@ -430,12 +448,12 @@ enum { FEAT_RES = 0, FEAT_VEL = 1, FEAT_PECLET = 2, FEAT_GEO = 3, FEAT_ZERO = 4 
 // along x on the cell's bottom and top edges are formed once and the R
 // nodes of the item read off them, with the arithmetic of CoarseWin::interp
 // (same bits).  Lanes take consecutive columns.
-template <typename T, int R, typename CWin>
+template <typename D, typename T, int R, typename CWin>
 __device__ __forceinline__ void interp_window(const CWin &cw, int I0, int J0, T *xs) {
-    using L = ResLayout;
+    using L = ResLayout<D>;
     constexpr int K = Log2<R>::v;
     constexpr T inv_r = T(1) / T(R);
-    // J0 is a multiple of 16, so the window's first row sits OFFY rows into its coarse cell
+    // J0 is a multiple of 8, so the window's first row sits OFFY rows into its coarse cell
     constexpr int OFFY = (R - L::YO % R) % R;
     constexpr int NKY = (L::HY + OFFY + R - 1) / R;
     for (int e = threadIdx.x; e < NKY * L::HX; e += blockDim.x) {
@@ -564,13 +582,14 @@ __device__ __forceinline__ void ld2(const double *p, double &a, double &b) {
 // convection comes from the per-cell contributions in cc.  The zero centre
 // column of the x-gradient/divergence stencils (zero centre row in y) is
 // skipped.  Window values and cell contributions are read as aligned pairs.
-// Nodes 2bx+1 = 33 and 2by+1 = 17 lie past the tile and are discarded.
-template <typename T, typename TX>
+// Nodes 2bx+1 = TXC+1 and 2by+1 = TYC+1 lie past the tile and are discarded.
+template <typename D, typename T, typename TX>
 __device__ __forceinline__ void block_residual(const MeshGeom &g, const FemCoef<T> &fc, const T *xs,
                                                const T *bs, const T *cc, const int *pid, int tpx, int tpy,
                                                int lS, int I0, int J0, int bx, int by, T *__restrict__ rf,
                                                TX *__restrict__ X, TX *rres) {
-    using L = ResLayout;
+    using L = ResLayout<D>;
+    constexpr int NYN = D::NYN;
     T Au[2][2], Av[2][2], Ap[2][2];   // [dy][dx]: velocity rows and pressure row of A(x~) x~
 #pragma unroll
     for (int dy = 0; dy < 2; ++dy)
@@ -681,14 +700,16 @@ __device__ __forceinline__ void block_residual(const MeshGeom &g, const FemCoef<
 // b_f window, xs the x~ window (R = 0) or cw the coarse window (R > 0), pid
 // the tile's patch numbers, geo_s the geometry features, fast the tile's
 // all-fluid flag.  Shared by the per-tile kernel and the persistent one.
-template <typename T, typename TX, int R, typename CWin>
+template <typename D, typename T, typename TX, int R, typename CWin>
 __device__ __forceinline__ void residual_tile(const MeshGeom &g, const FemCoef<T> &fc, const CWin &cw,
                                               double inflow_peak, T *xs, const T *bs, T *cc, T *un, const int *pid,
                                               unsigned char *cf, const T *geo_s, bool fast, int I0, int J0,
                                               T *__restrict__ rf, TX *__restrict__ X) {
-    using L = ResLayout;
+    using L = ResLayout<D>;
+    constexpr int TXC = D::TXC, TYC = D::TYC, NXN = D::NXN, NYN = D::NYN;
     const int lS = g.K + g.s - 1;   // S = s 2^K with s = 1, 2
     const int tpx = TXC >> lS, tpy = TYC >> lS;
+    const int *feat_tab = TXC == dnnmg::TXC ? g.feat_tab : g.feat_tab_small;
     if (!fast) {
         for (int idx = threadIdx.x; idx < L::FX * L::FY; idx += blockDim.x) {
             const int jj = idx / L::FX, ii = idx - jj * L::FX;
@@ -696,7 +717,7 @@ __device__ __forceinline__ void residual_tile(const MeshGeom &g, const FemCoef<T
         }
     }
     if constexpr (R > 0) {
-        interp_window<T, R>(cw, I0, J0, xs);
+        interp_window<D, T, R>(cw, I0, J0, xs);
         if (!fast) {
             // the Dirichlet velocity where a window node has one (fast tiles
             // have none within the cells they use)
@@ -724,11 +745,11 @@ __device__ __forceinline__ void residual_tile(const MeshGeom &g, const FemCoef<T
         for (int tp = warp; tp < tpx * tpy; tp += nw) {
             const int id = pid[tp];
             if (id < 0) continue;
-            const int lpy = tp >> (5 - lS), lpx = tp & (tpx - 1);
+            const int lpy = tp >> (D::LX - lS), lpx = tp & (tpx - 1);
             const T *xbase = xs + lpy * S * L::HX + lpx * S;
             TX *row = X + (size_t)id * g.ldx;
             for (int c = nres + lane; c < g.ldx; c += 32) {
-                const int e = __ldg(g.feat_tab + c);
+                const int e = __ldg(feat_tab + c);
                 const int kind = e >> 24, off = e & 0xFFFFFF;
                 const int o = kind <= FEAT_PECLET ? off : 0;
                 const T a = xbase[o], b = xbase[o + L::HP];
@@ -747,12 +768,12 @@ __device__ __forceinline__ void residual_tile(const MeshGeom &g, const FemCoef<T
         for (int tp = warp; tp < tpx * tpy; tp += nw) {
             const int id = pid[tp];
             if (id < 0) continue;
-            const int lpy = tp >> (5 - lS), lpx = tp & (tpx - 1);
+            const int lpy = tp >> (D::LX - lS), lpx = tp & (tpx - 1);
             const T *xbase = xs + lpy * S * L::HX + lpx * S;
             const TX *rbase = rres + lpy * S * L::RXP + lpx * S;
             TX *row = X + (size_t)id * g.ldx;
             for (int c = 2 * lane; c < g.ldx; c += 64) {
-                const int2 ee = __ldg(reinterpret_cast<const int2 *>(g.feat_tab + c));
+                const int2 ee = __ldg(reinterpret_cast<const int2 *>(feat_tab + c));
                 TX out[2];
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
@@ -810,14 +831,15 @@ __device__ __forceinline__ void residual_tile(const MeshGeom &g, const FemCoef<T
         // that holds it while idle warps write the other columns.
         constexpr bool kGather = 3 * L::RPL * sizeof(TX) <= L::LC * sizeof(T);
         TX *rres = kGather ? reinterpret_cast<TX *>(un) : nullptr;
-        // 16 blocks of one row per half-warp (contiguous pairs: conflict-free
+        // the blocks of one row on consecutive lanes (contiguous pairs: conflict-free
         // 64-bit loads), then the last block column
         constexpr int BW = (L::NB + 31) / 32;   // warps of the block pass
         if (threadIdx.x < L::NB) {
             const int t = threadIdx.x;
-            const bool main = t < 16 * L::NBY;
-            const int bx = main ? (t & 15) : L::NBX - 1, by = main ? (t >> 4) : t - 16 * L::NBY;
-            block_residual(g, fc, xs, bs, cc, pid, tpx, tpy, lS, I0, J0, bx, by, rf, X, rres);
+            constexpr int W = L::NBX - 1;
+            const bool main = t < W * L::NBY;
+            const int bx = main ? (t % W) : L::NBX - 1, by = main ? (t / W) : t - W * L::NBY;
+            block_residual<D>(g, fc, xs, bs, cc, pid, tpx, tpy, lS, I0, J0, bx, by, rf, X, rres);
         } else if (!kGather && threadIdx.x >= 32 * BW) {
             patch_inputs(BW, (int)(blockDim.x >> 5) - BW);
         }
@@ -953,11 +975,12 @@ __device__ __forceinline__ void residual_tile(const MeshGeom &g, const FemCoef<T
 // the caller); R = 2, 4, 8: x~ is interpolated from the coarse vector xc
 // inside the tile (S1 fused: x~ never reaches HBM), with the Dirichlet
 // values set where the tile touches a boundary.
-template <typename T, typename TX, int R>
-__global__ void __launch_bounds__(RES_THREADS)
+template <typename D, typename T, typename TX, int R>
+__global__ void __launch_bounds__(D::THREADS)
 k_residual_features(MeshGeom g, FemCoef<T> fc, const T *__restrict__ xf, const double *__restrict__ xc,
                     double inflow_peak, const T *__restrict__ bf, T *__restrict__ rf, TX *__restrict__ X) {
-    using L = ResLayout;
+    using L = ResLayout<D>;
+    constexpr int TXC = D::TXC, TYC = D::TYC, NYN = D::NYN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T geo_s[12];
     T *xs = reinterpret_cast<T *>(smem_raw);   // [3][HY][HX]   u, v, p
@@ -981,7 +1004,7 @@ k_residual_features(MeshGeom g, FemCoef<T> fc, const T *__restrict__ xf, const d
         stage_window<T, 3, L::HY, L::HX>(g, xf, I0 - L::XO, J0 - L::YO, xs);
     }
     for (int e = threadIdx.x; e < tpx * tpy; e += blockDim.x) {
-        const int py = e >> (5 - lS), px = e & (tpx - 1);
+        const int py = e >> (D::LX - lS), px = e & (tpx - 1);
         const int pi = (I0 >> lS) + px, pj = (J0 >> lS) + py;
         pid[e] = (pi < g.npx && pj < g.npy) ? g.patch_id[pj * g.npx + pi] : -1;
     }
@@ -989,9 +1012,9 @@ k_residual_features(MeshGeom g, FemCoef<T> fc, const T *__restrict__ xf, const d
     // fast tiles: every cell within two of the tile is fluid and exists, so
     // no tile node is a boundary node and node stencils apply everywhere
     // (the barrier inside also publishes the coarse window, pid and geo_s)
-    const bool fast = tile_fluid(g, blockIdx.x, blockIdx.y, 1);
+    const bool fast = tile_fluid(g, I0 / dnnmg::TXC, J0 / dnnmg::TYC, 1);
     __syncthreads();   // publishes the coarse window, pid and geo_s
-    residual_tile<T, TX, R>(g, fc, cw, inflow_peak, xs, bs, cc, un, pid, cf, geo_s, fast, I0, J0, rf, X);
+    residual_tile<D, T, TX, R>(g, fc, cw, inflow_peak, xs, bs, cc, un, pid, cf, geo_s, fast, I0, J0, rf, X);
 }
 
 // ------------------------------------------------------------------ S1 staging
@@ -999,13 +1022,13 @@ k_residual_features(MeshGeom g, FemCoef<T> fc, const T *__restrict__ xf, const d
 // that the step's tiles fetch coarse windows by TMA (the coarse planes have
 // an odd row length, which a TMA stride cannot express) and convert nothing.
 template <typename T>
-__global__ void __launch_bounds__(NTHREADS)
-k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int pc) {
+__device__ __forceinline__ void coarse_pad_cta(const MeshGeom &g, const double *__restrict__ xc, T *__restrict__ xcp,
+                                               int pc, int block, int nblocks) {
     // four consecutive outputs of one padded row per thread (pc is a multiple
     // of 32, so they never straddle rows and leave as one aligned store)
     const int nc1 = g.nxc + 1, quads = pc / 4;
     const long long nq = 3LL * (g.nyc + 1) * quads;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nq; e += (long long)gridDim.x * blockDim.x) {
+    for (long long e = (long long)block * blockDim.x + threadIdx.x; e < nq; e += (long long)nblocks * blockDim.x) {
         const long long row = e / quads;
         const int i = (int)(e - row * quads) * 4;
         const double *src = xc + row * nc1;   // rows of [3][nyc+1][nxc+1] are consecutive
@@ -1016,12 +1039,18 @@ k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int
     }
 }
 
+template <typename T>
+__global__ void __launch_bounds__(NTHREADS)
+k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int pc) {
+    coarse_pad_cta(g, xc, xcp, pc, blockIdx.x, gridDim.x);
+}
+
 // Shared-memory layout of the TMA-fed residual kernel (bytes; the TMA
 // destinations 128-byte aligned): the work buffers of ResLayout plus the
 // b_f window and the coarse window as TMA boxes.
-template <typename T, int R>
+template <typename D, typename T, int R>
 struct StepLayout {
-    using L = ResLayout;
+    using L = ResLayout<D>;
     using CWin = CoarseWin<T, R, L::HX, L::HY, 3, 4>;
     static constexpr size_t BS_BYTES = sizeof(T) * L::BS, CS_BYTES = sizeof(T) * CWin::N;
     static constexpr size_t BSB = 0;                                             // [2][NYN][BX]
@@ -1040,23 +1069,15 @@ struct StepLayout {
 // while the others load the patch numbers; then as residual_tile.  The wait
 // is bounded: on time-out the mesh status gets DNNMG_DEVERR_TIMEOUT and the
 // CTA returns once its copies have landed.
-template <typename T, typename TX, int R>
-__global__ void __launch_bounds__(RES_THREADS)
-k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmB,
-                const __grid_constant__ CUtensorMap tmC, double inflow_peak, TX *__restrict__ X,
-                const int *__restrict__ tile_list) {
-    using L = ResLayout;
-    using SL = StepLayout<T, R>;
+template <typename D, typename T, typename TX, int R>
+__device__ __forceinline__ void residual_step_cta(const MeshGeom &g, const FemCoef<T> &fc, const CUtensorMap *tmB,
+                                                  const CUtensorMap *tmC, double inflow_peak, TX *__restrict__ X, int tx,
+                                                  int ty) {
+    using L = ResLayout<D>;
+    using SL = StepLayout<D, T, R>;
+    constexpr int TXC = D::TXC, TYC = D::TYC;
     using CWin = typename SL::CWin;
     constexpr int K = Log2<R>::v;
-    // tile_list (when the closed-form kernel does the all-fluid tiles): the
-    // other tiles, one per CTA; otherwise the grid covers every tile
-    int tx = blockIdx.x, ty = blockIdx.y;
-    if (tile_list) {
-        const int tile = __ldg(tile_list + blockIdx.x);
-        ty = tile / g.ntx;
-        tx = tile - ty * g.ntx;
-    }
     extern __shared__ unsigned char smem_raw[];
     __shared__ T geo_s[12];
     // aligned by an offset from the shared-memory symbol itself, so that every
@@ -1081,18 +1102,18 @@ k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap t
         *abort_flag = 0;
         ptx::mbar_init_fence();
         ptx::expect_tx(mb_u, (uint32_t)(SL::BS_BYTES + SL::CS_BYTES));
-        ptx::tma_load_3d(ptx::smem_u32(base + SL::BSB), &tmB, I0, J0, 0, mb_u);
-        ptx::tma_load_3d(ptx::smem_u32(base + SL::CSB), &tmC, cw.ci0, cw.cj0, 0, mb_u);
+        ptx::tma_load_3d(ptx::smem_u32(base + SL::BSB), tmB, I0, J0, 0, mb_u);
+        ptx::tma_load_3d(ptx::smem_u32(base + SL::CSB), tmC, cw.ci0, cw.cj0, 0, mb_u);
     }
     const int lS = g.K + g.s - 1;
     const int tpx = TXC >> lS, tpy = TYC >> lS;
     for (int e = threadIdx.x; e < tpx * tpy; e += blockDim.x) {
-        const int py = e >> (5 - lS), px = e & (tpx - 1);
+        const int py = e >> (D::LX - lS), px = e & (tpx - 1);
         const int pi = (I0 >> lS) + px, pj = (J0 >> lS) + py;
         pid[e] = (pi < g.npx && pj < g.npy) ? __ldg(g.patch_id + pj * g.npx + pi) : -1;
     }
     if (threadIdx.x < 12) geo_s[threadIdx.x] = fc.geo[threadIdx.x];
-    const bool fast = tile_fluid(g, tx, ty, 1);
+    const bool fast = tile_fluid(g, I0 / dnnmg::TXC, J0 / dnnmg::TYC, 1);
     __syncthreads();   // the barrier is initialised; pid and geo_s are visible
     const bool ok = ptx::mbar_test(mb_u, 0) || ptx::mbar_wait(mb_u, 0, abort_flag);
     if (__syncthreads_or(!ok)) {
@@ -1103,7 +1124,23 @@ k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap t
         }
         return;
     }
-    residual_tile<T, TX, R>(g, fc, cw, inflow_peak, xs, bs, cc, un, pid, cf, geo_s, fast, I0, J0, nullptr, X);
+    residual_tile<D, T, TX, R>(g, fc, cw, inflow_peak, xs, bs, cc, un, pid, cf, geo_s, fast, I0, J0, nullptr, X);
+}
+
+template <typename D, typename T, typename TX, int R>
+__global__ void __launch_bounds__(D::THREADS)
+k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmB,
+                const __grid_constant__ CUtensorMap tmC, double inflow_peak, TX *__restrict__ X,
+                const int *__restrict__ tile_list) {
+    // tile_list (when the closed-form kernel does the all-fluid tiles): the
+    // other tiles, one per CTA; otherwise the grid covers every tile
+    int tx = blockIdx.x, ty = blockIdx.y;
+    if (tile_list) {
+        const int tile = __ldg(tile_list + blockIdx.x), ntx = (g.nxf + D::TXC - 1) / D::TXC;
+        ty = tile / ntx;
+        tx = tile - ty * ntx;
+    }
+    residual_step_cta<D, T, TX, R>(g, fc, &tmB, &tmC, inflow_peak, X, tx, ty);
 }
 
 // ------------------------------------------------------------------ S5
@@ -1228,23 +1265,26 @@ struct PatchWin {
 // exist): one 4-node run of one row per thread, with the patch numbers read
 // from the global patch map so that the loads of d are in flight while the
 // coarse window is staged.  Same arithmetic as the general path, same bits.
-template <typename T, int R, typename CWin>
+template <int PTY, typename T, int R, typename CWin>
 __device__ __forceinline__ void scatter_fast_tile(const MeshGeom &g, const T *__restrict__ d, const T *__restrict__ xf,
                                                   const double *__restrict__ xc, const T *__restrict__ xcp, int pc,
                                                   T *__restrict__ vc, CWin &cw, int I0, int J0) {
-    static_assert(NTHREADS == (PTX / 4) * PTY, "one run per thread");
-    const int Ib = I0 + 4 * (threadIdx.x & (PTX / 4 - 1)), J = J0 + threadIdx.x / (PTX / 4);
+    static_assert(NTHREADS >= (PTX / 4) * PTY, "at most one run per thread");
+    const bool mine = threadIdx.x < (PTX / 4) * PTY;
+    const int Ib = I0 + 4 * (threadIdx.x & (PTX / 4 - 1)), J = J0 + (mine ? threadIdx.x / (PTX / 4) : 0);
     const size_t node = (size_t)J * g.pitch + Ib;   // 4-aligned in a 64-aligned row
     T su[4], sv[4];
     int cnt[4];
-    PatchWin::run4(g, d, g.K + g.s - 1, Ib, J, su, sv, cnt);
+    if (mine) PatchWin::run4(g, d, g.K + g.s - 1, Ib, J, su, sv, cnt);
     T x[2][4];
     if constexpr (R > 0) {
         if (xcp) cw.stage_padded(g, xcp, pc, I0, J0);
         else cw.stage(g, xc, I0, J0);
         __syncthreads();   // publishes the staged coarse nodes
+        if (!mine) return;
         cw.interp4(Ib, J, x);
     } else {
+        if (!mine) return;
         load4(xf + node, x[0]);
         load4(xf + g.plane + node, x[1]);
     }
@@ -1254,28 +1294,26 @@ __device__ __forceinline__ void scatter_fast_tile(const MeshGeom &g, const T *__
     store4(vc + g.plane + node, x[1]);
 }
 
-// A CTA owns 64 x 16 nodes.  All-fluid tiles with S >= 4 take
+// A CTA owns 64 x PTY nodes (16; 4 on meshes of few tiles: four rows a thread
+// of a 64 x 16 tile took 15 us in FP64).  All-fluid tiles with S >= 4 take
 // scatter_fast_tile; otherwise lanes take consecutive nodes of a row (so the
 // reads of d are contiguous runs of each patch row), each thread 4 rows.
 // R = 0: v~ is read from xf; R = 2, 4, 8: v~ is interpolated from xc inside
 // the tile (S1 fused).  Registers are capped for the fast tiles' occupancy;
 // the rare general tiles may spill.
-template <typename T, int R>
-__global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 6 : 4)
-k_scatter_avg(MeshGeom g, const T *__restrict__ d, const T *__restrict__ xf, const double *__restrict__ xc,
-              const T *__restrict__ xcp, int pc, double inflow_peak, T *__restrict__ vc) {
+template <typename T, int R, int PTY>
+__device__ __forceinline__ void scatter_cta(const MeshGeom &g, const T *__restrict__ d, const T *__restrict__ xf,
+                                            const double *__restrict__ xc, const T *__restrict__ xcp, int pc,
+                                            double inflow_peak, T *__restrict__ vc, int bx, int by) {
     using CWin = CoarseWin<T, (R > 0 ? R : 2), PTX, PTY, 2>;
     __shared__ T cs_mem[R > 0 ? CWin::N : 1];
     __shared__ int pid_s[(PTX / 2 + 2) * (PTY / 2 + 2)];   // S = 2 holds the most patches
-    // the first and the two last tile rows (walls: general tiles, the slowest)
-    // are scheduled first, so that they do not form the grid's tail
-    const int ny = gridDim.y, by = blockIdx.y < 3 ? (blockIdx.y ? ny - blockIdx.y : 0) : blockIdx.y - 2;
-    const int I0 = blockIdx.x * PTX, J0 = by * PTY;
-    const bool fast = node_tile_fluid(g, blockIdx.x, by);
+    const int I0 = bx * PTX, J0 = by * PTY;
+    const bool fast = node_tile_fluid(g, bx, J0 / TYC);
     CWin cw;
     cw.cs = cs_mem;
     if (fast && g.K + g.s - 1 >= 2) {
-        scatter_fast_tile<T, R>(g, d, xf, xc, xcp, pc, vc, cw, I0, J0);
+        scatter_fast_tile<PTY, T, R>(g, d, xf, xc, xcp, pc, vc, cw, I0, J0);
         return;
     }
     PatchWin pw;
@@ -1338,11 +1376,22 @@ k_scatter_avg(MeshGeom g, const T *__restrict__ d, const T *__restrict__ xf, con
     }
 }
 
+template <typename T, int R, int PTY>
+__global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 6 : 4)
+k_scatter_avg(MeshGeom g, const T *__restrict__ d, const T *__restrict__ xf, const double *__restrict__ xc,
+              const T *__restrict__ xcp, int pc, double inflow_peak, T *__restrict__ vc) {
+    // the first and the two last tile rows (walls: general tiles, the slowest)
+    // are scheduled first, so that they do not form the grid's tail
+    const int ny = gridDim.y, by = blockIdx.y < 3 ? (blockIdx.y ? ny - blockIdx.y : 0) : blockIdx.y - 2;
+    scatter_cta<T, R, PTY>(g, d, xf, xc, xcp, pc, inflow_peak, vc, blockIdx.x, by);
+}
+
 // ------------------------------------------------------------------ S6
-// Node window of v_corr: columns I0-4 .. I0+35 (node I0+ii at column ii+4),
-// rows J0-1 .. J0+17 (node J0+jj at row jj+1).
-struct RhsLayout {
-    static constexpr int HX = 40, HY = NYN + 2, XO = 4, YO = 1, HP = HX * HY;
+// Node window of v_corr: columns I0-4 .. I0+TXC+3 (node I0+ii at column ii+4),
+// rows J0-1 .. J0+TYC+1 (node J0+jj at row jj+1).
+template <typename D> struct RhsLayout {
+    static constexpr int TXC = D::TXC, TYC = D::TYC, NYN = D::NYN;
+    static constexpr int HX = TXC + 8, HY = NYN + 2, XO = 4, YO = 1, HP = HX * HY;
     static constexpr int CX = TXC + 2, CY = TYC + 2;   // cells -1 .. 32 x -1 .. 16
     static constexpr int NCELL = CX * CY;
     static constexpr int NCP = NCELL + 4;              // corner arrays, as in ResLayout
@@ -1363,10 +1412,11 @@ struct RhsLayout {
 // the node stencil of the linear term plus the four cells' convection
 // corners, read as aligned pairs; 16 blocks of a row per half-warp.  Other
 // tiles: element by element with the cell codes cf.
-template <typename T>
+template <typename D, typename T>
 __device__ __forceinline__ void rhs_tile(const MeshGeom &g, const FemCoef<T> &fc, const T *vs, T *cc,
                                          const unsigned char *cf, bool fast, int I0, int J0, T *__restrict__ bf) {
-    using L = RhsLayout;
+    using L = RhsLayout<D>;
+    constexpr int TXC = D::TXC, TYC = D::TYC, NXN = D::NXN, NYN = D::NYN;
     if (fast) {
         using V = typename Packed<T>::type;
         const ConvK<V> k2(fc);
@@ -1396,7 +1446,7 @@ __device__ __forceinline__ void rhs_tile(const MeshGeom &g, const FemCoef<T> &fc
         }
         __syncthreads();
         if (threadIdx.x < (TXC / 2) * (TYC / 2)) {
-            const int bx = threadIdx.x & 15, by = threadIdx.x >> 4;   // nodes 2bx .. 2bx+1, 2by .. 2by+1
+            const int bx = threadIdx.x % (TXC / 2), by = threadIdx.x / (TXC / 2);   // nodes 2bx .. 2bx+1, 2by .. 2by+1
             // window rows 2by-1 .. 2by+2, columns 2bx-2 .. 2bx+3 (even start: aligned pairs)
             const T *w = vs + (2 * by + L::YO - 1) * L::HX + 2 * bx + L::XO - 2;
             T Bu[2][2], Bv[2][2];
@@ -1505,10 +1555,11 @@ __device__ __forceinline__ void rhs_tile(const MeshGeom &g, const FemCoef<T> &fc
 // outside the mesh read as zero) while the others classify the cells of
 // boundary tiles.  The wait is bounded: on time-out the mesh status gets
 // DNNMG_DEVERR_TIMEOUT and the CTA returns once its copy has landed.
-template <typename T>
-__global__ void __launch_bounds__(NTHREADS)
-k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__restrict__ bf) {
-    using L = RhsLayout;
+template <typename D, typename T>
+__device__ __forceinline__ void rhs_cta(const MeshGeom &g, const FemCoef<T> &fc, const CUtensorMap *tmV, T *__restrict__ bf,
+                                        int tx, int ty) {
+    using L = RhsLayout<D>;
+    constexpr int TXC = D::TXC, TYC = D::TYC;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((128u - (ptx::smem_u32(smem_raw) & 127u)) & 127u);
     T *vs = reinterpret_cast<T *>(base);   // [2][HY][HX]
@@ -1517,15 +1568,15 @@ k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__r
     uint64_t *mb = reinterpret_cast<uint64_t *>(base + (sizeof(T) * (L::VS + L::CC) + L::NCELL + 7) / 8 * 8);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(mb + 1);
     const uint32_t mb_u = ptx::smem_u32(mb);
-    const int I0 = blockIdx.x * TXC, J0 = blockIdx.y * TYC;
+    const int I0 = tx * TXC, J0 = ty * TYC;
     if (threadIdx.x == 0) {
         ptx::mbar_init(mb_u, 1);
         *abort_flag = 0;
         ptx::mbar_init_fence();
         ptx::expect_tx(mb_u, (uint32_t)(sizeof(T) * L::VS));
-        ptx::tma_load_3d(ptx::smem_u32(vs), &tmV, I0 - L::XO, J0 - L::YO, 0, mb_u);
+        ptx::tma_load_3d(ptx::smem_u32(vs), tmV, I0 - L::XO, J0 - L::YO, 0, mb_u);
     }
-    const bool fast = tile_fluid(g, blockIdx.x, blockIdx.y, 2);
+    const bool fast = tile_fluid(g, I0 / dnnmg::TXC, J0 / dnnmg::TYC, 2);
     if (!fast) {
         for (int idx = threadIdx.x; idx < L::NCELL; idx += blockDim.x) {
             const int jj = idx / L::CX, ii = idx - jj * L::CX;
@@ -1542,7 +1593,13 @@ k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__r
         }
         return;
     }
-    rhs_tile(g, fc, vs, cc, cf, fast, I0, J0, bf);
+    rhs_tile<D>(g, fc, vs, cc, cf, fast, I0, J0, bf);
+}
+
+template <typename D, typename T>
+__global__ void __launch_bounds__(D::THREADS)
+k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__restrict__ bf) {
+    rhs_cta<D>(g, fc, &tmV, bf, blockIdx.x, blockIdx.y);
 }
 
 // S5 + S6 fused for the correction step: the v_corr window of a right-hand
@@ -1558,7 +1615,7 @@ k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__r
 // the cell contributions of the right-hand side, then the cell codes.
 template <typename T>
 struct AvgRhsLayout {
-    using L = RhsLayout;
+    using L = RhsLayout<BigTile>;
     // patches holding the nodes I0-1 .. I0+33, J0-1 .. J0+17 that S6 reads
     static __host__ __device__ int npw(int lS) { return ((TXC + 1) >> lS) + 2; }
     static __host__ __device__ int nph(int lS) { return ((TYC + 1) >> lS) + 2; }
@@ -1577,7 +1634,7 @@ template <typename T, int R>
 __global__ void __launch_bounds__(NTHREADS)
 k_avg_rhs(MeshGeom g, FemCoef<T> fc, const T *__restrict__ d, const double *__restrict__ xc, double inflow_peak,
           T *__restrict__ bf, int region) {
-    using L = RhsLayout;
+    using L = RhsLayout<BigTile>;
     using AL = AvgRhsLayout<T>;
     using CWin = CoarseWin<T, R, L::HX, L::HY, 2>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1661,7 +1718,7 @@ k_avg_rhs(MeshGeom g, FemCoef<T> fc, const T *__restrict__ d, const double *__re
         vs[L::HP + e] = v;
     }
     __syncthreads();
-    rhs_tile(g, fc, vs, cc, cf, fast, I0, J0, bf);
+    rhs_tile<BigTile>(g, fc, vs, cc, cf, fast, I0, J0, bf);
 }
 
 // ------------------------------------------------------------------ S7
@@ -1712,8 +1769,8 @@ constexpr int RFW = 128 + 16, RXO = 8;
 // outside the mesh read as zero); the wait is bounded (on time-out the mesh
 // status gets DNNMG_DEVERR_TIMEOUT and the CTA returns once the copy has landed).
 template <typename T, typename Acc, int R>
-__global__ void __launch_bounds__(NTHREADS)
-k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restrict__ bc) {
+__device__ __forceinline__ void restrict_cta(const MeshGeom &g, const CUtensorMap *tmB, double *__restrict__ bc, int tx,
+                                             int ty) {
     using Row = typename Acc::Row;
     constexpr int TCX = 128 / R, TCY = 32 / R;              // coarse nodes per tile
     constexpr int FH = TCY * R + R - 1;                     // fine rows staged
@@ -1724,13 +1781,13 @@ k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restri
     uint64_t *mb = reinterpret_cast<uint64_t *>(rs + 2 * FH * TCX);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(mb + 1);
     const uint32_t mb_u = ptx::smem_u32(mb);
-    const int ci0 = blockIdx.x * TCX, cj0 = blockIdx.y * TCY;
+    const int ci0 = tx * TCX, cj0 = ty * TCY;
     if (threadIdx.x == 0) {
         ptx::mbar_init(mb_u, 1);
         *abort_flag = 0;
         ptx::mbar_init_fence();
         ptx::expect_tx(mb_u, (uint32_t)(sizeof(T) * 2 * FH * RFW));
-        ptx::tma_load_3d(ptx::smem_u32(fs), &tmB, ci0 * R - RXO, cj0 * R - (R - 1), 0, mb_u);
+        ptx::tma_load_3d(ptx::smem_u32(fs), tmB, ci0 * R - RXO, cj0 * R - (R - 1), 0, mb_u);
     }
     __syncthreads();   // the barrier is initialised
     const bool ok = ptx::mbar_test(mb_u, 0) || ptx::mbar_wait(mb_u, 0, abort_flag);
@@ -1783,22 +1840,33 @@ k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restri
 }
 
 template <typename T, typename Acc, int R>
+__global__ void __launch_bounds__(NTHREADS)
+k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restrict__ bc) {
+    restrict_cta<T, Acc, R>(g, &tmB, bc, blockIdx.x, blockIdx.y);
+}
+
+template <typename T, typename Acc, int R>
 size_t restrict_smem() {
     const size_t FH = (size_t)(32 / R) * R + R - 1;
     // fine window (TMA box), x-restricted rows, barrier and abort flag, alignment slack
     return 2 * FH * RFW * sizeof(T) + 2 * FH * (128 / R) * sizeof(typename Acc::Row) + 16 + 128;
 }
 
-template <typename T, typename Acc, int R>
-cudaError_t run_restrict(const MeshGeom &g, const T *bf, double *bc, cudaStream_t st) {
-    constexpr int TCX = 128 / R, TCY = 32 / R, FH = TCY * R + R - 1;
-    // b_f [2][nyf+1][pitch]: boxes of RFW columns x FH rows x 2 components
-    CUtensorMap tm;
+// b_f [2][nyf+1][pitch]: boxes of RFW columns x FH rows x 2 components
+template <typename T, int R> bool restrict_map(const MeshGeom &g, const T *bf, CUtensorMap *tm) {
+    constexpr int TCY = 32 / R, FH = TCY * R + R - 1;
     const CUtensorMapDataType dt = sizeof(T) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t dims[3] = {(cuuint64_t)g.nxf + 1, (cuuint64_t)g.nyf + 1, 2};
     const cuuint64_t str[2] = {(cuuint64_t)g.pitch * sizeof(T), (cuuint64_t)g.plane * sizeof(T)};
     const cuuint32_t box[3] = {(cuuint32_t)RFW, (cuuint32_t)FH, 2};
-    if (!tma_encode_tiled(&tm, dt, 3, const_cast<T *>(bf), dims, str, box)) return cudaErrorInvalidValue;
+    return tma_encode_tiled(tm, dt, 3, const_cast<T *>(bf), dims, str, box);
+}
+
+template <typename T, typename Acc, int R>
+cudaError_t run_restrict(const MeshGeom &g, const T *bf, double *bc, cudaStream_t st) {
+    constexpr int TCX = 128 / R, TCY = 32 / R;
+    CUtensorMap tm;
+    if (!restrict_map<T, R>(g, bf, &tm)) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)((g.nxc + TCX) / TCX), (unsigned)((g.nyc + TCY) / TCY));
     const size_t sm = restrict_smem<T, Acc, R>();
     cudaError_t e = cudaFuncSetAttribute(k_restrict<T, Acc, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -1843,8 +1911,8 @@ __global__ void k_mesh_maps(MeshGeom g, unsigned char *flags, unsigned char *mul
 dim3 node_grid(const MeshGeom &g) {
     return dim3((unsigned)((g.nxf + 1 + NTHREADS - 1) / NTHREADS), (unsigned)(g.nyf + 1));
 }
-dim3 tile_grid(const MeshGeom &g) {
-    return dim3((unsigned)((g.nxf + TXC - 1) / TXC), (unsigned)((g.nyf + TYC - 1) / TYC));
+template <typename D = BigTile> dim3 tile_grid(const MeshGeom &g) {
+    return dim3((unsigned)((g.nxf + D::TXC - 1) / D::TXC), (unsigned)((g.nyf + D::TYC - 1) / D::TYC));
 }
 dim3 node_tile_grid(const MeshGeom &g) {
     return dim3((unsigned)((g.nxf + PTX) / PTX), (unsigned)((g.nyf + PTY) / PTY));
@@ -1860,8 +1928,9 @@ cudaError_t set_smem(KernelT k, size_t bytes) {
 // Column sources of a feature row, in the order of Sec. 5.2 inputs:
 // residual (u, v, p) on the fine patch nodes, v~ (u, v) and the Peclet number
 // on the coarse patch nodes, 12 geometry values, zero padding to ldx.
-void feature_table(const MeshGeom &g, int *tab) {
-    using L = ResLayout;
+namespace {
+template <typename D> void feature_table_of(const MeshGeom &g, int *tab) {
+    using L = ResLayout<D>;
     const int S1 = g.S + 1, s1 = g.s + 1;
     int c = 0;
     for (int comp = 0; comp < 3; ++comp)
@@ -1876,8 +1945,27 @@ void feature_table(const MeshGeom &g, int *tab) {
     for (int k = 0; k < 12; ++k) tab[c++] = (FEAT_GEO << 24) | k;
     while (c < g.ldx) tab[c++] = FEAT_ZERO << 24;
 }
+}  // namespace
 
-int feature_table_capacity() { return ResLayout::MAX_LDX; }
+void feature_table(const MeshGeom &g, int *tab, bool small) {
+    if (small) feature_table_of<SmallTile>(g, tab);
+    else feature_table_of<BigTile>(g, tab);
+}
+
+int feature_table_capacity() { return ResLayout<BigTile>::MAX_LDX; }
+
+// The 8 x 8-cell tiles of the listed 32 x 16-cell tiles, in their own numbering.
+void small_tiles_of(const MeshGeom &g, const std::vector<int> &big, std::vector<int> *out) {
+    constexpr int SX = TXC / SmallTile::TXC, SY = TYC / SmallTile::TYC;
+    const int nsx = (g.nxf + SmallTile::TXC - 1) / SmallTile::TXC, nsy = (g.nyf + SmallTile::TYC - 1) / SmallTile::TYC;
+    out->clear();
+    for (int t : big)
+        for (int b = 0; b < SY; ++b)
+            for (int a = 0; a < SX; ++a) {
+                const int x = t % g.ntx * SX + a, y = t / g.ntx * SY + b;
+                if (x < nsx && y < nsy) out->push_back(y * nsx + x);
+            }
+}
 
 void tile_counts(const MeshGeom &g, int *ntx, int *nty) {
     *ntx = (g.nxf + TXC - 1) / TXC;
@@ -1924,27 +2012,34 @@ cudaError_t launch_prolongate(const MeshGeom &g, int prec, const double *xc, voi
     return run_prolongate(g, xc, (float *)xf, w, st);
 }
 
-template <typename T, typename TX, int R>
+template <typename D, typename T, typename TX, int R>
 cudaError_t run_residual(const MeshGeom &g, const FemCoef<T> &fc, const void *xf, const double *xc, double w,
                          const void *bf, void *rf, void *X, cudaStream_t st) {
-    auto k = k_residual_features<T, TX, R>;
-    const size_t sm = ResLayout::bytes<T>();
+    auto k = k_residual_features<D, T, TX, R>;
+    const size_t sm = ResLayout<D>::template bytes<T>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<tile_grid(g), RES_THREADS, sm, st>>>(g, fc, (const T *)xf, xc, w, (const T *)bf, (T *)rf, (TX *)X);
+    k<<<tile_grid<D>(g), D::THREADS, sm, st>>>(g, fc, (const T *)xf, xc, w, (const T *)bf, (T *)rf, (TX *)X);
     return cudaGetLastError();
+}
+
+template <typename D, typename T, typename TX>
+cudaError_t run_residual_d(const MeshGeom &g, const FemCoef<T> &fc, const void *xf, const double *xc, double w,
+                           const void *bf, void *rf, void *X, cudaStream_t st) {
+    if (!xc) return run_residual<D, T, TX, 0>(g, fc, xf, xc, w, bf, rf, X, st);
+    switch (g.r) {
+        case 2: return run_residual<D, T, TX, 2>(g, fc, xf, xc, w, bf, rf, X, st);
+        case 4: return run_residual<D, T, TX, 4>(g, fc, xf, xc, w, bf, rf, X, st);
+        case 8: return run_residual<D, T, TX, 8>(g, fc, xf, xc, w, bf, rf, X, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename T, typename TX>
 cudaError_t run_residual_r(const MeshGeom &g, const FemCoef<T> &fc, const void *xf, const double *xc, double w,
                            const void *bf, void *rf, void *X, cudaStream_t st) {
-    if (!xc) return run_residual<T, TX, 0>(g, fc, xf, xc, w, bf, rf, X, st);
-    switch (g.r) {
-        case 2: return run_residual<T, TX, 2>(g, fc, xf, xc, w, bf, rf, X, st);
-        case 4: return run_residual<T, TX, 4>(g, fc, xf, xc, w, bf, rf, X, st);
-        case 8: return run_residual<T, TX, 8>(g, fc, xf, xc, w, bf, rf, X, st);
-        default: return cudaErrorInvalidValue;
-    }
+    if (use_small(g, tiles_of(g))) return run_residual_d<SmallTile, T, TX>(g, fc, xf, xc, w, bf, rf, X, st);
+    return run_residual_d<BigTile, T, TX>(g, fc, xf, xc, w, bf, rf, X, st);
 }
 
 cudaError_t launch_residual_features(const MeshGeom &g, int prec, const FemCoef<double> &f64,
@@ -1973,47 +2068,61 @@ cudaError_t launch_coarse_pad(const MeshGeom &g, int prec, const double *xc, voi
     return run_coarse_pad(g, xc, (float *)xcp, st);
 }
 
-template <typename T, typename TX, int R>
-cudaError_t run_residual_step(const MeshGeom &g, const FemCoef<T> &fc, const T *xcp, double up, const T *bf, TX *X,
-                              cudaStream_t st, bool skip_fast) {
-    using L = ResLayout;
-    using SL = StepLayout<T, R>;
+template <typename D, typename T, int R>
+bool residual_maps(const MeshGeom &g, const T *bf, const T *xcp, CUtensorMap *tmB, CUtensorMap *tmC) {
+    using L = ResLayout<D>;
+    using SL = StepLayout<D, T, R>;
     const CUtensorMapDataType dt = sizeof(T) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     // b_f [2][nyf+1][pitch]: boxes of BX columns x NYN rows x 2 components
-    CUtensorMap tmB, tmC;
     const cuuint64_t bd[3] = {(cuuint64_t)g.nxf + 1, (cuuint64_t)g.nyf + 1, 2};
     const cuuint64_t bs[2] = {(cuuint64_t)g.pitch * sizeof(T), (cuuint64_t)g.plane * sizeof(T)};
-    const cuuint32_t bb[3] = {(cuuint32_t)L::BX, (cuuint32_t)NYN, 2};
+    const cuuint32_t bb[3] = {(cuuint32_t)L::BX, (cuuint32_t)D::NYN, 2};
     // padded coarse vector [3][nyc+1][pc]: boxes of the coarse window
     const int pc = coarse_pitch(g);
     const cuuint64_t cd[3] = {(cuuint64_t)g.nxc + 1, (cuuint64_t)g.nyc + 1, 3};
     const cuuint64_t cs[2] = {(cuuint64_t)pc * sizeof(T), (cuuint64_t)pc * (g.nyc + 1) * sizeof(T)};
     const cuuint32_t cb[3] = {(cuuint32_t)SL::CWin::CW, (cuuint32_t)SL::CWin::CH, 3};
-    if (!tma_encode_tiled(&tmB, dt, 3, const_cast<T *>(bf), bd, bs, bb) ||
-        !tma_encode_tiled(&tmC, dt, 3, const_cast<T *>(xcp), cd, cs, cb))
-        return cudaErrorInvalidValue;
-    auto k = k_residual_step<T, TX, R>;
+    return tma_encode_tiled(tmB, dt, 3, const_cast<T *>(bf), bd, bs, bb) &&
+           tma_encode_tiled(tmC, dt, 3, const_cast<T *>(xcp), cd, cs, cb);
+}
+
+template <typename D, typename T, typename TX, int R>
+cudaError_t run_residual_step(const MeshGeom &g, const FemCoef<T> &fc, const T *xcp, double up, const T *bf, TX *X,
+                              cudaStream_t st, bool skip_fast) {
+    using SL = StepLayout<D, T, R>;
+    CUtensorMap tmB, tmC;
+    if (!residual_maps<D, T, R>(g, bf, xcp, &tmB, &tmC)) return cudaErrorInvalidValue;
+    auto k = k_residual_step<D, T, TX, R>;
     const size_t sm = SL::BYTES;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     if (skip_fast) {
         if (g.n_slow_tiles == 0) return cudaSuccess;
-        k<<<g.n_slow_tiles, RES_THREADS, sm, st>>>(g, fc, tmB, tmC, up, X, g.slow_tiles);
+        constexpr bool big = D::TXC == TXC;
+        k<<<big ? g.n_slow_tiles : g.n_slow_small, D::THREADS, sm, st>>>(g, fc, tmB, tmC, up, X,
+                                                                       big ? g.slow_tiles : g.slow_small);
     } else {
-        k<<<tile_grid(g), RES_THREADS, sm, st>>>(g, fc, tmB, tmC, up, X, nullptr);
+        k<<<tile_grid<D>(g), D::THREADS, sm, st>>>(g, fc, tmB, tmC, up, X, nullptr);
     }
     return cudaGetLastError();
+}
+
+template <typename D, typename T, typename TX>
+cudaError_t run_residual_step_d(const MeshGeom &g, const FemCoef<T> &fc, const void *xcp, double up, const void *bf,
+                                void *X, cudaStream_t st, bool sf) {
+    switch (g.r) {
+        case 2: return run_residual_step<D, T, TX, 2>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
+        case 4: return run_residual_step<D, T, TX, 4>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
+        case 8: return run_residual_step<D, T, TX, 8>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename T, typename TX>
 cudaError_t run_residual_step_r(const MeshGeom &g, const FemCoef<T> &fc, const void *xcp, double up, const void *bf,
                                 void *X, cudaStream_t st, bool sf) {
-    switch (g.r) {
-        case 2: return run_residual_step<T, TX, 2>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
-        case 4: return run_residual_step<T, TX, 4>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
-        case 8: return run_residual_step<T, TX, 8>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
-        default: return cudaErrorInvalidValue;
-    }
+    if (use_small(g, sf ? g.n_slow_tiles : tiles_of(g))) return run_residual_step_d<SmallTile, T, TX>(g, fc, xcp, up, bf, X, st, sf);
+    return run_residual_step_d<BigTile, T, TX>(g, fc, xcp, up, bf, X, st, sf);
 }
 
 cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<double> &f64, const FemCoef<float> &f32,
@@ -2024,22 +2133,29 @@ cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<doub
     return run_residual_step_r<float, __nv_bfloat16>(g, f32, xcp, up, bf, X, st, skip_fast);
 }
 
-template <typename T>
-cudaError_t run_scatter(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
-                        cudaStream_t st) {
-    const dim3 grid = node_tile_grid(g);
+template <typename T, int PTY_>
+cudaError_t run_scatter_p(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
+                          cudaStream_t st) {
+    const dim3 grid((unsigned)((g.nxf + PTX) / PTX), (unsigned)((g.nyf + PTY_) / PTY_));
     const int pc = coarse_pitch(g);
     if (!xc && !xcp) {
-        k_scatter_avg<T, 0><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc);
+        k_scatter_avg<T, 0, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc);
         return cudaGetLastError();
     }
     switch (g.r) {
-        case 2: k_scatter_avg<T, 2><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
-        case 4: k_scatter_avg<T, 4><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
-        case 8: k_scatter_avg<T, 8><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
+        case 2: k_scatter_avg<T, 2, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
+        case 4: k_scatter_avg<T, 4, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
+        case 8: k_scatter_avg<T, 8, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t run_scatter(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
+                        cudaStream_t st) {
+    if (use_small(g, tiles_of(g))) return run_scatter_p<T, 4>(g, d, xf, xc, xcp, w, vc, st);
+    return run_scatter_p<T, PTY>(g, d, xf, xc, xcp, w, vc, st);
 }
 
 cudaError_t launch_scatter_avg(const MeshGeom &g, int prec, const void *d, const void *xf, const double *xc,
@@ -2050,21 +2166,32 @@ cudaError_t launch_scatter_avg(const MeshGeom &g, int prec, const void *d, const
     return run_scatter(g, (const float *)d, (const float *)xf, xc, (const float *)xcp, w, (float *)vcorr, st);
 }
 
-template <typename T>
-cudaError_t run_rhs(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st) {
-    using L = RhsLayout;
-    // v_corr [2][nyf+1][pitch]: boxes of the tile's node window
-    CUtensorMap tm;
+// v_corr [2][nyf+1][pitch]: boxes of the tile's node window
+template <typename D, typename T> bool rhs_map(const MeshGeom &g, const T *vcorr, CUtensorMap *tm) {
+    using L = RhsLayout<D>;
     const CUtensorMapDataType dt = sizeof(T) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t dims[3] = {(cuuint64_t)g.nxf + 1, (cuuint64_t)g.nyf + 1, 2};
     const cuuint64_t str[2] = {(cuuint64_t)g.pitch * sizeof(T), (cuuint64_t)g.plane * sizeof(T)};
     const cuuint32_t box[3] = {(cuuint32_t)L::HX, (cuuint32_t)L::HY, 2};
-    if (!tma_encode_tiled(&tm, dt, 3, const_cast<T *>(vcorr), dims, str, box)) return cudaErrorInvalidValue;
-    const size_t sm = L::bytes<T>();
-    cudaError_t e = set_smem(k_rhs<T>, sm);
+    return tma_encode_tiled(tm, dt, 3, const_cast<T *>(vcorr), dims, str, box);
+}
+
+template <typename D, typename T>
+cudaError_t run_rhs_d(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st) {
+    using L = RhsLayout<D>;
+    CUtensorMap tm;
+    if (!rhs_map<D, T>(g, vcorr, &tm)) return cudaErrorInvalidValue;
+    const size_t sm = L::template bytes<T>();
+    cudaError_t e = set_smem(k_rhs<D, T>, sm);
     if (e != cudaSuccess) return e;
-    k_rhs<T><<<tile_grid(g), NTHREADS, sm, st>>>(g, fc, tm, bf);
+    k_rhs<D, T><<<tile_grid<D>(g), D::THREADS, sm, st>>>(g, fc, tm, bf);
     return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t run_rhs(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st) {
+    if (use_small(g, tiles_of(g))) return run_rhs_d<SmallTile, T>(g, fc, vcorr, bf, st);
+    return run_rhs_d<BigTile, T>(g, fc, vcorr, bf, st);
 }
 
 cudaError_t launch_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f64,
