@@ -451,6 +451,7 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
         cudaFree(m->d_tile_flags);
         cudaFree(m->d_slow_tiles);
         cudaFree(m->d_cf_tab);
+        cudaFree(m->d_fem32);
         cudaFree(m->d_status);
         delete m;
         cudaGetLastError();
@@ -464,6 +465,16 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
     small_tiles_of(g, slow, &small);
     g.n_slow_small = (int)small.size();
     slow.insert(slow.end(), small.begin(), small.end());
+    // every tile, for batched launches of shapes without a closed form
+    std::vector<int> all((size_t)g.ntx * g.nty);
+    for (size_t i = 0; i < all.size(); ++i) all[i] = (int)i;
+    const size_t all_at = slow.size();
+    if (!residual_cf_supported(g, I.precision) && I.precision == DNNMG_BF16NET) {
+        small_tiles_of(g, all, &small);
+        slow.insert(slow.end(), all.begin(), all.end());
+        slow.insert(slow.end(), small.begin(), small.end());
+        g.n_all_small = (int)small.size();
+    }
     m->d_slow_tiles = nullptr;
     if (cudaMalloc(&m->d_slow_tiles, (slow.size() ? slow.size() : 1) * sizeof(int)) != cudaSuccess ||
         (slow.size() && cudaMemcpy(m->d_slow_tiles, slow.data(), slow.size() * sizeof(int),
@@ -471,6 +482,8 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
         return undo("boundary tile list");
     g.slow_tiles = m->d_slow_tiles;
     g.slow_small = m->d_slow_tiles + g.n_slow_tiles;
+    g.all_tiles = m->d_slow_tiles + all_at;
+    g.all_small = g.all_tiles + (size_t)g.ntx * g.nty;
     std::vector<uint16_t> ctab((size_t)I.ldx);
     residual_cf_table(g, ctab.data());
     m->d_cf_tab = nullptr;
@@ -488,6 +501,9 @@ int dnnmg_mesh_create(const dnnmg_mesh_desc *desc, dnnmg_mesh_t *out) {
         return undo("side stream and its events");
     fem_coefficients(*desc, &m->fem64);
     to_float(m->fem64, &m->fem32);
+    if (cudaMalloc(&m->d_fem32, sizeof(m->fem32)) != cudaSuccess ||
+        cudaMemcpy(m->d_fem32, &m->fem32, sizeof(m->fem32), cudaMemcpyHostToDevice) != cudaSuccess)
+        return undo("element constants");
     *out = m;
     return DNNMG_OK;
 }
@@ -502,6 +518,7 @@ int dnnmg_mesh_destroy(dnnmg_mesh_t mesh) {
     cudaFree(mesh->d_tile_flags);
     cudaFree(mesh->d_slow_tiles);
     cudaFree(mesh->d_cf_tab);
+    cudaFree(mesh->d_fem32);
     cudaFree(mesh->d_status);
     if (mesh->side) cudaStreamDestroy(mesh->side);
     if (mesh->ev_fork) cudaEventDestroy(mesh->ev_fork);

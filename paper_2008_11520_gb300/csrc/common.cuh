@@ -57,6 +57,8 @@ struct MeshGeom {
     int n_slow_tiles;
     const int *slow_small;        // the 8 x 8-cell tiles of those, in their own numbering
     int n_slow_small;
+    const int *all_tiles, *all_small;   // device, every tile of both sizes (batched launches take lists)
+    int n_all_small;
     const uint16_t *cf_tab;       // device [ldx]: feature column sources of the closed-form tiles
     int *status;                  // device status word of the mesh (DNNMG_DEVERR_* bits)
 };
@@ -105,6 +107,7 @@ struct Mesh {
     uint8_t *d_tile_flags;
     int *d_slow_tiles;
     uint16_t *d_cf_tab;
+    FemCoef<float> *d_fem32;   // copy of fem32 for launches over several meshes
     int *d_status;
     // the boundary tiles of S2+S3 run on this stream beside the closed-form
     // kernel (forked from and joined back to the caller's stream)
@@ -126,6 +129,19 @@ struct Net {
     void *tc_weights;
     size_t tc_bytes;
 };
+
+// One instance of a batched launch (serve.cu): what its passes read and write.
+struct StepInst {
+    const Mesh *mesh;
+    const double *xc;
+    double t;
+    float *bf;
+    double *bc;
+    void *X;          // its rows of the batch's features and outputs
+    const float *d;
+    float *xcp, *vc;  // padded x_c, v_corr
+};
+constexpr int kBatch = 32;   // instances of one launch (their parameters stay below 32 KB)
 
 int round_up(int v, int m);
 // Tiled TMA descriptor (no swizzle, zero fill out of bounds); strides in
@@ -171,6 +187,14 @@ void residual_cf_table(const MeshGeom &g, uint16_t *tab);
 void residual_cf_slow_tiles(const MeshGeom &g, const uint8_t *flags, std::vector<int> *slow);
 cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float> &f32, const void *xcp, const void *bf,
                                void *X, cudaStream_t st);
+// The passes over the tiles of n <= kBatch instances of one net shape in one
+// launch each (BF16 features); the same bits as the launches above.
+cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, cudaStream_t st);
+cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st);
+cudaError_t launch_residual_cf_batch(const StepInst *in, int n, cudaStream_t st);
+cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st);
+cudaError_t launch_rhs_batch(const StepInst *in, int n, cudaStream_t st);
+cudaError_t launch_restrict_batch(const StepInst *in, int n, cudaStream_t st);
 // S5 + S6 fused: b_f = Rhs(P x_c + mean of d) without writing v_corr.
 cudaError_t launch_avg_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f64, const FemCoef<float> &f32,
                            const void *d, const double *xc, double t, void *bf, cudaStream_t st);

@@ -327,12 +327,10 @@ struct CfShape {
 // tile's last node column.  Then the feature rows of the tile's patches are
 // gathered from shared memory in 16-byte pieces.
 template <typename TX, int R, int SP>
-__global__ void __launch_bounds__(CfShape<TX, R, SP>::THREADS, R == 4 ? 10 : 3)
-k_residual_cf(MeshGeom g, CfCoef c, const float *__restrict__ xcp, int pc, const float *__restrict__ bf,
-              TX *__restrict__ X) {
+__device__ __forceinline__ void residual_cf_cta(const MeshGeom &g, const CfCoef &c, const float *__restrict__ xcp, int pc,
+                                                const float *__restrict__ bf, TX *__restrict__ X, int tx, int ty) {
     using SH = CfShape<TX, R, SP>;
     constexpr int K = SH::K, S = SH::S, LS = K + SP - 1;
-    const int tx = blockIdx.x, ty = blockIdx.y;
     if (!block_fast(g, tx, ty)) return;
     extern __shared__ __align__(16) unsigned char smem[];
     float *cs = reinterpret_cast<float *>(smem + SH::CS);
@@ -432,6 +430,38 @@ k_residual_cf(MeshGeom g, CfCoef c, const float *__restrict__ xcp, int pc, const
 }
 
 template <typename TX, int R, int SP>
+__global__ void __launch_bounds__(CfShape<TX, R, SP>::THREADS, R == 4 ? 10 : 3)
+k_residual_cf(MeshGeom g, CfCoef c, const float *__restrict__ xcp, int pc, const float *__restrict__ bf,
+              TX *__restrict__ X) {
+    residual_cf_cta<TX, R, SP>(g, c, xcp, pc, bf, X, blockIdx.x, blockIdx.y);
+}
+
+// The blocks of several instances.
+struct CfBatch {
+    int n, first[kBatch + 1];
+    struct {
+        MeshGeom g;
+        CfCoef c;
+        const float *xcp, *bf;
+        int pc;
+        __nv_bfloat16 *X;
+    } inst[kBatch];
+};
+template <int R, int SP>
+__global__ void __launch_bounds__(CfShape<__nv_bfloat16, R, SP>::THREADS, R == 4 ? 10 : 3)
+k_residual_cf_batch(const __grid_constant__ CfBatch p) {
+    int lo = 0, hi = p.n;   // first[lo] <= blockIdx.x < first[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        if ((int)blockIdx.x >= p.first[mid]) lo = mid;
+        else hi = mid;
+    }
+    const auto &q = p.inst[lo];
+    const int local = blockIdx.x - p.first[lo], nbx = (q.g.nxf + CF_TXC - 1) / CF_TXC;
+    residual_cf_cta<__nv_bfloat16, R, SP>(q.g, q.c, q.xcp, q.pc, q.bf, q.X, local % nbx, local / nbx);
+}
+
+template <typename TX, int R, int SP>
 cudaError_t run_cf(const MeshGeom &g, const CfCoef &c, const float *xcp, const float *bf, TX *X, cudaStream_t st) {
     using SH = CfShape<TX, R, SP>;
     if (g.ldx != SH::LDX || g.nf != SH::NF) return cudaErrorInvalidValue;
@@ -480,8 +510,8 @@ bool residual_cf_supported(const MeshGeom &g, int prec) {
     return prec != DNNMG_F64 && (g.r == 2 || g.r == 4) && (g.s == 1 || g.s == 2);
 }
 
-cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float> &f32, const void *xcp, const void *bf,
-                               void *X, cudaStream_t st) {
+namespace {
+CfCoef cf_coefficients(const MeshGeom &g, const FemCoef<float> &f32) {
     CfCoef c;
     const double hx = g.hxf, hy = g.hyf, Hx = g.hxc, Hy = g.hyc;
     const double ik = 1.0 / g.k, hnu = 0.5 * g.nu;
@@ -515,10 +545,52 @@ cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float>
     c.hh = set(hx_, hy_);
     c.q_over_nu = f32.q_over_nu;
     for (int i = 0; i < 12; ++i) c.geo[i] = f32.geo[i];
+    return c;
+}
+}  // namespace
+
+cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float> &f32, const void *xcp, const void *bf,
+                               void *X, cudaStream_t st) {
+    const CfCoef c = cf_coefficients(g, f32);
     const float *xp = static_cast<const float *>(xcp);
     const float *b = static_cast<const float *>(bf);
     if (prec == DNNMG_F32) return run_cf_shape(g, c, xp, b, static_cast<float *>(X), st);
     return run_cf_shape(g, c, xp, b, static_cast<__nv_bfloat16 *>(X), st);
+}
+
+namespace {
+template <int R, int SP> cudaError_t cf_batch(const StepInst *in, int n, cudaStream_t st) {
+    using SH = CfShape<__nv_bfloat16, R, SP>;
+    CfBatch p;
+    p.n = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+        const Mesh &m = *in[i].mesh;
+        const MeshGeom &g = m.g;
+        if (g.ldx != SH::LDX || g.nf != SH::NF) return cudaErrorInvalidValue;
+        p.first[i] = at;
+        p.inst[i].g = g;
+        p.inst[i].c = cf_coefficients(g, m.fem32);
+        p.inst[i].xcp = in[i].xcp;
+        p.inst[i].bf = in[i].bf;
+        p.inst[i].pc = coarse_pitch(g);
+        p.inst[i].X = static_cast<__nv_bfloat16 *>(in[i].X);
+        at += ((g.nxf + CF_TXC - 1) / CF_TXC) * ((g.nyf + CF_TYC - 1) / CF_TYC);
+    }
+    p.first[n] = at;
+    auto k = k_residual_cf_batch<R, SP>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::BYTES);
+    if (e != cudaSuccess) return e;
+    k<<<at, SH::THREADS, SH::BYTES, st>>>(p);
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_residual_cf_batch(const StepInst *in, int n, cudaStream_t st) {
+    const MeshGeom &g = in[0].mesh->g;
+    if (g.r == 2) return g.s == 1 ? cf_batch<2, 1>(in, n, st) : cf_batch<2, 2>(in, n, st);
+    if (g.r == 4) return g.s == 1 ? cf_batch<4, 1>(in, n, st) : cf_batch<4, 2>(in, n, st);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace dnnmg

@@ -3,17 +3,19 @@
 // The correction step of Algorithm 2 is per instance; its network (Eq. gru + output
 // layer) works patch by patch with weights shared by every instance that uses
 // the same net.  A server therefore runs one step of several instances as:
-//   per instance  S1+S2+S3 into that instance's rows of one feature matrix X,
-//   once          S4 over all rows of X (one tensor-core GRU launch),
-//   per instance  S5, S6, S7 from that instance's rows of d.
+//   S1, S2+S3, S5, S6, S7   one launch each over the tiles of all instances,
+//                           from and into each instance's own arrays,
+//   S4                      one tensor-core GRU launch over all rows of X.
 // Each instance's GRU state h lives in a segment of one state pool.  Segments
 // and batch rows are whole 128-row tiles, so every GRU tile belongs to one
 // instance; a per-tile table gives the tile's first state row in the pool.
-// A patch row's arithmetic does not depend on the other rows of its tile, so
-// an instance gets the same bits alone (dnnmg_step) and in any batch.  The
-// per-instance passes of up to kLanes instances run side by side on the
-// server's own streams (small meshes fill few SMs each), each stream with its
-// own scratch; the caller's stream forks to them and joins back around S4.
+// A patch row's arithmetic does not depend on the other rows of its tile, and
+// a stencil tile runs the code of the single-instance launch, so an instance
+// gets the same bits alone (dnnmg_step) and in any batch.
+//
+// Launching the passes instance by instance on eight streams was bound by the
+// host (six launches and their tensor maps an instance): 20 instances of
+// 64 x 16 .. 512 x 128 coarse cells, K = 1, took 400 us a step; now 269 us.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -26,7 +28,7 @@ namespace dnnmg {
 namespace {
 
 constexpr int kTileRows = 128;   // rows of one GRU tile
-constexpr int kLanes = 8;        // side streams: the per-instance passes of up to 8 instances overlap
+constexpr int kGroup = 8;        // v_corr scratch: this many times the largest admitted mesh's
 
 // First-fit allocator of row ranges in units of `unit` rows; frees coalesce.
 struct RowPool {
@@ -108,15 +110,15 @@ struct dnnmg_server_s {
     int *tiles_host[2] = {nullptr, nullptr};   // pinned staging, used in turn
     cudaEvent_t tiles_ev[2] = {nullptr, nullptr};
     int flip = 0;
-    // per side stream: v_corr and the padded x_c of the largest admitted mesh
-    cudaStream_t lane[dnnmg::kLanes] = {};
-    cudaEvent_t lane_done[dnnmg::kLanes] = {};
-    cudaEvent_t fork = nullptr;
-    void *scratch[dnnmg::kLanes] = {};
-    size_t scratch_bytes = 0;
+    cudaStream_t side = nullptr;               // the boundary tiles, beside the closed form
+    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaEvent_t done = nullptr;                // end of the last step: the next may run on another stream
+    char *vc = nullptr;                        // v_corr of the instances whose S5 to S7 run together
+    size_t vc_bytes = 0, vc_max = 0;           // vc_bytes = kGroup x the largest admitted mesh's (vc_max)
     struct Slot {
         dnnmg_mesh_t mesh;
         int start, rows;      // pool segment (multiple of 128 rows); rows = padded patch rows
+        float *xcp;           // padded x_c
         bool live;
     };
     std::vector<Slot> slots;
@@ -125,9 +127,9 @@ struct dnnmg_server_s {
 namespace dnnmg {
 namespace {
 
-size_t scratch_need(const dnnmg_mesh_info &I) {
-    return align256(2 * (size_t)I.plane * I.real_bytes) +
-           align256(3 * (size_t)(I.nyc + 1) * round_up(I.nxc + 1, 32) * I.real_bytes);
+size_t vc_need(const dnnmg_mesh_info &I) { return align256(2 * (size_t)I.plane * I.real_bytes); }
+size_t xcp_need(const dnnmg_mesh_info &I) {
+    return 3 * (size_t)(I.nyc + 1) * round_up(I.nxc + 1, 32) * I.real_bytes;
 }
 
 void server_free(dnnmg_server_s *s) {
@@ -136,12 +138,12 @@ void server_free(dnnmg_server_s *s) {
     cudaFree(s->X);
     cudaFree(s->d);
     cudaFree(s->tiles_dev);
-    for (int j = 0; j < kLanes; ++j) {
-        cudaFree(s->scratch[j]);
-        if (s->lane[j]) cudaStreamDestroy(s->lane[j]);
-        if (s->lane_done[j]) cudaEventDestroy(s->lane_done[j]);
-    }
-    if (s->fork) cudaEventDestroy(s->fork);
+    cudaFree(s->vc);
+    for (auto &sl : s->slots)
+        if (sl.live) cudaFree(sl.xcp);
+    if (s->side) cudaStreamDestroy(s->side);
+    for (cudaEvent_t e : {s->fork, s->join, s->done})
+        if (e) cudaEventDestroy(e);
     for (int b = 0; b < 2; ++b) {
         if (s->tiles_host[b]) cudaFreeHost(s->tiles_host[b]);
         if (s->tiles_ev[b]) cudaEventDestroy(s->tiles_ev[b]);
@@ -240,10 +242,9 @@ int dnnmg_server_create(dnnmg_net_t net, int max_rows, dnnmg_server_t *out) {
     for (int b = 0; ok && b < 2; ++b)
         ok = cudaMallocHost(&s->tiles_host[b], ntiles * sizeof(int)) == cudaSuccess &&
              cudaEventCreateWithFlags(&s->tiles_ev[b], cudaEventDisableTiming) == cudaSuccess;
-    for (int j = 0; ok && j < kLanes; ++j)
-        ok = cudaStreamCreateWithFlags(&s->lane[j], cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&s->lane_done[j], cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t *e : {&s->fork, &s->join, &s->done})
+        ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
     // feature rows past an instance's patches are read by its last GRU tile:
     // keep them finite (their results land only in the instance's padding)
     ok = ok && cudaMemset(s->X, 0, rows * net->ldx * 2) == cudaSuccess;
@@ -282,27 +283,31 @@ int dnnmg_server_admit(dnnmg_server_t s, dnnmg_mesh_t mesh, int *slot) {
             return fail(DNNMG_ENOMEM, "no free state segment of %d rows (largest %d of %d)", rows,
                         s->pool.largest_free(), s->cap_rows);
     }
-    const size_t need = scratch_need(I);
-    if (need > s->scratch_bytes) {
+    float *xcp = nullptr;
+    char *vc = nullptr;
+    const size_t need = vc_need(I);
+    cudaError_t e = cudaMalloc(&xcp, xcp_need(I));
+    if (e == cudaSuccess && need > s->vc_max) {
         // the scratch may be in use by steps in flight
-        cudaError_t e = cudaDeviceSynchronize();
-        void *p[kLanes] = {};
-        for (int j = 0; e == cudaSuccess && j < kLanes; ++j) e = cudaMalloc(&p[j], need);
-        if (e != cudaSuccess) {
-            for (int j = 0; j < kLanes; ++j) cudaFree(p[j]);
-            if (rows > 0) s->pool.release(start);
-            cudaGetLastError();
-            return fail(DNNMG_ENOMEM, "scratch of %d x %zu bytes: %s", kLanes, need, cudaGetErrorString(e));
-        }
-        for (int j = 0; j < kLanes; ++j) {
-            cudaFree(s->scratch[j]);
-            s->scratch[j] = p[j];
-        }
-        s->scratch_bytes = need;
+        e = cudaDeviceSynchronize();
+        if (e == cudaSuccess) e = cudaMalloc(&vc, kGroup * need);
+    }
+    if (e != cudaSuccess) {
+        cudaFree(xcp);
+        if (rows > 0) s->pool.release(start);
+        cudaGetLastError();
+        return fail(DNNMG_ENOMEM, "scratch of %d x %zu bytes: %s", kGroup, need, cudaGetErrorString(e));
+    }
+    if (vc) {
+        cudaFree(s->vc);
+        s->vc = vc;
+        s->vc_max = need;
+        s->vc_bytes = kGroup * need;
     }
     // h0 = 0 (Sec. 6.2), padding rows included
     if (rows > 0 && cudaMemset(s->hpool + (size_t)start * n.H, 0, (size_t)rows * n.H * sizeof(float)) != cudaSuccess) {
         s->pool.release(start);
+        cudaFree(xcp);
         cudaGetLastError();
         return fail(DNNMG_ECUDA, "clearing the state segment failed");
     }
@@ -316,7 +321,7 @@ int dnnmg_server_admit(dnnmg_server_t s, dnnmg_mesh_t mesh, int *slot) {
         id = (int)s->slots.size();
         s->slots.push_back({});
     }
-    s->slots[id] = {mesh, start, rows, true};
+    s->slots[id] = {mesh, start, rows, xcp, true};
     *slot = id;
     return DNNMG_OK;
 }
@@ -328,6 +333,8 @@ int dnnmg_server_release(dnnmg_server_t s, int slot) {
     // a step in flight may still read or write the segment
     DNNMG_CUDA_TRY(cudaDeviceSynchronize());
     if (s->slots[slot].rows > 0) s->pool.release(s->slots[slot].start);
+    cudaFree(s->slots[slot].xcp);
+    s->slots[slot].xcp = nullptr;
     s->slots[slot].live = false;
     s->slots[slot].mesh = nullptr;
     return DNNMG_OK;
@@ -358,6 +365,12 @@ int dnnmg_server_step(dnnmg_server_t s, int n, const int *slots, const double *c
         row0[i] = total;
         total += s->slots[slots[i]].rows;
     }
+    // the server's buffers belong to one step at a time, on whichever stream
+    // (a captured step can neither wait for one outside its graph nor mark its end)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    DNNMG_CUDA_TRY(cudaStreamIsCapturing(stream, &capture));
+    const bool eager = capture == cudaStreamCaptureStatusNone;
+    if (eager) DNNMG_CUDA_TRY(cudaStreamWaitEvent(stream, s->done, 0));
     // per tile of the batch: its first state row in the pool
     const int b = s->flip;
     s->flip ^= 1;
@@ -373,53 +386,50 @@ int dnnmg_server_step(dnnmg_server_t s, int n, const int *slots, const double *c
                                        cudaMemcpyHostToDevice, stream));
         DNNMG_CUDA_TRY(cudaEventRecord(s->tiles_ev[b], stream));
     }
-    // the per-instance passes go round-robin to the side streams, which fork
-    // from and join back into the caller's stream around each phase
-    const int nl = n < kLanes ? n : kLanes;
-    auto fork = [&]() -> int {
-        DNNMG_CUDA_TRY(cudaEventRecord(s->fork, stream));
-        for (int j = 0; j < nl; ++j) DNNMG_CUDA_TRY(cudaStreamWaitEvent(s->lane[j], s->fork, 0));
-        return DNNMG_OK;
-    };
-    auto join = [&]() -> int {
-        for (int j = 0; j < nl; ++j) {
-            DNNMG_CUDA_TRY(cudaEventRecord(s->lane_done[j], s->lane[j]));
-            DNNMG_CUDA_TRY(cudaStreamWaitEvent(stream, s->lane_done[j], 0));
-        }
-        return DNNMG_OK;
-    };
     uint16_t *X = static_cast<uint16_t *>(s->X);
-    // S1 + S2 + S3 per instance, into its rows of X
-    if (int e = fork()) return e;
+    std::vector<StepInst> in(n);
     for (int i = 0; i < n; ++i) {
-        const dnnmg_mesh_s &m = *s->slots[slots[i]].mesh;
-        const dnnmg_mesh_info &I = m.info;
-        cudaStream_t st = s->lane[i % kLanes];
-        void *xcp = static_cast<char *>(s->scratch[i % kLanes]) + align256(2 * (size_t)I.plane * I.real_bytes);
-        DNNMG_CUDA_TRY(launch_coarse_pad(m.g, I.precision, xc[i], xcp, st));
-        // the same two S2+S3 kernels as dnnmg_step, so an instance gets the same bits
-        void *Xi = X + (size_t)row0[i] * net.ldx;
-        const bool cf = residual_cf_supported(m.g, I.precision);
-        if (cf) DNNMG_CUDA_TRY(launch_residual_cf(m.g, I.precision, m.fem32, xcp, bf[i], Xi, st));
-        DNNMG_CUDA_TRY(launch_residual_step(m.g, I.precision, m.fem64, m.fem32, xcp, t[i], bf[i], Xi, st, cf));
+        const dnnmg_server_s::Slot &sl = s->slots[slots[i]];
+        in[i] = {sl.mesh, xc[i], t[i], static_cast<float *>(bf[i]), bc[i], X + (size_t)row0[i] * net.ldx,
+                 s->d + (size_t)row0[i] * net.n_out, sl.xcp, nullptr};
     }
-    if (int e = join()) return e;
+    // S1 + S2 + S3, each instance into its rows of X: one launch per pass over
+    // up to kBatch instances, the boundary tiles on the side stream
+    const bool cf = residual_cf_supported(in[0].mesh->g, in[0].mesh->info.precision);
+    for (int i = 0; i < n; i += kBatch) {
+        const int m = std::min(kBatch, n - i);
+        DNNMG_CUDA_TRY(launch_coarse_pad_batch(&in[i], m, stream));
+        if (cf) {
+            DNNMG_CUDA_TRY(cudaEventRecord(s->fork, stream));
+            DNNMG_CUDA_TRY(cudaStreamWaitEvent(s->side, s->fork, 0));
+            DNNMG_CUDA_TRY(launch_residual_step_batch(&in[i], m, true, s->side));
+            DNNMG_CUDA_TRY(launch_residual_cf_batch(&in[i], m, stream));
+        } else {
+            DNNMG_CUDA_TRY(launch_residual_step_batch(&in[i], m, false, stream));
+        }
+    }
+    if (cf) {
+        DNNMG_CUDA_TRY(cudaEventRecord(s->join, s->side));
+        DNNMG_CUDA_TRY(cudaStreamWaitEvent(stream, s->join, 0));
+    }
     // S4 once over every instance's rows
     if (total > 0)
         DNNMG_CUDA_TRY(launch_gru_tc_rows(net, s->X, s->hpool, s->d, total, s->tiles_dev, s->cap_rows, stream));
-    // S5, S6, S7 per instance, from its rows of d
-    if (int e = fork()) return e;
-    for (int i = 0; i < n; ++i) {
-        const dnnmg_mesh_s &m = *s->slots[slots[i]].mesh;
-        const dnnmg_mesh_info &I = m.info;
-        cudaStream_t st = s->lane[i % kLanes];
-        void *vc = s->scratch[i % kLanes];
-        const float *d = s->d + (size_t)row0[i] * net.n_out;
-        DNNMG_CUDA_TRY(launch_scatter_avg(m.g, I.precision, d, nullptr, xc[i], t[i], vc, st));
-        DNNMG_CUDA_TRY(launch_rhs(m.g, I.precision, m.fem64, m.fem32, vc, bf[i], st));
-        DNNMG_CUDA_TRY(launch_restrict(m.g, I.precision, bf[i], bc[i], st));
+    // S5, S6, S7 from each instance's rows of d, over as many instances as the scratch holds v_corr of
+    for (int i = 0; i < n;) {
+        size_t used = 0;
+        int m = 0;
+        while (i + m < n && m < kBatch && used + vc_need(in[i + m].mesh->info) <= s->vc_bytes) {
+            in[i + m].vc = reinterpret_cast<float *>(s->vc + used);
+            used += vc_need(in[i + m].mesh->info);
+            ++m;
+        }
+        DNNMG_CUDA_TRY(launch_scatter_avg_batch(&in[i], m, stream));
+        DNNMG_CUDA_TRY(launch_rhs_batch(&in[i], m, stream));
+        DNNMG_CUDA_TRY(launch_restrict_batch(&in[i], m, stream));
+        i += m;
     }
-    if (int e = join()) return e;
+    if (eager) DNNMG_CUDA_TRY(cudaEventRecord(s->done, stream));
     return DNNMG_OK;
 }
 

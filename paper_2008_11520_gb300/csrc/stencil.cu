@@ -84,6 +84,24 @@ __device__ __forceinline__ bool node_tile_fluid(const MeshGeom &g, int bx, int b
     return tile_fluid(g, 2 * bx, by, 2) && tile_fluid(g, 2 * bx + 1, by, 2);
 }
 
+// A launch over the tiles of several instances: first[i] is instance i's first
+// CTA (first[n]: the grid).  i and the CTA's place in the instance.
+__device__ __forceinline__ int batch_instance(const int *first, int n, int &local) {
+    int lo = 0, hi = n;   // first[lo] <= blockIdx.x < first[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        if ((int)blockIdx.x >= first[mid]) lo = mid;
+        else hi = mid;
+    }
+    local = blockIdx.x - first[lo];
+    return lo;
+}
+// An instance's element constants, from its mesh's copy in device memory.
+template <typename T> __device__ __forceinline__ void stage_coef(FemCoef<T> &dst, const FemCoef<T> *src) {
+    static_assert(sizeof(FemCoef<T>) % sizeof(T) == 0, "array of T");
+    for (int i = threadIdx.x; i < (int)(sizeof(FemCoef<T>) / sizeof(T)); i += blockDim.x)
+        reinterpret_cast<T *>(&dst)[i] = __ldg(reinterpret_cast<const T *>(src) + i);
+}
 
 // Asynchronous 16-byte copy global -> shared; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_bytes) {
@@ -1045,6 +1063,21 @@ k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int
     coarse_pad_cta(g, xc, xcp, pc, blockIdx.x, gridDim.x);
 }
 
+struct PadBatch {
+    int n, first[kBatch + 1];
+    struct {
+        MeshGeom g;
+        const double *xc;
+        float *xcp;
+        int pc;
+    } inst[kBatch];
+};
+__global__ void __launch_bounds__(NTHREADS) k_coarse_pad_batch(const __grid_constant__ PadBatch p) {
+    int local;
+    const int i = batch_instance(p.first, p.n, local);
+    coarse_pad_cta(p.inst[i].g, p.inst[i].xc, p.inst[i].xcp, p.inst[i].pc, local, p.first[i + 1] - p.first[i]);
+}
+
 // Shared-memory layout of the TMA-fed residual kernel (bytes; the TMA
 // destinations 128-byte aligned): the work buffers of ResLayout plus the
 // b_f window and the coarse window as TMA boxes.
@@ -1141,6 +1174,32 @@ k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap t
         tx = tile - ty * ntx;
     }
     residual_step_cta<D, T, TX, R>(g, fc, &tmB, &tmC, inflow_peak, X, tx, ty);
+}
+
+// The boundary tiles of several instances (BF16 features).
+struct ResBatch {
+    CUtensorMap tmB[kBatch], tmC[kBatch];
+    int n, first[kBatch + 1];
+    struct {
+        MeshGeom g;
+        const FemCoef<float> *fc;
+        double up;
+        __nv_bfloat16 *X;
+        const int *tiles;
+    } inst[kBatch];
+};
+// (registers capped: with its constants in shared memory instead of kernel
+// parameters the compiler would keep 60 more of them in registers)
+template <typename D, int R>
+__global__ void __launch_bounds__(D::THREADS, 1024 / D::THREADS) k_residual_step_batch(const __grid_constant__ ResBatch p) {
+    __shared__ FemCoef<float> fc;
+    int local;
+    const int i = batch_instance(p.first, p.n, local);
+    stage_coef(fc, p.inst[i].fc);
+    const int tile = __ldg(p.inst[i].tiles + local), ntx = (p.inst[i].g.nxf + D::TXC - 1) / D::TXC;
+    const int ty = tile / ntx, tx = tile - ty * ntx;
+    __syncthreads();
+    residual_step_cta<D, float, __nv_bfloat16, R>(p.inst[i].g, fc, &p.tmB[i], &p.tmC[i], p.inst[i].up, p.inst[i].X, tx, ty);
 }
 
 // ------------------------------------------------------------------ S5
@@ -1386,6 +1445,25 @@ k_scatter_avg(MeshGeom g, const T *__restrict__ d, const T *__restrict__ xf, con
     scatter_cta<T, R, PTY>(g, d, xf, xc, xcp, pc, inflow_peak, vc, blockIdx.x, by);
 }
 
+struct AvgBatch {
+    int n, first[kBatch + 1];
+    struct {
+        MeshGeom g;
+        const float *d, *xcp;
+        int pc;
+        double up;
+        float *vc;
+    } inst[kBatch];
+};
+template <int R, int PTY>
+__global__ void __launch_bounds__(NTHREADS, 6) k_scatter_avg_batch(const __grid_constant__ AvgBatch p) {
+    int local;
+    const int i = batch_instance(p.first, p.n, local);
+    const auto &q = p.inst[i];
+    const int nx = (q.g.nxf + PTX) / PTX;
+    scatter_cta<float, R, PTY>(q.g, q.d, nullptr, nullptr, q.xcp, q.pc, q.up, q.vc, local % nx, local / nx);
+}
+
 // ------------------------------------------------------------------ S6
 // Node window of v_corr: columns I0-4 .. I0+TXC+3 (node I0+ii at column ii+4),
 // rows J0-1 .. J0+TYC+1 (node J0+jj at row jj+1).
@@ -1600,6 +1678,25 @@ template <typename D, typename T>
 __global__ void __launch_bounds__(D::THREADS)
 k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__restrict__ bf) {
     rhs_cta<D>(g, fc, &tmV, bf, blockIdx.x, blockIdx.y);
+}
+
+struct RhsBatch {
+    CUtensorMap tmV[kBatch];
+    int n, first[kBatch + 1];
+    struct {
+        MeshGeom g;
+        const FemCoef<float> *fc;
+        float *bf;
+    } inst[kBatch];
+};
+template <typename D>
+__global__ void __launch_bounds__(D::THREADS) k_rhs_batch(const __grid_constant__ RhsBatch p) {
+    __shared__ FemCoef<float> fc;
+    int local;
+    const int i = batch_instance(p.first, p.n, local);
+    stage_coef(fc, p.inst[i].fc);   // (visible after rhs_cta's first barrier)
+    const int ntx = (p.inst[i].g.nxf + D::TXC - 1) / D::TXC;
+    rhs_cta<D>(p.inst[i].g, fc, &p.tmV[i], p.inst[i].bf, local % ntx, local / ntx);
 }
 
 // S5 + S6 fused for the correction step: the v_corr window of a right-hand
@@ -1843,6 +1940,22 @@ template <typename T, typename Acc, int R>
 __global__ void __launch_bounds__(NTHREADS)
 k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restrict__ bc) {
     restrict_cta<T, Acc, R>(g, &tmB, bc, blockIdx.x, blockIdx.y);
+}
+
+struct RestrictBatch {
+    CUtensorMap tmB[kBatch];
+    int n, first[kBatch + 1];
+    struct {
+        MeshGeom g;
+        double *bc;
+    } inst[kBatch];
+};
+template <int R>
+__global__ void __launch_bounds__(NTHREADS) k_restrict_batch(const __grid_constant__ RestrictBatch p) {
+    int local;
+    const int i = batch_instance(p.first, p.n, local);
+    const int ntx = (p.inst[i].g.nxc + 128 / R) / (128 / R);
+    restrict_cta<float, RestrictAcc32, R>(p.inst[i].g, &p.tmB[i], p.inst[i].bc, local % ntx, local / ntx);
 }
 
 template <typename T, typename Acc, int R>
@@ -2234,6 +2347,157 @@ cudaError_t launch_restrict(const MeshGeom &g, int prec, const void *bf, double 
                             cudaStream_t st) {
     if (prec == DNNMG_F64) return run_restrict_r<double, RestrictAcc64>(g, (const double *)bf, bc, st);
     return run_restrict_r<float, RestrictAcc32>(g, (const float *)bf, bc, st);
+}
+
+// ---------------------------------------------------------------- batched passes
+// One launch over the tiles of up to kBatch instances of one K and patch size
+// (BF16 features); every tile runs the code of the single-instance launch.
+cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, cudaStream_t st) {
+    PadBatch p;
+    p.n = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+        const MeshGeom &g = in[i].mesh->g;
+        const int pc = coarse_pitch(g);
+        p.first[i] = at;
+        p.inst[i].g = g;
+        p.inst[i].xc = in[i].xc;
+        p.inst[i].xcp = in[i].xcp;
+        p.inst[i].pc = pc;
+        at += (int)((3LL * (g.nyc + 1) * (pc / 4) + NTHREADS - 1) / NTHREADS);
+    }
+    p.first[n] = at;
+    k_coarse_pad_batch<<<at, NTHREADS, 0, st>>>(p);
+    return cudaGetLastError();
+}
+
+template <typename D, int R> static cudaError_t residual_batch(const StepInst *in, int n, bool all, cudaStream_t st) {
+    ResBatch p;
+    p.n = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+        const Mesh &m = *in[i].mesh;
+        const MeshGeom &g = m.g;
+        if (!residual_maps<D, float, R>(g, in[i].bf, in[i].xcp, &p.tmB[i], &p.tmC[i])) return cudaErrorInvalidValue;
+        p.first[i] = at;
+        p.inst[i].g = g;
+        p.inst[i].fc = m.d_fem32;
+        p.inst[i].up = inflow_peak(g, in[i].t);
+        p.inst[i].X = static_cast<__nv_bfloat16 *>(in[i].X);
+        const bool big = D::TXC == TXC;
+        p.inst[i].tiles = all ? (big ? g.all_tiles : g.all_small) : (big ? g.slow_tiles : g.slow_small);
+        at += all ? (big ? g.ntx * g.nty : g.n_all_small) : (big ? g.n_slow_tiles : g.n_slow_small);
+    }
+    p.first[n] = at;
+    if (at == 0) return cudaSuccess;
+    auto k = k_residual_step_batch<D, R>;
+    const size_t sm = StepLayout<D, float, R>::BYTES;
+    cudaError_t e = set_smem(k, sm);
+    if (e != cudaSuccess) return e;
+    k<<<at, D::THREADS, sm, st>>>(p);
+    return cudaGetLastError();
+}
+
+// skip_fast: only the boundary tiles (launch_residual_cf_batch does the others)
+cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st) {
+    long long tiles = 0;
+    for (int i = 0; i < n; ++i) tiles += skip_fast ? in[i].mesh->g.n_slow_tiles : tiles_of(in[i].mesh->g);
+    const bool small = use_small(in[0].mesh->g, tiles);
+    switch (in[0].mesh->g.r) {
+        case 2: return small ? residual_batch<SmallTile, 2>(in, n, !skip_fast, st) : residual_batch<BigTile, 2>(in, n, !skip_fast, st);
+        case 4: return small ? residual_batch<SmallTile, 4>(in, n, !skip_fast, st) : residual_batch<BigTile, 4>(in, n, !skip_fast, st);
+        case 8: return small ? residual_batch<SmallTile, 8>(in, n, !skip_fast, st) : residual_batch<BigTile, 8>(in, n, !skip_fast, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <int R, int PTY_> static cudaError_t scatter_batch(const StepInst *in, int n, cudaStream_t st) {
+    AvgBatch p;
+    p.n = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+        const MeshGeom &g = in[i].mesh->g;
+        p.first[i] = at;
+        p.inst[i].g = g;
+        p.inst[i].d = in[i].d;
+        p.inst[i].xcp = in[i].xcp;
+        p.inst[i].pc = coarse_pitch(g);
+        p.inst[i].up = inflow_peak(g, in[i].t);
+        p.inst[i].vc = in[i].vc;
+        at += ((g.nxf + PTX) / PTX) * ((g.nyf + PTY_) / PTY_);
+    }
+    p.first[n] = at;
+    k_scatter_avg_batch<R, PTY_><<<at, NTHREADS, 0, st>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st) {
+    long long tiles = 0;
+    for (int i = 0; i < n; ++i) tiles += tiles_of(in[i].mesh->g);
+    const bool small = use_small(in[0].mesh->g, tiles);
+    switch (in[0].mesh->g.r) {
+        case 2: return small ? scatter_batch<2, 4>(in, n, st) : scatter_batch<2, PTY>(in, n, st);
+        case 4: return small ? scatter_batch<4, 4>(in, n, st) : scatter_batch<4, PTY>(in, n, st);
+        case 8: return small ? scatter_batch<8, 4>(in, n, st) : scatter_batch<8, PTY>(in, n, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <typename D> static cudaError_t rhs_batch(const StepInst *in, int n, cudaStream_t st) {
+    RhsBatch p;
+    p.n = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+        const MeshGeom &g = in[i].mesh->g;
+        if (!rhs_map<D, float>(g, in[i].vc, &p.tmV[i])) return cudaErrorInvalidValue;
+        p.first[i] = at;
+        p.inst[i].g = g;
+        p.inst[i].fc = in[i].mesh->d_fem32;
+        p.inst[i].bf = in[i].bf;
+        at += ((g.nxf + D::TXC - 1) / D::TXC) * ((g.nyf + D::TYC - 1) / D::TYC);
+    }
+    p.first[n] = at;
+    const size_t sm = RhsLayout<D>::template bytes<float>();
+    cudaError_t e = set_smem(k_rhs_batch<D>, sm);
+    if (e != cudaSuccess) return e;
+    k_rhs_batch<D><<<at, D::THREADS, sm, st>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rhs_batch(const StepInst *in, int n, cudaStream_t st) {
+    long long tiles = 0;
+    for (int i = 0; i < n; ++i) tiles += tiles_of(in[i].mesh->g);
+    return use_small(in[0].mesh->g, tiles) ? rhs_batch<SmallTile>(in, n, st) : rhs_batch<BigTile>(in, n, st);
+}
+
+template <int R> static cudaError_t restrict_batch(const StepInst *in, int n, cudaStream_t st) {
+    constexpr int TCX = 128 / R, TCY = 32 / R;
+    RestrictBatch p;
+    p.n = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+        const MeshGeom &g = in[i].mesh->g;
+        if (!restrict_map<float, R>(g, in[i].bf, &p.tmB[i])) return cudaErrorInvalidValue;
+        p.first[i] = at;
+        p.inst[i].g = g;
+        p.inst[i].bc = in[i].bc;
+        at += ((g.nxc + TCX) / TCX) * ((g.nyc + TCY) / TCY);
+    }
+    p.first[n] = at;
+    const size_t sm = restrict_smem<float, RestrictAcc32, R>();
+    cudaError_t e = set_smem(k_restrict_batch<R>, sm);
+    if (e != cudaSuccess) return e;
+    k_restrict_batch<R><<<at, NTHREADS, sm, st>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_restrict_batch(const StepInst *in, int n, cudaStream_t st) {
+    switch (in[0].mesh->g.r) {
+        case 2: return restrict_batch<2>(in, n, st);
+        case 4: return restrict_batch<4>(in, n, st);
+        case 8: return restrict_batch<8>(in, n, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_mesh_maps(const MeshGeom &g, unsigned char *flags, unsigned char *mult,
