@@ -153,8 +153,13 @@ __device__ __forceinline__ void store_h16(uint8_t *sAh, int row, int c0, const f
     }
 }
 
+// CTAs an SM: a state of 64 columns or fewer leaves room for two (registers,
+// shared and tensor memory), and one computes while the other waits for its
+// products (307 776 rows, 51 -> 64 -> 18: 84 -> 68 us).
+constexpr int ctas_per_sm(int H) { return H <= 64 ? 2 : 1; }
+
 template <int H>
-__global__ void __launch_bounds__(NTH, 1)
+__global__ void __launch_bounds__(NTH, ctas_per_sm(H))
 k_gru_tc(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmX3,
          const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmH3, float *__restrict__ d,
          int P, const int *__restrict__ hrow) {
@@ -676,8 +681,9 @@ cudaError_t launch_gru_tc_rows(const Net &n, const void *X, void *h, void *d, in
         if (!encode(&tmH3, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h, dims, strides, box)) return cudaErrorInvalidValue;
     }
     const size_t smem = smem_bytes(p);
-    // persistent: one CTA per SM (the shared memory allows no second), tiles strided over the grid
-    const int grid = std::min((P + TM - 1) / TM, sm_count());
+    // persistent: one or two CTAs per SM, tiles strided over the grid
+    const int per = 2 * (smem + 1024) <= 228 * 1024 && p.tmem_cols <= 256 ? ctas_per_sm(p.H) : 1;
+    const int grid = std::min((P + TM - 1) / TM, per * sm_count());
     cudaError_t e;
 #define DNNMG_LAUNCH_H(HH)                                                                                   \
     case HH:                                                                                                 \
