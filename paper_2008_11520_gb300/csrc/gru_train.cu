@@ -500,7 +500,9 @@ WinArgs window(dnnmg_trainer_s *t, const float *X) {
     g.n_in = t->n_in; g.ldx = t->ldx; g.n_out = t->n_out; g.nfc = round_up(t->n_out, 16);
     g.T = t->T; g.P = t->P; g.ntiles = win_tiles(t->P);
     g.xvec = t->ldx % 4 == 0 && aligned16(X);
-    g.part_cols = 3 * t->H + g.nfc;
+    g.kx2 = t->n_in > 64 ? round_up(t->n_in - 64, 16) / 16 : 0;
+    g.part_cols = (g.kx2 ? 6 : 3) * t->H + g.nfc;
+    g.GX = t->GX;
     g.X = X;
     g.z = t->z; g.r = t->r; g.c = t->c; g.hb = t->rh;
     g.part = t->wpart;
@@ -554,10 +556,10 @@ int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnm
     t->splits = (int)std::min<size_t>(256, std::max<size_t>(1, TP / 4096));
     const size_t mx = (size_t)std::max(3 * H, n_out) * std::max(std::max(n_in, H), 1);
     t->part_floats = (size_t)t->splits * mx;
-    // (z, r, rh and c hold whole 128-row tiles in the fused window)
+    // (GX, z, r, rh, c and dG hold whole 128-row tiles in the fused window)
     const size_t TPt = (size_t)T * win_tiles(P) * 128;
     struct { float **p; size_t n; } req[] = {
-        {&t->GX, TP * 3 * H}, {&t->hs, (TP + P) * H}, {&t->z, TPt * H}, {&t->r, TPt * H}, {&t->rh, TPt * H},
+        {&t->GX, TPt * 3 * H}, {&t->hs, (TP + P) * H}, {&t->z, TPt * H}, {&t->r, TPt * H}, {&t->rh, TPt * H},
         {&t->c, TPt * H}, {&t->GH, (size_t)P * 2 * H}, {&t->AH, (size_t)P * H}, {&t->dHfc, TP * H},
         {&t->dG, TPt * 3 * H}, {&t->dh, (size_t)P * H}, {&t->drh, (size_t)P * H}, {&t->carry, (size_t)P * H},
         {&t->part, t->part_floats}};
@@ -566,7 +568,7 @@ int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnm
     ok = ok && cudaMalloc(&t->red, kRedBlocks * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc(&t->d_status, sizeof(int)) == cudaSuccess && cudaMemset(t->d_status, 0, sizeof(int)) == cudaSuccess;
     if (win_supported(n_in, H, n_out))
-        ok = ok && cudaMalloc(&t->wpart, win_part_floats(H, n_out, T, P) * sizeof(float)) == cudaSuccess;
+        ok = ok && cudaMalloc(&t->wpart, win_part_floats(n_in, H, n_out, T, P) * sizeof(float)) == cudaSuccess;
     if (!ok) {
         trainer_free(t);
         cudaGetLastError();

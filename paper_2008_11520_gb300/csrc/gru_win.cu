@@ -10,7 +10,8 @@
 // per product (with FP32 intermediates and BF16 copies of every operand in
 // memory between them) took 4.07 ms for loss and gradients of 65 536 rows, T =
 // 10, H = 64; this takes 0.65 ms, of it forward 266 us, backward 256 us and
-// the sum of the partial gradients 15 us (ncu).
+// the sum of the partial gradients 15 us (ncu).  With 99 features (two chunks)
+// and 50 outputs 4.65 ms became 1.05 ms, forward 386 us, backward 399 us.
 //
 // Arithmetic is that of the kernel-per-product path (gru_train.cu): operands
 // are rounded to BF16 where it rounds them, X W_x^T and h U^T are accumulated
@@ -35,46 +36,65 @@
 namespace dnnmg {
 namespace {
 
-constexpr int FWD_TH = 256, BWD_TH = 512;
+constexpr int BWD_TH = 512;
 
 // ---------------------------------------------------------------- forward
-// Two CTAs an SM (each 256 threads, two per row, and half the tensor memory),
-// so that one computes while the other waits for its MMAs.  Tensor memory
+// XC = 1 (n_in <= 64): two CTAs an SM (each 256 threads, two per row, and half
+// the tensor memory), so that one computes while the other waits for its MMAs.
+// XC = 2 (n_in <= 128): the second chunk of W_x and X leaves room for one, of
+// 512 threads.  Tensor memory
 // columns: X W_zr^T [0, 2H), h U_zr^T [2H, 4H); once r has been read,
 // X W_h^T [H, 2H) and (r h) U_h^T [3H, 4H); then the output layer [0, nfc).
 // Bound by instruction issue (gate functions and conversions) and, close
 // behind, by memory (1.2 kB a row and step).
-template <int H> struct FwdLayout {
-    static constexpr int WX = 0, U = WX + 3 * H * 128, F = U + 3 * H * 128, X = F + 64 * 128, HI = X + IMG,
+template <int H, int XC> struct FwdLayout {
+    static constexpr int TH = XC == 1 ? 256 : 512, CTAS = XC == 1 ? 2 : 1;
+    static constexpr int WX = 0, U = WX + XC * 3 * H * 128, F = U + 3 * H * 128, X = F + 64 * 128, HI = X + XC * IMG,
                          BARS = HI + IMG, BYTES = BARS + 64 + 1024;
     static constexpr int COLS = 4 * H;
 };
 
-template <int H>
-__global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
-    using L = FwdLayout<H>;
-    constexpr int NH = H / 2;   // state columns of a thread
+template <int H, int XC>
+__global__ void __launch_bounds__(FwdLayout<H, XC>::TH, FwdLayout<H, XC>::CTAS) k_win_fwd(const WinArgs g) {
+    using L = FwdLayout<H, XC>;
+    constexpr int TH = L::TH, PARTS = TH / TM, NH = H / PARTS;   // threads a row, state columns of each
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = align1k(smem_raw);
     uint8_t *sX = base + L::X, *sH = base + L::HI;
     const uint32_t uWx = smem_u32(base + L::WX), uU = smem_u32(base + L::U), uF = smem_u32(base + L::F),
                    uX = smem_u32(sX), uH = smem_u32(sH);
-    build(base + L::WX, 3 * H, FWD_TH, [&](int r, int c) { return c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + c) : 0.f; });
-    build(base + L::U, 3 * H, FWD_TH, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)r * H + c) : 0.f; });
-    build(base + L::F, g.nfc, FWD_TH, [&](int r, int c) { return r < g.n_out && c < H ? __ldg(g.Wfc + (size_t)r * H + c) : 0.f; });
+    for (int x = 0; x < XC; ++x)
+        build(base + L::WX + x * 3 * H * 128, 3 * H, TH, [&](int r, int c) {
+            return 64 * x + c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + 64 * x + c) : 0.f;
+        });
+    build(base + L::U, 3 * H, TH, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)r * H + c) : 0.f; });
+    build(base + L::F, g.nfc, TH, [&](int r, int c) { return r < g.n_out && c < H ? __ldg(g.Wfc + (size_t)r * H + c) : 0.f; });
     Cta cta;
     cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 2, L::COLS);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp & 3, half = warp >> 2, row = q * 32 + lane, c0 = half * NH;
+    const int q = warp & 3, part = warp >> 2, row = q * 32 + lane, c0 = part * NH;
     const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
     uint32_t ph = 0;   // phase of the MMA barrier
     bool ok = true;
-    XTile<FWD_TH> xt;
+    XTile<TH> xt[XC];
+    auto load_x = [&](int s, int p0) {
+#pragma unroll
+        for (int x = 0; x < XC; ++x) xt[x].load(g, s, p0, 64 * x);
+    };
+    auto store_x = [&]() {
+#pragma unroll
+        for (int x = 0; x < XC; ++x) xt[x].store(g, sX + x * IMG, 64 * x);
+    };
+    // the products of columns [n0, n0 + N) of W_x with X
+    auto mma_x = [&](uint32_t d, int n0, int N) {
+        mma_k(d, uX, uWx + n0 * 128, N, 4, false);
+        if (XC == 2) mma_k(d, uX + IMG, uWx + (3 * H + n0) * 128, N, g.kx2, true);
+    };
     for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
         const int p0 = tile * TM, gp = p0 + row;
         const bool valid = gp < g.P;
         float hv[NH];
-        xt.load(g, 0, p0);
+        load_x(0, p0);
 #pragma unroll
         for (int i = 0; i < NH; i += 4) {
             hv[i] = hv[i + 1] = hv[i + 2] = hv[i + 3] = 0.f;
@@ -85,12 +105,12 @@ __global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
         for (int i = 0; i < NH; i += 4) st4(g.hb + (size_t)tile * tblk + blk(c0 + i, row), hv + i);
 #pragma unroll
         for (int i = 0; i < NH; i += 8) put8(sH, row, c0 + i, hv + i);
-        xt.store(g, sX);
+        store_x();
         for (int s = 0; s < g.T; ++s) {
             const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
             if (!(ok = cta.hand_over(ok))) break;
             if (tid == 0) {
-                mma_k(cta.tmem, uX, uWx, 2 * H, 4, false);
+                mma_x(cta.tmem, 0, 2 * H);
                 mma_k(cta.tmem + 2 * H, uH, uU, 2 * H, H / 16, false);
                 tc_commit(cta.bar0);
             }
@@ -116,7 +136,7 @@ __global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
             }
             if (!(ok = cta.hand_over(ok))) break;
             if (tid == 0) {
-                mma_k(cta.tmem + H, uX, uWx + 2 * H * 128, H, 4, false);
+                mma_x(cta.tmem + H, 2 * H, H);
                 mma_k(cta.tmem + 3 * H, uH, uU + 2 * H * 128, H, H / 16, false);
                 tc_commit(cta.bar0);
             }
@@ -149,7 +169,7 @@ __global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
                 put8(sH, row, c0 + i, hv + i);
             }
             if (s + 1 < g.T) {
-                xt.load(g, s + 1, p0);
+                load_x(s + 1, p0);
                 float *hb = g.hb + ((size_t)(s + 1) * g.ntiles + tile) * tblk;
 #pragma unroll
                 for (int i = 0; i < NH; i += 4) st4(hb + blk(c0 + i, row), hv + i);
@@ -162,12 +182,12 @@ __global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
                 mma_k(cta.tmem, uH, uF, g.nfc, H / 16, false);
                 tc_commit(cta.bar0);
             }
-            if (s + 1 < g.T) xt.store(g, sX);
+            if (s + 1 < g.T) store_x();
             ok = cta.wait(0, ph);
             ph ^= 1;
-            // outputs: blocks of 8 columns, alternating between the two threads of a row
+            // outputs: blocks of 8 columns, dealt to the threads of a row
             float *drow = g.D + ((size_t)s * g.P + gp) * g.n_out;
-            for (int b = half; b < g.nfc / 8; b += 2) {
+            for (int b = part; b < g.nfc / 8; b += PARTS) {
                 float v[8];
                 tmem_ld8(tl + 8 * b, v);
                 tmem_wait();
@@ -198,22 +218,27 @@ __global__ void __launch_bounds__(FWD_TH, 2) k_win_fwd(const WinArgs g) {
 //   MMA: [dA_z, dA_r] [U_z; U_r] and the next step's dD W_fc, then the
 //   weight gradients [X | h]^T [dA_z, dA_r], [X | r h]^T dA_c and h_{s+1}^T dD
 //   into their accumulators, which run while the next step's elements do.
-// Tensor memory: carry part [0, H), dD W_fc [64, 64 + H), d(r h) [128, 128 + H),
-// gradients [192, 192 + 2H), [320, 320 + H), [384, 384 + nfc).
+// Tensor memory, XC = 1: carry part [0, H), dD W_fc [64, 64 + H), d(r h) [128,
+// 128 + H), gradients [192, 192 + 2H), [320, 320 + H), [384, 384 + nfc).  XC = 2
+// (features 64 ..) has gradients of its own, so the carry's products add to
+// dD W_fc, and d(r h) takes their place once they have been read.
 // Bound by the chain of the two MMA round trips a step and the element work
 // between them; memory (1.4 kB a row and step) is close behind.
-template <int H> struct BwdLayout {
-    static constexpr int X = 0, HP = X + IMG, RH = HP + IMG, HN = RH + IMG, GZR = HN + IMG,
+template <int H, int XC> struct BwdLayout {
+    static constexpr int X = 0, HP = X + XC * IMG, RH = HP + IMG, HN = RH + IMG, GZR = HN + IMG,
                          GC = GZR + (H == 64 ? 2 : 1) * IMG, DD = GC + IMG, WF = DD + 2 * IMG, UC = WF + H * 128,
                          UZR = UC + H * 128, BARS = UZR + (H == 64 ? 2 : 1) * H * 128, BYTES = BARS + 64 + 1024;
     static constexpr int COLS = 512;
+    static constexpr int CARRY = 0, DH = XC == 1 ? 64 : 0, DRH = XC == 1 ? 128 : 0;
+    // [X | h]^T [dA_z dA_r], [X | r h]^T dA_c, h_{s+1}^T dD (rows 64 .. of it with XC = 2), second chunk
+    static constexpr int G1 = XC == 1 ? 192 : 64, G2 = G1 + 128, G3 = XC == 1 ? 384 : 448, G4 = 256, G5 = 384;
 };
-constexpr int T_CARRY = 0, T_DH = 64, T_DRH = 128, T_G1 = 192, T_G2 = 320, T_G3 = 384;
 
-template <int H>
+template <int H, int XC>
 __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
-    using L = BwdLayout<H>;
+    using L = BwdLayout<H, XC>;
     constexpr int NC = H / 4;   // state columns of a thread: 16 or 8
+    constexpr int T_CARRY = L::CARRY, T_DH = L::DH, T_DRH = L::DRH;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = align1k(smem_raw);
     const uint32_t u = smem_u32(base);
@@ -280,6 +305,7 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
         load_dd(g.T - 1, p0);
         load_step(g.T - 1, tile);
         xt.load(g, g.T - 1, p0);
+        if (XC == 2) xt.prefetch(g, g.T - 1, p0, 64);
         if (!(ok = cta.hand_over(ok))) break;
         if (tid == 0) {
             mma_k(cta.tmem + T_DH, u + L::DD + ((g.T - 1) & 1) * IMG, u + L::WF, H, kfc, false);
@@ -293,14 +319,14 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8];
                 tmem_ld8(tl + T_DH + c0 + i, a);
-                tmem_ld8(tl + T_CARRY + c0 + i, b);
+                if (XC == 1) tmem_ld8(tl + T_CARRY + c0 + i, b);
                 tmem_wait();
                 keep(a);
-                keep(b);
+                if (XC == 1) keep(b);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
-                    const float carry = s == g.T - 1 ? 0.f : b[j] + cpart[k];
+                    const float carry = s == g.T - 1 ? 0.f : (XC == 1 ? b[j] + cpart[k] : cpart[k]);
                     dh[k] = a[j] + carry;
                     const float dc = dh[k] * (1.0f - zv[k]), dz = dh[k] * (hp[k] - cv[k]);
                     az[k] = dz * zv[k] * (1.0f - zv[k]);
@@ -331,6 +357,10 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
                 tc_commit(cta.bar0 + 16);
             }
             xt.store(g, base + L::X);
+            if (XC == 2) {
+                xt.load(g, s, p0, 64);
+                xt.store(g, base + L::X + IMG, 64);
+            }
             if (s > 0) load_dd(s - 1, p0);
             ok = cta.wait(2, ph2);
             ph2 ^= 1;
@@ -353,16 +383,24 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
             if (s > 0) {
                 load_step(s - 1, tile);
                 xt.load(g, s - 1, p0);
+                if (XC == 2) xt.prefetch(g, s - 1, p0, 64);
             }
             if (!(ok = cta.hand_over(ok))) break;
             if (tid == 0) {
                 mma_k(cta.tmem + T_CARRY, u + L::GZR, u + L::UZR, H, 4, false);
                 if (H == 64) mma_k(cta.tmem + T_CARRY, u + L::GZR + IMG, u + L::UZR + H * 128, H, 4, true);
-                if (s > 0) mma_k(cta.tmem + T_DH, u + L::DD + ((s - 1) & 1) * IMG, u + L::WF, H, kfc, false);
+                if (s > 0) mma_k(cta.tmem + T_DH, u + L::DD + ((s - 1) & 1) * IMG, u + L::WF, H, kfc, XC == 2);
                 tc_commit(cta.bar0);
-                mma_mn(cta.tmem + T_G1, desc_mn(u + L::X, L::HP - L::X), desc_mn(u + L::GZR, IMG), 2 * H, grads);
-                mma_mn(cta.tmem + T_G2, desc_mn(u + L::X, L::RH - L::X), desc_mn(u + L::GC, IMG), H, grads);
-                mma_mn(cta.tmem + T_G3, desc_mn(u + L::HN, L::HP - L::X), desc_mn(u + L::DD + (s & 1) * IMG, IMG), g.nfc, grads);
+                mma_mn(cta.tmem + L::G1, desc_mn(u + L::X, L::HP - L::X), desc_mn(u + L::GZR, IMG), 2 * H, grads);
+                mma_mn(cta.tmem + L::G2, desc_mn(u + L::X, L::RH - L::X), desc_mn(u + L::GC, IMG), H, grads);
+                if (XC == 1) {
+                    mma_mn(cta.tmem + L::G3, desc_mn(u + L::HN, L::HP - L::X), desc_mn(u + L::DD + (s & 1) * IMG, IMG), g.nfc, grads);
+                } else {
+                    const uint64_t a = desc_mn(u + L::X + IMG, L::HN - L::X - IMG);   // [X's second chunk | h_{s+1}]
+                    mma_mn(cta.tmem + L::G4, a, desc_mn(u + L::GZR, IMG), 2 * H, grads);
+                    mma_mn(cta.tmem + L::G5, a, desc_mn(u + L::GC, IMG), H, grads);
+                    mma_mn(cta.tmem + L::G3, a, desc_mn(u + L::DD + (s & 1) * IMG, IMG), g.nfc, grads);
+                }
                 tc_commit(cta.bar0 + 8);
             }
             grads = true;
@@ -388,17 +426,19 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
         }
         ok = cta.hand_over(ok);   // (the same answer in every thread)
     }
-    // this CTA's sums: [column][lane], gradients of W_x (lanes 0 .. 63) and U (64 ..), then of W_fc
+    // this CTA's sums: [column][lane], gradients of W_x (lanes 0 .. 63) and U (64 ..), then of W_fc,
+    // then of W_x's second chunk
     if (ok && grads) {
         ok = cta.wait(1, ph1);
         ph1 ^= 1;
     }
     if (ok && !*cta.abort_flag) {
         float *o = g.part + (size_t)blockIdx.x * g.part_cols * TM;
-        const int ncol = 3 * H + g.nfc;
+        const int ncol = g.part_cols, x2 = 3 * H + g.nfc;
         for (int b = part; b < ncol / 8; b += 4) {
             const int c = 8 * b;
-            const int t = c < 2 * H ? T_G1 + c : (c < 3 * H ? T_G2 + c - 2 * H : T_G3 + c - 3 * H);
+            int t = c < 2 * H ? L::G1 + c : (c < 3 * H ? L::G2 + c - 2 * H : L::G3 + c - 3 * H);
+            if (XC == 2 && c >= x2) t = c - x2 < 2 * H ? L::G4 + c - x2 : L::G5 + c - x2 - 2 * H;
             float v[8];
             tmem_ld8(tl + t, v);
             tmem_wait();
@@ -413,7 +453,7 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
 // Sums of the CTAs' partial gradients, in the order of the CTAs and without
 // their rounding errors (TwoSum: an FP32 sum of 152 parts in sequence is off
 // by about as much as everything before it).
-__global__ void __launch_bounds__(TM) k_win_reduce(const WinArgs g, int H, int nparts) {
+__global__ void __launch_bounds__(TM) k_win_reduce(const WinArgs g, int H, int nparts, int fc_lane) {
     const int c = blockIdx.x, m = threadIdx.x;
     const float *p = g.part + (size_t)c * TM + m;
     const size_t stride = (size_t)g.part_cols * TM;
@@ -428,38 +468,51 @@ __global__ void __launch_bounds__(TM) k_win_reduce(const WinArgs g, int H, int n
     if (c < 3 * H) {
         if (m < g.n_in && m < 64) g.gWx[(size_t)c * g.n_in + m] = s;
         if (m >= 64 && m < 64 + H) g.gUh[(size_t)c * H + m - 64] = s;
-    } else if (c - 3 * H < g.n_out && m < H) {
-        g.gWfc[(size_t)(c - 3 * H) * H + m] = s;
+    } else if (c < 3 * H + g.nfc) {
+        if (c - 3 * H < g.n_out && m >= fc_lane && m < fc_lane + H) g.gWfc[(size_t)(c - 3 * H) * H + m - fc_lane] = s;
+    } else if (m < 64 && 64 + m < g.n_in) {
+        g.gWx[(size_t)(c - 3 * H - g.nfc) * g.n_in + 64 + m] = s;
     }
 }
 
 }  // namespace
 
-// Shapes the window kernels take: one 64-column chunk of features, H = 32 or
-// 64, up to 64 outputs (the K = 1 networks of the training workload); the
-// others run one kernel per product.
-bool win_supported(int n_in, int H, int n_out) { return n_in <= 64 && (H == 32 || H == 64) && n_out <= 64; }
+// Shapes the window kernels take: one or two 64-column chunks of features, H =
+// 32 or 64, up to 64 outputs (the K = 1 and K = 2 networks of one-cell
+// patches); the others run one kernel per product.
+bool win_supported(int n_in, int H, int n_out) { return n_in <= 128 && (H == 32 || H == 64) && n_out <= 64; }
 int win_tiles(int P) { return (P + TM - 1) / TM; }
-size_t win_part_floats(int H, int n_out, int T, int P) {
-    return (size_t)win32_parts(T, P) * (3 * H + round_up(n_out, 16)) * TM;   // (at least win_tiles(P) or one per SM)
+size_t win_part_floats(int n_in, int H, int n_out, int T, int P) {
+    return (size_t)win32_parts(T, P) * ((n_in > 64 ? 6 : 3) * H + round_up(n_out, 16)) * TM;   // (at least win_tiles(P) or one per SM)
 }
 
+namespace {
+template <int H, int XC> cudaError_t forward(const WinArgs &g, cudaStream_t st) {
+    using L = FwdLayout<H, XC>;
+    return launch(k_win_fwd<H, XC>, std::min(g.ntiles, L::CTAS * sm_count()), L::TH, L::BYTES, g, st);
+}
+template <int H, int XC> cudaError_t backward(const WinArgs &g, int grid, cudaStream_t st) {
+    return launch(k_win_bwd<H, XC>, grid, BWD_TH, BwdLayout<H, XC>::BYTES, g, st);
+}
+}  // namespace
+
 cudaError_t win_forward(const WinArgs &g, int H, cudaStream_t st) {
-    const int grid = std::min(g.ntiles, 2 * sm_count());
-    if (H == 64) return launch(k_win_fwd<64>, grid, FWD_TH, FwdLayout<64>::BYTES, g, st);
-    return launch(k_win_fwd<32>, grid, FWD_TH, FwdLayout<32>::BYTES, g, st);
+    if (H == 64) return g.kx2 ? forward<64, 2>(g, st) : forward<64, 1>(g, st);
+    return g.kx2 ? forward<32, 2>(g, st) : forward<32, 1>(g, st);
 }
 
 cudaError_t win_backward(const WinArgs &g, int H, cudaStream_t st) {
     const int grid = std::min(g.ntiles, sm_count());
-    cudaError_t e = H == 64 ? launch(k_win_bwd<64>, grid, BWD_TH, BwdLayout<64>::BYTES, g, st)
-                            : launch(k_win_bwd<32>, grid, BWD_TH, BwdLayout<32>::BYTES, g, st);
+    cudaError_t e;
+    if (H == 64) e = g.kx2 ? backward<64, 2>(g, grid, st) : backward<64, 1>(g, grid, st);
+    else e = g.kx2 ? backward<32, 2>(g, grid, st) : backward<32, 1>(g, grid, st);
     if (e != cudaSuccess) return e;
-    return win_reduce(g, H, grid, st);
+    return win_reduce(g, H, grid, g.kx2 ? 64 : 0, st);
 }
 
-cudaError_t win_reduce(const WinArgs &g, int H, int nparts, cudaStream_t st) {
-    k_win_reduce<<<3 * H + g.nfc, TM, 0, st>>>(g, H, nparts);
+// fc_lane: the lane of the first row of W_fc's gradient
+cudaError_t win_reduce(const WinArgs &g, int H, int nparts, int fc_lane, cudaStream_t st) {
+    k_win_reduce<<<g.part_cols, TM, 0, st>>>(g, H, nparts, fc_lane);
     return cudaGetLastError();
 }
 

@@ -16,7 +16,9 @@
 // rate; the CUDA cores' FMAs give 74.  With the fused window (see gru_win.cu,
 // whose layouts these kernels share) loss and gradients of 65 536 rows, T =
 // 10, H = 64 take 1.23 ms instead of 5.5 ms with one FP32 kernel per
-// product, and of 762 rows, H = 32, 0.46 ms instead of 2.7 ms.
+// product, and of 762 rows, H = 32, 0.46 ms instead of 2.7 ms; with 99
+// features and 50 outputs 1.9 ms instead of 6.5 ms (X W_x^T 217 us, forward
+// 385, state gradients 423, weight gradients 368 and 230).
 //
 // Values beyond the largest BF16 number are clamped to it (an infinite
 // feature saturates the gates as it does in FP32); a NaN stays one.
@@ -105,7 +107,6 @@ template <bool CL = false> __device__ __forceinline__ void put4_3(uint8_t *img, 
 #pragma unroll
     for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2 *>(img + p * step + at) = make_uint2(a[p], b[p]);
 }
-__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 template <typename F> __device__ __forceinline__ void build3(uint8_t *img, int step, int rows, F src) {
     for (int e = threadIdx.x; e < rows * 8; e += W32_TH) {
@@ -116,12 +117,12 @@ template <typename F> __device__ __forceinline__ void build3(uint8_t *img, int s
         put8_3<true>(img, step, r, c, v);   // (8-row groups are 1024 bytes apart: row * 128 throughout)
     }
 }
-__device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &x, uint8_t *img) {
+__device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &x, uint8_t *img, int x0 = 0) {
+    const int n = g.n_in - x0;
 #pragma unroll
     for (int i = 0; i < XTile<W32_TH>::NV; ++i) {
         const int e = threadIdx.x + i * W32_TH, row = e >> 4, c = (e & 15) * 4;
-        const float v[4] = {x.v[i].x, c + 1 < g.n_in ? x.v[i].y : 0.f, c + 2 < g.n_in ? x.v[i].z : 0.f,
-                            c + 3 < g.n_in ? x.v[i].w : 0.f};
+        const float v[4] = {x.v[i].x, c + 1 < n ? x.v[i].y : 0.f, c + 2 < n ? x.v[i].z : 0.f, c + 3 < n ? x.v[i].w : 0.f};
         put4_3<true>(img, IMG, row, c, v);
     }
 }
@@ -133,21 +134,93 @@ __device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &
 // for X W_x^T, r h for the candidate.  Tensor memory: X W_x^T [0, 3H),
 // h U_zr^T [3H, 5H), (r h) U_h^T [5H, 6H), outputs [6H, 6H + nfc).
 // Bound by the chain of three MMA round trips a step with the splits and gate
-// functions between them.
-template <int H> struct Fwd32Layout {
+// functions between them.  Two chunks of features (XC = 2) leave no room for
+// W_x: X W_x^T comes from memory (k_win32_x).
+template <int H, int XC> struct Fwd32Layout {
     static constexpr int WS = 3 * H * 128, FS = 64 * 128;   // bytes of one part
-    static constexpr int WX = 0, U = WX + 3 * WS, F = U + 3 * WS, A = F + 3 * FS, BARS = A + 3 * IMG, BYTES = BARS + 64 + 1024;
+    static constexpr int WX = 0, U = WX + (XC == 1 ? 3 * WS : 0), F = U + 3 * WS, A = F + 3 * FS, BARS = A + 3 * IMG, BYTES = BARS + 64 + 1024;
     static constexpr int COLS = H == 64 ? 512 : 256;
 };
 
+// X W_x^T of every step for two chunks of features, [step][tile][column / 4][row][4].
+// Each chunk's products are accumulated apart (W_x and one chunk's images fill
+// the shared memory) and added in FP32.  Bound by the chain of split, products
+// and read-out, two of them a tile.
+template <int H> struct X32Layout {
+    static constexpr int WS = 3 * H * 128;
+    static constexpr int W = 0, A = W + 6 * WS, BARS = A + 3 * IMG, BYTES = BARS + 64 + 1024;   // W: 3 parts of each chunk
+    static constexpr int COLS = H == 64 ? 512 : 256;
+};
 template <int H>
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_x(const WinArgs g) {
+    using L = X32Layout<H>;
+    constexpr int NC = 3 * H / 4;   // columns of a thread
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = align1k(smem_raw), *sA = base + L::A;
+    const uint32_t u = smem_u32(base);
+    for (int x = 0; x < 2; ++x)
+        build3(base + L::W + 3 * x * L::WS, L::WS, 3 * H, [&](int r, int c) {
+            return 64 * x + c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + 64 * x + c) : 0.f;
+        });
+    Cta cta;
+    cta.init(reinterpret_cast<uint64_t *>(base + L::BARS), 2, L::COLS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = warp & 3, part = warp >> 2, row = q * 32 + lane, c0 = part * NC;
+    const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
+    uint32_t ph = 0;
+    bool ok = true;
+    const int n = g.T * g.ntiles;
+    XTile<W32_TH> xt;
+    if ((int)blockIdx.x < n) xt.load(g, blockIdx.x / g.ntiles, blockIdx.x % g.ntiles * TM);
+    for (int it = blockIdx.x; ok && it < n; it += gridDim.x) {
+        const int s = it / g.ntiles, p0 = it % g.ntiles * TM;
+        store_x3(g, xt, sA);
+        xt.load(g, s, p0, 64);
+        if (!(ok = cta.hand_over(ok))) break;
+        if (tid == 0) {
+            mma3_k(cta.tmem, u + L::A, IMG, u + L::W, L::WS, 3 * H, 4);
+            tc_commit(cta.bar0);
+        }
+        ok = cta.wait(0, ph);
+        ph ^= 1;
+        store_x3(g, xt, sA, 64);
+        if (!(ok = cta.hand_over(ok))) break;
+        if (tid == 0) {
+            mma3_k(cta.tmem + 3 * H, u + L::A, IMG, u + L::W + 3 * L::WS, L::WS, 3 * H, g.kx2);
+            tc_commit(cta.bar0);
+        }
+        const int nx = it + gridDim.x;
+        if (nx < n) xt.load(g, nx / g.ntiles, nx % g.ntiles * TM);
+        ok = cta.wait(0, ph);
+        ph ^= 1;
+        float *o = g.GX + (size_t)it * (3 * TM * H);
+#pragma unroll
+        for (int i = 0; i < NC; i += 8) {
+            float a[8], b[8];
+            tmem_ld8(tl + c0 + i, a);
+            tmem_ld8(tl + 3 * H + c0 + i, b);
+            tmem_wait();
+            keep(a);
+            keep(b);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) a[j] = whole(a[j], 4) + whole(b[j], g.kx2);
+            st4(o + blk(c0 + i, row), a);
+            st4(o + blk(c0 + i + 4, row), a + 4);
+        }
+    }
+    ok = cta.hand_over(ok);
+    cta.finish(1, L::COLS, g.status);
+}
+
+template <int H, int XC>
 __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
-    using L = Fwd32Layout<H>;
+    using L = Fwd32Layout<H, XC>;
     constexpr int NC = H / 4;   // state columns of a thread
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = align1k(smem_raw), *sA = base + L::A;
     const uint32_t u = smem_u32(base), uA = u + L::A;
-    build3(base + L::WX, L::WS, 3 * H, [&](int r, int c) { return c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + c) : 0.f; });
+    if (XC == 1)
+        build3(base + L::WX, L::WS, 3 * H, [&](int r, int c) { return c < g.n_in ? __ldg(g.Wx + (size_t)r * g.n_in + c) : 0.f; });
     build3(base + L::U, L::WS, 3 * H, [&](int r, int c) { return c < H ? __ldg(g.Uh + (size_t)r * H + c) : 0.f; });
     build3(base + L::F, L::FS, g.nfc, [&](int r, int c) { return r < g.n_out && c < H ? __ldg(g.Wfc + (size_t)r * H + c) : 0.f; });
     Cta cta;
@@ -169,7 +242,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
             if (g.h0 && valid) ld4(g.h0 + (size_t)gp * H + c0 + i, hv + i);
             st4(g.hb + (size_t)tile * tblk + blk(c0 + i, row), hv + i);
         }
-        xt.load(g, 0, p0);
+        if (XC == 1) xt.load(g, 0, p0);
 #pragma unroll
         for (int i = 0; i < NC; i += 8) put8_3(sA, IMG, row, c0 + i, hv + i);
         if (!(ok = cta.hand_over(ok))) break;
@@ -201,28 +274,36 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
         };
         for (int s = 0; s < g.T; ++s) {
             const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
-            ok = cta.wait(0, ph);
-            ph ^= 1;
-            store_x3(g, xt, sA);
-            if (!(ok = cta.hand_over(ok))) break;
-            if (tid == 0) {
-                mma3_k(cta.tmem, uA, IMG, u + L::WX, L::WS, 3 * H, 4);
-                tc_commit(cta.bar0);
+            float gr[XC == 2 ? NC : 1], gz[XC == 2 ? NC : 1], gc[XC == 2 ? NC : 1];   // X W_x^T from memory
+            const float *gx = g.GX + 3 * sb;
+            if (XC == 2) {
+#pragma unroll
+                for (int i = 0; i < NC; i += 4) ld4(gx + blk(H + c0 + i, row), gr + i);
             }
-            if (s > 0) outputs(s - 1);
             ok = cta.wait(0, ph);
             ph ^= 1;
+            if (XC == 1) {
+                store_x3(g, xt, sA);
+                if (!(ok = cta.hand_over(ok))) break;
+                if (tid == 0) {
+                    mma3_k(cta.tmem, uA, IMG, u + L::WX, L::WS, 3 * H, 4);
+                    tc_commit(cta.bar0);
+                }
+                if (s > 0) outputs(s - 1);
+                ok = cta.wait(0, ph);
+                ph ^= 1;
+            }
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8], rr[8];
-                tmem_ld8(tl + H + c0 + i, a);
+                if (XC == 1) tmem_ld8(tl + H + c0 + i, a);
                 tmem_ld8(tl + 4 * H + c0 + i, b);
                 tmem_wait();
-                keep(a);
+                if (XC == 1) keep(a);
                 keep(b);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    rr[j] = sigm(whole(a[j], 4) + whole(b[j], H / 16));
+                    rr[j] = sigm((XC == 1 ? whole(a[j], 4) : gr[(i + j) % (XC == 2 ? NC : 1)]) + whole(b[j], H / 16));
                     a[j] = rr[j] * hv[i + j];
                 }
                 st4(g.r + sb + blk(c0 + i, row), rr);
@@ -234,25 +315,39 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
                 mma3_k(cta.tmem + 5 * H, uA, IMG, u + L::U + 2 * H * 128, L::WS, H, H / 16);
                 tc_commit(cta.bar0);
             }
-            if (s + 1 < g.T) xt.load(g, s + 1, p0);
+            if (XC == 1) {
+                if (s + 1 < g.T) xt.load(g, s + 1, p0);
+            } else {
+                if (s > 0) outputs(s - 1);
+#pragma unroll
+                for (int i = 0; i < NC; i += 4) {
+                    ld4(gx + blk(c0 + i, row), gz + i);
+                    ld4(gx + blk(2 * H + c0 + i, row), gc + i);
+                }
+            }
             ok = cta.wait(0, ph);
             ph ^= 1;
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8], zz[8], cc[8];
-                tmem_ld8(tl + c0 + i, a);
+                if (XC == 1) {
+                    tmem_ld8(tl + c0 + i, a);
+                    tmem_ld8(tl + 2 * H + c0 + i, zz);
+                }
                 tmem_ld8(tl + 3 * H + c0 + i, b);
-                tmem_ld8(tl + 2 * H + c0 + i, zz);
                 tmem_ld8(tl + 5 * H + c0 + i, cc);
                 tmem_wait();
-                keep(a);
+                if (XC == 1) {
+                    keep(a);
+                    keep(zz);
+                }
                 keep(b);
-                keep(zz);
                 keep(cc);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const float z = sigm(whole(a[j], 4) + whole(b[j], H / 16)),
-                                c = tanhf(whole(zz[j], 4) + whole(cc[j], H / 16));
+                    const int k = (i + j) % (XC == 2 ? NC : 1);
+                    const float z = sigm((XC == 1 ? whole(a[j], 4) : gz[k]) + whole(b[j], H / 16)),
+                                c = tanhf((XC == 1 ? whole(zz[j], 4) : gc[k]) + whole(cc[j], H / 16));
                     zz[j] = z;
                     cc[j] = c;
                     hv[i + j] = z * hv[i + j] + (1.0f - z) * c;
@@ -464,7 +559,9 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
 // shared memory): a CTA takes a contiguous range of blocks, accumulates each
 // in tensor memory, adds it to FP32 registers and these, every few blocks, to
 // a sum kept in tensor memory (a sum in one run of 67 blocks loses twice as much).
-// Bound by memory (2.6 kB a row and step at H = 64) and the splits.
+// Bound by memory (2.6 kB a row and step at H = 64) and the splits.  X2: the
+// products of the second chunk of features with dA alone, in a launch of its
+// own (their sums have no room beside the others).
 constexpr int GR = 64, GIMG = GR * 128;   // rows of a block, one image
 constexpr int G32_RUN = 8;                // blocks added up in registers before they join the sum in tensor memory
 template <int H> struct Grad32Layout {
@@ -477,9 +574,10 @@ template <int H> struct Grad32Layout {
     static constexpr int NB = (3 * H + 64) / 8 / 4;   // blocks of 8 gradient columns a thread adds up
 };
 
-template <int H>
+template <int H, bool X2>
 __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
     using L = Grad32Layout<H>;
+    constexpr int X0 = X2 ? 64 : 0, NB = X2 ? 3 * H / 32 : L::NB;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = align1k(smem_raw);
     const uint32_t u = smem_u32(base);
@@ -490,11 +588,11 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q = warp & 3, part = warp >> 2, row = q * 32 + lane;
     const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
-    const int ncol = 3 * H + g.nfc;
+    const int ncol = 3 * H + (X2 ? 0 : g.nfc), out0 = X2 ? 3 * H + g.nfc : 0;
     const size_t tblk = (size_t)TM * H;
-    float acc[L::NB][8];
+    float acc[NB][8];
 #pragma unroll
-    for (int b = 0; b < L::NB; ++b)
+    for (int b = 0; b < NB; ++b)
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[b][j] = 0.f;
     const long long n = 2LL * g.T * g.ntiles;   // blocks: (tile, half, step), steps fastest
@@ -505,7 +603,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
         ok = cta.wait(0, ph);
         ph ^= 1;
 #pragma unroll
-        for (int b = 0; b < L::NB; ++b) {
+        for (int b = 0; b < NB; ++b) {
             const int c = 8 * (part + 4 * b);
             if (c < ncol) {
                 float v[8];
@@ -520,7 +618,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
     bool summed = false;
     auto flush = [&]() {   // the registers' sums into tensor memory
 #pragma unroll
-        for (int b = 0; b < L::NB; ++b) {
+        for (int b = 0; b < NB; ++b) {
             const int c = 8 * (part + 4 * b);
             if (c < ncol) {
                 if (summed) {
@@ -552,18 +650,20 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
         const float *hnp = last ? g.hT + (size_t)(tile * TM + tr) * H + lc : g.hb + o + (size_t)g.ntiles * tblk;
         const int hstep = last ? 4 : 4 * TM;
         const bool hnok = !last || tile * TM + tr < g.P;
-        const int xr = tid >> 3, xc = (tid & 7) * 8, gp = tile * TM + r0 + xr;   // X and dD: 8 threads a row
+        const int xr = tid >> 3, xc = (tid & 7) * 8, fc = X0 + xc, gp = tile * TM + r0 + xr;   // X and dD: 8 threads a row
         const float *dsrc = g.dD + ((size_t)s * g.P + gp) * g.n_out + xc;
         float hp[8], rr[8], xv[8];
         if (mine) {
-            ld4(g.hb + o, hp); ld4(g.hb + o + 4 * TM, hp + 4);
-            ld4(g.r + o, rr); ld4(g.r + o + 4 * TM, rr + 4);
+            if (!X2) {
+                ld4(g.hb + o, hp); ld4(g.hb + o + 4 * TM, hp + 4);
+                ld4(g.r + o, rr); ld4(g.r + o + 4 * TM, rr + 4);
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 prefetch_l2(g.dG + gz + k * tblk);
                 prefetch_l2(g.dG + gz + k * tblk + 4 * TM);
             }
-            if (hnok) {
+            if (!X2 && hnok) {
                 prefetch_l2(hnp);
                 prefetch_l2(hnp + hstep);
             }
@@ -571,17 +671,17 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) xv[j] = 0.f;
         if (gp < g.P) {
-            const float *src = g.X + ((size_t)s * g.P + gp) * g.ldx + xc;
+            const float *src = g.X + ((size_t)s * g.P + gp) * g.ldx + fc;
             if (g.xvec) {
-                if (xc < g.n_in) ld4(src, xv);
-                if (xc + 4 < g.n_in) ld4(src + 4, xv + 4);
+                if (fc < g.n_in) ld4(src, xv);
+                if (fc + 4 < g.n_in) ld4(src + 4, xv + 4);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) xv[j] = xc + j < g.n_in ? xv[j] : 0.f;
+                for (int j = 0; j < 8; ++j) xv[j] = fc + j < g.n_in ? xv[j] : 0.f;
             } else {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) xv[j] = xc + j < g.n_in ? __ldg(src + j) : 0.f;
+                for (int j = 0; j < 8; ++j) xv[j] = fc + j < g.n_in ? __ldg(src + j) : 0.f;
             }
-            if (xc < g.n_out) prefetch_l2(dsrc);
+            if (!X2 && xc < g.n_out) prefetch_l2(dsrc);
         }
         if (it > i0) {
             drain();   // the images are free again
@@ -594,14 +694,16 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
         }
         put8_3<true>(base + L::X, GIMG, xr, xc, xv);
         if (mine) {
-            put8_3(base + L::HP, GIMG, lr, lc, hp);
+            if (!X2) {
+                put8_3(base + L::HP, GIMG, lr, lc, hp);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) rr[j] *= hp[j];
-            put8_3(base + L::RH, GIMG, lr, lc, rr);
+                for (int j = 0; j < 8; ++j) rr[j] *= hp[j];
+                put8_3(base + L::RH, GIMG, lr, lc, rr);
+            }
             ld4(g.dG + gz + 2 * tblk, hp); ld4(g.dG + gz + 2 * tblk + 4 * TM, hp + 4);   // dA_c
 #pragma unroll
             for (int j = 0; j < 8; ++j) rr[j] = 0.f;
-            if (hnok) {
+            if (!X2 && hnok) {
                 ld4(hnp, rr);
                 ld4(hnp + hstep, rr + 4);
             }
@@ -610,20 +712,20 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
             if (H == 64) put8_3(base + L::GRR, GIMG, lr, lc, ar);
             else put8_3(base + L::GZ, GIMG, lr, H + lc, ar);
         }
-        if (xc < g.nfc) {
+        if (!X2 && xc < g.nfc) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) xv[j] = gp < g.P && xc + j < g.n_out ? __ldg(dsrc + j) : 0.f;
             put8_3<true>(base + L::DD, GIMG, xr, xc, xv);
         }
         if (mine) {
             put8_3(base + L::GC, GIMG, lr, lc, hp);
-            put8_3(base + L::HN, GIMG, lr, lc, rr);
+            if (!X2) put8_3(base + L::HN, GIMG, lr, lc, rr);
         }
         if (!(ok = cta.hand_over(ok))) break;
         if (tid == 0) {
             mma3_mn(cta.tmem, u + L::X, GIMG, L::HP - L::X, u + L::GZ, GIMG, L::GRR - L::GZ, 2 * H, GR);
             mma3_mn(cta.tmem + 2 * H, u + L::X, GIMG, L::RH - L::X, u + L::GC, GIMG, GIMG, H, GR);
-            mma3_mn(cta.tmem + 3 * H, u + L::HN, GIMG, L::HP - L::X, u + L::DD, GIMG, GIMG, g.nfc, GR);
+            if (!X2) mma3_mn(cta.tmem + 3 * H, u + L::HN, GIMG, L::HP - L::X, u + L::DD, GIMG, GIMG, g.nfc, GR);
             tc_commit(cta.bar0);
         }
     }
@@ -634,7 +736,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
     if (ok && summed && !*cta.abort_flag) {
         float *o = g.part + (size_t)blockIdx.x * g.part_cols * TM;
 #pragma unroll
-        for (int b = 0; b < L::NB; ++b) {
+        for (int b = 0; b < NB; ++b) {
             const int c = 8 * (part + 4 * b);
             if (c >= ncol) continue;
             float v[8];
@@ -642,7 +744,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
             tmem_wait();
             keep(v);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) o[(size_t)(c + j) * TM + row] = v[j];
+            for (int j = 0; j < 8; ++j) o[(size_t)(out0 + c + j) * TM + row] = v[j];
         }
     }
     cta.finish(1, L::COLS, g.status);
@@ -650,21 +752,26 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
 
 }  // namespace
 
-cudaError_t win32_forward(const WinArgs &g, int H, cudaStream_t st) {
-    const int grid = std::min(g.ntiles, sm_count());
-    if (H == 64) return launch(k_win32_fwd<64>, grid, W32_TH, Fwd32Layout<64>::BYTES, g, st);
-    return launch(k_win32_fwd<32>, grid, W32_TH, Fwd32Layout<32>::BYTES, g, st);
+namespace {
+template <int H> cudaError_t forward(const WinArgs &g, cudaStream_t st) {
+    const int sms = sm_count(), grid = std::min(g.ntiles, sms);
+    if (!g.kx2) return launch(k_win32_fwd<H, 1>, grid, W32_TH, Fwd32Layout<H, 1>::BYTES, g, st);
+    const cudaError_t e = launch(k_win32_x<H>, (int)std::min<long long>((long long)g.T * g.ntiles, sms), W32_TH,
+                                 X32Layout<H>::BYTES, g, st);
+    return e != cudaSuccess ? e : launch(k_win32_fwd<H, 2>, grid, W32_TH, Fwd32Layout<H, 2>::BYTES, g, st);
 }
+template <int H> cudaError_t backward(const WinArgs &g, cudaStream_t st) {
+    const int grid = std::min(g.ntiles, sm_count()), ggrid = win32_parts(g.T, g.P);
+    cudaError_t e = launch(k_win32_bwd<H>, grid, W32_TH, Bwd32Layout<H>::BYTES, g, st);
+    if (e == cudaSuccess) e = launch(k_win32_grad<H, false>, ggrid, W32_TH, Grad32Layout<H>::BYTES, g, st);
+    if (e == cudaSuccess && g.kx2) e = launch(k_win32_grad<H, true>, ggrid, W32_TH, Grad32Layout<H>::BYTES, g, st);
+    return e != cudaSuccess ? e : win_reduce(g, H, ggrid, 0, st);
+}
+}  // namespace
 
+cudaError_t win32_forward(const WinArgs &g, int H, cudaStream_t st) { return H == 64 ? forward<64>(g, st) : forward<32>(g, st); }
 cudaError_t win32_backward(const WinArgs &g, int H, cudaStream_t st) {
-    const int sms = sm_count(), grid = std::min(g.ntiles, sms), ggrid = win32_parts(g.T, g.P);
-    cudaError_t e = H == 64 ? launch(k_win32_bwd<64>, grid, W32_TH, Bwd32Layout<64>::BYTES, g, st)
-                            : launch(k_win32_bwd<32>, grid, W32_TH, Bwd32Layout<32>::BYTES, g, st);
-    if (e != cudaSuccess) return e;
-    e = H == 64 ? launch(k_win32_grad<64>, ggrid, W32_TH, Grad32Layout<64>::BYTES, g, st)
-                : launch(k_win32_grad<32>, ggrid, W32_TH, Grad32Layout<32>::BYTES, g, st);
-    if (e != cudaSuccess) return e;
-    return win_reduce(g, H, ggrid, st);
+    return H == 64 ? backward<64>(g, st) : backward<32>(g, st);
 }
 
 // CTAs of the weight-gradient kernel, each with a partial sum of its own

@@ -113,14 +113,16 @@ __device__ __forceinline__ void st4(float *p, const float *v) {
 // saved activations: element (column c, row) of a tile's block
 __device__ __forceinline__ size_t blk(int c, int row) { return (size_t)(c >> 2) * (4 * TM) + 4 * row; }
 
-// The feature rows of a tile, coalesced: 16 lanes take one row's 64 columns.
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// 64 columns, from x0 on, of a tile's feature rows, coalesced: 16 lanes take one row's.
 template <int NTH> struct XTile {
     static constexpr int NV = TM * 16 / NTH;
     float4 v[NV];
-    __device__ __forceinline__ void load(const WinArgs &g, int s, int p0) {
+    __device__ __forceinline__ void load(const WinArgs &g, int s, int p0, int x0 = 0) {
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
-            const int e = threadIdx.x + i * NTH, row = e >> 4, c = (e & 15) * 4;
+            const int e = threadIdx.x + i * NTH, row = e >> 4, c = x0 + (e & 15) * 4;
             v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (p0 + row >= g.P || c >= g.n_in) continue;
             const float *src = g.X + ((size_t)s * g.P + p0 + row) * g.ldx + c;
@@ -134,12 +136,20 @@ template <int NTH> struct XTile {
             }
         }
     }
-    __device__ __forceinline__ void store(const WinArgs &g, uint8_t *img) const {
+    __device__ __forceinline__ void prefetch(const WinArgs &g, int s, int p0, int x0) const {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int e = threadIdx.x + i * NTH, row = e >> 4, c = x0 + (e & 15) * 4;
+            if (p0 + row < g.P && c < g.n_in) prefetch_l2(g.X + ((size_t)s * g.P + p0 + row) * g.ldx + c);
+        }
+    }
+    __device__ __forceinline__ void store(const WinArgs &g, uint8_t *img, int x0 = 0) const {
+        const int n = g.n_in - x0;
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
             const int e = threadIdx.x + i * NTH, row = e >> 4, c = (e & 15) * 4;
-            const float a = v[i].x, b = c + 1 < g.n_in ? v[i].y : 0.f, d = c + 2 < g.n_in ? v[i].z : 0.f,
-                        f = c + 3 < g.n_in ? v[i].w : 0.f;   // (columns past n_in are not read as features)
+            const float a = v[i].x, b = c + 1 < n ? v[i].y : 0.f, d = c + 2 < n ? v[i].z : 0.f,
+                        f = c + 3 < n ? v[i].w : 0.f;   // (columns past n_in are not read as features)
             *reinterpret_cast<uint2 *>(img + swz(row, c >> 3) + (c & 4) * 2) = make_uint2(pack(a, b), pack(d, f));
         }
     }
