@@ -140,6 +140,7 @@ struct StepInst {
     void *X;          // its rows of the batch's features and outputs
     const float *d;
     float *xcp, *vc;  // padded x_c, v_corr
+    int tile0, ntiles, row;   // its GRU tiles in the batch; its first state row
 };
 constexpr int kBatch = 32;   // instances of one launch (their parameters stay below 32 KB)
 
@@ -189,7 +190,8 @@ cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float>
                                void *X, cudaStream_t st);
 // The passes over the tiles of n <= kBatch instances of one net shape in one
 // launch each (BF16 features); the same bits as the launches above.
-cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, cudaStream_t st);
+// (the coarse one also writes the first state row of every GRU tile of the instances to hrow)
+cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, int *hrow, cudaStream_t st);
 cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st);
 cudaError_t launch_residual_cf_batch(const StepInst *in, int n, cudaStream_t st);
 cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st);

