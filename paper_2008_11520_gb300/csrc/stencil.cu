@@ -1684,23 +1684,172 @@ k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__r
     rhs_cta<D>(g, fc, &tmV, bf, blockIdx.x, blockIdx.y);
 }
 
+// The all-fluid pairs of tiles of an FP32 right-hand side, without shared
+// memory: a warp walks up NS rows of 62 node columns.  A lane holds the nodes
+// E and E + 1 (E even) and works on the cells E - 1 and E and on its two nodes
+// in packed arithmetic; columns E - 1 and E + 2 and the contributions of cell
+// E + 1 come from its neighbours (lane 31 has none and stores nothing).  A
+// row's nodes are read once and enter the three node rows they touch, a cell
+// row's contributions the two, in the order of rhs_tile: the same bits.
+// rhs_tile is bound by its shared-memory traffic (16 stores and 26 loads for
+// two nodes; 87% of the pipe); this takes 8 shuffles: 8192 x 2048 cells 115 ->
+// 87 us, 4096 x 1024 33 -> 27.  Bound by the latency of the row reads at the 24
+// warps an SM that its registers allow (80 a thread; 64 spill: 102 us, 84 with
+// two CTAs: 104 us; reading two rows ahead: 97 us).
+template <int NS>
+__device__ __forceinline__ void rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const float *__restrict__ vc,
+                                          float *__restrict__ bf, int wx, int strip) {
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, E = 62 * wx + 2 * lane, J0 = strip * NS, ty = J0 / TYC, bx = E >> 6;
+    const bool fast = lane < 31 && tile_fluid(g, 2 * bx, ty, 1) && tile_fluid(g, 2 * bx + 1, ty, 1);
+    if (!__any_sync(ALL, fast)) return;
+    // (an all-fluid tile has neighbours on every side: rows J0 - 1 .. J0 + NS exist)
+    const bool in = E < g.pitch, edge = lane == 0 && E > 0;
+    const float *q = vc + (size_t)(J0 - 1) * g.pitch + E;
+    struct Row {
+        float2 u, v;
+        float lu, lv;
+    };
+    auto load = [&](const float *p) {
+        Row r;
+        r.u = r.v = make_float2(0.f, 0.f);
+        r.lu = r.lv = 0.f;
+        if (in) {
+            r.u = __ldg(reinterpret_cast<const float2 *>(p));
+            r.v = __ldg(reinterpret_cast<const float2 *>(p + g.plane));
+        }
+        if (edge) {
+            r.lu = __ldg(p - 1);
+            r.lv = __ldg(p + g.plane - 1);
+        }
+        return r;
+    };
+    // columns (E - 1, E), (E, E + 1), (E + 1, E + 2) of a row
+    auto spread = [&](float2 a, float left, F2 (&o)[3]) {
+        const float l = __shfl_up_sync(ALL, a.y, 1), r = __shfl_down_sync(ALL, a.x, 1);
+        o[0] = pack2(lane == 0 ? left : l, a.x);
+        o[1] = pack2(a.x, a.y);
+        o[2] = pack2(a.y, r);
+    };
+    // corners of the cells (E, E + 1) from those of (E - 1, E)
+    auto east = [&](F2 c) {
+        float lo, hi;
+        unpack2(c, lo, hi);
+        return pack2(hi, __shfl_down_sync(ALL, lo, 1));
+    };
+    const ConvK<F2> k2(fc);
+    // (scalar coefficients from the parameters: packed ones would take 18 registers)
+    auto stencil = [&](int sy, const F2 (&r)[3], F2 acc) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            float a, b, c, d;
+            unpack2(acc, a, b);
+            unpack2(r[x], c, d);
+            acc = pack2(fmaf(fc.nB[sy][x], c, a), fmaf(fc.nB[sy][x], d, b));
+        }
+        return acc;
+    };
+    const F2 zero = pack2(0.f, 0.f);
+    F2 pu[2], pv[2];                             // the row below
+    F2 u1 = zero, v1 = zero, u2, v2;             // linear terms of the row below and of this one, so far
+    F2 bu = zero, bv = zero;                     // the contributions of the cell row below the row below
+    {
+        const Row r = load(q);
+        F2 u[3], v[3];
+        spread(r.u, r.lu, u);
+        spread(r.v, r.lv, v);
+        pu[0] = u[0]; pu[1] = u[1];
+        pv[0] = v[0]; pv[1] = v[1];
+        u2 = stencil(0, u, zero);
+        v2 = stencil(0, v, zero);
+    }
+    Row nx = load(q + g.pitch);
+    float *out = bf + (size_t)(J0 - 1) * g.pitch + E;
+#pragma unroll 2
+    for (int j = 0; j <= NS; ++j) {   // node row J0 + j comes in, row J0 + j - 1 goes out
+        const Row r = nx;
+        q += g.pitch;
+        if (j < NS) nx = load(q + g.pitch);
+        F2 u[3], v[3];
+        spread(r.u, r.lu, u);
+        spread(r.v, r.lv, v);
+        const F2 cu4[4] = {pu[0], pu[1], u[0], u[1]}, cv4[4] = {pv[0], pv[1], v[0], v[1]};
+        F2 cu[4], cv[4];
+        convection(k2, cu4, cv4, cu, cv);
+        const F2 su = stencil(2, u, u1), sv = stencil(2, v, v1);
+        u1 = stencil(1, u, u2);
+        v1 = stencil(1, v, v2);
+        u2 = stencil(0, u, zero);
+        v2 = stencil(0, v, zero);
+        pu[0] = u[0]; pu[1] = u[1];
+        pv[0] = v[0]; pv[1] = v[1];
+        const F2 ru = vsub(su, vadd(bu, vadd(cu[1], east(cu[0])))), rv = vsub(sv, vadd(bv, vadd(cv[1], east(cv[0]))));
+        bu = vadd(cu[3], east(cu[2]));
+        bv = vadd(cv[3], east(cv[2]));
+        if (fast && j > 0) {
+            float a, b;
+            unpack2(ru, a, b);
+            store2(out, a, b);
+            unpack2(rv, a, b);
+            store2(out + g.plane, a, b);
+        }
+        out += g.pitch;
+    }
+}
+
+// The tiles that rhs_march leaves out first, one a CTA, then 8 of its warps a
+// CTA.  `local` is the CTA's place in the mesh's grid of rhs_march_ctas.
+constexpr int MARCH_THREADS = 256, MARCH_CTAS = 3;
+__host__ __device__ __forceinline__ int march_columns(const MeshGeom &g) { return (g.nxf + 62) / 62; }
+template <int NS> int rhs_march_ctas(const MeshGeom &g) {
+    const long long warps = (long long)march_columns(g) * (g.nty * (TYC / NS));
+    return g.n_slow_tiles + (int)((warps + MARCH_THREADS / 32 - 1) / (MARCH_THREADS / 32));
+}
+template <int NS>
+__device__ __forceinline__ void rhs_big(const MeshGeom &g, const FemCoef<float> &fc, const CUtensorMap *tmV,
+                                        const float *__restrict__ vc, float *__restrict__ bf, int local) {
+    if (local < g.n_slow_tiles) {
+        const int tile = __ldg(g.slow_tiles + local), ty = tile / g.ntx;
+        rhs_cta<BigTile>(g, fc, tmV, bf, tile - ty * g.ntx, ty);
+        return;
+    }
+    const int w = (local - g.n_slow_tiles) * (MARCH_THREADS / 32) + (int)(threadIdx.x >> 5), nc = march_columns(g);
+    if (w < nc * (g.nty * (TYC / NS))) rhs_march<NS>(g, fc, vc, bf, w % nc, w / nc);
+}
+template <int NS>
+__global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS)
+k_rhs_march(MeshGeom g, FemCoef<float> fc, const __grid_constant__ CUtensorMap tmV, const float *__restrict__ vc,
+            float *__restrict__ bf) {
+    rhs_big<NS>(g, fc, &tmV, vc, bf, blockIdx.x);
+}
+
 struct RhsBatch {
     CUtensorMap tmV[kBatch];
     int n, first[kBatch + 1];
     struct {
         MeshGeom g;
         const FemCoef<float> *fc;
+        const float *vc;
         float *bf;
     } inst[kBatch];
 };
-template <typename D>
-__global__ void __launch_bounds__(D::THREADS) k_rhs_batch(const __grid_constant__ RhsBatch p) {
+__global__ void __launch_bounds__(SmallTile::THREADS) k_rhs_batch_small(const __grid_constant__ RhsBatch p) {
+    using D = SmallTile;
     __shared__ FemCoef<float> fc;
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);   // (visible after rhs_cta's first barrier)
     const int ntx = (p.inst[i].g.nxf + D::TXC - 1) / D::TXC;
     rhs_cta<D>(p.inst[i].g, fc, &p.tmV[i], p.inst[i].bf, local % ntx, local / ntx);
+}
+template <int NS>
+__global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS) k_rhs_batch_march(const __grid_constant__ RhsBatch p) {
+    __shared__ FemCoef<float> fc;
+    int local;
+    const int i = batch_instance(p.first, p.n, local);
+    stage_coef(fc, p.inst[i].fc);
+    __syncthreads();
+    rhs_big<NS>(p.inst[i].g, fc, &p.tmV[i], p.inst[i].vc, p.inst[i].bf, local);
 }
 
 // S5 + S6 fused for the correction step: the v_corr window of a right-hand
@@ -2305,10 +2454,25 @@ cudaError_t run_rhs_d(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T
     return cudaGetLastError();
 }
 
+// Rows a warp of rhs_march walks: 16 from 4096 tiles on (2 100 warps and
+// more), else 4, whose warps work on five cell rows for them.
+inline bool march_tall(long long tiles) { return tiles >= 4096; }
+template <int NS>
+cudaError_t run_rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const float *vcorr, float *bf, cudaStream_t st) {
+    CUtensorMap tm;
+    if (!rhs_map<BigTile, float>(g, vcorr, &tm)) return cudaErrorInvalidValue;
+    const size_t sm = RhsLayout<BigTile>::bytes<float>();
+    cudaError_t e = set_smem(k_rhs_march<NS>, sm);
+    if (e != cudaSuccess) return e;
+    k_rhs_march<NS><<<rhs_march_ctas<NS>(g), MARCH_THREADS, sm, st>>>(g, fc, tm, vcorr, bf);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t run_rhs(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st) {
     if (use_small(g, tiles_of(g))) return run_rhs_d<SmallTile, T>(g, fc, vcorr, bf, st);
-    return run_rhs_d<BigTile, T>(g, fc, vcorr, bf, st);
+    if constexpr (sizeof(T) == 8) return run_rhs_d<BigTile, T>(g, fc, vcorr, bf, st);
+    else return march_tall(tiles_of(g)) ? run_rhs_march<16>(g, fc, vcorr, bf, st) : run_rhs_march<4>(g, fc, vcorr, bf, st);
 }
 
 cudaError_t launch_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f64,
@@ -2451,7 +2615,7 @@ cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st)
     }
 }
 
-template <typename D> static cudaError_t rhs_batch(const StepInst *in, int n, cudaStream_t st) {
+template <typename D, int NS> static cudaError_t rhs_batch(const StepInst *in, int n, cudaStream_t st) {
     RhsBatch p;
     p.n = n;
     int at = 0;
@@ -2461,21 +2625,26 @@ template <typename D> static cudaError_t rhs_batch(const StepInst *in, int n, cu
         p.first[i] = at;
         p.inst[i].g = g;
         p.inst[i].fc = in[i].mesh->d_fem32;
+        p.inst[i].vc = in[i].vc;
         p.inst[i].bf = in[i].bf;
-        at += ((g.nxf + D::TXC - 1) / D::TXC) * ((g.nyf + D::TYC - 1) / D::TYC);
+        if constexpr (NS > 0) at += rhs_march_ctas<NS>(g);
+        else at += ((g.nxf + D::TXC - 1) / D::TXC) * ((g.nyf + D::TYC - 1) / D::TYC);
     }
     p.first[n] = at;
     const size_t sm = RhsLayout<D>::template bytes<float>();
-    cudaError_t e = set_smem(k_rhs_batch<D>, sm);
+    auto k = k_rhs_batch_small;
+    if constexpr (NS > 0) k = k_rhs_batch_march<NS>;
+    cudaError_t e = set_smem(k, sm);
     if (e != cudaSuccess) return e;
-    k_rhs_batch<D><<<at, D::THREADS, sm, st>>>(p);
+    k<<<at, D::THREADS, sm, st>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rhs_batch(const StepInst *in, int n, cudaStream_t st) {
     long long tiles = 0;
     for (int i = 0; i < n; ++i) tiles += tiles_of(in[i].mesh->g);
-    return use_small(in[0].mesh->g, tiles) ? rhs_batch<SmallTile>(in, n, st) : rhs_batch<BigTile>(in, n, st);
+    if (use_small(in[0].mesh->g, tiles)) return rhs_batch<SmallTile, 0>(in, n, st);
+    return march_tall(tiles) ? rhs_batch<BigTile, 16>(in, n, st) : rhs_batch<BigTile, 4>(in, n, st);
 }
 
 template <int R> static cudaError_t restrict_batch(const StepInst *in, int n, cudaStream_t st) {
