@@ -697,7 +697,7 @@ int dnnmg_rhs_restrict(dnnmg_mesh_t mesh, const void *vcorr, void *bf, double *b
     if (vcorr == bf) return fail(DNNMG_EINVAL, "vcorr and bf must not alias");
     if (!aligned16(vcorr) || !aligned16(bf)) return fail(DNNMG_EINVAL, "fine fields must be 16-byte aligned");
     DNNMG_CUDA_TRY(launch_rhs(mesh->g, mesh->info.precision, mesh->fem64, mesh->fem32, vcorr, bf, stream));
-    DNNMG_CUDA_TRY(launch_restrict(mesh->g, mesh->info.precision, bf, bc, stream));
+    DNNMG_CUDA_TRY(launch_restrict(mesh->g, mesh->info.precision, bf, bc, stream, true));
     return DNNMG_OK;
 }
 
@@ -785,6 +785,9 @@ static int step_body(dnnmg_mesh_t mesh, dnnmg_net_t net, const double *xc, void 
     const int prec = mesh->info.precision;
     const MeshGeom &g = mesh->g;
     int nev = 0;
+    // (on large meshes the next kernel's CTAs, waiting beside the last ones of this
+    // one, cost more than its launch: 623 -> 631 us at 32 768 tiles)
+    const bool chain = !ev && (long long)g.ntx * g.nty < 4096;
     auto mark = [&]() -> cudaError_t { return ev ? cudaEventRecord(ev[nev++], s) : cudaSuccess; };
     DNNMG_CUDA_TRY(mark());
     // S1 is fused into S2+S3 and into S5: both interpolate x~ from xc inside
@@ -820,11 +823,11 @@ static int step_body(dnnmg_mesh_t mesh, dnnmg_net_t net, const double *xc, void 
         DNNMG_CUDA_TRY(launch_gru(*net, w.X, h, w.d, mesh->info.P, s));
         DNNMG_CUDA_TRY(mark());
     }
-    DNNMG_CUDA_TRY(launch_scatter_avg(g, prec, w.d, nullptr, xc, t, w.vc, s, w.xcp));
+    DNNMG_CUDA_TRY(launch_scatter_avg(g, prec, w.d, nullptr, xc, t, w.vc, s, w.xcp, chain && mesh->info.P > 0));
     DNNMG_CUDA_TRY(mark());
-    DNNMG_CUDA_TRY(launch_rhs(g, prec, mesh->fem64, mesh->fem32, w.vc, bf, s));
+    DNNMG_CUDA_TRY(launch_rhs(g, prec, mesh->fem64, mesh->fem32, w.vc, bf, s, chain));
     DNNMG_CUDA_TRY(mark());
-    DNNMG_CUDA_TRY(launch_restrict(g, prec, bf, bc, s));
+    DNNMG_CUDA_TRY(launch_restrict(g, prec, bf, bc, s, chain));
     DNNMG_CUDA_TRY(mark());
     return DNNMG_OK;
 }

@@ -145,6 +145,33 @@ struct StepInst {
 constexpr int kBatch = 32;   // instances of one launch (their parameters stay below 32 KB)
 
 int round_up(int v, int m);
+
+#ifdef __CUDACC__
+// Kernels of the step that follow one another on a stream are launched so that
+// each may be put on the SMs while the one before it drains (programmatic
+// launch): 1 to 2 us less per kernel on small meshes.  pdl_enter() is the first
+// thing every thread does: it lets the next kernel in and waits until the one
+// before has completed and its writes are visible.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");
+}
+// chained: the kernel before on the stream is one of this library's, nothing in between
+template <typename... P, typename... A>
+cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A &&...a) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);
+}
+#endif
 // Tiled TMA descriptor (no swizzle, zero fill out of bounds); strides in
 // bytes for dimensions 1 .. rank-1.  False if the driver entry point is
 // missing or the layout is not expressible.
@@ -164,9 +191,9 @@ cudaError_t launch_residual_features(const MeshGeom &g, int prec, const FemCoef<
 // xcp (may be null): the step's padded copy of x_c in the fine type, read
 // instead of xc for the coarse window (the same values)
 cudaError_t launch_scatter_avg(const MeshGeom &g, int prec, const void *d, const void *xf, const double *xc,
-                               double t, void *vcorr, cudaStream_t st, const void *xcp = nullptr);
+                               double t, void *vcorr, cudaStream_t st, const void *xcp = nullptr, bool chained = false);
 cudaError_t launch_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f64,
-                       const FemCoef<float> &f32, const void *vcorr, void *bf, cudaStream_t st);
+                       const FemCoef<float> &f32, const void *vcorr, void *bf, cudaStream_t st, bool chained = false);
 // The coarse vector in the fine arithmetic type, rows padded to pc (a
 // multiple of 32) so that tiles can fetch coarse windows by TMA: xcp
 // [3][nyc+1][pc], zero past nxc.
@@ -194,14 +221,15 @@ cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float>
 cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, int *hrow, cudaStream_t st);
 cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st);
 cudaError_t launch_residual_cf_batch(const StepInst *in, int n, cudaStream_t st);
-cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st);
+// (chained: right after the network; the two passes after it always are)
+cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st, bool chained);
 cudaError_t launch_rhs_batch(const StepInst *in, int n, cudaStream_t st);
 cudaError_t launch_restrict_batch(const StepInst *in, int n, cudaStream_t st);
 // S5 + S6 fused: b_f = Rhs(P x_c + mean of d) without writing v_corr.
 cudaError_t launch_avg_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f64, const FemCoef<float> &f32,
                            const void *d, const double *xc, double t, void *bf, cudaStream_t st);
 cudaError_t launch_restrict(const MeshGeom &g, int prec, const void *bf, double *bc,
-                            cudaStream_t st);
+                            cudaStream_t st, bool chained = false);
 cudaError_t launch_mesh_maps(const MeshGeom &g, unsigned char *flags, unsigned char *mult,
                              cudaStream_t st);
 cudaError_t launch_gru(const Net &net, const void *X, void *h, void *d, int P, cudaStream_t st);

@@ -222,6 +222,7 @@ template <typename T, int TP, int JT, int PT, int THREADS, bool SW>
 __global__ void __launch_bounds__(THREADS)
 k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, const T *WxT, const T *UhT, const T *WfcT, T *__restrict__ h, T *__restrict__ d, int P) {
     static_assert(TP % PT == 0, "whole tiles");
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int LP = TP + (TP > 4 ? 16 / (int)sizeof(T) : 0);   // staged row length (padded against bank conflicts)
     T *xs = reinterpret_cast<T *>(smem_raw);   // [n_in][LP] features

@@ -400,7 +400,7 @@ int dnnmg_server_step(dnnmg_server_t s, int n, const int *slots, const double *c
             used += vc_need(in[i + m].mesh->info);
             ++m;
         }
-        DNNMG_CUDA_TRY(launch_scatter_avg_batch(&in[i], m, stream));
+        DNNMG_CUDA_TRY(launch_scatter_avg_batch(&in[i], m, stream, total > 0 || i > 0));
         DNNMG_CUDA_TRY(launch_rhs_batch(&in[i], m, stream));
         DNNMG_CUDA_TRY(launch_restrict_batch(&in[i], m, stream));
         i += m;

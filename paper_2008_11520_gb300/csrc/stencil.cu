@@ -1060,6 +1060,7 @@ __device__ __forceinline__ void coarse_pad_cta(const MeshGeom &g, const double *
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int pc) {
+    pdl_enter();
     coarse_pad_cta(g, xc, xcp, pc, blockIdx.x, gridDim.x);
 }
 
@@ -1074,6 +1075,7 @@ struct PadBatch {
     } inst[kBatch];
 };
 __global__ void __launch_bounds__(NTHREADS) k_coarse_pad_batch(const __grid_constant__ PadBatch p) {
+    pdl_enter();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     if (local == 0)
@@ -1169,6 +1171,7 @@ __global__ void __launch_bounds__(D::THREADS)
 k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmC, double inflow_peak, TX *__restrict__ X,
                 const int *__restrict__ tile_list) {
+    pdl_enter();
     // tile_list (when the closed-form kernel does the all-fluid tiles): the
     // other tiles, one per CTA; otherwise the grid covers every tile
     int tx = blockIdx.x, ty = blockIdx.y;
@@ -1197,6 +1200,7 @@ struct ResBatch {
 template <typename D, int R>
 __global__ void __launch_bounds__(D::THREADS, 1024 / D::THREADS) k_residual_step_batch(const __grid_constant__ ResBatch p) {
     __shared__ FemCoef<float> fc;
+    pdl_enter();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);
@@ -1446,6 +1450,7 @@ k_scatter_avg(MeshGeom g, const T *__restrict__ d, const T *__restrict__ xf, con
     // the first and the two last tile rows (walls: general tiles, the slowest)
     // are scheduled first, so that they do not form the grid's tail
     const int ny = gridDim.y, by = blockIdx.y < 3 ? (blockIdx.y ? ny - blockIdx.y : 0) : blockIdx.y - 2;
+    pdl_enter();
     scatter_cta<T, R, PTY>(g, d, xf, xc, xcp, pc, inflow_peak, vc, blockIdx.x, by);
 }
 
@@ -1461,6 +1466,7 @@ struct AvgBatch {
 };
 template <int R, int PTY>
 __global__ void __launch_bounds__(NTHREADS, 6) k_scatter_avg_batch(const __grid_constant__ AvgBatch p) {
+    pdl_enter();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     const auto &q = p.inst[i];
@@ -1681,6 +1687,7 @@ __device__ __forceinline__ void rhs_cta(const MeshGeom &g, const FemCoef<T> &fc,
 template <typename D, typename T>
 __global__ void __launch_bounds__(D::THREADS)
 k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__restrict__ bf) {
+    pdl_enter();
     rhs_cta<D>(g, fc, &tmV, bf, blockIdx.x, blockIdx.y);
 }
 
@@ -1820,6 +1827,7 @@ template <int NS>
 __global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS)
 k_rhs_march(MeshGeom g, FemCoef<float> fc, const __grid_constant__ CUtensorMap tmV, const float *__restrict__ vc,
             float *__restrict__ bf) {
+    pdl_enter();
     rhs_big<NS>(g, fc, &tmV, vc, bf, blockIdx.x);
 }
 
@@ -1836,6 +1844,7 @@ struct RhsBatch {
 __global__ void __launch_bounds__(SmallTile::THREADS) k_rhs_batch_small(const __grid_constant__ RhsBatch p) {
     using D = SmallTile;
     __shared__ FemCoef<float> fc;
+    pdl_enter();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);   // (visible after rhs_cta's first barrier)
@@ -1845,6 +1854,7 @@ __global__ void __launch_bounds__(SmallTile::THREADS) k_rhs_batch_small(const __
 template <int NS>
 __global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS) k_rhs_batch_march(const __grid_constant__ RhsBatch p) {
     __shared__ FemCoef<float> fc;
+    pdl_enter();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);
@@ -2092,6 +2102,7 @@ __device__ __forceinline__ void restrict_cta(const MeshGeom &g, const CUtensorMa
 template <typename T, typename Acc, int R>
 __global__ void __launch_bounds__(NTHREADS)
 k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restrict__ bc) {
+    pdl_enter();
     restrict_cta<T, Acc, R>(g, &tmB, bc, blockIdx.x, blockIdx.y);
 }
 
@@ -2105,6 +2116,7 @@ struct RestrictBatch {
 };
 template <int R>
 __global__ void __launch_bounds__(NTHREADS) k_restrict_batch(const __grid_constant__ RestrictBatch p) {
+    pdl_enter();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     const int ntx = (p.inst[i].g.nxc + 128 / R) / (128 / R);
@@ -2129,7 +2141,7 @@ template <typename T, int R> bool restrict_map(const MeshGeom &g, const T *bf, C
 }
 
 template <typename T, typename Acc, int R>
-cudaError_t run_restrict(const MeshGeom &g, const T *bf, double *bc, cudaStream_t st) {
+cudaError_t run_restrict(const MeshGeom &g, const T *bf, double *bc, cudaStream_t st, bool chained) {
     constexpr int TCX = 128 / R, TCY = 32 / R;
     CUtensorMap tm;
     if (!restrict_map<T, R>(g, bf, &tm)) return cudaErrorInvalidValue;
@@ -2137,16 +2149,15 @@ cudaError_t run_restrict(const MeshGeom &g, const T *bf, double *bc, cudaStream_
     const size_t sm = restrict_smem<T, Acc, R>();
     cudaError_t e = cudaFuncSetAttribute(k_restrict<T, Acc, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_restrict<T, Acc, R><<<grid, NTHREADS, sm, st>>>(g, tm, bc);
-    return cudaGetLastError();
+    return launch_chained(chained, k_restrict<T, Acc, R>, grid, NTHREADS, sm, st, g, tm, bc);
 }
 
 template <typename T, typename Acc>
-cudaError_t run_restrict_r(const MeshGeom &g, const T *bf, double *bc, cudaStream_t st) {
+cudaError_t run_restrict_r(const MeshGeom &g, const T *bf, double *bc, cudaStream_t st, bool chained) {
     switch (g.r) {
-        case 2: return run_restrict<T, Acc, 2>(g, bf, bc, st);
-        case 4: return run_restrict<T, Acc, 4>(g, bf, bc, st);
-        case 8: return run_restrict<T, Acc, 8>(g, bf, bc, st);
+        case 2: return run_restrict<T, Acc, 2>(g, bf, bc, st, chained);
+        case 4: return run_restrict<T, Acc, 4>(g, bf, bc, st, chained);
+        case 8: return run_restrict<T, Acc, 8>(g, bf, bc, st, chained);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -2401,35 +2412,32 @@ cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<doub
 
 template <typename T, int PTY_>
 cudaError_t run_scatter_p(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
-                          cudaStream_t st) {
+                          cudaStream_t st, bool chained) {
     const dim3 grid((unsigned)((g.nxf + PTX) / PTX), (unsigned)((g.nyf + PTY_) / PTY_));
     const int pc = coarse_pitch(g);
-    if (!xc && !xcp) {
-        k_scatter_avg<T, 0, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc);
-        return cudaGetLastError();
-    }
-    switch (g.r) {
-        case 2: k_scatter_avg<T, 2, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
-        case 4: k_scatter_avg<T, 4, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
-        case 8: k_scatter_avg<T, 8, PTY_><<<grid, NTHREADS, 0, st>>>(g, d, xf, xc, xcp, pc, w, vc); break;
+    auto k = k_scatter_avg<T, 0, PTY_>;
+    if (xc || xcp) switch (g.r) {
+        case 2: k = k_scatter_avg<T, 2, PTY_>; break;
+        case 4: k = k_scatter_avg<T, 4, PTY_>; break;
+        case 8: k = k_scatter_avg<T, 8, PTY_>; break;
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+    return launch_chained(chained, k, grid, NTHREADS, 0, st, g, d, xf, xc, xcp, pc, w, vc);
 }
 
 template <typename T>
 cudaError_t run_scatter(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
-                        cudaStream_t st) {
-    if (use_small(g, tiles_of(g))) return run_scatter_p<T, 4>(g, d, xf, xc, xcp, w, vc, st);
-    return run_scatter_p<T, PTY>(g, d, xf, xc, xcp, w, vc, st);
+                        cudaStream_t st, bool chained) {
+    if (use_small(g, tiles_of(g))) return run_scatter_p<T, 4>(g, d, xf, xc, xcp, w, vc, st, chained);
+    return run_scatter_p<T, PTY>(g, d, xf, xc, xcp, w, vc, st, chained);
 }
 
 cudaError_t launch_scatter_avg(const MeshGeom &g, int prec, const void *d, const void *xf, const double *xc,
-                               double t, void *vcorr, cudaStream_t st, const void *xcp) {
+                               double t, void *vcorr, cudaStream_t st, const void *xcp, bool chained) {
     const double w = inflow_peak(g, t);
     if (prec == DNNMG_F64)
-        return run_scatter(g, (const double *)d, (const double *)xf, xc, (const double *)xcp, w, (double *)vcorr, st);
-    return run_scatter(g, (const float *)d, (const float *)xf, xc, (const float *)xcp, w, (float *)vcorr, st);
+        return run_scatter(g, (const double *)d, (const double *)xf, xc, (const double *)xcp, w, (double *)vcorr, st, chained);
+    return run_scatter(g, (const float *)d, (const float *)xf, xc, (const float *)xcp, w, (float *)vcorr, st, chained);
 }
 
 // v_corr [2][nyf+1][pitch]: boxes of the tile's node window
@@ -2443,42 +2451,42 @@ template <typename D, typename T> bool rhs_map(const MeshGeom &g, const T *vcorr
 }
 
 template <typename D, typename T>
-cudaError_t run_rhs_d(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st) {
+cudaError_t run_rhs_d(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st, bool chained) {
     using L = RhsLayout<D>;
     CUtensorMap tm;
     if (!rhs_map<D, T>(g, vcorr, &tm)) return cudaErrorInvalidValue;
     const size_t sm = L::template bytes<T>();
     cudaError_t e = set_smem(k_rhs<D, T>, sm);
     if (e != cudaSuccess) return e;
-    k_rhs<D, T><<<tile_grid<D>(g), D::THREADS, sm, st>>>(g, fc, tm, bf);
-    return cudaGetLastError();
+    return launch_chained(chained, k_rhs<D, T>, tile_grid<D>(g), D::THREADS, sm, st, g, fc, tm, bf);
 }
 
 // Rows a warp of rhs_march walks: 16 from 4096 tiles on (2 100 warps and
 // more), else 4, whose warps work on five cell rows for them.
 inline bool march_tall(long long tiles) { return tiles >= 4096; }
 template <int NS>
-cudaError_t run_rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const float *vcorr, float *bf, cudaStream_t st) {
+cudaError_t run_rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const float *vcorr, float *bf, cudaStream_t st,
+                          bool chained) {
     CUtensorMap tm;
     if (!rhs_map<BigTile, float>(g, vcorr, &tm)) return cudaErrorInvalidValue;
     const size_t sm = RhsLayout<BigTile>::bytes<float>();
     cudaError_t e = set_smem(k_rhs_march<NS>, sm);
     if (e != cudaSuccess) return e;
-    k_rhs_march<NS><<<rhs_march_ctas<NS>(g), MARCH_THREADS, sm, st>>>(g, fc, tm, vcorr, bf);
-    return cudaGetLastError();
+    return launch_chained(chained, k_rhs_march<NS>, dim3(rhs_march_ctas<NS>(g)), MARCH_THREADS, sm, st, g, fc, tm, vcorr, bf);
 }
 
 template <typename T>
-cudaError_t run_rhs(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st) {
-    if (use_small(g, tiles_of(g))) return run_rhs_d<SmallTile, T>(g, fc, vcorr, bf, st);
-    if constexpr (sizeof(T) == 8) return run_rhs_d<BigTile, T>(g, fc, vcorr, bf, st);
-    else return march_tall(tiles_of(g)) ? run_rhs_march<16>(g, fc, vcorr, bf, st) : run_rhs_march<4>(g, fc, vcorr, bf, st);
+cudaError_t run_rhs(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st, bool chained) {
+    if (use_small(g, tiles_of(g))) return run_rhs_d<SmallTile, T>(g, fc, vcorr, bf, st, chained);
+    if constexpr (sizeof(T) == 8) return run_rhs_d<BigTile, T>(g, fc, vcorr, bf, st, chained);
+    else return march_tall(tiles_of(g)) ? run_rhs_march<16>(g, fc, vcorr, bf, st, chained)
+                                       : run_rhs_march<4>(g, fc, vcorr, bf, st, chained);
 }
 
 cudaError_t launch_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f64,
-                       const FemCoef<float> &f32, const void *vcorr, void *bf, cudaStream_t st) {
-    if (prec == DNNMG_F64) return run_rhs(g, f64, (const double *)vcorr, (double *)bf, st);
-    return run_rhs(g, f32, (const float *)vcorr, (float *)bf, st);
+                       const FemCoef<float> &f32, const void *vcorr, void *bf, cudaStream_t st, bool chained) {
+    if (prec == DNNMG_F64) return run_rhs(g, f64, (const double *)vcorr, (double *)bf, st, chained);
+    return run_rhs(g, f32, (const float *)vcorr, (float *)bf, st, chained);
 }
 
 template <typename T, int R>
@@ -2512,9 +2520,9 @@ cudaError_t launch_avg_rhs(const MeshGeom &g, int prec, const FemCoef<double> &f
 }
 
 cudaError_t launch_restrict(const MeshGeom &g, int prec, const void *bf, double *bc,
-                            cudaStream_t st) {
-    if (prec == DNNMG_F64) return run_restrict_r<double, RestrictAcc64>(g, (const double *)bf, bc, st);
-    return run_restrict_r<float, RestrictAcc32>(g, (const float *)bf, bc, st);
+                            cudaStream_t st, bool chained) {
+    if (prec == DNNMG_F64) return run_restrict_r<double, RestrictAcc64>(g, (const double *)bf, bc, st, chained);
+    return run_restrict_r<float, RestrictAcc32>(g, (const float *)bf, bc, st, chained);
 }
 
 // ---------------------------------------------------------------- batched passes
@@ -2583,7 +2591,7 @@ cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast
     }
 }
 
-template <int R, int PTY_> static cudaError_t scatter_batch(const StepInst *in, int n, cudaStream_t st) {
+template <int R, int PTY_> static cudaError_t scatter_batch(const StepInst *in, int n, cudaStream_t st, bool chained) {
     AvgBatch p;
     p.n = n;
     int at = 0;
@@ -2599,18 +2607,17 @@ template <int R, int PTY_> static cudaError_t scatter_batch(const StepInst *in, 
         at += ((g.nxf + PTX) / PTX) * ((g.nyf + PTY_) / PTY_);
     }
     p.first[n] = at;
-    k_scatter_avg_batch<R, PTY_><<<at, NTHREADS, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(chained, k_scatter_avg_batch<R, PTY_>, dim3(at), NTHREADS, 0, st, p);
 }
 
-cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st) {
+cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st, bool chained) {
     long long tiles = 0;
     for (int i = 0; i < n; ++i) tiles += tiles_of(in[i].mesh->g);
     const bool small = use_small(in[0].mesh->g, tiles);
     switch (in[0].mesh->g.r) {
-        case 2: return small ? scatter_batch<2, 4>(in, n, st) : scatter_batch<2, PTY>(in, n, st);
-        case 4: return small ? scatter_batch<4, 4>(in, n, st) : scatter_batch<4, PTY>(in, n, st);
-        case 8: return small ? scatter_batch<8, 4>(in, n, st) : scatter_batch<8, PTY>(in, n, st);
+        case 2: return small ? scatter_batch<2, 4>(in, n, st, chained) : scatter_batch<2, PTY>(in, n, st, chained);
+        case 4: return small ? scatter_batch<4, 4>(in, n, st, chained) : scatter_batch<4, PTY>(in, n, st, chained);
+        case 8: return small ? scatter_batch<8, 4>(in, n, st, chained) : scatter_batch<8, PTY>(in, n, st, chained);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -2636,8 +2643,7 @@ template <typename D, int NS> static cudaError_t rhs_batch(const StepInst *in, i
     if constexpr (NS > 0) k = k_rhs_batch_march<NS>;
     cudaError_t e = set_smem(k, sm);
     if (e != cudaSuccess) return e;
-    k<<<at, D::THREADS, sm, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(true, k, dim3(at), D::THREADS, sm, st, p);
 }
 
 cudaError_t launch_rhs_batch(const StepInst *in, int n, cudaStream_t st) {
@@ -2664,8 +2670,7 @@ template <int R> static cudaError_t restrict_batch(const StepInst *in, int n, cu
     const size_t sm = restrict_smem<float, RestrictAcc32, R>();
     cudaError_t e = set_smem(k_restrict_batch<R>, sm);
     if (e != cudaSuccess) return e;
-    k_restrict_batch<R><<<at, NTHREADS, sm, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(true, k_restrict_batch<R>, dim3(at), NTHREADS, sm, st, p);
 }
 
 cudaError_t launch_restrict_batch(const StepInst *in, int n, cudaStream_t st) {
