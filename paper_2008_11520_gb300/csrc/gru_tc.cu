@@ -2,7 +2,7 @@
 // Eq. gru (reset gate before U_h, no biases) and the output layer, BF16
 // operands, FP32 accumulators in tensor memory.
 //
-// One persistent CTA per SM walks 128-patch tiles (one TMEM lane per patch
+// One persistent CTA per SM (two for H <= 64) walks 128-patch tiles (one TMEM lane per patch
 // row).  Per tile, with the z, r and candidate pre-activations accumulating
 // in TMEM columns [0,H), [H,2H), [2H,3H):
 //   X groups:  for each 64-column chunk of X:

@@ -9,9 +9,9 @@
 // the window's inputs, outputs and saved activations touch memory.  A kernel
 // per product (with FP32 intermediates and BF16 copies of every operand in
 // memory between them) took 4.07 ms for loss and gradients of 65 536 rows, T =
-// 10, H = 64; this takes 0.65 ms, of it forward 266 us, backward 256 us and
+// 10, H = 64; this takes 0.62 ms, of it forward 266 us, backward 256 us and
 // the sum of the partial gradients 15 us (ncu).  With 99 features (two chunks)
-// and 50 outputs 4.65 ms became 1.05 ms, forward 386 us, backward 399 us.
+// and 50 outputs 4.65 ms became 0.96 ms, forward 383 us, backward 399 us.
 //
 // Arithmetic is that of the kernel-per-product path (gru_train.cu): operands
 // are rounded to BF16 where it rounds them, X W_x^T and h U^T are accumulated

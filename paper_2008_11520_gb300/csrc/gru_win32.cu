@@ -15,10 +15,10 @@
 // Six tcgen05 products of BF16 are 316 TFLOP/s of FP32 at the measured BF16
 // rate; the CUDA cores' FMAs give 74.  With the fused window (see gru_win.cu,
 // whose layouts these kernels share) loss and gradients of 65 536 rows, T =
-// 10, H = 64 take 1.23 ms instead of 5.5 ms with one FP32 kernel per
+// 10, H = 64 take 1.2 ms instead of 5.5 ms with one FP32 kernel per
 // product, and of 762 rows, H = 32, 0.46 ms instead of 2.7 ms; with 99
-// features and 50 outputs 1.9 ms instead of 6.5 ms (X W_x^T 217 us, forward
-// 385, state gradients 423, weight gradients 368 and 230).
+// features and 50 outputs 1.8 ms instead of 6.5 ms (X W_x^T 214 us, forward
+// 383, state gradients 422, weight gradients 363 and 229).
 //
 // Values beyond the largest BF16 number are clamped to it (an infinite
 // feature saturates the gates as it does in FP32); a NaN stays one.
