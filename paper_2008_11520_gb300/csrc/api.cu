@@ -33,7 +33,7 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 cudaError_t launch_gru_cuda_core(const Net &n, const void *X, void *h, void *d, int P,
-                                 cudaStream_t st);
+                                 cudaStream_t st, bool chained);
 
 namespace {
 
@@ -816,11 +816,11 @@ static int step_body(dnnmg_mesh_t mesh, dnnmg_net_t net, const double *xc, void 
             DNNMG_CUDA_TRY(launch_residual_cf(g, prec, mesh->fem32, w.xcp, bf, w.X, s));
             DNNMG_CUDA_TRY(mark());
         }
-        DNNMG_CUDA_TRY(launch_residual_step(g, prec, mesh->fem64, mesh->fem32, w.xcp, t, bf, w.X, s, cf));
+        DNNMG_CUDA_TRY(launch_residual_step(g, prec, mesh->fem64, mesh->fem32, w.xcp, t, bf, w.X, s, cf, chain && !cf));
         DNNMG_CUDA_TRY(mark());
     }
     if (mesh->info.P) {
-        DNNMG_CUDA_TRY(launch_gru(*net, w.X, h, w.d, mesh->info.P, s));
+        DNNMG_CUDA_TRY(launch_gru(*net, w.X, h, w.d, mesh->info.P, s, chain && !cf));
         DNNMG_CUDA_TRY(mark());
     }
     DNNMG_CUDA_TRY(launch_scatter_avg(g, prec, w.d, nullptr, xc, t, w.vc, s, w.xcp, chain && mesh->info.P > 0));
@@ -915,9 +915,9 @@ int dnnmg_step_launches(dnnmg_mesh_t mesh, dnnmg_net_t net) {
 }  // extern "C"
 
 namespace dnnmg {
-cudaError_t launch_gru(const Net &net, const void *X, void *h, void *d, int P, cudaStream_t st) {
+cudaError_t launch_gru(const Net &net, const void *X, void *h, void *d, int P, cudaStream_t st, bool chained) {
     if (net.tc) return launch_gru_tc(net, X, h, d, P, st);
-    return launch_gru_cuda_core(net, X, h, d, P, st);
+    return launch_gru_cuda_core(net, X, h, d, P, st, chained);
 }
 int gru_launch_count(const Net &) { return 1; }
 }  // namespace dnnmg

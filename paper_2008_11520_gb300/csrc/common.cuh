@@ -153,8 +153,10 @@ int round_up(int v, int m);
 // thing every thread does: it lets the next kernel in and waits until the one
 // before has completed and its writes are visible.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");
+    pdl_trigger();
+    pdl_wait();
 }
 // chained: the kernel before on the stream is one of this library's, nothing in between
 template <typename... P, typename... A>
@@ -204,7 +206,7 @@ cudaError_t launch_coarse_pad(const MeshGeom &g, int prec, const double *xc, voi
 // launch_residual_features with xc; rf is not written).
 cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<double> &f64, const FemCoef<float> &f32,
                                  const void *xcp, double t, const void *bf, void *X, cudaStream_t st,
-                                 bool skip_fast = false);
+                                 bool skip_fast = false, bool chained = false);
 // S2 + S3 of the step on the all-fluid tiles in closed form (residual_cf.cu):
 // FP32 fields, K = 1 or 2.  launch_residual_step(..., skip_fast = true) then
 // does the other tiles.
@@ -232,9 +234,9 @@ cudaError_t launch_restrict(const MeshGeom &g, int prec, const void *bf, double 
                             cudaStream_t st, bool chained = false);
 cudaError_t launch_mesh_maps(const MeshGeom &g, unsigned char *flags, unsigned char *mult,
                              cudaStream_t st);
-cudaError_t launch_gru(const Net &net, const void *X, void *h, void *d, int P, cudaStream_t st);
+cudaError_t launch_gru(const Net &net, const void *X, void *h, void *d, int P, cudaStream_t st, bool chained = false);
 int gru_launch_count(const Net &net);
-cudaError_t launch_gru_cuda_core(const Net &n, const void *X, void *h, void *d, int P, cudaStream_t st);
+cudaError_t launch_gru_cuda_core(const Net &n, const void *X, void *h, void *d, int P, cudaStream_t st, bool chained);
 cudaError_t launch_gru_tc(const Net &n, const void *X, void *h, void *d, int P, cudaStream_t st);
 cudaError_t launch_gru_tc_rows(const Net &n, const void *X, void *h, void *d, int P, const int *hrow, int h_rows,
                                cudaStream_t st);

@@ -249,6 +249,7 @@ k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, 
             ws += cnt[m];
         }
     }
+    pdl_wait();   // (the weights do not change: staged above while the kernel before drains)
     for (long long q0 = (long long)blockIdx.x * TP; q0 < P; q0 += (long long)gridDim.x * TP) {
         const int p0 = (int)q0, np = min(TP, P - p0);
         for (int i = threadIdx.x; i < TP * n_in; i += THREADS) {
@@ -333,7 +334,7 @@ size_t rt_bytes(const Net &n, int LP, size_t elem) {
 }
 
 template <typename T, int TP, int JT, int PT, int THREADS, bool SW>
-cudaError_t run_rt(const Net &n, const void *X, void *h, void *d, int P, cudaStream_t st) {
+cudaError_t run_rt(const Net &n, const void *X, void *h, void *d, int P, cudaStream_t st, bool chained) {
     constexpr int LP = TP + (TP > 4 ? 16 / (int)sizeof(T) : 0);
     const size_t sm = sizeof(T) * ((size_t)LP * (n.n_in + 4 * n.H) + (SW ? weight_count(n) : 0));
     auto k = k_gru_rt<T, TP, JT, PT, THREADS, SW>;
@@ -345,9 +346,8 @@ cudaError_t run_rt(const Net &n, const void *X, void *h, void *d, int P, cudaStr
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, THREADS, sm)) != cudaSuccess) return e;
         grid = std::min(grid, std::max(1, per) * sm_count());
     }
-    k<<<grid, THREADS, sm, st>>>(n.n_in, n.ldx, n.H, n.n_out, n.ldo, (const T *)X, (const T *)n.WxT,
-                                              (const T *)n.UhT, (const T *)n.WfcTp, (T *)h, (T *)d, P);
-    return cudaGetLastError();
+    return launch_chained(chained, k, dim3(grid), THREADS, sm, st, n.n_in, n.ldx, n.H, n.n_out, n.ldo, (const T *)X,
+                          (const T *)n.WxT, (const T *)n.UhT, (const T *)n.WfcTp, (T *)h, (T *)d, P);
 }
 
 template <typename T, typename TW, int TP>
@@ -366,7 +366,7 @@ cudaError_t run(const Net &n, const void *X, void *h, void *d, int P, cudaStream
 }  // namespace
 
 cudaError_t launch_gru_cuda_core(const Net &n, const void *X, void *h, void *d, int P,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, bool chained) {
     if (P == 0) return cudaSuccess;
     // the register-tiled kernel, its weights in shared memory where they fit; else
     // one column a thread
@@ -377,12 +377,12 @@ cudaError_t launch_gru_cuda_core(const Net &n, const void *X, void *h, void *d, 
             // (99 -> 64 -> 50: 4000 patches 25 against 35 us); more tiles: several CTAs an SM
             // read them from L2 (16 336 patches 58 against 78 us)
             if ((P + 31) / 32 <= sm_count() && rt_bytes(n, 36, 4) <= lim)
-                return run_rt<float, 32, 4, 4, 384, true>(n, X, h, d, P, st);
-            return run_rt<float, 32, 4, 8, 192, false>(n, X, h, d, P, st);
+                return run_rt<float, 32, 4, 4, 384, true>(n, X, h, d, P, st, chained);
+            return run_rt<float, 32, 4, 8, 192, false>(n, X, h, d, P, st, chained);
         }
         if (n.precision == DNNMG_F64) {
-            if (rt_bytes(n, 2, 8) <= lim) return run_rt<double, 2, 2, 1, 128, true>(n, X, h, d, P, st);
-            return run_rt<double, 2, 2, 1, 128, false>(n, X, h, d, P, st);
+            if (rt_bytes(n, 2, 8) <= lim) return run_rt<double, 2, 2, 1, 128, true>(n, X, h, d, P, st, chained);
+            return run_rt<double, 2, 2, 1, 128, false>(n, X, h, d, P, st, chained);
         }
     }
     if (n.precision == DNNMG_F64) return run<double, double, 8>(n, X, h, d, P, st);

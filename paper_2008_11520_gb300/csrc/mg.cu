@@ -262,7 +262,6 @@ __global__ void __launch_bounds__(MR_THREADS) k_mg_rows(const __grid_constant__ 
 // so that a pass may start while the one before it drains; what depends on
 // that one comes after the wait (which ends when the pass before has
 // completed and its writes are visible).
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // One colour pass of the Vanka smoother for J(x) d = rhs: every fluid cell
 // (ci, cj) with ci = cx (mod 4), cj = cy (mod 4) solves the 12 x 12 block of

@@ -2365,7 +2365,7 @@ bool residual_maps(const MeshGeom &g, const T *bf, const T *xcp, CUtensorMap *tm
 
 template <typename D, typename T, typename TX, int R>
 cudaError_t run_residual_step(const MeshGeom &g, const FemCoef<T> &fc, const T *xcp, double up, const T *bf, TX *X,
-                              cudaStream_t st, bool skip_fast) {
+                              cudaStream_t st, bool skip_fast, bool chained) {
     using SL = StepLayout<D, T, R>;
     CUtensorMap tmB, tmC;
     if (!residual_maps<D, T, R>(g, bf, xcp, &tmB, &tmC)) return cudaErrorInvalidValue;
@@ -2378,36 +2378,37 @@ cudaError_t run_residual_step(const MeshGeom &g, const FemCoef<T> &fc, const T *
         constexpr bool big = D::TXC == TXC;
         k<<<big ? g.n_slow_tiles : g.n_slow_small, D::THREADS, sm, st>>>(g, fc, tmB, tmC, up, X,
                                                                        big ? g.slow_tiles : g.slow_small);
-    } else {
-        k<<<tile_grid<D>(g), D::THREADS, sm, st>>>(g, fc, tmB, tmC, up, X, nullptr);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
+    return launch_chained(chained, k, tile_grid<D>(g), D::THREADS, sm, st, g, fc, tmB, tmC, up, X, nullptr);
 }
 
 template <typename D, typename T, typename TX>
 cudaError_t run_residual_step_d(const MeshGeom &g, const FemCoef<T> &fc, const void *xcp, double up, const void *bf,
-                                void *X, cudaStream_t st, bool sf) {
+                                void *X, cudaStream_t st, bool sf, bool chained) {
     switch (g.r) {
-        case 2: return run_residual_step<D, T, TX, 2>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
-        case 4: return run_residual_step<D, T, TX, 4>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
-        case 8: return run_residual_step<D, T, TX, 8>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf);
+        case 2: return run_residual_step<D, T, TX, 2>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf, chained);
+        case 4: return run_residual_step<D, T, TX, 4>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf, chained);
+        case 8: return run_residual_step<D, T, TX, 8>(g, fc, (const T *)xcp, up, (const T *)bf, (TX *)X, st, sf, chained);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <typename T, typename TX>
 cudaError_t run_residual_step_r(const MeshGeom &g, const FemCoef<T> &fc, const void *xcp, double up, const void *bf,
-                                void *X, cudaStream_t st, bool sf) {
-    if (use_small(g, sf ? g.n_slow_tiles : tiles_of(g))) return run_residual_step_d<SmallTile, T, TX>(g, fc, xcp, up, bf, X, st, sf);
-    return run_residual_step_d<BigTile, T, TX>(g, fc, xcp, up, bf, X, st, sf);
+                                void *X, cudaStream_t st, bool sf, bool chained) {
+    if (use_small(g, sf ? g.n_slow_tiles : tiles_of(g)))
+        return run_residual_step_d<SmallTile, T, TX>(g, fc, xcp, up, bf, X, st, sf, chained);
+    return run_residual_step_d<BigTile, T, TX>(g, fc, xcp, up, bf, X, st, sf, chained);
 }
 
 cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<double> &f64, const FemCoef<float> &f32,
-                                 const void *xcp, double t, const void *bf, void *X, cudaStream_t st, bool skip_fast) {
+                                 const void *xcp, double t, const void *bf, void *X, cudaStream_t st, bool skip_fast,
+                                 bool chained) {
     const double up = inflow_peak(g, t);
-    if (prec == DNNMG_F64) return run_residual_step_r<double, double>(g, f64, xcp, up, bf, X, st, skip_fast);
-    if (prec == DNNMG_F32) return run_residual_step_r<float, float>(g, f32, xcp, up, bf, X, st, skip_fast);
-    return run_residual_step_r<float, __nv_bfloat16>(g, f32, xcp, up, bf, X, st, skip_fast);
+    if (prec == DNNMG_F64) return run_residual_step_r<double, double>(g, f64, xcp, up, bf, X, st, skip_fast, chained);
+    if (prec == DNNMG_F32) return run_residual_step_r<float, float>(g, f32, xcp, up, bf, X, st, skip_fast, chained);
+    return run_residual_step_r<float, __nv_bfloat16>(g, f32, xcp, up, bf, X, st, skip_fast, chained);
 }
 
 template <typename T, int PTY_>
