@@ -152,6 +152,11 @@ int round_up(int v, int m);
 // launch): 1 to 2 us less per kernel on small meshes.  pdl_enter() is the first
 // thing every thread does: it lets the next kernel in and waits until the one
 // before has completed and its writes are visible.
+// What an earlier kernel of the chain writes (X, d, v_corr, the padded x_c, the
+// correction of a sweep) is read by plain loads through pointers without __restrict__: a
+// chained kernel lives while that one still writes, and the read-only path
+// (__ldg, const __restrict__) is for data that nothing writes meanwhile, its
+// loads free to move above the wait.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {

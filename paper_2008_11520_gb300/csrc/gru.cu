@@ -220,7 +220,7 @@ __device__ __forceinline__ void RTile<double, 2, 1>::mac(const double *W, int ld
 
 template <typename T, int TP, int JT, int PT, int THREADS, bool SW>
 __global__ void __launch_bounds__(THREADS)
-k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, const T *WxT, const T *UhT, const T *WfcT, T *__restrict__ h, T *__restrict__ d, int P) {
+k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *X, const T *WxT, const T *UhT, const T *WfcT, T *__restrict__ h, T *__restrict__ d, int P) {
     static_assert(TP % PT == 0, "whole tiles");
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -254,7 +254,7 @@ k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *__restrict__ X, 
         const int p0 = (int)q0, np = min(TP, P - p0);
         for (int i = threadIdx.x; i < TP * n_in; i += THREADS) {
             const int p = i / n_in, k = i - p * n_in;
-            xs[k * LP + p] = p < np ? __ldg(X + (size_t)(p0 + p) * ldx + k) : T(0);
+            xs[k * LP + p] = p < np ? X[(size_t)(p0 + p) * ldx + k] : T(0);
         }
         for (int i = threadIdx.x; i < TP * H; i += THREADS) {
             const int p = i / H, k = i - p * H;

@@ -182,8 +182,7 @@ struct CoarseWin {
     }
     // The same window from the padded copy [NC..][nyc+1][pc] of x_c in the
     // fine type that the step keeps (the same values: both round x_c once).
-    __device__ __forceinline__ void stage_padded(const MeshGeom &g, const T *__restrict__ xcp, int pc, int Ilo,
-                                                 int Jlo) {
+    __device__ __forceinline__ void stage_padded(const MeshGeom &g, const T *xcp, int pc, int Ilo, int Jlo) {
         ci0 = Ilo >> K;
         cj0 = Jlo >> K;
         const size_t cplane = (size_t)pc * (g.nyc + 1);
@@ -192,7 +191,7 @@ struct CoarseWin {
             const int b = rem / CW, a = rem - b * CW;
             const int ci = ci0 + a, cj = cj0 + b;
             T v = T(0);
-            if (ci >= 0 && cj >= 0 && ci <= g.nxc && cj <= g.nyc) v = __ldg(xcp + c * cplane + (size_t)cj * pc + ci);
+            if (ci >= 0 && cj >= 0 && ci <= g.nxc && cj <= g.nyc) v = xcp[c * cplane + (size_t)cj * pc + ci];
             cs[e] = v;
         }
     }
@@ -1234,7 +1233,7 @@ struct PatchWin {
     // several nodes before using any: the node's own patch (first), then on
     // patch edges the left, lower and lower-left neighbours.
     template <typename T>
-    __device__ __forceinline__ void own_patch(const MeshGeom &g, const T *__restrict__ d, int I, int J, T &su, T &sv,
+    __device__ __forceinline__ void own_patch(const MeshGeom &g, const T *d, int I, int J, T &su, T &sv,
                                               int &cnt) const {
         const int S = 1 << lS;
         const int id = pid[((J >> lS) - py0) * npw + (I >> lS) - px0];
@@ -1242,13 +1241,13 @@ struct PatchWin {
         cnt = 0;
         if (id >= 0) {
             const T *q = d + (size_t)id * g.n_out + (J & (S - 1)) * (S + 1) + (I & (S - 1));
-            su = __ldg(q);
-            sv = __ldg(q + g.nf);
+            su = *q;
+            sv = q[g.nf];
             cnt = 1;
         }
     }
     template <typename T>
-    __device__ __forceinline__ void edge_patches(const MeshGeom &g, const T *__restrict__ d, int I, int J, T &su, T &sv,
+    __device__ __forceinline__ void edge_patches(const MeshGeom &g, const T *d, int I, int J, T &su, T &sv,
                                                  int &cnt) const {
         const int S = 1 << lS;
         const int row = (J >> lS) - py0, lj = J & (S - 1), col = (I >> lS) - px0, li = I & (S - 1);
@@ -1260,8 +1259,8 @@ struct PatchWin {
             const int id = pid[(row - oy) * npw + col - ox];
             if (id < 0) continue;
             const T *q = d + (size_t)id * g.n_out + (lj + oy * S) * (S + 1) + li + ox * S;
-            su += __ldg(q);
-            sv += __ldg(q + g.nf);
+            su += *q;
+            sv += q[g.nf];
             ++cnt;
         }
     }
@@ -1281,7 +1280,7 @@ struct PatchWin {
     // be issued before the tile's staging barrier.  Sums are formed in the
     // order of own_patch + edge_patches (same bits).
     template <typename T>
-    static __device__ __forceinline__ void run4(const MeshGeom &g, const T *__restrict__ d, int lS, int Ib, int J,
+    static __device__ __forceinline__ void run4(const MeshGeom &g, const T *d, int lS, int Ib, int J,
                                                 T (&su)[4], T (&sv)[4], int (&cnt)[4]) {
         const int S = 1 << lS, S1 = S + 1, nf = g.nf;
         const int pi = Ib >> lS, pj = J >> lS, li = Ib & (S - 1), lj = J & (S - 1);
@@ -1299,30 +1298,30 @@ struct PatchWin {
             const T *p = d + (size_t)id * g.n_out + lj * S1 + li;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                su[q] = __ldg(p + q);
-                sv[q] = __ldg(p + nf + q);
+                su[q] = p[q];
+                sv[q] = p[nf + q];
                 cnt[q] = 1;
             }
         }
         if (il >= 0) {   // left patch, its last column
             const T *p = d + (size_t)il * g.n_out + lj * S1 + S;
-            su[0] += __ldg(p);
-            sv[0] += __ldg(p + nf);
+            su[0] += *p;
+            sv[0] += p[nf];
             ++cnt[0];
         }
         if (ib >= 0) {   // lower patch, its last row
             const T *p = d + (size_t)ib * g.n_out + S * S1 + li;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                su[q] += __ldg(p + q);
-                sv[q] += __ldg(p + nf + q);
+                su[q] += p[q];
+                sv[q] += p[nf + q];
                 ++cnt[q];
             }
         }
         if (ibl >= 0) {   // lower-left patch, its last node
             const T *p = d + (size_t)ibl * g.n_out + S * S1 + S;
-            su[0] += __ldg(p);
-            sv[0] += __ldg(p + nf);
+            su[0] += *p;
+            sv[0] += p[nf];
             ++cnt[0];
         }
     }
@@ -1333,8 +1332,8 @@ struct PatchWin {
 // from the global patch map so that the loads of d are in flight while the
 // coarse window is staged.  Same arithmetic as the general path, same bits.
 template <int PTY, typename T, int R, typename CWin>
-__device__ __forceinline__ void scatter_fast_tile(const MeshGeom &g, const T *__restrict__ d, const T *__restrict__ xf,
-                                                  const double *__restrict__ xc, const T *__restrict__ xcp, int pc,
+__device__ __forceinline__ void scatter_fast_tile(const MeshGeom &g, const T *d, const T *__restrict__ xf,
+                                                  const double *__restrict__ xc, const T *xcp, int pc,
                                                   T *__restrict__ vc, CWin &cw, int I0, int J0) {
     static_assert(NTHREADS >= (PTX / 4) * PTY, "at most one run per thread");
     const bool mine = threadIdx.x < (PTX / 4) * PTY;
@@ -1369,8 +1368,8 @@ __device__ __forceinline__ void scatter_fast_tile(const MeshGeom &g, const T *__
 // the tile (S1 fused).  Registers are capped for the fast tiles' occupancy;
 // the rare general tiles may spill.
 template <typename T, int R, int PTY>
-__device__ __forceinline__ void scatter_cta(const MeshGeom &g, const T *__restrict__ d, const T *__restrict__ xf,
-                                            const double *__restrict__ xc, const T *__restrict__ xcp, int pc,
+__device__ __forceinline__ void scatter_cta(const MeshGeom &g, const T *d, const T *__restrict__ xf,
+                                            const double *__restrict__ xc, const T *xcp, int pc,
                                             double inflow_peak, T *__restrict__ vc, int bx, int by) {
     using CWin = CoarseWin<T, (R > 0 ? R : 2), PTX, PTY, 2>;
     __shared__ T cs_mem[R > 0 ? CWin::N : 1];
@@ -1445,8 +1444,8 @@ __device__ __forceinline__ void scatter_cta(const MeshGeom &g, const T *__restri
 
 template <typename T, int R, int PTY>
 __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 6 : 4)
-k_scatter_avg(MeshGeom g, const T *__restrict__ d, const T *__restrict__ xf, const double *__restrict__ xc,
-              const T *__restrict__ xcp, int pc, double inflow_peak, T *__restrict__ vc) {
+k_scatter_avg(MeshGeom g, const T *d, const T *__restrict__ xf, const double *__restrict__ xc,
+              const T *xcp, int pc, double inflow_peak, T *__restrict__ vc) {
     // the first and the two last tile rows (walls: general tiles, the slowest)
     // are scheduled first, so that they do not form the grid's tail
     const int ny = gridDim.y, by = blockIdx.y < 3 ? (blockIdx.y ? ny - blockIdx.y : 0) : blockIdx.y - 2;
@@ -1704,7 +1703,7 @@ k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__r
 // warps an SM that its registers allow (80 a thread; 64 spill: 102 us, 84 with
 // two CTAs: 104 us; reading two rows ahead: 97 us).
 template <int NS>
-__device__ __forceinline__ void rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const float *__restrict__ vc,
+__device__ __forceinline__ void rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const float *vc,
                                           float *__restrict__ bf, int wx, int strip) {
     constexpr unsigned ALL = 0xffffffffu;
     const int lane = threadIdx.x & 31, E = 62 * wx + 2 * lane, J0 = strip * NS, ty = J0 / TYC, bx = E >> 6;
@@ -1722,12 +1721,12 @@ __device__ __forceinline__ void rhs_march(const MeshGeom &g, const FemCoef<float
         r.u = r.v = make_float2(0.f, 0.f);
         r.lu = r.lv = 0.f;
         if (in) {
-            r.u = __ldg(reinterpret_cast<const float2 *>(p));
-            r.v = __ldg(reinterpret_cast<const float2 *>(p + g.plane));
+            r.u = *reinterpret_cast<const float2 *>(p);
+            r.v = *reinterpret_cast<const float2 *>(p + g.plane);
         }
         if (edge) {
-            r.lu = __ldg(p - 1);
-            r.lv = __ldg(p + g.plane - 1);
+            r.lu = p[-1];
+            r.lv = p[(ptrdiff_t)g.plane - 1];
         }
         return r;
     };
@@ -1814,7 +1813,7 @@ template <int NS> int rhs_march_ctas(const MeshGeom &g) {
 }
 template <int NS>
 __device__ __forceinline__ void rhs_big(const MeshGeom &g, const FemCoef<float> &fc, const CUtensorMap *tmV,
-                                        const float *__restrict__ vc, float *__restrict__ bf, int local) {
+                                        const float *vc, float *__restrict__ bf, int local) {
     if (local < g.n_slow_tiles) {
         const int tile = __ldg(g.slow_tiles + local), ty = tile / g.ntx;
         rhs_cta<BigTile>(g, fc, tmV, bf, tile - ty * g.ntx, ty);
@@ -1825,7 +1824,7 @@ __device__ __forceinline__ void rhs_big(const MeshGeom &g, const FemCoef<float> 
 }
 template <int NS>
 __global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS)
-k_rhs_march(MeshGeom g, FemCoef<float> fc, const __grid_constant__ CUtensorMap tmV, const float *__restrict__ vc,
+k_rhs_march(MeshGeom g, FemCoef<float> fc, const __grid_constant__ CUtensorMap tmV, const float *vc,
             float *__restrict__ bf) {
     pdl_enter();
     rhs_big<NS>(g, fc, &tmV, vc, bf, blockIdx.x);
