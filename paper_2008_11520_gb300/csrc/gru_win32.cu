@@ -20,8 +20,11 @@
 // features and 50 outputs 1.8 ms instead of 6.5 ms (X W_x^T 214 us, forward
 // 383, state gradients 422, weight gradients 363 and 229).
 //
-// Values beyond the largest BF16 number are clamped to it (an infinite
-// feature saturates the gates as it does in FP32); a NaN stays one.
+// An infinite operand, or a finite one beyond the BF16 range, has no such
+// parts: its remainders are NaNs, and every sum it enters is one.  So results
+// are looked at, and a tile (in the weight gradients: a CTA's blocks) with a
+// state, output or gradient that is not finite is computed again with FP32
+// FMAs (plain_*), which give FP32's infinities, NaNs and saturated gates.
 #include <algorithm>
 #include <cstring>
 
@@ -68,18 +71,14 @@ __device__ __forceinline__ void mma3_mn(uint32_t d, uint32_t a, uint32_t astep, 
 // long sums of products do not keep the bias.
 __device__ __forceinline__ float whole(float v, int ksteps) { return fmaf(v, 2.1e-8f * (float)ksteps, v); }
 
-__device__ __forceinline__ float clamp_bf16(float x) {
-    float y;
-    asm("{\n.reg .f32 t;\nmin.NaN.f32 t, %1, 0f7F7F0000;\nmax.NaN.f32 %0, t, 0fFF7F0000;\n}\n" : "=f"(y) : "f"(x));
-    return y;
-}
-// the three parts of two values, each pair packed; CL: of values that may be
-// beyond the BF16 range (the caller's arrays; states, gates and gradients are not)
-template <bool CL> __device__ __forceinline__ void split2(float x, float y, uint32_t (&o)[3]) {
-    if (CL) {
-        x = clamp_bf16(x);
-        y = clamp_bf16(y);
-    }
+// Whether every value seen is finite (0 x is not 0 for one that is not)
+struct Finite {
+    float m = 0.f;
+    __device__ __forceinline__ void see(float x) { m = fmaf(0.f, x, m); }
+    __device__ __forceinline__ bool failed() const { return m != 0.f; }
+};
+// the three parts of two values, each pair packed
+__device__ __forceinline__ void split2(float x, float y, uint32_t (&o)[3]) {
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const __nv_bfloat162 t = __floats2bfloat162_rn(x, y);
@@ -89,20 +88,20 @@ template <bool CL> __device__ __forceinline__ void split2(float x, float y, uint
     }
 }
 // 8 consecutive columns of a row into the three images, `step` bytes apart
-template <bool CL = false> __device__ __forceinline__ void put8_3(uint8_t *img, int step, int row, int c, const float *v) {
+__device__ __forceinline__ void put8_3(uint8_t *img, int step, int row, int c, const float *v) {
     uint32_t o[4][3];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) split2<CL>(v[2 * i], v[2 * i + 1], o[i]);
+    for (int i = 0; i < 4; ++i) split2(v[2 * i], v[2 * i + 1], o[i]);
     const uint32_t at = swz(row, c >> 3);
 #pragma unroll
     for (int p = 0; p < 3; ++p)
         *reinterpret_cast<uint4 *>(img + p * step + at) = make_uint4(o[0][p], o[1][p], o[2][p], o[3][p]);
 }
 // 4 consecutive columns (c a multiple of 4)
-template <bool CL = false> __device__ __forceinline__ void put4_3(uint8_t *img, int step, int row, int c, const float *v) {
+__device__ __forceinline__ void put4_3(uint8_t *img, int step, int row, int c, const float *v) {
     uint32_t a[3], b[3];
-    split2<CL>(v[0], v[1], a);
-    split2<CL>(v[2], v[3], b);
+    split2(v[0], v[1], a);
+    split2(v[2], v[3], b);
     const uint32_t at = swz(row, c >> 3) + (c & 4) * 2;
 #pragma unroll
     for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2 *>(img + p * step + at) = make_uint2(a[p], b[p]);
@@ -114,7 +113,7 @@ template <typename F> __device__ __forceinline__ void build3(uint8_t *img, int s
         float v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = src(r, c + i);
-        put8_3<true>(img, step, r, c, v);   // (8-row groups are 1024 bytes apart: row * 128 throughout)
+        put8_3(img, step, r, c, v);   // (8-row groups are 1024 bytes apart: row * 128 throughout)
     }
 }
 __device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &x, uint8_t *img, int x0 = 0) {
@@ -123,7 +122,141 @@ __device__ __forceinline__ void store_x3(const WinArgs &g, const XTile<W32_TH> &
     for (int i = 0; i < XTile<W32_TH>::NV; ++i) {
         const int e = threadIdx.x + i * W32_TH, row = e >> 4, c = (e & 15) * 4;
         const float v[4] = {x.v[i].x, c + 1 < n ? x.v[i].y : 0.f, c + 2 < n ? x.v[i].z : 0.f, c + 3 < n ? x.v[i].w : 0.f};
-        put4_3<true>(img, IMG, row, c, v);
+        put4_3(img, IMG, row, c, v);
+    }
+}
+
+// ---------------------------------------------------------------- FP32 FMAs
+// A tile (128 rows) with values that are not finite, computed again: a warp
+// takes a row; rows past the last patch are zero.  buf: 16 x 512 floats of
+// shared memory.  Called by all threads of a CTA.
+__device__ __forceinline__ size_t elem(int c, int row) { return blk(c, row) + (c & 3); }
+// y = W x, W [rows][n] (one dot product at a time, lanes along n)
+__device__ __forceinline__ void rows_times(const float *__restrict__ W, int rows, int n, const float *x, float *y) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 4
+    for (int c = 0; c < rows; ++c) {
+        float a = 0.f;
+        for (int k = lane; k < n; k += 32) a = fmaf(__ldg(W + (size_t)c * n + k), x[k], a);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) y[c] = a;
+    }
+}
+// sum over k of W[k][j] x[k], rows of W H long (lanes along j)
+__device__ __forceinline__ float column_times(const float *__restrict__ W, int H, int n, int j, const float *x) {
+    float a = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) a = fmaf(__ldg(W + (size_t)k * H + j), x[k], a);
+    return a;
+}
+
+// forward of all steps
+template <int H> __device__ __noinline__ void plain_fwd(const WinArgs &g, int tile, float *buf) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const size_t tblk = (size_t)TM * H;
+    float *x = buf + warp * 512, *h = x + 128, *rh = h + 64, *ax = rh + 64, *ah = ax + 64;
+    for (int row = warp; row < TM; row += W32_TH / 32) {
+        const int gp = tile * TM + row;
+        const bool valid = gp < g.P;
+        __syncwarp();
+        for (int j = lane; j < H; j += 32) h[j] = valid && g.h0 ? g.h0[(size_t)gp * H + j] : 0.f;
+        for (int s = 0; s < g.T; ++s) {
+            const size_t sb = ((size_t)s * g.ntiles + tile) * tblk, prow = (size_t)s * g.P + gp;
+            if (valid)
+                for (int k = lane; k < g.n_in; k += 32) x[k] = __ldg(g.X + prow * g.ldx + k);
+            for (int j = lane; j < H; j += 32) g.hb[sb + elem(j, row)] = h[j];
+            for (int gate = 1; gate >= 0; --gate) {   // r, then z
+                __syncwarp();
+                if (valid) {
+                    rows_times(g.Wx + (size_t)gate * H * g.n_in, H, g.n_in, x, ax);
+                    rows_times(g.Uh + (size_t)gate * H * H, H, H, h, ah);
+                }
+                __syncwarp();
+                for (int j = lane; j < H; j += 32) {
+                    const float v = valid ? sigm(ax[j] + ah[j]) : 0.f;
+                    (gate ? g.r : g.z)[sb + elem(j, row)] = v;
+                    if (gate) rh[j] = v * h[j];
+                }
+            }
+            __syncwarp();
+            if (valid) {
+                rows_times(g.Wx + (size_t)2 * H * g.n_in, H, g.n_in, x, ax);
+                rows_times(g.Uh + (size_t)2 * H * H, H, H, rh, ah);
+            }
+            __syncwarp();
+            for (int j = lane; j < H; j += 32) {
+                const float c = valid ? tanhf(ax[j] + ah[j]) : 0.f, z = g.z[sb + elem(j, row)];
+                g.c[sb + elem(j, row)] = c;
+                if (valid) h[j] = z * h[j] + (1.0f - z) * c;
+            }
+            __syncwarp();
+            if (valid) rows_times(g.Wfc, g.n_out, H, h, ax);
+            __syncwarp();
+            if (valid)
+                for (int o = lane; o < g.n_out; o += 32) g.D[prow * g.n_out + o] = ax[o];
+        }
+        if (valid)
+            for (int j = lane; j < H; j += 32) g.hT[(size_t)gp * H + j] = h[j];
+    }
+}
+
+// state gradients of all steps
+template <int H> __device__ __noinline__ void plain_bwd(const WinArgs &g, int tile, float *buf) {
+    constexpr int NJ = H / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const size_t tblk = (size_t)TM * H;
+    float *dd = buf + warp * 512, *az = dd + 64, *ar = az + 64, *ac = ar + 64;
+    for (int row = warp; row < TM; row += W32_TH / 32) {
+        const int gp = tile * TM + row;
+        const bool valid = gp < g.P;
+        float carry[NJ];
+#pragma unroll
+        for (int i = 0; i < NJ; ++i) carry[i] = 0.f;
+        for (int s = g.T - 1; s >= 0; --s) {
+            const size_t sb = ((size_t)s * g.ntiles + tile) * tblk, gb = 3 * sb;
+            __syncwarp();
+            if (valid)
+                for (int o = lane; o < g.n_out; o += 32) dd[o] = __ldg(g.dD + ((size_t)s * g.P + gp) * g.n_out + o);
+            __syncwarp();
+            float dh[NJ], drh[NJ];
+#pragma unroll
+            for (int i = 0; i < NJ; ++i) {
+                const int j = lane + 32 * i;
+                const size_t e = sb + elem(j, row);
+                az[j] = ac[j] = dh[i] = 0.f;
+                if (!valid) continue;
+                dh[i] = column_times(g.Wfc, H, g.n_out, j, dd) + carry[i];
+                const float z = g.z[e], c = g.c[e], dc = dh[i] * (1.0f - z), dz = dh[i] * (g.hb[e] - c);
+                az[j] = dz * z * (1.0f - z);
+                ac[j] = dc * (1.0f - c * c);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < NJ; ++i) {
+                const int j = lane + 32 * i;
+                const size_t e = sb + elem(j, row);
+                ar[j] = drh[i] = 0.f;
+                if (!valid) continue;
+                drh[i] = column_times(g.Uh + (size_t)2 * H * H, H, H, j, ac);
+                ar[j] = drh[i] * g.hb[e] * g.r[e] * (1.0f - g.r[e]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < NJ; ++i) {
+                const int j = lane + 32 * i;
+                const size_t e = sb + elem(j, row), d = gb + elem(j, row);
+                g.dG[d] = az[j];
+                g.dG[d + tblk] = ar[j];
+                g.dG[d + 2 * tblk] = ac[j];
+                if (!valid) continue;
+                carry[i] = dh[i] * g.z[e] + drh[i] * g.r[e];
+                carry[i] += column_times(g.Uh, H, H, j, az) + column_times(g.Uh + (size_t)H * H, H, H, j, ar);
+            }
+        }
+        if (valid && g.dh0)
+#pragma unroll
+            for (int i = 0; i < NJ; ++i) g.dh0[(size_t)gp * H + lane + 32 * i] = carry[i];
     }
 }
 
@@ -152,7 +285,7 @@ template <int H> struct X32Layout {
     static constexpr int COLS = H == 64 ? 512 : 256;
 };
 template <int H>
-__global__ void __launch_bounds__(W32_TH, 1) k_win32_x(const WinArgs g) {
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_x(const __grid_constant__ WinArgs g) {
     using L = X32Layout<H>;
     constexpr int NC = 3 * H / 4;   // columns of a thread
     extern __shared__ uint8_t smem_raw[];
@@ -213,7 +346,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_x(const WinArgs g) {
 }
 
 template <int H, int XC>
-__global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__ WinArgs g) {
     using L = Fwd32Layout<H, XC>;
     constexpr int NC = H / 4;   // state columns of a thread
     extern __shared__ uint8_t smem_raw[];
@@ -254,12 +387,17 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
             float *drow = g.D + ((size_t)s * g.P + gp) * g.n_out;
             for (int b = part; b < g.nfc / 8; b += 4) {
                 float v[8];
+                Finite fin;
                 tmem_ld8(tl + 6 * H + 8 * b, v);
                 tmem_wait();
                 keep(v);
                 if (!valid) continue;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = whole(v[j], H / 16);
+                for (int j = 0; j < 8; ++j) {
+                    v[j] = whole(v[j], H / 16);
+                    fin.see(v[j]);
+                }
+                if (fin.failed()) cta.mark();
 #pragma unroll
                 for (int j = 0; j < 8; j += 2) {
                     const int c = 8 * b + j;
@@ -330,6 +468,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8], zz[8], cc[8];
+                Finite fin;
                 if (XC == 1) {
                     tmem_ld8(tl + c0 + i, a);
                     tmem_ld8(tl + 2 * H + c0 + i, zz);
@@ -351,7 +490,9 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
                     zz[j] = z;
                     cc[j] = c;
                     hv[i + j] = z * hv[i + j] + (1.0f - z) * c;
+                    fin.see(hv[i + j]);
                 }
+                if (fin.failed()) cta.mark();
                 st4(g.z + sb + blk(c0 + i, row), zz);
                 st4(g.z + sb + blk(c0 + i + 4, row), zz + 4);
                 st4(g.c + sb + blk(c0 + i, row), cc);
@@ -379,6 +520,10 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const WinArgs g) {
             if (ok) outputs(g.T - 1);
         }
         ok = cta.hand_over(ok);   // (the same answer in every thread)
+        if (ok && cta.marked()) {
+            plain_fwd<H>(g, tile, reinterpret_cast<float *>(sA));
+            cta.unmark();
+        }
     }
     cta.finish(1, L::COLS, g.status);
 }
@@ -397,7 +542,7 @@ template <int H> struct Bwd32Layout {
 };
 
 template <int H>
-__global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__ WinArgs g) {
     using L = Bwd32Layout<H>;
     constexpr int NC = H / 4;
     constexpr int T_DH = 0, T_DRH = 64, T_CZ = 128, T_CR = 192;
@@ -433,7 +578,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
 #pragma unroll
         for (int i = 0; i < DDN; ++i) {
             const int c = 4 * (part + 4 * i);
-            if (c < g.nfc) put4_3<true>(img, IMG, row, c, dd[i]);
+            if (c < g.nfc) put4_3(img, IMG, row, c, dd[i]);
         }
     };
     for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
@@ -502,6 +647,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8];
+                Finite fin;   // (a dA that is not finite shows in the step before)
                 tmem_ld8(tl + T_DRH + c0 + i, a);
                 tmem_wait();
                 keep(a);
@@ -510,8 +656,10 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
                     const int k = i + j;
                     a[j] = whole(a[j], H / 16);
                     cpart[k] = dh[k] * zv[k] + a[j] * rv[k];
+                    fin.see(cpart[k]);
                     a[j] = a[j] * hp[k] * rv[k] * (1.0f - rv[k]);
                 }
+                if (fin.failed()) cta.mark();
                 put8_3(B1, IMG, row, c0 + i, a);
 #pragma unroll
                 for (int j = 0; j < 8; j += 4) st4(g.dG + gb + tblk + blk(c0 + i + j, row), a + j);
@@ -534,13 +682,18 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
 #pragma unroll
                 for (int i = 0; i < NC; i += 8) {
                     float b[8], c[8];
+                    Finite fin;
                     tmem_ld8(tl + T_CZ + c0 + i, b);
                     tmem_ld8(tl + T_CR + c0 + i, c);
                     tmem_wait();
                     keep(b);
                     keep(c);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) b[j] = whole(b[j] + c[j], H / 16) + cpart[i + j];
+                    for (int j = 0; j < 8; ++j) {
+                        b[j] = whole(b[j] + c[j], H / 16) + cpart[i + j];
+                        fin.see(b[j]);
+                    }
+                    if (fin.failed()) cta.mark();
                     if (gp < g.P) {
                         st4(g.dh0 + (size_t)gp * H + c0 + i, b);
                         st4(g.dh0 + (size_t)gp * H + c0 + i + 4, b + 4);
@@ -549,6 +702,10 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const WinArgs g) {
             }
         }
         ok = cta.hand_over(ok);   // (the same answer in every thread)
+        if (ok && cta.marked()) {
+            plain_bwd<H>(g, tile, reinterpret_cast<float *>(B0));
+            cta.unmark();
+        }
     }
     cta.finish(1, L::COLS, g.status);
 }
@@ -574,8 +731,50 @@ template <int H> struct Grad32Layout {
     static constexpr int NB = (3 * H + 64) / 8 / 4;   // blocks of 8 gradient columns a thread adds up
 };
 
+// A CTA's blocks [b0, b1) with FP32 FMAs, for a warp with a sum that is not finite:
+// its own lanes and columns, to where the sums were.
+template <int H, bool X2> __device__ __noinline__ void plain_grad(const WinArgs &g, long long b0, long long b1, uint32_t tmem) {
+    const int warp = threadIdx.x >> 5, q = warp & 3, part = warp >> 2, m = q * 32 + (threadIdx.x & 31);
+    const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
+    const int ncol = 3 * H + (X2 ? 0 : g.nfc), fx = (X2 ? 64 : 0) + m, mh = m - 64;   // feature and state column of this lane
+    const size_t tblk = (size_t)TM * H;
+    for (int c = 8 * part; c < ncol; c += 32) {
+        const int gate = c / H;
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = 0.f;
+        for (long long it = b0; it < b1; ++it) {
+            const int s = (int)(it % g.T), th = (int)(it / g.T), tile = th >> 1, r0 = (th & 1) * GR;
+            const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+            const bool last = s + 1 == g.T;
+            for (int r = r0; r < min(r0 + GR, g.P - tile * TM); ++r) {
+                const int gp = tile * TM + r;
+                const size_t prow = (size_t)s * g.P + gp;
+                float a = 0.f;
+                if (c >= 3 * H) {
+                    if (m < H) a = last ? g.hT[(size_t)gp * H + m] : g.hb[sb + (size_t)g.ntiles * tblk + elem(m, r)];
+                } else if (m < 64) {
+                    if (fx < g.n_in) a = __ldg(g.X + prow * g.ldx + fx);
+                } else if (!X2 && mh < H) {
+                    a = g.hb[sb + elem(mh, r)];
+                    if (gate == 2) a *= g.r[sb + elem(mh, r)];
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float b;
+                    if (c < 3 * H) b = g.dG[3 * sb + gate * tblk + elem(c - gate * H + j, r)];
+                    else b = c - 3 * H + j < g.n_out ? __ldg(g.dD + prow * g.n_out + c - 3 * H + j) : 0.f;
+                    v[j] = fmaf(a, b, v[j]);
+                }
+            }
+        }
+        tmem_st8(tl + Grad32Layout<H>::SUM + c, v);
+    }
+    tmem_wait_st();
+}
+
 template <int H, bool X2>
-__global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
+__global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const __grid_constant__ WinArgs g) {
     using L = Grad32Layout<H>;
     constexpr int X0 = X2 ? 64 : 0, NB = X2 ? 3 * H / 32 : L::NB;
     extern __shared__ uint8_t smem_raw[];
@@ -692,7 +891,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
             ld4(g.dG + gz, az); ld4(g.dG + gz + 4 * TM, az + 4);
             ld4(g.dG + gz + tblk, ar); ld4(g.dG + gz + tblk + 4 * TM, ar + 4);
         }
-        put8_3<true>(base + L::X, GIMG, xr, xc, xv);
+        put8_3(base + L::X, GIMG, xr, xc, xv);
         if (mine) {
             if (!X2) {
                 put8_3(base + L::HP, GIMG, lr, lc, hp);
@@ -715,7 +914,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
         if (!X2 && xc < g.nfc) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) xv[j] = gp < g.P && xc + j < g.n_out ? __ldg(dsrc + j) : 0.f;
-            put8_3<true>(base + L::DD, GIMG, xr, xc, xv);
+            put8_3(base + L::DD, GIMG, xr, xc, xv);
         }
         if (mine) {
             put8_3(base + L::GC, GIMG, lr, lc, hp);
@@ -735,16 +934,27 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const WinArgs g) {
     }
     if (ok && summed && !*cta.abort_flag) {
         float *o = g.part + (size_t)blockIdx.x * g.part_cols * TM;
+        auto write = [&]() {
+            Finite fin;
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const int c = 8 * (part + 4 * b);
-            if (c >= ncol) continue;
-            float v[8];
-            tmem_ld8(tl + L::SUM + c, v);
-            tmem_wait();
-            keep(v);
+            for (int b = 0; b < NB; ++b) {
+                const int c = 8 * (part + 4 * b);
+                if (c >= ncol) continue;
+                float v[8];
+                tmem_ld8(tl + L::SUM + c, v);
+                tmem_wait();
+                keep(v);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) o[(size_t)(out0 + c + j) * TM + row] = v[j];
+                for (int j = 0; j < 8; ++j) {
+                    fin.see(v[j]);
+                    o[(size_t)(out0 + c + j) * TM + row] = v[j];
+                }
+            }
+            return fin.failed();
+        };
+        if (__any_sync(0xffffffffu, write())) {
+            plain_grad<H, X2>(g, i0, i1, cta.tmem);
+            write();
         }
     }
     cta.finish(1, L::COLS, g.status);

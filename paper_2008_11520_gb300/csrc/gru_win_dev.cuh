@@ -165,7 +165,7 @@ struct Cta {
         bar0 = smem_u32(bars);
         if (threadIdx.x == 0) {
             for (int i = 0; i < nbar; ++i) mbar_init(bar0 + 8 * i, 1);
-            *abort_flag = 0;
+            abort_flag[0] = abort_flag[1] = 0;
             mbar_init_fence();
         }
         if (threadIdx.x < 32) {
@@ -187,6 +187,13 @@ struct Cta {
         const bool bad = __syncthreads_or(!ok);
         tc_after_sync();
         return !bad;
+    }
+    // a value that is not finite has been seen (read by all threads after a hand-over, and set back by one)
+    __device__ __forceinline__ void mark() { abort_flag[1] = 1; }
+    __device__ __forceinline__ bool marked() const { return abort_flag[1]; }
+    __device__ __forceinline__ void unmark() {
+        __syncthreads();
+        if (threadIdx.x == 0) abort_flag[1] = 0;
     }
     __device__ __forceinline__ bool wait(int b, uint32_t parity) {
         const bool ok = mbar_wait_inl(bar0 + 8 * b, parity, abort_flag);
