@@ -264,11 +264,19 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
     const size_t tblk = (size_t)TM * H;
     XTile<BWD_TH> xt;
     float zv[NC], rv[NC], cv[NC], hp[NC];
+    // (rows past the last patch add nothing to the weight gradients, also where
+    // an infinite weight makes NaNs of them: activations and gradients of 0)
     auto load_step = [&](int s, int tile) {
         const size_t sb = ((size_t)s * g.ntiles + tile) * tblk;
+        const bool valid = tile * TM + row < g.P;
 #pragma unroll
         for (int i = 0; i < NC; i += 4) {
             const size_t o = sb + blk(c0 + i, row);
+            if (!valid) {
+#pragma unroll
+                for (int j = i; j < i + 4; ++j) zv[j] = rv[j] = cv[j] = hp[j] = 0.f;
+                continue;
+            }
             ld4(g.z + o, zv + i);
             ld4(g.r + o, rv + i);
             ld4(g.c + o, cv + i);
@@ -293,6 +301,7 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
     const int kfc = g.nfc / 16;
     for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
         const int p0 = tile * TM, gp = p0 + row;
+        const bool valid = gp < g.P;
         float cpart[NC];
 #pragma unroll
         for (int i = 0; i < NC; ++i) cpart[i] = 0.f;
@@ -327,7 +336,7 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
                     const float carry = s == g.T - 1 ? 0.f : (XC == 1 ? b[j] + cpart[k] : cpart[k]);
-                    dh[k] = a[j] + carry;
+                    dh[k] = valid ? a[j] + carry : 0.f;
                     const float dc = dh[k] * (1.0f - zv[k]), dz = dh[k] * (hp[k] - cv[k]);
                     az[k] = dz * zv[k] * (1.0f - zv[k]);
                     ac[k] = dc * (1.0f - cv[k] * cv[k]);
@@ -373,6 +382,7 @@ __global__ void __launch_bounds__(BWD_TH, 1) k_win_bwd(const WinArgs g) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
+                    if (!valid) a[j] = 0.f;
                     cpart[k] = dh[k] * zv[k] + a[j] * rv[k];
                     a[j] = a[j] * hp[k] * rv[k] * (1.0f - rv[k]);
                 }

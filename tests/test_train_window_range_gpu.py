@@ -1,6 +1,6 @@
 """Training windows with operands that are infinite, not numbers, or near the
 ends of the FP32 range: outputs, state and gradients have the infinities, NaNs
-and values that FP32 products give."""
+and values that FP32 products give, and in BF16 those of rounded operands."""
 
 import pytest
 import torch
@@ -95,6 +95,13 @@ def check_range(dn, prec, where, value, size):
     if value in (INF, -INF):
         a[a.shape[0] // 2, 1] = -value
     agree(run(dn, prec, **t), reference(**t, bf16=prec == "bf16"), TOL[prec])
+
+
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("where,value", CASES)
+def test_bf16_range(dn, where, value, size):
+    # (sizes whose last tile has rows past the last patch)
+    check_range(dn, "bf16", where, value, size)
 
 
 @pytest.mark.parametrize("scale", [1e-30, 1e-33])
