@@ -10,7 +10,12 @@
 // registers.  Measured against 64 bits on N(0, 1) operands: 0.8e-7 for K = 64
 // and 1.3e-7 for K = 128, against 1.5e-7 and 2.1e-7 for FP32 FMA in sequence
 // (the leading product first: 7e-7 and 1.4e-6); sums of 4096 terms drained
-// every 128: 1.6e-7 against 1.1e-6.
+// every 128: 1.6e-7 against 1.1e-6.  Each accumulation at a sum's full
+// magnitude, one per 16 terms, drops up to an ulp, all of one sign; outputs and
+// gradients of a window (65 536 rows, T = 10, H = 64) are off by 1.5e-7 and
+// 2.3e-7, with FP32 FMAs by 2.1e-7 and 1.2e-6.  Putting back the average loss
+// would make that 1.2e-7 and 1.8e-7, but also change sums that lost nothing:
+// a sum of one product is exact wherever FP32's is.
 //
 // Six tcgen05 products of BF16 are 316 TFLOP/s of FP32 at the measured BF16
 // rate; the CUDA cores' FMAs give 74.  With the fused window (see gru_win.cu,
@@ -64,12 +69,6 @@ __device__ __forceinline__ void mma3_mn(uint32_t d, uint32_t a, uint32_t astep, 
         }
     }
 }
-
-// Each accumulation at a product's full magnitude (one per 16 terms of its
-// leading part) drops on average 2.1e-8 of the sum (measured: 0.85e-7 for K =
-// 64, 1.7e-7 for K = 128, all of one sign).  That much is put back, so that
-// long sums of products do not keep the bias.
-__device__ __forceinline__ float whole(float v, int ksteps) { return fmaf(v, 2.1e-8f * (float)ksteps, v); }
 
 // Whether every value seen is finite (0 x is not 0 for one that is not)
 struct Finite {
@@ -336,7 +335,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_x(const __grid_constant__ W
             keep(a);
             keep(b);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) a[j] = whole(a[j], 4) + whole(b[j], g.kx2);
+            for (int j = 0; j < 8; ++j) a[j] += b[j];
             st4(o + blk(c0 + i, row), a);
             st4(o + blk(c0 + i + 4, row), a + 4);
         }
@@ -393,10 +392,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
                 keep(v);
                 if (!valid) continue;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    v[j] = whole(v[j], H / 16);
-                    fin.see(v[j]);
-                }
+                for (int j = 0; j < 8; ++j) fin.see(v[j]);
                 if (fin.failed()) cta.mark();
 #pragma unroll
                 for (int j = 0; j < 8; j += 2) {
@@ -441,7 +437,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
                 keep(b);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    rr[j] = sigm((XC == 1 ? whole(a[j], 4) : gr[(i + j) % (XC == 2 ? NC : 1)]) + whole(b[j], H / 16));
+                    rr[j] = sigm((XC == 1 ? a[j] : gr[(i + j) % (XC == 2 ? NC : 1)]) + b[j]);
                     a[j] = rr[j] * hv[i + j];
                 }
                 st4(g.r + sb + blk(c0 + i, row), rr);
@@ -485,8 +481,8 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = (i + j) % (XC == 2 ? NC : 1);
-                    const float z = sigm((XC == 1 ? whole(a[j], 4) : gz[k]) + whole(b[j], H / 16)),
-                                c = tanhf((XC == 1 ? whole(zz[j], 4) : gc[k]) + whole(cc[j], H / 16));
+                    const float z = sigm((XC == 1 ? a[j] : gz[k]) + b[j]),
+                                c = tanhf((XC == 1 ? zz[j] : gc[k]) + cc[j]);
                     zz[j] = z;
                     cc[j] = c;
                     hv[i + j] = z * hv[i + j] + (1.0f - z) * c;
@@ -622,8 +618,8 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
-                    const float carry = s == g.T - 1 ? 0.f : whole(b[j] + c[j], H / 16) + cpart[k];
-                    dh[k] = whole(a[j], kfc) + carry;
+                    const float carry = s == g.T - 1 ? 0.f : b[j] + c[j] + cpart[k];
+                    dh[k] = a[j] + carry;
                     const float dc = dh[k] * (1.0f - zv[k]), dz = dh[k] * (hp[k] - cv[k]);
                     az[j] = dz * zv[k] * (1.0f - zv[k]);
                     ac[j] = dc * (1.0f - cv[k] * cv[k]);
@@ -654,7 +650,6 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
-                    a[j] = whole(a[j], H / 16);
                     cpart[k] = dh[k] * zv[k] + a[j] * rv[k];
                     fin.see(cpart[k]);
                     a[j] = a[j] * hp[k] * rv[k] * (1.0f - rv[k]);
@@ -690,7 +685,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
                     keep(c);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        b[j] = whole(b[j] + c[j], H / 16) + cpart[i + j];
+                        b[j] = b[j] + c[j] + cpart[i + j];
                         fin.see(b[j]);
                     }
                     if (fin.failed()) cta.mark();
@@ -810,7 +805,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const __grid_constant_
                 tmem_wait();
                 keep(v);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[b][j] += whole(v[j], GR / 16);
+                for (int j = 0; j < 8; ++j) acc[b][j] += v[j];
             }
         }
     };
