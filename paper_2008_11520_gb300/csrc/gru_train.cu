@@ -257,11 +257,17 @@ __global__ void k_bwd_reset(int P, int H, const float *__restrict__ drh, const f
 }
 
 // ---------------------------------------------------------------- loss, Adam
+__device__ __forceinline__ float two_sum(float &s, float x) {   // s += x; returns what the sum lost
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s), e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+    s = t;
+    return e;
+}
 // dD = 2 (D - Y) / P (FP32) and per-block partial sums of (D - Y)^2 / P,
 // accumulated in FP64.  FP64 adds and conversions (two a clock and SM) took
 // three times as long as the memory, so where the arrays start on 16 bytes
-// (VEC) a thread adds 16 squares exactly as an FP32 sum and its error (TwoSum)
-// and only these two in FP64: 32.8 million values 158 -> 62 us.
+// (VEC) a thread adds 16 squares as an FP32 sum, the sum of its errors (TwoSum)
+// and the errors of that, off by less than 2^-68 of them, and only these three
+// in FP64: 32.8 million values 158 -> 62 us (memory).
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_l2_loss(long long n, int P, float two_over_p, const float *__restrict__ D,
                                                  const float *__restrict__ Y, float *__restrict__ dD,
@@ -292,16 +298,13 @@ __global__ void __launch_bounds__(256) k_l2_loss(long long n, int P, float two_o
                 p[4 * k + 2] = f.z * f.z;
                 p[4 * k + 3] = f.w * f.w;
             }
-            float hi = 0.f, lo = 0.f;
+            float hi = 0.f, lo = 0.f, ll = 0.f;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const float t = __fadd_rn(hi, p[k]), bb = __fsub_rn(t, hi);
-                lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bb)), __fsub_rn(p[k], bb)));
-                hi = t;
-            }
+            for (int k = 0; k < 16; ++k) ll = __fadd_rn(ll, two_sum(lo, two_sum(hi, p[k])));
             if (isfinite(hi)) {
                 s += (double)hi;
                 s += (double)lo;
+                s += (double)ll;
             } else {   // beyond the FP32 range, or a value is not a number
                 for (int k = 0; k < 16; ++k) s += (double)p[k];
             }
