@@ -146,7 +146,9 @@ class PatchNetTrainer:
         return L2Loss.apply(D, Y, self.P), D
 
     def train_window(self, X, Y, h0=None):
-        """One Adam update on one window; returns (loss incl. Tikhonov, h_T)."""
+        """One Adam update on one window; returns (loss incl. Tikhonov, h_T).
+        DnnmgError if a bounded wait of the window's kernels ran out: outputs
+        and gradients were incomplete, so this update's weights are not to be used."""
         for p in self.params:
             p.grad = None
         L, _ = self.loss(X, Y, h0)
@@ -157,7 +159,11 @@ class PatchNetTrainer:
                 dnnmg.dnnmg_adam_step(p, p.grad, m, v, self.step_no, lr=self.lr, alpha=self.alpha)
             reg = sum(dnnmg.dnnmg_sumsq(p) for p in self.params)
         hT = self.trainer.state().clone()
-        return float(L.detach()) + self.alpha * float(reg), hT
+        loss = float(L.detach()) + self.alpha * float(reg)
+        status = self.trainer.status()   # (the device has finished: read with the loss)
+        if status:
+            raise dnnmg.DnnmgError(2, f"update {self.step_no}: the window's device status is {status}")
+        return loss, hT
 
 
 def patch_node_index(mesh):
