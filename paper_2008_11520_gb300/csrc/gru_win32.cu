@@ -159,7 +159,8 @@ template <int H> __device__ __noinline__ void plain_fwd(const WinArgs &g, int ti
         const int gp = tile * TM + row;
         const bool valid = gp < g.P;
         __syncwarp();
-        for (int j = lane; j < H; j += 32) h[j] = valid && g.h0 ? g.h0[(size_t)gp * H + j] : 0.f;
+        // (h_0 as saved: the caller's array may be the state that has been written meanwhile)
+        for (int j = lane; j < H; j += 32) h[j] = g.hb[(size_t)tile * tblk + elem(j, row)];
         for (int s = 0; s < g.T; ++s) {
             const size_t sb = ((size_t)s * g.ntiles + tile) * tblk, prow = (size_t)s * g.P + gp;
             if (valid)

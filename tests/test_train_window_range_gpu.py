@@ -113,3 +113,20 @@ def test_small_gradients_keep_their_digits(dn, size, scale):
     t = {k: torch.tensor(a, dtype=torch.float32) for k, a in zip(("X", "h0", "Wx", "Uh", "Wfc"), (X, h0, *W))}
     t["dD"] = torch.randn(T, P, n_out, generator=torch.Generator().manual_seed(2)) * scale
     agree(run(dn, "f32", **t), reference(**t, bf16=False), TOL["f32"])
+
+
+def test_state_of_the_window_before_as_h0(dn):
+    """h0 may be the trainer's own state, which the window overwrites."""
+    T, P, n_in, H, n_out = 2, 140, 51, 64, 18
+    (X, h0, Y), W = problem(T, P, n_in, n_in, H, n_out, seed=7)
+    t = {k: torch.tensor(a, dtype=torch.float32) for k, a in zip(("X", "h0", "Wx", "Uh", "Wfc"), (X, h0, *W))}
+    t["X"][0, 3, 5] = INF
+    tr = dn.Trainer(n_in, n_in, H, n_out, T, P)
+    Xg, Wg = t["X"].cuda(), [t[k].cuda() for k in ("Wx", "Uh", "Wfc")]
+    D = torch.empty(T, P, n_out, device="cuda")
+    tr.forward(torch.nan_to_num(Xg, posinf=1.0), t["h0"].cuda(), *Wg, D)
+    h1 = tr.state().cpu()
+    tr.forward(Xg, tr.state(), *Wg, D)
+    dD = torch.zeros(T, P, n_out)
+    want = reference(t["X"], h1, t["Wx"], t["Uh"], t["Wfc"], dD, False)
+    agree([D.cpu(), tr.state().cpu()], want, TOL["f32"])
