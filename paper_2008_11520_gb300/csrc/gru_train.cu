@@ -376,10 +376,13 @@ unsigned blocks_for(long long n) { return (unsigned)((n + 255) / 256); }
 
 struct dnnmg_trainer_s {
     int n_in, ldx, H, n_out, T, P, device;
-    // saved activations of the last forward window
-    float *GX;      // [T P][3H]
-    float *hs;      // [(T+1) P][H]: h_0 .. h_T
-    float *z, *r, *rh, *c;   // [T P][H] each
+    // Activations of the last forward, one kernel per product: GX [T P][3H],
+    // hs [(T+1) P][H] (h_0 .. h_T), z, r, rh = r h, c [T P][H] each.  Fused window
+    // (wpart): z, r, c and, in rh, h_0 .. h_{T-1} in whole 128-row tiles (gru_win.cu),
+    // hs [2 P][H] (a copy of an unaligned h_0; h_T), and of the scratch only dG
+    // (FP32 products; GX is the same array, used before it) and carry.
+    float *GX, *hs, *hT;
+    float *z, *r, *rh, *c;
     // scratch
     float *GH;      // [P][2H]
     float *AH;      // [P][H]
@@ -549,12 +552,12 @@ WinArgs window(dnnmg_trainer_s *t, const float *X) {
     g.xvec = t->ldx % 4 == 0 && aligned16(X);
     g.kx2 = t->n_in > 64 ? round_up(t->n_in - 64, 16) / 16 : 0;
     g.part_cols = (g.kx2 ? 6 : 3) * t->H + g.nfc;
-    g.GX = t->GX;
+    g.GX = t->dG;
     g.X = X;
     g.z = t->z; g.r = t->r; g.c = t->c; g.hb = t->rh;
     g.part = t->wpart;
     g.dG = t->dG;
-    g.hT = t->hs + (size_t)t->T * t->P * t->H;
+    g.hT = t->hT;
     g.status = t->d_status;
     return g;
 }
@@ -603,19 +606,19 @@ int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnm
     t->splits = (int)std::min<size_t>(256, std::max<size_t>(1, TP / 4096));
     const size_t mx = (size_t)std::max(3 * H, n_out) * std::max(std::max(n_in, H), 1);
     t->part_floats = (size_t)t->splits * mx;
-    // (GX, z, r, rh, c and dG hold whole 128-row tiles in the fused window)
-    const size_t TPt = (size_t)T * win_tiles(P) * 128;
-    struct { float **p; size_t n; } req[] = {
-        {&t->GX, TPt * 3 * H}, {&t->hs, (TP + P) * H}, {&t->z, TPt * H}, {&t->r, TPt * H}, {&t->rh, TPt * H},
-        {&t->c, TPt * H}, {&t->GH, (size_t)P * 2 * H}, {&t->AH, (size_t)P * H}, {&t->dHfc, TP * H},
-        {&t->dG, TPt * 3 * H}, {&t->dh, (size_t)P * H}, {&t->drh, (size_t)P * H}, {&t->carry, (size_t)P * H},
-        {&t->part, t->part_floats}};
+    const bool win = win_supported(n_in, H, n_out);
+    const size_t PH = (size_t)P * H, rows = win ? (size_t)T * win_tiles(P) * 128 : TP;
+    struct { float **p; size_t n; bool need; } req[] = {
+        {&t->z, rows * H, true}, {&t->r, rows * H, true}, {&t->rh, rows * H, true}, {&t->c, rows * H, true},
+        {&t->dG, rows * 3 * H, true}, {&t->carry, PH, true}, {&t->hs, win ? 2 * PH : (TP + P) * H, true},
+        {&t->wpart, win ? win_part_floats(n_in, H, n_out, T, P) : 0, win},
+        {&t->GX, TP * 3 * H, !win}, {&t->GH, 2 * PH, !win}, {&t->AH, PH, !win}, {&t->dHfc, TP * H, !win},
+        {&t->dh, PH, !win}, {&t->drh, PH, !win}, {&t->part, t->part_floats, !win}};
     bool ok = true;
-    for (auto &q : req) ok = ok && cudaMalloc(q.p, q.n * sizeof(float)) == cudaSuccess;
+    for (auto &q : req) ok = ok && (!q.need || cudaMalloc(q.p, q.n * sizeof(float)) == cudaSuccess);
+    t->hT = t->hs + (win ? PH : TP * H);
     ok = ok && cudaMalloc(&t->red, kRedBlocks * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc(&t->d_status, sizeof(int)) == cudaSuccess && cudaMemset(t->d_status, 0, sizeof(int)) == cudaSuccess;
-    if (win_supported(n_in, H, n_out))
-        ok = ok && cudaMalloc(&t->wpart, win_part_floats(n_in, H, n_out, T, P) * sizeof(float)) == cudaSuccess;
     if (!ok) {
         trainer_free(t);
         cudaGetLastError();
@@ -638,12 +641,23 @@ int dnnmg_trainer_set_precision(dnnmg_trainer_t t, int precision) {
     if (int e = check_trainer(t)) return e;
     if (precision != DNNMG_F32 && precision != DNNMG_BF16NET)
         return fail(DNNMG_EINVAL, "trainer precision must be DNNMG_F32 or DNNMG_BF16NET, got %d", precision);
-    t->bf16 = 0;
-    if (precision == DNNMG_F32) return DNNMG_OK;
-    if (t->wpart) {   // the fused window: no operand copies
-        t->bf16 = 1;
+    if (t->wpart) {   // the fused window: no operand copies, and only FP32 products keep dA in memory
+        if (precision == DNNMG_BF16NET) {
+            cudaFree(t->dG);
+            t->dG = nullptr;
+        } else if (!t->dG) {
+            const size_t n = (size_t)t->T * win_tiles(t->P) * 128 * 3 * t->H;
+            if (cudaMalloc(&t->dG, n * sizeof(float)) != cudaSuccess) {
+                t->dG = nullptr;
+                cudaGetLastError();
+                return fail(DNNMG_ENOMEM, "FP32 gate gradients (%zu values) could not be allocated", n);
+            }
+        }
+        t->bf16 = precision == DNNMG_BF16NET;
         return DNNMG_OK;
     }
+    t->bf16 = 0;
+    if (precision == DNNMG_F32) return DNNMG_OK;
     // BF16 copies of the window's operands, K contiguous, each region 256-byte aligned
     const int H = t->H, P = t->P, TP = t->T * t->P;
     t->kx = kpad(t->n_in); t->kh = kpad(H); t->k2 = kpad(2 * H); t->ko = kpad(t->n_out);
@@ -757,7 +771,7 @@ int dnnmg_gru_seq_forward(dnnmg_trainer_t t, const float *X, const float *h0, co
 int dnnmg_gru_seq_state(dnnmg_trainer_t t, float **hT) {
     clear_error();
     if (!t || !hT) return fail(DNNMG_EINVAL, "NULL argument");
-    *hT = t->hs + (size_t)t->T * t->P * t->H;
+    *hT = t->hT;
     return DNNMG_OK;
 }
 

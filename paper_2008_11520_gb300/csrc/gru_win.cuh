@@ -15,8 +15,8 @@ struct WinArgs {
     float *D, *hT;                             // outputs of every step, state after the last
     float *z, *r, *c, *hb;                     // saved activations, [T][ntiles][H / 4][128][4]
     float *gWx, *gUh, *gWfc, *dh0, *part;
-    float *GX;                                 // FP32, two chunks: X W_x^T, [T][ntiles][3H / 4][128][4]
-    float *dG;                                 // FP32: gate gradients, [T][ntiles][3][H / 4][128][4]
+    float *GX;                                 // FP32 forward, two chunks: X W_x^T, [T][ntiles][3H / 4][128][4]
+    float *dG;                                 // FP32 backward: gate gradients, [T][ntiles][3][H / 4][128][4] (may be GX)
     int *status;
 };
 
