@@ -2,7 +2,7 @@
 // Eq. gru (reset gate before U_h, no biases) and the output layer, BF16
 // operands, FP32 accumulators in tensor memory.
 //
-// One persistent CTA per SM (two for H <= 64) walks 128-patch tiles (one TMEM lane per patch
+// One persistent CTA per SM (or two, for H <= 64) walks 128-patch tiles (one TMEM lane per patch
 // row).  Per tile, with the z, r and candidate pre-activations accumulating
 // in TMEM columns [0,H), [H,2H), [2H,3H):
 //   X groups:  for each 64-column chunk of X:
@@ -153,13 +153,11 @@ __device__ __forceinline__ void store_h16(uint8_t *sAh, int row, int c0, const f
     }
 }
 
-// CTAs an SM: a state of 64 columns or fewer leaves room for two (registers,
-// shared and tensor memory), and one computes while the other waits for its
-// products (307 776 rows, 51 -> 64 -> 18: 84 -> 68 us).
-constexpr int ctas_per_sm(int H) { return H <= 64 ? 2 : 1; }
-
-template <int H>
-__global__ void __launch_bounds__(NTH, ctas_per_sm(H))
+// CTAS: CTAs an SM.  A state of 64 columns or fewer leaves room for two, and one
+// computes while the other waits for its products; their registers are capped
+// at half (launch_gru_tc_rows has the rule and the figures).
+template <int H, int CTAS>
+__global__ void __launch_bounds__(NTH, CTAS)
 k_gru_tc(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmX3,
          const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmH3, float *__restrict__ d,
          int P, const int *__restrict__ hrow) {
@@ -682,25 +680,26 @@ cudaError_t launch_gru_tc_rows(const Net &n, const void *X, void *h, void *d, in
         if (!encode(&tmH3, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h, dims, strides, box)) return cudaErrorInvalidValue;
     }
     const size_t smem = smem_bytes(p);
-    // persistent: one or two CTAs per SM, tiles strided over the grid
-    const int per = 2 * (smem + 1024) <= 228 * 1024 && p.tmem_cols <= 256 ? ctas_per_sm(p.H) : 1;
-    const int grid = std::min((P + TM - 1) / TM, per * sm_count());
-    cudaError_t e;
-#define DNNMG_LAUNCH_H(HH)                                                                                   \
-    case HH:                                                                                                 \
-        e = cudaFuncSetAttribute(k_gru_tc<HH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
-        if (e != cudaSuccess) return e;                                                                      \
-        k_gru_tc<HH><<<grid, NTH, smem, st>>>(p, tmX3, tmX, tmH3, (float *)d, P, hrow);                      \
-        break;
+    // persistent, tiles strided over the grid.  Two CTAs an SM where shared and
+    // tensor memory hold them and there are more tiles than SMs (51 -> 64 -> 18:
+    // 307 776 rows 84 -> 68 us, 65 536 rows 24 -> 21; but 16 384 rows, 128 tiles, 10.7 -> 12.3
+    // with the capped registers, and 262 144 rows of 267 -> 64 -> 162, which leaves room for one, 148 -> 190).
+    const int tiles = (P + TM - 1) / TM, sms = sm_count();
+    const bool two = p.H <= 64 && 2 * (smem + 1024) <= 228 * 1024 && p.tmem_cols <= 256 && tiles > sms;
+    const int grid = std::min(tiles, (two ? 2 : 1) * sms);
+    auto run = [&](auto k) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k<<<grid, NTH, smem, st>>>(p, tmX3, tmX, tmH3, (float *)d, P, hrow);
+        return cudaGetLastError();
+    };
     switch (p.H) {
-        DNNMG_LAUNCH_H(32)
-        DNNMG_LAUNCH_H(64)
-        DNNMG_LAUNCH_H(96)
-        DNNMG_LAUNCH_H(128)
+        case 32: return two ? run(k_gru_tc<32, 2>) : run(k_gru_tc<32, 1>);
+        case 64: return two ? run(k_gru_tc<64, 2>) : run(k_gru_tc<64, 1>);
+        case 96: return run(k_gru_tc<96, 1>);
+        case 128: return run(k_gru_tc<128, 1>);
         default: return cudaErrorInvalidValue;
     }
-#undef DNNMG_LAUNCH_H
-    return cudaGetLastError();
 }
 
 }  // namespace dnnmg
