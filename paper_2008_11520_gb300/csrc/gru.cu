@@ -250,6 +250,7 @@ k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *X, const T *WxT,
         }
     }
     pdl_wait();   // (the weights do not change: staged above while the kernel before drains)
+    // (the grid has a CTA for every tile; as straight code FP32 came out 1.3 times slower)
     for (long long q0 = (long long)blockIdx.x * TP; q0 < P; q0 += (long long)gridDim.x * TP) {
         const int p0 = (int)q0, np = min(TP, P - p0);
         for (int i = threadIdx.x; i < TP * n_in; i += THREADS) {
@@ -340,11 +341,16 @@ cudaError_t run_rt(const Net &n, const void *X, void *h, void *d, int P, cudaStr
     auto k = k_gru_rt<T, TP, JT, PT, THREADS, SW>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    int grid = (P + TP - 1) / TP;
-    if (SW) {   // persistent: as many CTAs as fit
+    const int grid = (P + TP - 1) / TP;
+    if constexpr (SW && sizeof(T) == 8) {
+        // FP64 keeps the weights in shared memory while every CTA has one tile; beyond that
+        // the few CTAs an SM that fit beside them fall behind those that read them from L2
+        // (99 -> 32 -> 50: 300 patches 30 against 44 us, 700 patches 73 against 48,
+        // 16 336 patches 1209 against 553)
         int per = 1;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, THREADS, sm)) != cudaSuccess) return e;
-        grid = std::min(grid, std::max(1, per) * sm_count());
+        if (grid > std::max(1, per) * sm_count())
+            return run_rt<T, TP, JT, PT, THREADS, false>(n, X, h, d, P, st, chained);
     }
     return launch_chained(chained, k, dim3(grid), THREADS, sm, st, n.n_in, n.ldx, n.H, n.n_out, n.ldo, (const T *)X,
                           (const T *)n.WxT, (const T *)n.UhT, (const T *)n.WfcTp, (T *)h, (T *)d, P);
