@@ -785,9 +785,7 @@ static int step_body(dnnmg_mesh_t mesh, dnnmg_net_t net, const double *xc, void 
     const int prec = mesh->info.precision;
     const MeshGeom &g = mesh->g;
     int nev = 0;
-    // (on large meshes the next kernel's CTAs, waiting beside the last ones of this
-    // one, cost more than its launch: 623 -> 631 us at 32 768 tiles)
-    const bool chain = !ev && (long long)g.ntx * g.nty < 4096;
+    const bool chain = !ev;
     auto mark = [&]() -> cudaError_t { return ev ? cudaEventRecord(ev[nev++], s) : cudaSuccess; };
     DNNMG_CUDA_TRY(mark());
     // S1 is fused into S2+S3 and into S5: both interpolate x~ from xc inside

@@ -148,10 +148,15 @@ int round_up(int v, int m);
 
 #ifdef __CUDACC__
 // Kernels of the step that follow one another on a stream are launched so that
-// each may be put on the SMs while the one before it drains (programmatic
-// launch): 1 to 2 us less per kernel on small meshes.  pdl_enter() is the first
-// thing every thread does: it lets the next kernel in and waits until the one
-// before has completed and its writes are visible.
+// each is put on the SMs as soon as every CTA of the one before has exited
+// (programmatic launch): 1 to 2 us less per kernel on small meshes.  pdl_wait()
+// is the first thing every thread does: the kernel before has completed and its
+// writes are visible.  The step's kernels do not let the next one in earlier
+// (pdl_trigger): its CTAs would take the SMs that happen to have room, many of
+// them one SM's, and wait there, so that its work is spread unevenly
+// (384 x 96 cells, K = s = 2, FP64: a step takes 172 us so, 452 with the trigger
+// at the start of every kernel, 185 launched in plain order; 800 x 200 cells,
+// K = 2, FP32 with the BF16 net: 52, 57 and 59 us).
 // What an earlier kernel of the chain writes (X, d, v_corr, the padded x_c, the
 // correction of a sweep) is read by plain loads through pointers without __restrict__: a
 // chained kernel lives while that one still writes, and the read-only path
@@ -159,10 +164,6 @@ int round_up(int v, int m);
 // loads free to move above the wait.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_enter() {
-    pdl_trigger();
-    pdl_wait();
-}
 // chained: the kernel before on the stream is one of this library's, nothing in between
 template <typename... P, typename... A>
 cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A &&...a) {

@@ -222,7 +222,6 @@ template <typename T, int TP, int JT, int PT, int THREADS, bool SW>
 __global__ void __launch_bounds__(THREADS)
 k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *X, const T *WxT, const T *UhT, const T *WfcT, T *__restrict__ h, T *__restrict__ d, int P) {
     static_assert(TP % PT == 0, "whole tiles");
-    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int LP = TP + (TP > 4 ? 16 / (int)sizeof(T) : 0);   // staged row length (padded against bank conflicts)
     T *xs = reinterpret_cast<T *>(smem_raw);   // [n_in][LP] features
@@ -249,7 +248,7 @@ k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *X, const T *WxT,
             ws += cnt[m];
         }
     }
-    pdl_wait();   // (the weights do not change: staged above while the kernel before drains)
+    pdl_wait();   // (the weights do not change: staged above before the other kernel has completed)
     // (the grid has a CTA for every tile; as straight code FP32 came out 1.3 times slower)
     for (long long q0 = (long long)blockIdx.x * TP; q0 < P; q0 += (long long)gridDim.x * TP) {
         const int p0 = (int)q0, np = min(TP, P - p0);

@@ -161,7 +161,6 @@ __global__ void __launch_bounds__(NTH, CTAS)
 k_gru_tc(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmX3,
          const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmH3, float *__restrict__ d,
          int P, const int *__restrict__ hrow) {
-    pdl_trigger();
     constexpr int NH = H / 2;           // state columns per epilogue thread
     extern __shared__ uint8_t smem_raw[];
     // aligned by an offset from the shared-memory symbol itself, so that every

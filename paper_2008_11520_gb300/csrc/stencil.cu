@@ -1059,7 +1059,7 @@ __device__ __forceinline__ void coarse_pad_cta(const MeshGeom &g, const double *
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 k_coarse_pad(MeshGeom g, const double *__restrict__ xc, T *__restrict__ xcp, int pc) {
-    pdl_enter();
+    pdl_wait();
     coarse_pad_cta(g, xc, xcp, pc, blockIdx.x, gridDim.x);
 }
 
@@ -1074,7 +1074,7 @@ struct PadBatch {
     } inst[kBatch];
 };
 __global__ void __launch_bounds__(NTHREADS) k_coarse_pad_batch(const __grid_constant__ PadBatch p) {
-    pdl_enter();
+    pdl_wait();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     if (local == 0)
@@ -1170,7 +1170,7 @@ __global__ void __launch_bounds__(D::THREADS)
 k_residual_step(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmC, double inflow_peak, TX *__restrict__ X,
                 const int *__restrict__ tile_list) {
-    pdl_enter();
+    pdl_wait();
     // tile_list (when the closed-form kernel does the all-fluid tiles): the
     // other tiles, one per CTA; otherwise the grid covers every tile
     int tx = blockIdx.x, ty = blockIdx.y;
@@ -1199,7 +1199,7 @@ struct ResBatch {
 template <typename D, int R>
 __global__ void __launch_bounds__(D::THREADS, 1024 / D::THREADS) k_residual_step_batch(const __grid_constant__ ResBatch p) {
     __shared__ FemCoef<float> fc;
-    pdl_enter();
+    pdl_wait();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);
@@ -1449,7 +1449,7 @@ k_scatter_avg(MeshGeom g, const T *d, const T *__restrict__ xf, const double *__
     // the first and the two last tile rows (walls: general tiles, the slowest)
     // are scheduled first, so that they do not form the grid's tail
     const int ny = gridDim.y, by = blockIdx.y < 3 ? (blockIdx.y ? ny - blockIdx.y : 0) : blockIdx.y - 2;
-    pdl_enter();
+    pdl_wait();
     scatter_cta<T, R, PTY>(g, d, xf, xc, xcp, pc, inflow_peak, vc, blockIdx.x, by);
 }
 
@@ -1465,7 +1465,7 @@ struct AvgBatch {
 };
 template <int R, int PTY>
 __global__ void __launch_bounds__(NTHREADS, 6) k_scatter_avg_batch(const __grid_constant__ AvgBatch p) {
-    pdl_enter();
+    pdl_wait();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     const auto &q = p.inst[i];
@@ -1686,7 +1686,7 @@ __device__ __forceinline__ void rhs_cta(const MeshGeom &g, const FemCoef<T> &fc,
 template <typename D, typename T>
 __global__ void __launch_bounds__(D::THREADS)
 k_rhs(MeshGeom g, FemCoef<T> fc, const __grid_constant__ CUtensorMap tmV, T *__restrict__ bf) {
-    pdl_enter();
+    pdl_wait();
     rhs_cta<D>(g, fc, &tmV, bf, blockIdx.x, blockIdx.y);
 }
 
@@ -1826,7 +1826,7 @@ template <int NS>
 __global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS)
 k_rhs_march(MeshGeom g, FemCoef<float> fc, const __grid_constant__ CUtensorMap tmV, const float *vc,
             float *__restrict__ bf) {
-    pdl_enter();
+    pdl_wait();
     rhs_big<NS>(g, fc, &tmV, vc, bf, blockIdx.x);
 }
 
@@ -1843,7 +1843,7 @@ struct RhsBatch {
 __global__ void __launch_bounds__(SmallTile::THREADS) k_rhs_batch_small(const __grid_constant__ RhsBatch p) {
     using D = SmallTile;
     __shared__ FemCoef<float> fc;
-    pdl_enter();
+    pdl_wait();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);   // (visible after rhs_cta's first barrier)
@@ -1853,7 +1853,7 @@ __global__ void __launch_bounds__(SmallTile::THREADS) k_rhs_batch_small(const __
 template <int NS>
 __global__ void __launch_bounds__(MARCH_THREADS, MARCH_CTAS) k_rhs_batch_march(const __grid_constant__ RhsBatch p) {
     __shared__ FemCoef<float> fc;
-    pdl_enter();
+    pdl_wait();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     stage_coef(fc, p.inst[i].fc);
@@ -2101,7 +2101,7 @@ __device__ __forceinline__ void restrict_cta(const MeshGeom &g, const CUtensorMa
 template <typename T, typename Acc, int R>
 __global__ void __launch_bounds__(NTHREADS)
 k_restrict(MeshGeom g, const __grid_constant__ CUtensorMap tmB, double *__restrict__ bc) {
-    pdl_enter();
+    pdl_wait();
     restrict_cta<T, Acc, R>(g, &tmB, bc, blockIdx.x, blockIdx.y);
 }
 
@@ -2115,7 +2115,7 @@ struct RestrictBatch {
 };
 template <int R>
 __global__ void __launch_bounds__(NTHREADS) k_restrict_batch(const __grid_constant__ RestrictBatch p) {
-    pdl_enter();
+    pdl_wait();
     int local;
     const int i = batch_instance(p.first, p.n, local);
     const int ntx = (p.inst[i].g.nxc + 128 / R) / (128 / R);
