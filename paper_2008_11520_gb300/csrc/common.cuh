@@ -145,6 +145,13 @@ struct StepInst {
 constexpr int kBatch = 32;   // instances of one launch (their parameters stay below 32 KB)
 
 int round_up(int v, int m);
+// SMs of the current device
+inline int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return n > 0 ? n : 1;
+}
 
 #ifdef __CUDACC__
 // Kernels of the step that follow one another on a stream are launched so that

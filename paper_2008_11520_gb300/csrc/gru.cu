@@ -321,12 +321,6 @@ k_gru_rt(int n_in, int ldx, int H, int n_out, int ldo, const T *X, const T *WxT,
     }
 }
 
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 1;
-    return n > 0 ? n : 1;
-}
 size_t weight_count(const Net &n) { return (size_t)3 * n.H * (n.n_in + n.H) + (size_t)n.H * n.ldo; }
 // bytes of the weights and the staged values of TP patches (row length LP)
 size_t rt_bytes(const Net &n, int LP, size_t elem) {

@@ -509,13 +509,6 @@ size_t smem_bytes(const TcParams &p) {
     return (size_t)p.xb + (size_t)p.ahb + (size_t)p.wb + SMEM_EXTRA;
 }
 
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 1;
-    return n > 0 ? n : 1;
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     if (!fn) {

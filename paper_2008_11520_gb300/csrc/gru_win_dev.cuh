@@ -221,13 +221,6 @@ struct Cta {
 
 __device__ __forceinline__ uint8_t *align1k(uint8_t *p) { return p + ((1024u - (smem_u32(p) & 1023u)) & 1023u); }
 
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 1;
-    return n > 0 ? n : 1;
-}
-
 template <typename K> cudaError_t launch(K k, int grid, int threads, int smem, const WinArgs &g, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

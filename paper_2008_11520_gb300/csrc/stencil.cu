@@ -36,10 +36,19 @@ using BigTile = TileDim<TXC, TYC, 256>;
 // right-hand side 29 -> 9 us; 256 x 64 in FP32 (32 tiles): 24.5 -> 9 and
 // 5.7 -> 4.6 us; bound by the chain of staging, cell and node passes.
 using SmallTile = TileDim<8, 8, 128>;
-// Whether a launch over n tiles of 32 x 16 cells takes 8 x 8 ones instead:
-// where the large ones would not fill the chip twice over (patches have to
-// fit a tile).  Every node's arithmetic is the same in both.
-inline bool use_small(const MeshGeom &g, long long n) { return g.S <= SmallTile::TXC && n < 304; }
+// Whether a launch over n tiles of 32 x 16 cells takes 8 x 8 ones instead
+// (patches have to fit a tile).  Every node's arithmetic is the same in both.
+// FP32: where the large ones would not fill the chip twice over.  FP64 is bound
+// by its FMAs and the small tiles' halos add half to them: where the large ones
+// fill at most three fifths of their waves, one tile an SM (steps, large against
+// small ones: 72 tiles 366 / 330 and 203 / 175 us, 91 tiles 400 / 376, 98 tiles
+// 438 / 428 and 237 / 246, 128 tiles 209 / 227, 153 tiles 319 / 301, 200 tiles
+// 413 / 408, 242 tiles 463 / 479, 288 tiles 371 / 410).
+inline bool use_small(const MeshGeom &g, long long n, bool f64) {
+    const long long sms = sm_count();
+    if (g.S > SmallTile::TXC || n >= 2 * sms) return false;
+    return !f64 || 5 * n <= 3 * sms * ((n + sms - 1) / sms);
+}
 inline long long tiles_of(const MeshGeom &g) { return (long long)g.ntx * g.nty; }
 
 template <typename TX, typename T> __device__ __forceinline__ TX store_as(T v) { return (TX)v; }
@@ -2314,7 +2323,7 @@ cudaError_t run_residual_d(const MeshGeom &g, const FemCoef<T> &fc, const void *
 template <typename T, typename TX>
 cudaError_t run_residual_r(const MeshGeom &g, const FemCoef<T> &fc, const void *xf, const double *xc, double w,
                            const void *bf, void *rf, void *X, cudaStream_t st) {
-    if (use_small(g, tiles_of(g))) return run_residual_d<SmallTile, T, TX>(g, fc, xf, xc, w, bf, rf, X, st);
+    if (use_small(g, tiles_of(g), sizeof(T) == 8)) return run_residual_d<SmallTile, T, TX>(g, fc, xf, xc, w, bf, rf, X, st);
     return run_residual_d<BigTile, T, TX>(g, fc, xf, xc, w, bf, rf, X, st);
 }
 
@@ -2396,7 +2405,7 @@ cudaError_t run_residual_step_d(const MeshGeom &g, const FemCoef<T> &fc, const v
 template <typename T, typename TX>
 cudaError_t run_residual_step_r(const MeshGeom &g, const FemCoef<T> &fc, const void *xcp, double up, const void *bf,
                                 void *X, cudaStream_t st, bool sf, bool chained) {
-    if (use_small(g, sf ? g.n_slow_tiles : tiles_of(g)))
+    if (use_small(g, sf ? g.n_slow_tiles : tiles_of(g), sizeof(T) == 8))
         return run_residual_step_d<SmallTile, T, TX>(g, fc, xcp, up, bf, X, st, sf, chained);
     return run_residual_step_d<BigTile, T, TX>(g, fc, xcp, up, bf, X, st, sf, chained);
 }
@@ -2428,7 +2437,7 @@ cudaError_t run_scatter_p(const MeshGeom &g, const T *d, const T *xf, const doub
 template <typename T>
 cudaError_t run_scatter(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
                         cudaStream_t st, bool chained) {
-    if (use_small(g, tiles_of(g))) return run_scatter_p<T, 4>(g, d, xf, xc, xcp, w, vc, st, chained);
+    if (use_small(g, tiles_of(g), sizeof(T) == 8)) return run_scatter_p<T, 4>(g, d, xf, xc, xcp, w, vc, st, chained);
     return run_scatter_p<T, PTY>(g, d, xf, xc, xcp, w, vc, st, chained);
 }
 
@@ -2477,7 +2486,7 @@ cudaError_t run_rhs_march(const MeshGeom &g, const FemCoef<float> &fc, const flo
 
 template <typename T>
 cudaError_t run_rhs(const MeshGeom &g, const FemCoef<T> &fc, const T *vcorr, T *bf, cudaStream_t st, bool chained) {
-    if (use_small(g, tiles_of(g))) return run_rhs_d<SmallTile, T>(g, fc, vcorr, bf, st, chained);
+    if (use_small(g, tiles_of(g), sizeof(T) == 8)) return run_rhs_d<SmallTile, T>(g, fc, vcorr, bf, st, chained);
     if constexpr (sizeof(T) == 8) return run_rhs_d<BigTile, T>(g, fc, vcorr, bf, st, chained);
     else return march_tall(tiles_of(g)) ? run_rhs_march<16>(g, fc, vcorr, bf, st, chained)
                                        : run_rhs_march<4>(g, fc, vcorr, bf, st, chained);
@@ -2582,7 +2591,7 @@ template <typename D, int R> static cudaError_t residual_batch(const StepInst *i
 cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st) {
     long long tiles = 0;
     for (int i = 0; i < n; ++i) tiles += skip_fast ? in[i].mesh->g.n_slow_tiles : tiles_of(in[i].mesh->g);
-    const bool small = use_small(in[0].mesh->g, tiles);
+    const bool small = use_small(in[0].mesh->g, tiles, false);
     switch (in[0].mesh->g.r) {
         case 2: return small ? residual_batch<SmallTile, 2>(in, n, !skip_fast, st) : residual_batch<BigTile, 2>(in, n, !skip_fast, st);
         case 4: return small ? residual_batch<SmallTile, 4>(in, n, !skip_fast, st) : residual_batch<BigTile, 4>(in, n, !skip_fast, st);
@@ -2613,7 +2622,7 @@ template <int R, int PTY_> static cudaError_t scatter_batch(const StepInst *in, 
 cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st, bool chained) {
     long long tiles = 0;
     for (int i = 0; i < n; ++i) tiles += tiles_of(in[i].mesh->g);
-    const bool small = use_small(in[0].mesh->g, tiles);
+    const bool small = use_small(in[0].mesh->g, tiles, false);
     switch (in[0].mesh->g.r) {
         case 2: return small ? scatter_batch<2, 4>(in, n, st, chained) : scatter_batch<2, PTY>(in, n, st, chained);
         case 4: return small ? scatter_batch<4, 4>(in, n, st, chained) : scatter_batch<4, PTY>(in, n, st, chained);
@@ -2649,7 +2658,7 @@ template <typename D, int NS> static cudaError_t rhs_batch(const StepInst *in, i
 cudaError_t launch_rhs_batch(const StepInst *in, int n, cudaStream_t st) {
     long long tiles = 0;
     for (int i = 0; i < n; ++i) tiles += tiles_of(in[i].mesh->g);
-    if (use_small(in[0].mesh->g, tiles)) return rhs_batch<SmallTile, 0>(in, n, st);
+    if (use_small(in[0].mesh->g, tiles, false)) return rhs_batch<SmallTile, 0>(in, n, st);
     return march_tall(tiles) ? rhs_batch<BigTile, 16>(in, n, st) : rhs_batch<BigTile, 4>(in, n, st);
 }
 
