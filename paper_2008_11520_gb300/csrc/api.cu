@@ -801,11 +801,19 @@ static int step_body(dnnmg_mesh_t mesh, dnnmg_net_t net, const double *xc, void 
     const bool cf = residual_cf_supported(g, prec);
     if (cf && !ev && g.n_slow_tiles > 0) {
         // the two S2+S3 kernels write disjoint rows of X: the boundary tiles
-        // (few, slow CTAs) run on the side stream while the closed form runs
+        // (few, slow CTAs) run on the side stream while the closed form runs.
+        // 8 x 8-cell ones go second: they spread over every SM at once, and the
+        // closed form, which wants another split of shared memory and L1, would
+        // wait for them where the GPU is not still busy with other work (lone
+        // steps of 512 x 128 cells, K = 2, BF16 net: 65 us so, 81 the other way
+        // round; 1600 x 400: 100 and 114).  Large ones, on few SMs, go first
+        // (2400 x 600, K = s = 2: 118 us, 126 the other way round).
+        const bool second = residual_step_small(g, prec);
         DNNMG_CUDA_TRY(cudaEventRecord(mesh->ev_fork, s));
         DNNMG_CUDA_TRY(cudaStreamWaitEvent(mesh->side, mesh->ev_fork, 0));
+        if (second) DNNMG_CUDA_TRY(launch_residual_cf(g, prec, mesh->fem32, w.xcp, bf, w.X, s));
         DNNMG_CUDA_TRY(launch_residual_step(g, prec, mesh->fem64, mesh->fem32, w.xcp, t, bf, w.X, mesh->side, true));
-        DNNMG_CUDA_TRY(launch_residual_cf(g, prec, mesh->fem32, w.xcp, bf, w.X, s));
+        if (!second) DNNMG_CUDA_TRY(launch_residual_cf(g, prec, mesh->fem32, w.xcp, bf, w.X, s));
         DNNMG_CUDA_TRY(cudaEventRecord(mesh->ev_join, mesh->side));
         DNNMG_CUDA_TRY(cudaStreamWaitEvent(s, mesh->ev_join, 0));
     } else {

@@ -220,6 +220,8 @@ cudaError_t launch_coarse_pad(const MeshGeom &g, int prec, const double *xc, voi
 cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<double> &f64, const FemCoef<float> &f32,
                                  const void *xcp, double t, const void *bf, void *X, cudaStream_t st,
                                  bool skip_fast = false, bool chained = false);
+// Whether that launch takes 8 x 8-cell tiles for the tiles left to it.
+bool residual_step_small(const MeshGeom &g, int prec);
 // S2 + S3 of the step on the all-fluid tiles in closed form (residual_cf.cu):
 // FP32 fields, K = 1 or 2.  launch_residual_step(..., skip_fast = true) then
 // does the other tiles.
@@ -235,6 +237,7 @@ cudaError_t launch_residual_cf(const MeshGeom &g, int prec, const FemCoef<float>
 // (the coarse one also writes the first state row of every GRU tile of the instances to hrow)
 cudaError_t launch_coarse_pad_batch(const StepInst *in, int n, int *hrow, cudaStream_t st);
 cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st);
+bool residual_step_batch_small(const StepInst *in, int n, bool skip_fast);   // as residual_step_small
 cudaError_t launch_residual_cf_batch(const StepInst *in, int n, cudaStream_t st);
 // (chained: right after the network; the two passes after it always are)
 cudaError_t launch_scatter_avg_batch(const StepInst *in, int n, cudaStream_t st, bool chained);

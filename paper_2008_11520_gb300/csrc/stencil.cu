@@ -2419,6 +2419,8 @@ cudaError_t launch_residual_step(const MeshGeom &g, int prec, const FemCoef<doub
     return run_residual_step_r<float, __nv_bfloat16>(g, f32, xcp, up, bf, X, st, skip_fast, chained);
 }
 
+bool residual_step_small(const MeshGeom &g, int prec) { return use_small(g, g.n_slow_tiles, prec == DNNMG_F64); }
+
 template <typename T, int PTY_>
 cudaError_t run_scatter_p(const MeshGeom &g, const T *d, const T *xf, const double *xc, const T *xcp, double w, T *vc,
                           cudaStream_t st, bool chained) {
@@ -2587,11 +2589,15 @@ template <typename D, int R> static cudaError_t residual_batch(const StepInst *i
     return cudaGetLastError();
 }
 
-// skip_fast: only the boundary tiles (launch_residual_cf_batch does the others)
-cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st) {
+bool residual_step_batch_small(const StepInst *in, int n, bool skip_fast) {
     long long tiles = 0;
     for (int i = 0; i < n; ++i) tiles += skip_fast ? in[i].mesh->g.n_slow_tiles : tiles_of(in[i].mesh->g);
-    const bool small = use_small(in[0].mesh->g, tiles, false);
+    return use_small(in[0].mesh->g, tiles, false);
+}
+
+// skip_fast: only the boundary tiles (launch_residual_cf_batch does the others)
+cudaError_t launch_residual_step_batch(const StepInst *in, int n, bool skip_fast, cudaStream_t st) {
+    const bool small = residual_step_batch_small(in, n, skip_fast);
     switch (in[0].mesh->g.r) {
         case 2: return small ? residual_batch<SmallTile, 2>(in, n, !skip_fast, st) : residual_batch<BigTile, 2>(in, n, !skip_fast, st);
         case 4: return small ? residual_batch<SmallTile, 4>(in, n, !skip_fast, st) : residual_batch<BigTile, 4>(in, n, !skip_fast, st);
