@@ -11,11 +11,11 @@
 // and 1.3e-7 for K = 128, against 1.5e-7 and 2.1e-7 for FP32 FMA in sequence
 // (the leading product first: 7e-7 and 1.4e-6); sums of 4096 terms drained
 // every 128: 1.6e-7 against 1.1e-6.  Each accumulation at a sum's full
-// magnitude, one per 16 terms, drops up to an ulp, all of one sign; outputs and
-// gradients of a window (65 536 rows, T = 10, H = 64) are off by 1.5e-7 and
-// 2.3e-7, with FP32 FMAs by 2.1e-7 and 1.2e-6.  Putting back the average loss
-// would make that 1.2e-7 and 1.8e-7, but also change sums that lost nothing:
-// a sum of one product is exact wherever FP32's is.
+// magnitude, one per 16 terms of the leading product, drops up to an ulp, all of
+// one sign; the average is put back (whole), so that a chain of products does not
+// gather it.  Outputs and gradients of a window (65 536 rows, T = 10, H = 64) are
+// off by 0.8e-7 and at most 1.2e-7, without that by 1.2e-7 and 2.0e-7, with FP32
+// FMAs by 1.7e-7 and 2.2e-7 (762 rows: 0.8e-7, 1.7e-7, 1.3e-6).
 //
 // Six tcgen05 products of BF16 are 316 TFLOP/s of FP32 at the measured BF16
 // rate; the CUDA cores' FMAs give 74.  With the fused window (see gru_win.cu,
@@ -68,6 +68,27 @@ __device__ __forceinline__ void mma3_mn(uint32_t d, uint32_t a, uint32_t astep, 
             acc = 1;
         }
     }
+}
+
+// Each accumulation at a product's full magnitude (one per 16 terms of its
+// leading part) drops on average 2.1e-8 of the sum (measured on N(0, 1) operands:
+// 0.85e-7 for K = 64, 1.7e-7 for K = 128, all of one sign).  That much is put
+// back.  steps: those that hold data, which are the only ones that can drop
+// anything: of one, it is less than half an ulp and a representable sum stays.
+__device__ __forceinline__ float whole(float v, int steps) { return fmaf(v, 2.1e-8f * (float)steps, v); }
+// The steps of a row that hold data: each of its four threads (part) leaves a mask
+// of the 16-column steps in which it has a value other than zero, in the row's
+// word of an operand's 512 bytes; to be read after a hand-over.
+constexpr int STEPS = TM * 4;
+__device__ __forceinline__ void put_steps(uint8_t *f, int row, int part, unsigned mask) { f[4 * row + part] = (uint8_t)mask; }
+__device__ __forceinline__ int get_steps(const uint8_t *f, int row) {
+    unsigned w = *reinterpret_cast<const unsigned *>(f + 4 * row);
+    w |= w >> 16;
+    return __popc((w | w >> 8) & 15u);
+}
+// of H / 4 consecutive columns a thread; bits: all its values' bits (of zeros, no more than the sign)
+template <int H> __device__ __forceinline__ unsigned step_mask(unsigned bits, int part) {
+    return bits << 1 ? 1u << (H == 64 ? part : part >> 1) : 0u;
 }
 
 // Whether every value seen is finite (0 x is not 0 for one that is not)
@@ -271,7 +292,7 @@ template <int H> __device__ __noinline__ void plain_bwd(const WinArgs &g, int ti
 // W_x: X W_x^T comes from memory (k_win32_x).
 template <int H, int XC> struct Fwd32Layout {
     static constexpr int WS = 3 * H * 128, FS = 64 * 128;   // bytes of one part
-    static constexpr int WX = 0, U = WX + (XC == 1 ? 3 * WS : 0), F = U + 3 * WS, A = F + 3 * FS, BARS = A + 3 * IMG, BYTES = BARS + 64 + 1024;
+    static constexpr int WX = 0, U = WX + (XC == 1 ? 3 * WS : 0), F = U + 3 * WS, A = F + 3 * FS, SH = A + 3 * IMG, SR = SH + STEPS, BARS = SR + STEPS, BYTES = BARS + 64 + 1024;   // SH, SR: steps of h, r h
     static constexpr int COLS = H == 64 ? 512 : 256;
 };
 
@@ -336,7 +357,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_x(const __grid_constant__ W
             keep(a);
             keep(b);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) a[j] += b[j];
+            for (int j = 0; j < 8; ++j) a[j] = whole(a[j], 4) + whole(b[j], g.kx2);
             st4(o + blk(c0 + i, row), a);
             st4(o + blk(c0 + i + 4, row), a + 4);
         }
@@ -362,6 +383,9 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
     const int q = warp & 3, part = warp >> 2, row = q * 32 + lane, c0 = part * NC;
     const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
     const size_t tblk = (size_t)TM * H;
+    uint8_t *fh = base + L::SH, *fr = base + L::SR;
+    const int kx = (min(g.n_in, 64) + 15) / 16;
+    int kh = 0;   // steps of the state that h U^T and the outputs in tensor memory come from
     uint32_t ph = 0;
     bool ok = true;
     XTile<W32_TH> xt;
@@ -375,6 +399,13 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
             if (g.h0 && valid) ld4(g.h0 + (size_t)gp * H + c0 + i, hv + i);
             st4(g.hb + (size_t)tile * tblk + blk(c0 + i, row), hv + i);
         }
+        auto put_h = [&]() {
+            unsigned any = 0;
+#pragma unroll
+            for (int i = 0; i < NC; ++i) any |= __float_as_uint(hv[i]);
+            put_steps(fh, row, part, step_mask<H>(any, part));
+        };
+        put_h();
         if (XC == 1) xt.load(g, 0, p0);
 #pragma unroll
         for (int i = 0; i < NC; i += 8) put8_3(sA, IMG, row, c0 + i, hv + i);
@@ -393,7 +424,10 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
                 keep(v);
                 if (!valid) continue;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) fin.see(v[j]);
+                for (int j = 0; j < 8; ++j) {
+                    v[j] = whole(v[j], kh);
+                    fin.see(v[j]);
+                }
                 if (fin.failed()) cta.mark();
 #pragma unroll
                 for (int j = 0; j < 8; j += 2) {
@@ -417,6 +451,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
             }
             ok = cta.wait(0, ph);
             ph ^= 1;
+            kh = get_steps(fh, row);
             if (XC == 1) {
                 store_x3(g, xt, sA);
                 if (!(ok = cta.hand_over(ok))) break;
@@ -428,6 +463,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
                 ok = cta.wait(0, ph);
                 ph ^= 1;
             }
+            unsigned any = 0;
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8], rr[8];
@@ -438,13 +474,15 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
                 keep(b);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    rr[j] = sigm((XC == 1 ? a[j] : gr[(i + j) % (XC == 2 ? NC : 1)]) + b[j]);
+                    rr[j] = sigm((XC == 1 ? whole(a[j], kx) : gr[(i + j) % (XC == 2 ? NC : 1)]) + whole(b[j], kh));
                     a[j] = rr[j] * hv[i + j];
+                    any |= __float_as_uint(a[j]);
                 }
                 st4(g.r + sb + blk(c0 + i, row), rr);
                 st4(g.r + sb + blk(c0 + i + 4, row), rr + 4);
                 put8_3(sA, IMG, row, c0 + i, a);
             }
+            put_steps(fr, row, part, step_mask<H>(any, part));
             if (!(ok = cta.hand_over(ok))) break;
             if (tid == 0) {
                 mma3_k(cta.tmem + 5 * H, uA, IMG, u + L::U + 2 * H * 128, L::WS, H, H / 16);
@@ -462,6 +500,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
             }
             ok = cta.wait(0, ph);
             ph ^= 1;
+            const int kr = get_steps(fr, row);
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8], zz[8], cc[8];
@@ -482,8 +521,8 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = (i + j) % (XC == 2 ? NC : 1);
-                    const float z = sigm((XC == 1 ? a[j] : gz[k]) + b[j]),
-                                c = tanhf((XC == 1 ? zz[j] : gc[k]) + cc[j]);
+                    const float z = sigm((XC == 1 ? whole(a[j], kx) : gz[k]) + whole(b[j], kh)),
+                                c = tanhf((XC == 1 ? whole(zz[j], kx) : gc[k]) + whole(cc[j], kr));
                     zz[j] = z;
                     cc[j] = c;
                     hv[i + j] = z * hv[i + j] + (1.0f - z) * c;
@@ -496,6 +535,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
                 st4(g.c + sb + blk(c0 + i + 4, row), cc + 4);
                 put8_3(sA, IMG, row, c0 + i, hv + i);
             }
+            put_h();
             if (s + 1 < g.T) {
                 float *hb = g.hb + ((size_t)(s + 1) * g.ntiles + tile) * tblk;
 #pragma unroll
@@ -514,6 +554,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
         if (ok) {
             ok = cta.wait(0, ph);
             ph ^= 1;
+            kh = get_steps(fh, row);
             if (ok) outputs(g.T - 1);
         }
         ok = cta.hand_over(ok);   // (the same answer in every thread)
@@ -534,7 +575,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_fwd(const __grid_constant__
 template <int H> struct Bwd32Layout {
     static constexpr int WS = H * 128;
     static constexpr int WF = 0, UC = WF + 3 * WS, UZ = UC + 3 * WS, UR = UZ + 3 * WS, B0 = UR + 3 * WS, B1 = B0 + 3 * IMG,
-                         BARS = B1 + 3 * IMG, BYTES = BARS + 64 + 1024;
+                         SD = B1 + 3 * IMG, BARS = SD + STEPS, BYTES = BARS + 64 + 1024;   // SD: steps of dD
     static constexpr int COLS = 256;
 };
 
@@ -557,6 +598,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
     const uint32_t tl = cta.tmem + ((uint32_t)(q * 32) << 16);
     const size_t tblk = (size_t)TM * H;
     const int kfc = g.nfc / 16;
+    uint8_t *fd = base + L::SD;   // (dA has values in all its steps wherever it has any)
     uint32_t ph = 0;
     bool ok = true;
     // dD of a step: each thread up to 16 columns of its row (blocks of 4 dealt to the row's threads)
@@ -572,11 +614,15 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
         }
     };
     auto put_dd = [&](uint8_t *img) {
+        unsigned mask = 0;   // (block i lies in step i)
 #pragma unroll
         for (int i = 0; i < DDN; ++i) {
             const int c = 4 * (part + 4 * i);
             if (c < g.nfc) put4_3(img, IMG, row, c, dd[i]);
+            const unsigned any = __float_as_uint(dd[i][0]) | __float_as_uint(dd[i][1]) | __float_as_uint(dd[i][2]) | __float_as_uint(dd[i][3]);
+            mask |= any << 1 ? 1u << i : 0u;
         }
+        put_steps(fd, row, part, mask);
     };
     for (int tile = blockIdx.x; ok && tile < g.ntiles; tile += gridDim.x) {
         const int p0 = tile * TM, gp = p0 + row;
@@ -606,6 +652,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
             ok = cta.wait(0, ph);
             ph ^= 1;
             float dh[NC];
+            const int kd = get_steps(fd, row);
 #pragma unroll
             for (int i = 0; i < NC; i += 8) {
                 float a[8], b[8], c[8], az[8], ac[8];
@@ -619,8 +666,8 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
-                    const float carry = s == g.T - 1 ? 0.f : b[j] + c[j] + cpart[k];
-                    dh[k] = a[j] + carry;
+                    const float carry = s == g.T - 1 ? 0.f : whole(b[j] + c[j], H / 16) + cpart[k];
+                    dh[k] = whole(a[j], kd) + carry;
                     const float dc = dh[k] * (1.0f - zv[k]), dz = dh[k] * (hp[k] - cv[k]);
                     az[j] = dz * zv[k] * (1.0f - zv[k]);
                     ac[j] = dc * (1.0f - cv[k] * cv[k]);
@@ -651,6 +698,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = i + j;
+                    a[j] = whole(a[j], H / 16);
                     cpart[k] = dh[k] * zv[k] + a[j] * rv[k];
                     fin.see(cpart[k]);
                     a[j] = a[j] * hp[k] * rv[k] * (1.0f - rv[k]);
@@ -686,7 +734,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_bwd(const __grid_constant__
                     keep(c);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        b[j] = b[j] + c[j] + cpart[i + j];
+                        b[j] = whole(b[j] + c[j], H / 16) + cpart[i + j];
                         fin.see(b[j]);
                     }
                     if (fin.failed()) cta.mark();
@@ -794,21 +842,26 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const __grid_constant_
     const long long i0 = n * blockIdx.x / gridDim.x, i1 = n * (blockIdx.x + 1) / gridDim.x;
     uint32_t ph = 0;
     bool ok = true;
-    auto drain = [&]() {   // the block's products into the registers
+    const long long full = (long long)g.T * (g.P / GR);   // blocks before have all their rows, those from full + T on none
+    auto drain = [&](long long it) {   // the block's products into the registers
         ok = cta.wait(0, ph);
         ph ^= 1;
+        auto add = [&](int steps) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const int c = 8 * (part + 4 * b);
-            if (c < ncol) {
-                float v[8];
-                tmem_ld8(tl + c, v);
-                tmem_wait();
-                keep(v);
+            for (int b = 0; b < NB; ++b) {
+                const int c = 8 * (part + 4 * b);
+                if (c < ncol) {
+                    float v[8];
+                    tmem_ld8(tl + c, v);
+                    tmem_wait();
+                    keep(v);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[b][j] += v[j];
+                    for (int j = 0; j < 8; ++j) acc[b][j] += whole(v[j], steps);
+                }
             }
-        }
+        };
+        if (it < full) add(GR / 16);
+        else add(it < full + g.T ? (g.P % GR + 15) / 16 : 0);
     };
     bool summed = false;
     auto flush = [&]() {   // the registers' sums into tensor memory
@@ -879,7 +932,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const __grid_constant_
             if (!X2 && xc < g.n_out) prefetch_l2(dsrc);
         }
         if (it > i0) {
-            drain();   // the images are free again
+            drain(it - 1);   // the images are free again
             if ((it - i0) % G32_RUN == 0) flush();
         }
         float az[8], ar[8];
@@ -925,7 +978,7 @@ __global__ void __launch_bounds__(W32_TH, 1) k_win32_grad(const __grid_constant_
         }
     }
     if (ok && i1 > i0) {
-        drain();
+        drain(i1 - 1);
         flush();
     }
     if (ok && summed && !*cta.abort_flag) {
