@@ -445,15 +445,18 @@ void dnnmg_pool_destroy(dnnmg_pool_t pool);
  * Forward and backward of Eq. gru followed by the output layer (Sec. 6.2),
  * unrolled over a window of T steps of P patch rows, for truncated
  * backpropagation through time; the l2 loss of Sec. 6.3 and its gradient;
- * Adam with the Tikhonov term of Sec. 6.3.  FP32 products on the CUDA cores,
- * or BF16 products on the tensor cores (dnnmg_trainer_set_precision);
- * weight-gradient sums are split over the T P rows in a fixed order, so
- * results repeat bit for bit.  All arrays are caller-owned device memory:
+ * Adam with the Tikhonov term of Sec. 6.3.  FP32 or BF16 products
+ * (dnnmg_trainer_set_precision); weight-gradient sums are split over the T P
+ * rows in a fixed order, so results repeat bit for bit.  Networks of n_in <=
+ * 128, H = 32 or 64 and n_out <= 64 take the whole window in a few persistent
+ * tensor-core kernels, the others one kernel per product.  All arrays are
+ * caller-owned device memory:
  *   X [T][P][ldx] (columns n_in..ldx-1 ignored), h0 / dh0 [P][H],
  *   Wx / gWx [3H][n_in], Uh / gUh [3H][H] (gates z, r, h), Wfc / gWfc [n_out][H],
  *   D / dD [T][P][n_out].
- * A trainer owns the activations of one window (about T P (12 H) floats) and
- * serves one forward/backward pair at a time.
+ * A trainer owns the activations of one window (about T P (12 H) floats; the
+ * window kernels T P (7 H), with BF16 products T P (4 H)) and serves one
+ * forward/backward pair at a time.
  */
 typedef struct dnnmg_trainer_s *dnnmg_trainer_t;
 int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnmg_trainer_t *out);
@@ -463,18 +466,29 @@ int dnnmg_trainer_destroy(dnnmg_trainer_t trainer);
  * Arithmetic of the trainer's matrix products (the pointwise steps, the
  * reductions and every array stay FP32; the training workload of Sec. 6.3
  * asks for BF16 products with FP32 master weights):
- *   DNNMG_F32      FP32 products on the CUDA cores (the default);
+ *   DNNMG_F32      FP32 products (the default).  In the window kernels each
+ *                  operand is split into three BF16 parts and six products
+ *                  of the parts are accumulated in FP32 on the tensor cores,
+ *                  with FP32's error or less; a tile (128 rows) or gradient
+ *                  block with an infinity, a NaN or an operand beyond the
+ *                  BF16 range is computed again with FP32 FMAs and gives what
+ *                  these give.  Otherwise FP32 FMAs on the CUDA cores.
  *   DNNMG_BF16NET  BF16 operands, FP32 accumulation, on the tensor cores
- *                  (tcgen05): each product's operands are rounded to BF16
- *                  once per tensor (transposed where the product needs it)
- *                  into scratch the trainer allocates here (about
- *                  T P (2 n_in + 6 H + 2 n_out) BF16 values).
+ *                  (tcgen05).  Outside the window kernels each product's
+ *                  operands are rounded to BF16 once per tensor (transposed
+ *                  where the product needs it) into scratch the trainer
+ *                  allocates here (about T P (2 n_in + 6 H + 2 n_out) BF16
+ *                  values); in them the gate gradients' FP32 scratch
+ *                  (T P (3 H) floats) is given back, and allocated again on
+ *                  the way back to DNNMG_F32.
  * DNNMG_EINVAL for another value, DNNMG_ENOMEM if the scratch cannot be had.
  */
 int dnnmg_trainer_set_precision(dnnmg_trainer_t trainer, int precision);
 /*
  * Device status bits of the trainer's tensor-core products (DNNMG_DEVERR_*,
- * e.g. a bounded wait that timed out); reset clears them.  Synchronous.
+ * e.g. a bounded wait that timed out), which FP32 window kernels have too;
+ * reset clears them.  Synchronous.  Once a bit is set, outputs and gradients
+ * of that window are incomplete: read it before gradients are used for good.
  */
 int dnnmg_trainer_status(dnnmg_trainer_t trainer, int *status, int reset);
 /*

@@ -147,7 +147,7 @@ k_gru(int n_in, int ldx, int H, int n_out, const TW *__restrict__ X, const TW *_
 // after the other from zero, as k_gru's does: the same bits.
 // FP32: 8 patches and 4 columns a thread, operations on patch pairs in packed
 // form.  16 336 patches, 99 inputs, H = 64, 50 outputs: k_gru 123 us,
-// this 58 us; bound by latency (the weights' way from L2, staging).  FP64 runs at two FMA a clock and SM, so
+// this 57 us; bound by latency (the weights' way from L2, staging).  FP64 runs at two FMA a clock and SM, so
 // there the tile is small (2 columns of 1 patch) and few patches are spread
 // over the chip: 254 patches, 51 inputs, H = 32: k_gru 83 us (32 CTAs), this
 // 38 us (both under ncu, cold caches).

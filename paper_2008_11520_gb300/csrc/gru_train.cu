@@ -1,9 +1,12 @@
 // Training the patch network (Eq. gru + output layer, Sec. 6.2 and 6.3):
 // the GRU unrolled over a window of T steps, and its gradient by truncated
-// backpropagation through time, in FP32 on the CUDA cores.
+// backpropagation through time.  Networks that win_supported() names run the
+// fused window kernels (gru_win.cu: BF16 products, gru_win32.cu: FP32); this
+// file has the trainer, the loss and Adam, and the window of the others, with
+// FP32 products on the CUDA cores or BF16 ones on the tensor cores (gemm_tc.cu).
 //
-// Every product of the network is a matrix product over the patch rows, so a
-// window is a short sequence of GEMMs and fused pointwise kernels:
+// There every product of the network is a matrix product over the patch rows,
+// so a window is a short sequence of GEMMs and fused pointwise kernels:
 //   forward   GX = X W_x^T for all steps at once; per step t
 //             GH = h_{t-1} [U_z; U_r]^T, gates (z, r, r*h), AH = (r*h) U_h^T,
 //             candidate and new state; then D = H W_fc^T for all steps.

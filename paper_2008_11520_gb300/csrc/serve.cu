@@ -15,7 +15,9 @@
 //
 // Launching the passes instance by instance on eight streams was bound by the
 // host (six launches and their tensor maps an instance): 20 instances of
-// 64 x 16 .. 512 x 128 coarse cells, K = 1, took 400 us a step; now 240 us.
+// 64 x 16 .. 512 x 128 coarse cells, K = 1, took 390 us a step; now 235 us.
+// Eight of 256 x 64 .. 512 x 128, K = 2: back to back 318 and 326 us, waited for 387
+// and 360.
 #include <algorithm>
 #include <cstring>
 #include <map>

@@ -32,8 +32,8 @@ template <int X, int Y, int TH> struct TileDim {
 using BigTile = TileDim<TXC, TYC, 256>;
 // Few tiles: a 32 x 16 tile is 16 us of latency in FP32 and 80 us of work in
 // FP64 (two FMA a clock and SM) on one SM while the rest of the chip idles.
-// 64 x 16 cells in FP64 (2 tiles): residual and features 80 -> 26 us,
-// right-hand side 29 -> 9 us; 256 x 64 in FP32 (32 tiles): 24.5 -> 9 and
+// 64 x 16 cells in FP64 (2 tiles): residual and features 80 -> 22 us,
+// right-hand side 29 -> 7 us; 256 x 64 in FP32 (32 tiles): 24.5 -> 9 and
 // 5.7 -> 4.6 us; bound by the chain of staging, cell and node passes.
 using SmallTile = TileDim<8, 8, 128>;
 // Whether a launch over n tiles of 32 x 16 cells takes 8 x 8 ones instead

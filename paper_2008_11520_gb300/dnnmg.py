@@ -654,9 +654,12 @@ def gemm_bf16_nt(A, B, C, accumulate=False, status=None, stream=None):
 class Trainer:
     """Owning wrapper of a dnnmg_trainer_t: the activations of one window of
     T steps of P patch rows (FP32), for dnnmg_gru_seq_forward / _backward.
-    precision "f32" multiplies in FP32 on the CUDA cores, "bf16" rounds each
-    product's operands to BF16 and multiplies on the tensor cores (FP32
-    accumulation; the FP32 master weights are the caller's)."""
+    precision "f32" multiplies in FP32 (n_in <= 128, H = 32 or 64, n_out <= 64:
+    on the tensor cores, in three BF16 parts per operand; other networks on the
+    CUDA cores), "bf16" rounds each product's operands to BF16 and multiplies
+    on the tensor cores (FP32 accumulation; the FP32 master weights are the
+    caller's).  status() tells whether a bounded wait of the tensor-core
+    kernels ran out: outputs and gradients are incomplete then."""
 
     def __init__(self, n_in, ldx, H, n_out, T, P, precision="f32"):
         h = ctypes.c_void_p()

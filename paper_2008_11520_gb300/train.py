@@ -109,8 +109,8 @@ class PatchNetTrainer:
                  device="cuda", precision="f32", head=False):
         """Initial weights N(0, std^2); the output layer N(0, out_std^2) if given
         (0: zero, so that the untrained net predicts d = 0).  precision: "f32"
-        products on the CUDA cores, or "bf16" products on the tensor cores
-        (FP32 master weights and Adam state either way).  head: train the
+        or "bf16" products (dnnmg.Trainer; FP32 master weights and Adam state
+        either way).  head: train the
         convolutional head of Sec. 6.2 too (``head_init``; its parameters are
         the fourth entry of ``params``)."""
         Wx, Uh, Wfc = synth.net_weights(n_in, H, n_out, seed=seed, std=std)
