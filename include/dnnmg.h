@@ -460,6 +460,9 @@ void dnnmg_pool_destroy(dnnmg_pool_t pool);
  */
 typedef struct dnnmg_trainer_s *dnnmg_trainer_t;
 int dnnmg_trainer_create(int n_in, int ldx, int H, int n_out, int T, int P, dnnmg_trainer_t *out);
+/* The same in the given precision (dnnmg_trainer_set_precision), without FP32 scratch that BF16 products do not use. */
+int dnnmg_trainer_create_precision(int n_in, int ldx, int H, int n_out, int T, int P, int precision,
+                                   dnnmg_trainer_t *out);
 /* Wait for the device, then free the trainer (NULL is allowed). */
 int dnnmg_trainer_destroy(dnnmg_trainer_t trainer);
 /*

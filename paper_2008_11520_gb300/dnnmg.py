@@ -110,6 +110,7 @@ def _load():
         "dnnmg_pool_free": [P, I],
         "dnnmg_pool_stats": [P, ctypes.POINTER(I), ctypes.POINTER(I)],
         "dnnmg_trainer_create": [I, I, I, I, I, I, ctypes.POINTER(P)],
+        "dnnmg_trainer_create_precision": [I, I, I, I, I, I, I, ctypes.POINTER(P)],
         "dnnmg_trainer_destroy": [P],
         "dnnmg_trainer_set_precision": [P, I],
         "dnnmg_trainer_status": [P, ctypes.POINTER(I), I],
@@ -663,12 +664,10 @@ class Trainer:
 
     def __init__(self, n_in, ldx, H, n_out, T, P, precision="f32"):
         h = ctypes.c_void_p()
-        _check(_lib.dnnmg_trainer_create(n_in, ldx, H, n_out, T, P, ctypes.byref(h)))
+        _check(_lib.dnnmg_trainer_create_precision(n_in, ldx, H, n_out, T, P, PRECISIONS[precision], ctypes.byref(h)))
         self.handle = h
         self.n_in, self.ldx, self.H, self.n_out, self.T, self.P = n_in, ldx, H, n_out, T, P
         self.precision = precision
-        if precision != "f32":
-            _check(_lib.dnnmg_trainer_set_precision(h, PRECISIONS[precision]))
 
     def status(self, reset=False):
         """Device status bits (DNNMG_DEVERR_*) of the tensor-core products."""
